@@ -84,15 +84,18 @@ def draw(rng):
     cams = _log(rng, 1 if kind == "render" else (2, 8, 16, 24)[degree], 200)
     width = rng.randint(100, 1600)
     height = max(64, int(width * rng.uniform(0.55, 1.0)))
-    # between the largest listed cases in pairs, target bytes and per-camera sums
-    while n * cams > 3e8 or width * height * cams * channels > 3e9 or (degree and n * cams * (1 + channels) > 1.2e9):
+    sets = rng.choice([2, 3, 4]) if kind == "sets" else 1
+    # below the largest listed cases in pairs, walked pixels, target bytes and per-camera sums
+    walks = {"train": 3, "refine": 2}.get(kind, sets)
+    channels_all = channels * sets
+    while (n * cams * walks > 4e8 or width * height * cams * walks > 3e8 or width * height * cams * channels_all > 3e9
+           or (degree and n * cams * (1 + channels_all) > 1.2e9)):
         if cams > 36:
             cams = cams * 2 // 3
-        elif width * height * cams * channels > 3e9:
+        elif width * height * cams * max(walks, 0.1 * channels_all) > 3e8:
             width, height = width * 4 // 5, height * 4 // 5
         else:
             n = max(1000, n // 2)
-    sets = rng.choice([2, 3, 4]) if kind == "sets" else 1
     precision = "plain" if rng.random() < 0.15 else "mixed"
     return _case(None, kind, n, cams, width, height, degree, channels, dtype, fov, content, precision, sets)
 
