@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "icgs_device.cuh"
+#include "groupwalk.cuh"
 #include "icgs_internal.h"
 #include "walk.cuh"
 
@@ -182,59 +183,52 @@ __global__ void __launch_bounds__(kThreads, KC <= 8 ? 5 : 4) k_blend_accumulate(
   if (k0 == 0) add_pair_count(npairs, status);
 }
 
-// The same accumulation for up to 3 channels with two pixels per thread: CTAs of 128 threads, each
-// warp covering an 8x8 block, 10 CTAs (48 registers a thread) per SM. A hit's fixed costs (the ballot loop, the shared loads, the vote, the
-// warp reduction and the shared atomic) are shared by 64 pixels instead of 32: each thread adds its
-// two pixels' contributions before the reduction. The pixels of a thread are walked independently
-// (own transmittance, own stop), in the same depth order, through the same blend_step().
-constexpr int kThreads2 = kThreads / 2;
-
+// The same accumulation for up to 7 channels by 8-lane groups (groupwalk.cuh): 128 threads, two pixels
+// each, a hit list per 4x4 block. A group reduces its own hits, kHits at a time (two for up to 3
+// channels), over its 8 lanes: NT = kHits NP values leave one warp-wide butterfly of 7 shuffles with
+// one sum per lane, stored (no atomics: a group takes a Gaussian once per batch) in the group's
+// row of s_part; after the batch two threads per Gaussian add the rows of the groups that list it, and
+// one atomic group per (Gaussian, tile) lands in the accumulator.
 template <int KC>
-__global__ void __launch_bounds__(kThreads2, 10) k_blend_accumulate2(
-    const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
-    const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
-    const void* __restrict__ targets, int dtype, int K, int k0, int cam0, const float* __restrict__ sub_img,
-    float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
-  static_assert(KC <= 3, "two pixels per thread: up to 3 channels");
-  constexpr int NV = KC + 1;
-  constexpr int NP = NextPow2<NV>::value;
-  constexpr int NP2 = 2 * NP;                     // two hits per reduction
-  constexpr int SHIFT2 = 5 - Log2<NP2>::value;
-  __shared__ float4 s_geo[kBatch], s_aux[kBatch];
-  __shared__ float2 s_half[kBatch];
-  __shared__ uint32_t s_id[kBatch];
-  __shared__ float s_acc[kBatch][NV];
-  const TileCtx c = tile_ctx<2>(tile_off, capacity, tiles, tiles_x, width, height);
-  const unsigned long long* list = tile_list(entries, c.b);
-  const int lane = threadIdx.x & 31;
-  const bool inside1 = c.inside && c.py + 4 < height;
-  const float pyf1 = c.pyf + 4.0f;
-  float tv0[KC], tv1[KC];
+struct GroupAcc {
+  static_assert(KC >= 1 && KC <= 7, "1..7 channels");
+  static constexpr int NV = KC + 1;                 // V and S_0..S_{KC-1}
+  static constexpr int NP = NextPow2<NV>::value;    // 2, 4 or 8: floats of a partial row
+  static constexpr int kHits = NP <= 4 ? 2 : 1;
+  static constexpr int NT = NP * kHits;             // values of a group reduction (4 or 8)
+  static constexpr int SHIFT = 3 - Log2<NT>::value; // lane l of a group returns value l >> SHIFT
+  float part[kGroups][kBatch][NP];
+};
+
+// Group sums of NT values held in lane-permuted slots (warp_permuted_reduce over 8 lanes).
+template <int NT>
+__device__ __forceinline__ float group_permuted_reduce(float (&v)[NT]) {
+  constexpr int P = Log2<NT>::value;
 #pragma unroll
-  for (int k = 0; k < KC; ++k) tv0[k] = tv1[k] = 0.0f;
-  const int64_t row = (int64_t)width * K;
-  if (c.inside) {
-    const int64_t base = (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K + k0;
-    const int64_t ib = (((int64_t)c.j * height + c.py) * width + c.px) * K + k0;
+  for (int lvl = 0; lvl < P; ++lvl) {
+    const int half = NT >> (lvl + 1);
 #pragma unroll
-    for (int k = 0; k < KC; ++k) {
-      if (k0 + k < K) {
-        tv0[k] = load_target(targets, base + k, dtype);
-        if (sub_img) tv0[k] -= sub_img[ib + k];  // refinement: residual targets t - img
-        if (inside1) {
-          tv1[k] = load_target(targets, base + 4 * row + k, dtype);
-          if (sub_img) tv1[k] -= sub_img[ib + 4 * row + k];
-        }
-      }
-    }
-    check_finite(tv0, status);
-    check_finite(tv1, status);
+    for (int i = 0; i < half; ++i) v[i] += __shfl_xor_sync(kFull, v[i + half], 4 >> lvl);
   }
-  // Value h NP + k of a hit pair is hit h's weights times u[k], u = (1, t_0, .., t_{KC-1}, 0, ..),
-  // summed over the thread's two pixels. This lane keeps it in slot (h NP + k) ^ m
-  // (warp_permuted_reduce), so u is permuted here once, by one conditional swap per bit of mk, and
-  // the pair's two hits trade places when mh is set.
-  const int m = lane >> SHIFT2;
+  float r = v[0];
+#pragma unroll
+  for (int off = 4 >> P; off > 0; off >>= 1) r += __shfl_xor_sync(kFull, r, off);
+  return r;
+}
+
+// The walk of one tile for target values tv0, tv1 of the thread's two pixels.
+template <int KC>
+__device__ __forceinline__ void group_accumulate(GroupBatch& s, GroupAcc<KC>& sa, const GroupCtx& c,
+                                                 const unsigned long long* list, const ProjRec* __restrict__ rec_cam,
+                                                 int64_t n, const float (&tv0)[KC], const float (&tv1)[KC],
+                                                 float* __restrict__ acc_cam, int RS, int K, int k0, DevStatus* status) {
+  using S = GroupAcc<KC>;
+  constexpr int NV = S::NV, NP = S::NP, NT = S::NT;
+  const int lane = threadIdx.x & 31;
+  // Value h NP + k of a step is hit h's weights times u[k], u = (1, t_0, .., t_{KC-1}, 0, ..), summed
+  // over the thread's two pixels. This lane keeps it in slot (h NP + k) ^ m, so u is permuted here
+  // once, by one conditional swap per bit of mk, and two hits trade places when mh is set.
+  const int m = (lane & 7) >> S::SHIFT;
   const bool mh = (m & NP) != 0;
   const int mk = m & (NP - 1);
   float u0[NP], u1[NP];
@@ -257,72 +251,154 @@ __global__ void __launch_bounds__(kThreads2, 10) k_blend_accumulate2(
       u1[k | bit] = sw ? x1 : y1;
     }
   }
-  for (int k = threadIdx.x; k < kBatch * NV; k += kThreads2) (&s_acc[0][0])[k] = 0.0f;
-  const ProjRec* rec_cam = rec + (int64_t)c.j * n;
-  float* acc_cam = acc + (int64_t)c.j * acc_cam_stride;
-  float T0 = 1.0f, T1 = 1.0f;
-  bool done0 = !c.inside, done1 = !inside1;
+  f2 U0[NP / 2], U1[NP / 2];
+#pragma unroll
+  for (int k = 0; k < NP / 2; ++k) {
+    U0[k] = pack2(u0[2 * k], u0[2 * k + 1]);
+    U1[k] = pack2(u1[2 * k], u1[2 * k + 1]);
+  }
+  const bool writer = ((lane & 7) & ((1 << S::SHIFT) - 1)) == 0 && mk < NV;
+  char* const my_part = reinterpret_cast<char*>(&sa.part[c.group][0][mk]);
+  const uint16_t* const my_list = s.list[c.group];
+  float2 T = make_float2(c.in0 ? 1.0f : 0.0f, c.in1 ? 1.0f : 0.0f);
   uint32_t npairs = 0;
-  for (uint32_t start = 0; start < c.len; start += kBatch) {
+  int buf = 0;
+  group_stage(list, c.b, (int)min((uint32_t)kBatch, c.len), rec_cam, n, c.ox, c.oy, s, buf);
+  __syncthreads();
+  // two barriers a batch: the next batch is staged between them, when the walk of this one has ended
+  for (uint32_t start = 0; start < c.len; start += kBatch, buf ^= 1) {
     const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    __syncthreads();
-    load_batch(list, start, nb, rec_cam, n, c.ox, c.oy, s_geo, s_aux, s_half, s_id);
-    __syncthreads();
-    if (!__all_sync(kFull, done0 && done1)) {
+    const int steps = group_lists(s, c, nb, group_alive(T.x > 0.0f || T.y > 0.0f));
+    for (int i = 0; i < steps; i += S::kHits) {
+      if constexpr (S::kHits == 2) {
+        const uint32_t pair = *reinterpret_cast<const uint32_t*>(my_list + i);
+        const uint32_t o1 = pair & 0xFFFFu, o2 = pair >> 16;
+        const GroupAlpha a1 = group_alpha(s, o1, c), a2 = group_alpha(s, o2, c);  // independent of T
+        const float2 w1 = group_take(a1.alpha, T, npairs), w2 = group_take(a2.alpha, T, npairs);
+        const float p0 = mh ? w2.x : w1.x, p1 = mh ? w2.y : w1.y;
+        const float q0 = mh ? w1.x : w2.x, q1 = mh ? w1.y : w2.y;
+        float v[NT];
 #pragma unroll
-      for (int half = 0; half < kBatch / 32; ++half) {
-        uint32_t bits = warp_hit_bits<true>(s_geo, s_aux, s_half, half * 32, nb, c);
-        while (bits) {
-          const int g1 = half * 32 + __ffs(bits) - 1;
-          bits &= bits - 1;
-          const int g2 = bits ? half * 32 + __ffs(bits) - 1 : -1;
-          bits &= bits - 1;
-          float w20 = 0.0f, w21 = 0.0f;
-          const float4 geo1 = s_geo[g1], aux1 = s_aux[g1];
-          const float w10 = blend_weight<true>(geo1, aux1, c.pxf, c.pyf, T0, done0, npairs);
-          const float w11 = blend_weight<true>(geo1, aux1, c.pxf, pyf1, T1, done1, npairs);
-          if (g2 >= 0) {
-            const float4 geo = s_geo[g2], aux = s_aux[g2];
-            w20 = blend_weight<true>(geo, aux, c.pxf, c.pyf, T0, done0, npairs);
-            w21 = blend_weight<true>(geo, aux, c.pxf, pyf1, T1, done1, npairs);
-          }
-          const float w1 = __fadd_rn(w10, w11), w2 = __fadd_rn(w20, w21);
-          if (__any_sync(kFull, w1 > 0.0f || w2 > 0.0f)) {
-            const float a0 = mh ? w20 : w10, a1 = mh ? w21 : w11;
-            const float c0 = mh ? w10 : w20, c1 = mh ? w11 : w21;
-            float v[NP2];
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-              v[k] = __fmaf_rn(a0, u0[k], __fmul_rn(a1, u1[k]));
-              v[NP + k] = __fmaf_rn(c0, u0[k], __fmul_rn(c1, u1[k]));
-            }
-            const float r = warp_permuted_reduce<NP2>(v);  // the warp sum of value index m
-            const int gg = mh ? g2 : g1;
-            if ((lane & ((1 << SHIFT2) - 1)) == 0 && mk < NV && gg >= 0) atomicAdd(&s_acc[gg][mk], r);
-          }
+        for (int k = 0; k < NP / 2; ++k) {
+          const float2 x = unpack2(fma2(pack2(p0, p0), U0[k], mul2(pack2(p1, p1), U1[k])));
+          const float2 y = unpack2(fma2(pack2(q0, q0), U0[k], mul2(pack2(q1, q1), U1[k])));
+          v[2 * k] = x.x;
+          v[2 * k + 1] = x.y;
+          v[NP + 2 * k] = y.x;
+          v[NP + 2 * k + 1] = y.y;
         }
+        const float r = group_permuted_reduce<NT>(v);  // the group's sum of value index m
+        const uint32_t o = mh ? o2 : o1;
+        if (writer && o != kGPad) *reinterpret_cast<float*>(my_part + o * NP / 4) = r;
+      } else {
+        const uint32_t o = my_list[i];
+        const float2 w = group_take(group_alpha(s, o, c).alpha, T, npairs);
+        float v[NT];
+#pragma unroll
+        for (int k = 0; k < NP / 2; ++k) {
+          const float2 x = unpack2(fma2(pack2(w.x, w.x), U0[k], mul2(pack2(w.y, w.y), U1[k])));
+          v[2 * k] = x.x;
+          v[2 * k + 1] = x.y;
+        }
+        const float r = group_permuted_reduce<NT>(v);
+        if (writer && o != kGPad) *reinterpret_cast<float*>(my_part + o * NP / 4) = r;
       }
     }
     __syncthreads();
-    if ((int)threadIdx.x < nb) {
-      const int g = threadIdx.x;
-      if (s_acc[g][0] > 0.0f) {
-        float* dst = acc_cam + (int64_t)s_id[g] * RS;
+    {
+      const int g = threadIdx.x >> 1, half = threadIdx.x & 1;
+      float sum[NP];
+#pragma unroll
+      for (int k = 0; k < NP; ++k) sum[k] = 0.0f;
+      if (g < nb) {
+        const uint32_t hits = *reinterpret_cast<const uint16_t*>(&s.hits[g][2 * half]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (hits & (1u << (q < 4 ? q : q + 4))) {
+            const float* row = sa.part[half * 8 + q][g];
+            if constexpr (NP == 2) {
+              const float2 x = *reinterpret_cast<const float2*>(row);
+              sum[0] += x.x;
+              sum[1] += x.y;
+            } else {
+#pragma unroll
+              for (int k = 0; k < NP; k += 4) {
+                const float4 x = *reinterpret_cast<const float4*>(row + k);
+                sum[k] += x.x;
+                sum[k + 1] += x.y;
+                sum[k + 2] += x.z;
+                sum[k + 3] += x.w;
+              }
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < NV; ++k) sum[k] += __shfl_xor_sync(kFull, sum[k], 1);
+      if (half == 0 && g < nb && sum[0] > 0.0f) {
+        float* dst = acc_cam + (int64_t)s.id[buf][g] * RS;
         if (KC == 3 && K == 3) {
-          atomicAdd(reinterpret_cast<float4*>(dst), make_float4(s_acc[g][0], s_acc[g][1], s_acc[g][2], s_acc[g][3]));
+          atomicAdd(reinterpret_cast<float4*>(dst), make_float4(sum[0], sum[1], sum[2], sum[NP > 3 ? 3 : 0]));
         } else {
-          if (k0 == 0) atomicAdd(dst, s_acc[g][0]);
+          if (k0 == 0) atomicAdd(dst, sum[0]);
 #pragma unroll
           for (int k = 0; k < KC; ++k)
-            if (k0 + k < K) atomicAdd(dst + 1 + k0 + k, s_acc[g][k + 1]);
+            if (k0 + k < K) atomicAdd(dst + 1 + k0 + k, sum[k + 1]);
         }
-#pragma unroll
-        for (int k = 0; k < NV; ++k) s_acc[g][k] = 0.0f;
       }
     }
-    if (__syncthreads_and(done0 && done1)) break;
+    const uint32_t next = start + kBatch;
+    if (next < c.len)
+      group_stage(list, c.b + next, (int)min((uint32_t)kBatch, c.len - next), rec_cam, n, c.ox, c.oy, s, buf ^ 1);
+    if (!__syncthreads_or(T.x > 0.0f || T.y > 0.0f)) break;
   }
   if (k0 == 0) add_pair_count(npairs, status);
+}
+
+template <int KC>
+__global__ void __launch_bounds__(kGThreads, KC <= 3 ? 9 : 5) k_blend_accumulate2(
+    const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
+    const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
+    const void* __restrict__ targets, int dtype, int K, int k0, int cam0, const float* __restrict__ sub_img,
+    float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
+  __shared__ GroupBatch s;
+  __shared__ __align__(16) GroupAcc<KC> sa;
+  const GroupCtx c = group_ctx(tile_off, capacity, tiles, tiles_x, width, height);
+  group_batch_init(s);
+  float tv0[KC], tv1[KC];
+#pragma unroll
+  for (int k = 0; k < KC; ++k) tv0[k] = tv1[k] = 0.0f;
+  const int64_t row2 = 2 * (int64_t)width * K;
+  if (c.in0) {
+    const int64_t base = (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K + k0;
+    const int64_t ib = (((int64_t)c.j * height + c.py) * width + c.px) * K + k0;
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+      if (k0 + k < K) {
+        tv0[k] = load_target(targets, base + k, dtype);
+        if (c.in1) tv1[k] = load_target(targets, base + row2 + k, dtype);
+      }
+    }
+    if (KC > 3) {
+      check_finite(tv0, status);
+      check_finite(tv1, status);
+    }
+    if (sub_img) {  // refinement: residual targets t - img, img of this pass's cameras
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        if (k0 + k < K) {
+          tv0[k] -= sub_img[ib + k];
+          if (c.in1) tv1[k] -= sub_img[ib + row2 + k];
+        }
+      }
+    }
+    if (KC <= 3) {
+      check_finite(tv0, status);
+      check_finite(tv1, status);
+    }
+  }
+  group_accumulate<KC>(s, sa, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n, tv0, tv1,
+                       acc + (int64_t)c.j * acc_cam_stride, RS, K, k0, status);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -383,80 +459,110 @@ __global__ void __launch_bounds__(kThreads) k_blend_render(
   }
 }
 
-// The render with two pixels per thread (up to 4 channels): CTAs of 128 threads, each warp
-// covering an 8x8 block; the pixels (x, y) and (x, y + 4) of a thread are walked independently.
-// A hit costs little here (no reduction), so the warp keeps the plain box test.
+// The render by 8-lane groups (groupwalk.cuh) for up to 4 channels: two pixels a thread, a hit list per
+// 4x4 block. The colours are staged twice each, so that a channel of both pixels is one packed FMA.
+// A skipped step adds 0 c, which is exact for a finite c; once a staged colour is not finite (weird)
+// the tile's steps test the weight instead.
+struct GroupColours {
+  float4 c01[kBatch + 1], c23[kBatch + 1];  // (c0, c0, c1, c1), (c2, c2, c3, c3); slot kBatch: zeros
+};
+
+// The thread's staged Gaussian's channels: the even thread of a pair stages c0, c1, the odd one c2, c3.
 template <int KC>
-__global__ void __launch_bounds__(kThreads2, 10) k_blend_render2(
+__device__ __forceinline__ void stage_colours(const float* __restrict__ pay_cam, uint32_t id, int nb, int K, int k0,
+                                              GroupColours& col, int* weird) {
+  const int g = threadIdx.x >> 1, half = threadIdx.x & 1;
+  if (g >= nb || (KC <= 2 && half == 1)) return;
+  const float* src = pay_cam + (int64_t)id * K + k0 + 2 * half;
+  const float x = 2 * half < KC && k0 + 2 * half < K ? src[0] : 0.0f;
+  const float y = 2 * half + 1 < KC && k0 + 2 * half + 1 < K ? src[1] : 0.0f;
+  (half ? col.c23 : col.c01)[g] = make_float4(x, x, y, y);
+  if (!isfinite(x) || !isfinite(y)) *weird = 1;
+}
+
+template <int KC>
+__device__ __forceinline__ void group_render(GroupBatch& s, GroupColours& col, int* weird, const GroupCtx& c,
+                                             const unsigned long long* list, const ProjRec* __restrict__ rec_cam,
+                                             int64_t n, const float* __restrict__ pay_cam, int K, int k0,
+                                             f2 (&img)[KC]) {
+  if (threadIdx.x == 0) {
+    *weird = 0;
+    col.c01[kBatch] = col.c23[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  }
+#pragma unroll
+  for (int k = 0; k < KC; ++k) img[k] = pack2(0.0f, 0.0f);
+  const uint16_t* const my_list = s.list[c.group];
+  float2 T = make_float2(c.in0 ? 1.0f : 0.0f, c.in1 ? 1.0f : 0.0f);
+  uint32_t unused = 0;
+  __syncthreads();
+  auto stage = [&](uint32_t first, int nb) {
+    const uint32_t id = group_stage(list, first, nb, rec_cam, n, c.ox, c.oy, s, 0);
+    stage_colours<KC>(pay_cam, id, nb, K, k0, col, weird);
+  };
+  stage(c.b, (int)min((uint32_t)kBatch, c.len));
+  __syncthreads();
+  for (uint32_t start = 0; start < c.len; start += kBatch) {
+    const int nb = (int)min((uint32_t)kBatch, c.len - start);
+    const int steps = group_lists(s, c, nb, group_alive(T.x > 0.0f || T.y > 0.0f));
+    auto blend = [&](uint32_t o, const float2 w, bool guard) {
+      const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(reinterpret_cast<const char*>(col.c01) + o);
+      ulonglong2 c23 = make_ulonglong2(0ull, 0ull);
+      if constexpr (KC > 2) c23 = *reinterpret_cast<const ulonglong2*>(reinterpret_cast<const char*>(col.c23) + o);
+      const f2 ck[4] = {c01.x, c01.y, c23.x, c23.y};
+      const f2 w2 = pack2(w.x, w.y);
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        const f2 v = fma2(w2, ck[k], img[k]);
+        if (!guard) {
+          img[k] = v;
+        } else {
+          const float2 a = unpack2(v), b = unpack2(img[k]);
+          img[k] = pack2(w.x > 0.0f ? a.x : b.x, w.y > 0.0f ? a.y : b.y);
+        }
+      }
+    };
+    auto walk = [&](bool guard) {
+      for (int i = 0; i < steps; i += 2) {
+        const uint32_t pair = *reinterpret_cast<const uint32_t*>(my_list + i);
+        const uint32_t o1 = pair & 0xFFFFu, o2 = pair >> 16;
+        const GroupAlpha a1 = group_alpha(s, o1, c), a2 = group_alpha(s, o2, c);
+        blend(o1, group_take<false>(a1.alpha, T, unused), guard);
+        blend(o2, group_take<false>(a2.alpha, T, unused), guard);
+      }
+    };
+    if (*weird) walk(true);
+    else walk(false);
+    if (!__syncthreads_or(T.x > 0.0f || T.y > 0.0f)) break;
+    const uint32_t next = start + kBatch;
+    if (next < c.len) stage(c.b + next, (int)min((uint32_t)kBatch, c.len - next));
+    __syncthreads();
+  }
+}
+
+template <int KC>
+__global__ void __launch_bounds__(kGThreads, 10) k_blend_render2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const float* __restrict__ payload, int K, int k0, int cam0, float* __restrict__ images) {
-  static_assert(KC <= 4, "two pixels per thread: up to 4 channels");
-  __shared__ float4 s_geo[kBatch], s_aux[kBatch];
-  __shared__ float2 s_half[kBatch];
-  __shared__ uint32_t s_id[kBatch];
-  __shared__ float s_col[kBatch][KC];
-  const TileCtx c = tile_ctx<2>(tile_off, capacity, tiles, tiles_x, width, height);
-  const unsigned long long* list = tile_list(entries, c.b);
-  const bool inside1 = c.inside && c.py + 4 < height;
-  const float pyf1 = c.pyf + 4.0f;
-  const ProjRec* rec_cam = rec + (int64_t)c.j * n;
-  const float* pay_cam = payload + (int64_t)c.j * n * K;
-  float img0[KC], img1[KC];
-#pragma unroll
-  for (int k = 0; k < KC; ++k) img0[k] = img1[k] = 0.0f;
-  float T0 = 1.0f, T1 = 1.0f;
-  bool done0 = !c.inside, done1 = !inside1;
-  for (uint32_t start = 0; start < c.len; start += kBatch) {
-    const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    __syncthreads();
-    load_batch(list, start, nb, rec_cam, n, c.ox, c.oy, s_geo, s_aux, s_half, s_id);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nb * KC; idx += kThreads2) {
-      const int g = idx / KC, k = idx - g * KC;
-      s_col[g][k] = k0 + k < K ? pay_cam[(int64_t)s_id[g] * K + k0 + k] : 0.0f;
-    }
-    __syncthreads();
-    if (!__all_sync(kFull, done0 && done1)) {
-#pragma unroll
-      for (int half = 0; half < kBatch / 32; ++half) {
-        uint32_t bits = warp_hit_bits(s_geo, s_aux, s_half, half * 32, nb, c);
-        while (bits && !(done0 && done1)) {
-          const int g = half * 32 + __ffs(bits) - 1;
-          bits &= bits - 1;
-          const float4 geo = s_geo[g], aux = s_aux[g];
-          float al, ex;
-          bool cap;
-          if (!done0) {
-            const float w = blend_step(geo, aux, c.pxf, c.pyf, T0, done0, al, ex, cap);
-            if (w > 0.0f) {
-#pragma unroll
-              for (int k = 0; k < KC; ++k) img0[k] = fmaf(w, s_col[g][k], img0[k]);
-            }
-          }
-          if (!done1) {
-            const float w = blend_step(geo, aux, c.pxf, pyf1, T1, done1, al, ex, cap);
-            if (w > 0.0f) {
-#pragma unroll
-              for (int k = 0; k < KC; ++k) img1[k] = fmaf(w, s_col[g][k], img1[k]);
-            }
-          }
-        }
-      }
-    }
-    if (__syncthreads_and(done0 && done1)) break;
-  }
-  if (c.inside) {
+  static_assert(KC <= 4, "up to 4 channels");
+  __shared__ GroupBatch s;
+  __shared__ GroupColours col;
+  __shared__ int weird;
+  const GroupCtx c = group_ctx(tile_off, capacity, tiles, tiles_x, width, height);
+  group_batch_init(s);
+  f2 img[KC];
+  group_render<KC>(s, col, &weird, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n,
+                   payload + (int64_t)c.j * n * K, K, k0, img);
+  if (c.in0) {
     float* dst = images + (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K + k0;
+    const int64_t row2 = 2 * (int64_t)width * K;
 #pragma unroll
     for (int k = 0; k < KC; ++k)
-      if (k0 + k < K) dst[k] = img0[k];
-    if (inside1) {
-      dst += 4 * (int64_t)width * K;
-#pragma unroll
-      for (int k = 0; k < KC; ++k)
-        if (k0 + k < K) dst[k] = img1[k];
-    }
+      if (k0 + k < K) {
+        const float2 v = unpack2(img[k]);
+        dst[k] = v.x;
+        if (c.in1) dst[row2 + k] = v.y;
+      }
   }
 }
 
@@ -608,365 +714,254 @@ __global__ void __launch_bounds__(kThreads, KC <= 4 ? 6 : (KC <= 16 ? 4 : (KC <=
   }
 }
 
-// Pass 1 of the adjoint walk for one pixel and one staged Gaussian: F += g w and dL/dt += w a,
-// with g = a . t + beta.
+// The adjoint walk by 8-lane groups (groupwalk.cuh) for up to 4 channels: two pixels a thread, a hit
+// list per 4x4 block, the payload staged twice each for packed arithmetic. Pass 2 adds a thread's two
+// pixels, reduces two hits at a time over the group's 8 lanes (3 shuffles) and stores the sums in the
+// group's row; after the batch two threads per Gaussian add the rows and one atomic lands in grad_o.
+// A skipped step adds 0 a, exact for finite values; with a staged payload value or a target of the
+// tile that is not finite (weird) the steps test the weight instead.
 template <int KC>
-__device__ __forceinline__ void adjoint_gather(const float4 geo, const float4 aux, const float* pay,
-                                               const float (&tv)[KC], float pxf, float pyf, float& T, bool& done,
-                                               float& F, float (&gt)[KC]) {
-  float al, ex;
-  bool cap;
-  const float w = blend_step(geo, aux, pxf, pyf, T, done, al, ex, cap);
-  if (w > 0.0f) {
-    float gg = pay[KC];
+struct GroupPayload {
+  static constexpr int NQ = (KC + 2) / 2;      // float4 rows of two doubled values: a_0.., beta
+  float4 q[NQ][kBatch + 1];
+};
+
+template <int KC>
+__device__ __forceinline__ void stage_payload(const float* __restrict__ pay_cam, uint32_t id, int nb, int K,
+                                              GroupPayload<KC>& pay, int* weird) {
+  const int g = threadIdx.x >> 1, half = threadIdx.x & 1;
+  if (g >= nb) return;
+  const float* src = pay_cam + (int64_t)id * (K + 1);  // K == KC
+  bool bad = false;
 #pragma unroll
-    for (int k = 0; k < KC; ++k) {
-      gg = fmaf(pay[k], tv[k], gg);
-      gt[k] = fmaf(w, pay[k], gt[k]);
-    }
-    F = fmaf(gg, w, F);
+  for (int r = 0; r < GroupPayload<KC>::NQ; ++r) {
+    if ((r & 1) != half) continue;
+    const float x = src[2 * r], y = 2 * r + 1 <= KC ? src[2 * r + 1 <= KC ? 2 * r + 1 : 0] : 0.0f;
+    pay.q[r][g] = make_float4(x, x, y, y);
+    bad |= !isfinite(x) || !isfinite(y);
+  }
+  if (bad) *weird = 1;
+}
+
+// The staged payload of the Gaussian at byte offset o: a[0..KC-1], beta in a[KC].
+template <int KC>
+__device__ __forceinline__ void load_group_payload(const GroupPayload<KC>& pay, uint32_t o, f2 (&a)[KC + 1]) {
+#pragma unroll
+  for (int r = 0; r < GroupPayload<KC>::NQ; ++r) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(reinterpret_cast<const char*>(pay.q[r]) + o);
+    a[2 * r] = v.x;
+    if (2 * r + 1 <= KC) a[2 * r + 1 <= KC ? 2 * r + 1 : 0] = v.y;
   }
 }
 
-// Pass 2 for one pixel and one staged Gaussian m: dL/dalpha_m = g_m T_m - (F - P_m) / (1 - alpha_m),
-// returned times dalpha/do = exp(-q/2) (0 when skipped or when alpha was capped); advances T and P.
 template <int KC>
-__device__ __forceinline__ float adjoint_step(const float4 geo, const float4 aux, const float* pay,
-                                              const float (&tv)[KC], float pxf, float pyf, float F, float& T,
-                                              float& P, bool& done) {
-  if (done) return 0.0f;
-  const float Tm = T;
-  float al = 0.0f, ex = 0.0f;
-  bool cap = false;
-  const float w = blend_step(geo, aux, pxf, pyf, T, done, al, ex, cap);
-  if (!(w > 0.0f)) return 0.0f;
-  float gg = pay[KC];
-#pragma unroll
-  for (int k = 0; k < KC; ++k) gg = fmaf(pay[k], tv[k], gg);
-  P = fmaf(gg, w, P);
-  const float dalpha = gg * Tm - __fdividef(F - P, 1.0f - al);
-  return cap ? 0.0f : dalpha * ex;
-}
-
-// The adjoint walk with two pixels per thread (up to 4 channels): CTAs of 128 threads, each warp
-// covering an 8x8 block. Pass 2 adds a thread's two pixels before the warp reduction, so one
-// reduction of a hit pair serves 64 pixels.
-template <int KC>
-__global__ void __launch_bounds__(kThreads2, KC <= 2 ? 10 : 8) k_blend_adjoint2(
+__global__ void __launch_bounds__(kGThreads, 8) k_blend_adjoint2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, const float* __restrict__ payload, int K, int cam0,
     float* __restrict__ grad_t, float* __restrict__ grad_o) {
-  static_assert(KC <= 4, "two pixels per thread: up to 4 channels");
-  __shared__ float4 s_geo[kBatch], s_aux[kBatch];
-  __shared__ float2 s_half[kBatch];
-  __shared__ uint32_t s_id[kBatch];
-  __shared__ float s_pay[kBatch][KC + 1];
-  __shared__ float s_go[kBatch];
-  const TileCtx c = tile_ctx<2>(tile_off, capacity, tiles, tiles_x, width, height);
-  const unsigned long long* list = tile_list(entries, c.b);
+  static_assert(KC <= 4, "up to 4 channels");
+  __shared__ GroupBatch s;
+  __shared__ GroupPayload<KC> pay;
+  __shared__ float s_go[kGroups][kBatch];
+  __shared__ int weird;
+  const GroupCtx c = group_ctx(tile_off, capacity, tiles, tiles_x, width, height);
+  const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const int lane = threadIdx.x & 31;
-  const bool inside1 = c.inside && c.py + 4 < height;
-  const float pyf1 = c.pyf + 4.0f;
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;
   const float* pay_cam = payload + (int64_t)c.j * n * (K + 1);
-  float tv0[KC], tv1[KC];
+  if (threadIdx.x == 0) {
+    weird = 0;
 #pragma unroll
-  for (int k = 0; k < KC; ++k) tv0[k] = tv1[k] = 0.0f;
-  const int64_t pix0 = ((int64_t)(cam0 + c.j) * height + c.py) * width + c.px;
-  const int64_t pix1 = pix0 + 4 * (int64_t)width;
-  if (c.inside) {
-#pragma unroll
-    for (int k = 0; k < KC; ++k)
-      if (k < K) {
-        tv0[k] = load_target(targets, pix0 * K + k, dtype);
-        if (inside1) tv1[k] = load_target(targets, pix1 * K + k, dtype);
-      }
+    for (int r = 0; r < GroupPayload<KC>::NQ; ++r) pay.q[r][kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
-  // pass 1: F = sum_n g_n w_n and dL/dt = sum_n w_n a_n, per pixel
-  float F0 = 0.0f, F1 = 0.0f;
-  {
-    float gt0[KC], gt1[KC];
+  group_batch_init(s);
+  __syncthreads();
+  const int64_t pix0 = ((int64_t)(cam0 + c.j) * height + c.py) * width + c.px;
+  const int64_t pix1 = pix0 + 2 * (int64_t)width;
+  f2 tv[KC];
 #pragma unroll
-    for (int k = 0; k < KC; ++k) gt0[k] = gt1[k] = 0.0f;
-    float T0 = 1.0f, T1 = 1.0f;
-    bool done0 = !c.inside, done1 = !inside1;
+  for (int k = 0; k < KC; ++k) {
+    const float x = c.in0 ? load_target(targets, pix0 * K + k, dtype) : 0.0f;
+    const float y = c.in1 ? load_target(targets, pix1 * K + k, dtype) : 0.0f;
+    tv[k] = pack2(x, y);
+    if (!isfinite(x) || !isfinite(y)) weird = 1;
+  }
+  auto stage = [&](uint32_t first, int nb, int buf) {
+    const uint32_t id = group_stage(list, first, nb, rec_cam, n, c.ox, c.oy, s, buf);
+    stage_payload<KC>(pay_cam, id, nb, K, pay, &weird);
+  };
+  // g = a . t + beta
+  auto gain = [&](const f2 (&a)[KC + 1]) -> f2 {
+    f2 g = a[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) g = fma2(a[k], tv[k], g);
+    return g;
+  };
+  // x with each half replaced by old's where that pixel's weight is 0 (weird tiles only)
+  auto guarded = [&](bool guard, const float2 w, f2 x, f2 old) -> f2 {
+    if (!guard) return x;
+    const float2 a = unpack2(x), b = unpack2(old);
+    return pack2(w.x > 0.0f ? a.x : b.x, w.y > 0.0f ? a.y : b.y);
+  };
+  const uint16_t* const my_list = s.list[c.group];
+  uint32_t unused = 0;
+  const float2 T_start = make_float2(c.in0 ? 1.0f : 0.0f, c.in1 ? 1.0f : 0.0f);
+  // pass 1: F = sum_n g_n w_n and dL/dt = sum_n w_n a_n, per pixel
+  f2 F = pack2(0.0f, 0.0f);
+  {
+    f2 gt[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) gt[k] = pack2(0.0f, 0.0f);
+    float2 T = T_start;
+    stage(c.b, (int)min((uint32_t)kBatch, c.len), 0);
+    __syncthreads();
     for (uint32_t start = 0; start < c.len; start += kBatch) {
       const int nb = (int)min((uint32_t)kBatch, c.len - start);
-      __syncthreads();
-      load_batch(list, start, nb, rec_cam, n, c.ox, c.oy, s_geo, s_aux, s_half, s_id);
-      __syncthreads();
-      load_payload<KC, kThreads2>(pay_cam, nb, K, s_id, s_pay);
-      __syncthreads();
-      if (!__all_sync(kFull, done0 && done1)) {
+      const int steps = group_lists(s, c, nb, group_alive(T.x > 0.0f || T.y > 0.0f));
+      auto gather = [&](uint32_t o, const float2 w, bool guard) {
+        f2 a[KC + 1];
+        load_group_payload<KC>(pay, o, a);
+        const f2 w2 = pack2(w.x, w.y);
 #pragma unroll
-        for (int half = 0; half < kBatch / 32; ++half) {
-          uint32_t bits = warp_hit_bits<true>(s_geo, s_aux, s_half, half * 32, nb, c);
-          while (bits && !(done0 && done1)) {
-            const int g = half * 32 + __ffs(bits) - 1;
-            bits &= bits - 1;
-            const float4 geo = s_geo[g], aux = s_aux[g];
-            if (!done0) adjoint_gather<KC>(geo, aux, s_pay[g], tv0, c.pxf, c.pyf, T0, done0, F0, gt0);
-            if (!done1) adjoint_gather<KC>(geo, aux, s_pay[g], tv1, c.pxf, pyf1, T1, done1, F1, gt1);
-          }
+        for (int k = 0; k < KC; ++k) gt[k] = guarded(guard, w, fma2(w2, a[k], gt[k]), gt[k]);
+        F = guarded(guard, w, fma2(gain(a), w2, F), F);
+      };
+      auto walk = [&](bool guard) {
+        for (int i = 0; i < steps; i += 2) {
+          const uint32_t pair = *reinterpret_cast<const uint32_t*>(my_list + i);
+          const uint32_t o1 = pair & 0xFFFFu, o2 = pair >> 16;
+          const GroupAlpha a1 = group_alpha(s, o1, c), a2 = group_alpha(s, o2, c);
+          gather(o1, group_take<false>(a1.alpha, T, unused), guard);
+          gather(o2, group_take<false>(a2.alpha, T, unused), guard);
         }
-      }
-      if (__syncthreads_and(done0 && done1)) break;
+      };
+      if (weird) walk(true);
+      else walk(false);
+      if (!__syncthreads_or(T.x > 0.0f || T.y > 0.0f)) break;
+      const uint32_t next = start + kBatch;
+      if (next < c.len) stage(c.b + next, (int)min((uint32_t)kBatch, c.len - next), 0);
+      __syncthreads();
     }
-    if (grad_t && c.inside) {
+    if (grad_t && c.in0) {
 #pragma unroll
-      for (int k = 0; k < KC; ++k)
-        if (k < K) {
-          grad_t[pix0 * K + k] = gt0[k];
-          if (inside1) grad_t[pix1 * K + k] = gt1[k];
-        }
+      for (int k = 0; k < KC; ++k) {
+        const float2 v = unpack2(gt[k]);
+        grad_t[pix0 * K + k] = v.x;
+        if (c.in1) grad_t[pix1 * K + k] = v.y;
+      }
     }
   }
   if (!grad_o) return;
-  // pass 2: dL/dalpha_m = g_m T_m - (F - P_m) / (1 - alpha_m), P_m = sum_{n<=m} g_n w_n
-  for (int k = threadIdx.x; k < kBatch; k += kThreads2) s_go[k] = 0.0f;
-  float T0 = 1.0f, T1 = 1.0f, P0 = 0.0f, P1 = 0.0f;
-  bool done0 = !c.inside, done1 = !inside1;
-  for (uint32_t start = 0; start < c.len; start += kBatch) {
+  // pass 2: dL/dalpha_m = g_m T_m - (F - P_m) / (1 - alpha_m), P_m = sum_{n<=m} g_n w_n; times
+  // dalpha/do = exp(-q/2), 0 where skipped or where alpha was capped
+  __syncthreads();
+  float2 T = T_start;
+  f2 P = pack2(0.0f, 0.0f);
+  const bool second = (lane & 4) != 0;  // this lane's half of the group returns the second hit's sum
+  float* const my_go = s_go[c.group];
+  int buf = 0;
+  stage(c.b, (int)min((uint32_t)kBatch, c.len), buf);
+  __syncthreads();
+  for (uint32_t start = 0; start < c.len; start += kBatch, buf ^= 1) {
     const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    __syncthreads();
-    load_batch(list, start, nb, rec_cam, n, c.ox, c.oy, s_geo, s_aux, s_half, s_id);
-    __syncthreads();
-    load_payload<KC, kThreads2>(pay_cam, nb, K, s_id, s_pay);
-    __syncthreads();
-    if (!__all_sync(kFull, done0 && done1)) {
-#pragma unroll
-      for (int half = 0; half < kBatch / 32; ++half) {
-        uint32_t bits = warp_hit_bits<true>(s_geo, s_aux, s_half, half * 32, nb, c);
-        // two consecutive hits (in depth order) share one warp reduction of their two values
-        while (bits) {
-          const int g1 = half * 32 + __ffs(bits) - 1;
-          bits &= bits - 1;
-          const int g2 = bits ? half * 32 + __ffs(bits) - 1 : -1;
-          bits &= bits - 1;
-          float d1, d2 = 0.0f;
-          {
-            const float4 geo = s_geo[g1], aux = s_aux[g1];
-            d1 = adjoint_step<KC>(geo, aux, s_pay[g1], tv0, c.pxf, c.pyf, F0, T0, P0, done0) +
-                 adjoint_step<KC>(geo, aux, s_pay[g1], tv1, c.pxf, pyf1, F1, T1, P1, done1);
-          }
-          if (g2 >= 0) {
-            const float4 geo = s_geo[g2], aux = s_aux[g2];
-            d2 = adjoint_step<KC>(geo, aux, s_pay[g2], tv0, c.pxf, c.pyf, F0, T0, P0, done0) +
-                 adjoint_step<KC>(geo, aux, s_pay[g2], tv1, c.pxf, pyf1, F1, T1, P1, done1);
-          }
-          if (__any_sync(kFull, d1 != 0.0f || d2 != 0.0f)) {
-            // lanes < 16 end with the sum of d1, lanes >= 16 with the sum of d2
-            const bool upper = (lane & 16) != 0;
-            float r = (upper ? d2 : d1) + __shfl_xor_sync(kFull, upper ? d1 : d2, 16);
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
-            if (lane == 0) atomicAdd(&s_go[g1], r);
-            if (lane == 16 && g2 >= 0) atomicAdd(&s_go[g2], r);
-          }
-        }
+    const int steps = group_lists(s, c, nb, group_alive(T.x > 0.0f || T.y > 0.0f));
+    auto step = [&](uint32_t o, const GroupAlpha& al, bool guard) -> float {
+      const f2 Tm = pack2(T.x, T.y);
+      const float2 w = group_take<false>(al.alpha, T, unused);
+      f2 a[KC + 1];
+      load_group_payload<KC>(pay, o, a);
+      const f2 g = gain(a);
+      P = guarded(guard, w, fma2(g, pack2(w.x, w.y), P), P);
+      const float2 rest = unpack2(fma2(P, pack2(-1.0f, -1.0f), F));  // F - P
+      const float2 om = unpack2(fma2(pack2(al.alpha.x, al.alpha.y), pack2(-1.0f, -1.0f), pack2(1.0f, 1.0f)));
+      const f2 da = fma2(g, Tm, pack2(-__fdividef(rest.x, om.x), -__fdividef(rest.y, om.y)));
+      const float2 d = unpack2(mul2(da, pack2(al.e.x, al.e.y)));
+      const float d0 = w.x > 0.0f && al.oe.x < kAlphaMax ? d.x : 0.0f;
+      const float d1 = w.y > 0.0f && al.oe.y < kAlphaMax ? d.y : 0.0f;
+      return d0 + d1;
+    };
+    auto walk = [&](bool guard) {
+      for (int i = 0; i < steps; i += 2) {
+        const uint32_t pair = *reinterpret_cast<const uint32_t*>(my_list + i);
+        const uint32_t o1 = pair & 0xFFFFu, o2 = pair >> 16;
+        const GroupAlpha a1 = group_alpha(s, o1, c), a2 = group_alpha(s, o2, c);
+        const float d1 = step(o1, a1, guard), d2 = step(o2, a2, guard);
+        float v[2] = {second ? d2 : d1, second ? d1 : d2};
+        const float r = group_permuted_reduce<2>(v);
+        const uint32_t o = second ? o2 : o1;
+        if ((lane & 3) == 0 && o != kGPad) my_go[o / 16] = r;
       }
-    }
+    };
+    if (weird) walk(true);
+    else walk(false);
     __syncthreads();
-    if ((int)threadIdx.x < nb) {
-      const float v = s_go[threadIdx.x];
-      if (v != 0.0f) {
-        atomicAdd(grad_o + s_id[threadIdx.x], v);
-        s_go[threadIdx.x] = 0.0f;
+    {
+      const int g = threadIdx.x >> 1, half = threadIdx.x & 1;
+      float sum = 0.0f;
+      if (g < nb) {
+        const uint32_t hits = *reinterpret_cast<const uint16_t*>(&s.hits[g][2 * half]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (hits & (1u << (q < 4 ? q : q + 4))) sum += s_go[half * 8 + q][g];
       }
+      sum += __shfl_xor_sync(kFull, sum, 1);
+      if (half == 0 && g < nb && sum != 0.0f) atomicAdd(grad_o + s.id[buf][g], sum);
     }
-    if (__syncthreads_and(done0 && done1)) break;
+    const uint32_t next = start + kBatch;
+    if (next < c.len) stage(c.b + next, (int)min((uint32_t)kBatch, c.len - next), buf ^ 1);
+    if (!__syncthreads_or(T.x > 0.0f || T.y > 0.0f)) break;
   }
 }
 
-// One refinement walk (Alg. 1 lines 8-9) for up to 3 channels, two pixels per thread: pass 1
-// renders the current colours of the thread's pixels (as k_blend_render2), pass 2 accumulates the
-// residual targets t - img (as k_blend_accumulate2 with a rendered image subtracted), over the tile
-// list sorted once. Same arithmetic as the two separate walks, without the image round trip.
+// One refinement walk (Alg. 1 lines 8-9) for up to 3 channels by 8-lane groups: pass 1 renders the
+// current colours of the thread's pixels (as k_blend_render2), pass 2 accumulates the residual targets
+// t - img (as k_blend_accumulate2 with a rendered image subtracted), over the tile list sorted once.
+// Same arithmetic as the two separate walks, without the image round trip. The colours of pass 1 share
+// the shared memory of pass 2's partial sums.
 template <int KC>
-__global__ void __launch_bounds__(kThreads2, 10) k_blend_refine2(
+__global__ void __launch_bounds__(kGThreads, 9) k_blend_refine2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, int K, int cam0, const float* __restrict__ payload,
     float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
-  static_assert(KC <= 3, "two pixels per thread: up to 3 channels");
-  constexpr int NV = KC + 1;
-  constexpr int NP = NextPow2<NV>::value;
-  constexpr int NP2 = 2 * NP;
-  constexpr int SHIFT2 = 5 - Log2<NP2>::value;
-  __shared__ float4 s_geo[kBatch], s_aux[kBatch];
-  __shared__ float2 s_half[kBatch];
-  __shared__ uint32_t s_id[kBatch];
-  __shared__ float s_acc[kBatch][NV];
-  __shared__ float s_col[kBatch][KC];
-  const TileCtx c = tile_ctx<2>(tile_off, capacity, tiles, tiles_x, width, height);
-  const unsigned long long* list = tile_list(entries, c.b);
-  const int lane = threadIdx.x & 31;
-  const bool inside1 = c.inside && c.py + 4 < height;
-  const float pyf1 = c.pyf + 4.0f;
+  static_assert(KC <= 3, "up to 3 channels");
+  static_assert(sizeof(GroupColours) <= sizeof(GroupAcc<KC>), "the colours fit where the sums go");
+  __shared__ GroupBatch s;
+  __shared__ __align__(16) GroupAcc<KC> sa;
+  __shared__ int weird;
+  const GroupCtx c = group_ctx(tile_off, capacity, tiles, tiles_x, width, height);
+  group_batch_init(s);
+  const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;
-  const float* pay_cam = payload + (int64_t)c.j * n * K;
-  // pass 1: the current render of both pixels
-  float img0[KC], img1[KC];
-#pragma unroll
-  for (int k = 0; k < KC; ++k) img0[k] = img1[k] = 0.0f;
-  {
-    float T0 = 1.0f, T1 = 1.0f;
-    bool done0 = !c.inside, done1 = !inside1;
-    for (uint32_t start = 0; start < c.len; start += kBatch) {
-      const int nb = (int)min((uint32_t)kBatch, c.len - start);
-      __syncthreads();
-      load_batch(list, start, nb, rec_cam, n, c.ox, c.oy, s_geo, s_aux, s_half, s_id);
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < nb * KC; idx += kThreads2) {
-        const int g = idx / KC, k = idx - g * KC;
-        s_col[g][k] = k < K ? pay_cam[(int64_t)s_id[g] * K + k] : 0.0f;
-      }
-      __syncthreads();
-      if (!__all_sync(kFull, done0 && done1)) {
-#pragma unroll
-        for (int half = 0; half < kBatch / 32; ++half) {
-          uint32_t bits = warp_hit_bits(s_geo, s_aux, s_half, half * 32, nb, c);
-          while (bits && !(done0 && done1)) {
-            const int g = half * 32 + __ffs(bits) - 1;
-            bits &= bits - 1;
-            const float4 geo = s_geo[g], aux = s_aux[g];
-            float al, ex;
-            bool cap;
-            if (!done0) {
-              const float w = blend_step(geo, aux, c.pxf, c.pyf, T0, done0, al, ex, cap);
-              if (w > 0.0f) {
-#pragma unroll
-                for (int k = 0; k < KC; ++k) img0[k] = fmaf(w, s_col[g][k], img0[k]);
-              }
-            }
-            if (!done1) {
-              const float w = blend_step(geo, aux, c.pxf, pyf1, T1, done1, al, ex, cap);
-              if (w > 0.0f) {
-#pragma unroll
-                for (int k = 0; k < KC; ++k) img1[k] = fmaf(w, s_col[g][k], img1[k]);
-              }
-            }
-          }
-        }
-      }
-      if (__syncthreads_and(done0 && done1)) break;
-    }
-  }
-  // residual targets t - img
+  f2 img[KC];
+  group_render<KC>(s, reinterpret_cast<GroupColours&>(sa), &weird, c, list, rec_cam, n,
+                   payload + (int64_t)c.j * n * K, K, 0, img);
   float tv0[KC], tv1[KC];
 #pragma unroll
   for (int k = 0; k < KC; ++k) tv0[k] = tv1[k] = 0.0f;
-  if (c.inside) {
+  if (c.in0) {
     const int64_t base = (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K;
-    const int64_t row = (int64_t)width * K;
+    const int64_t row2 = 2 * (int64_t)width * K;
 #pragma unroll
     for (int k = 0; k < KC; ++k) {
-      if (k < K) {
-        tv0[k] = load_target(targets, base + k, dtype) - img0[k];
-        if (inside1) tv1[k] = load_target(targets, base + 4 * row + k, dtype) - img1[k];
-      }
+      const float2 v = unpack2(img[k]);
+      tv0[k] = load_target(targets, base + k, dtype) - v.x;
+      if (c.in1) tv1[k] = load_target(targets, base + row2 + k, dtype) - v.y;
     }
     check_finite(tv0, status);
     check_finite(tv1, status);
   }
-  // pass 2: the accumulate walk of k_blend_accumulate2 on the residuals
-  const int m = lane >> SHIFT2;
-  const bool mh = (m & NP) != 0;
-  const int mk = m & (NP - 1);
-  float u0[NP], u1[NP];
-  u0[0] = u1[0] = 1.0f;
-#pragma unroll
-  for (int k = 1; k < NP; ++k) {
-    u0[k] = k <= KC ? tv0[k <= KC ? k - 1 : 0] : 0.0f;
-    u1[k] = k <= KC ? tv1[k <= KC ? k - 1 : 0] : 0.0f;
-  }
-#pragma unroll
-  for (int bit = 1; bit < NP; bit <<= 1) {  // u[k] <- u[k ^ mk], one conditional swap per bit of mk
-    const bool sw = (mk & bit) != 0;
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      if (k & bit) continue;
-      const float x0 = u0[k], y0 = u0[k | bit], x1 = u1[k], y1 = u1[k | bit];
-      u0[k] = sw ? y0 : x0;
-      u0[k | bit] = sw ? x0 : y0;
-      u1[k] = sw ? y1 : x1;
-      u1[k | bit] = sw ? x1 : y1;
-    }
-  }
-  for (int k = threadIdx.x; k < kBatch * NV; k += kThreads2) (&s_acc[0][0])[k] = 0.0f;
-  float* acc_cam = acc + (int64_t)c.j * acc_cam_stride;
-  float T0 = 1.0f, T1 = 1.0f;
-  bool done0 = !c.inside, done1 = !inside1;
-  uint32_t npairs = 0;
-  for (uint32_t start = 0; start < c.len; start += kBatch) {
-    const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    __syncthreads();
-    load_batch(list, start, nb, rec_cam, n, c.ox, c.oy, s_geo, s_aux, s_half, s_id);
-    __syncthreads();
-    if (!__all_sync(kFull, done0 && done1)) {
-#pragma unroll
-      for (int half = 0; half < kBatch / 32; ++half) {
-        uint32_t bits = warp_hit_bits<true>(s_geo, s_aux, s_half, half * 32, nb, c);
-        while (bits) {
-          const int g1 = half * 32 + __ffs(bits) - 1;
-          bits &= bits - 1;
-          const int g2 = bits ? half * 32 + __ffs(bits) - 1 : -1;
-          bits &= bits - 1;
-          float w20 = 0.0f, w21 = 0.0f;
-          const float4 geo1 = s_geo[g1], aux1 = s_aux[g1];
-          const float w10 = blend_weight<true>(geo1, aux1, c.pxf, c.pyf, T0, done0, npairs);
-          const float w11 = blend_weight<true>(geo1, aux1, c.pxf, pyf1, T1, done1, npairs);
-          if (g2 >= 0) {
-            const float4 geo = s_geo[g2], aux = s_aux[g2];
-            w20 = blend_weight<true>(geo, aux, c.pxf, c.pyf, T0, done0, npairs);
-            w21 = blend_weight<true>(geo, aux, c.pxf, pyf1, T1, done1, npairs);
-          }
-          const float w1 = __fadd_rn(w10, w11), w2 = __fadd_rn(w20, w21);
-          if (__any_sync(kFull, w1 > 0.0f || w2 > 0.0f)) {
-            const float a0 = mh ? w20 : w10, a1 = mh ? w21 : w11;
-            const float c0 = mh ? w10 : w20, c1 = mh ? w11 : w21;
-            float v[NP2];
-#pragma unroll
-            for (int k = 0; k < NP; ++k) {
-              v[k] = __fmaf_rn(a0, u0[k], __fmul_rn(a1, u1[k]));
-              v[NP + k] = __fmaf_rn(c0, u0[k], __fmul_rn(c1, u1[k]));
-            }
-            const float r = warp_permuted_reduce<NP2>(v);  // the warp sum of value index m
-            const int gg = mh ? g2 : g1;
-            if ((lane & ((1 << SHIFT2) - 1)) == 0 && mk < NV && gg >= 0) atomicAdd(&s_acc[gg][mk], r);
-          }
-        }
-      }
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < nb) {
-      const int g = threadIdx.x;
-      if (s_acc[g][0] > 0.0f) {
-        float* dst = acc_cam + (int64_t)s_id[g] * RS;
-        if (KC == 3 && K == 3) {
-          atomicAdd(reinterpret_cast<float4*>(dst), make_float4(s_acc[g][0], s_acc[g][1], s_acc[g][2], s_acc[g][3]));
-        } else {
-          atomicAdd(dst, s_acc[g][0]);
-#pragma unroll
-          for (int k = 0; k < KC; ++k)
-            if (k < K) atomicAdd(dst + 1 + k, s_acc[g][k + 1]);
-        }
-#pragma unroll
-        for (int k = 0; k < NV; ++k) s_acc[g][k] = 0.0f;
-      }
-    }
-    if (__syncthreads_and(done0 && done1)) break;
-  }
-  add_pair_count(npairs, status);
+  __syncthreads();
+  group_accumulate<KC>(s, sa, c, list, rec_cam, n, tv0, tv1, acc + (int64_t)c.j * acc_cam_stride, RS, K, 0, status);
 }
 
 template <int KC>
 void accumulate_chunk(const Problem& p, int cb, int cam0, const void* targets, int dtype, int k0,
                       const float* sub_img, const Workspace& ws, cudaStream_t s) {
   const int64_t stride = p.L == 0 ? 0 : p.n * (int64_t)p.acc_stride;
-  if constexpr (KC <= 3) {
-    k_blend_accumulate2<KC><<<cb * p.tiles, kThreads2, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,
+  if constexpr (KC <= 7) {
+    k_blend_accumulate2<KC><<<cb * p.tiles, kGThreads, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,
                                                                p.width, p.height, p.tiles_x, p.tiles, targets, dtype,
                                                                p.K, k0, cam0, sub_img, ws.acc, p.acc_stride, stride,
                                                                ws.status);
@@ -983,7 +978,7 @@ template <int KC>
 void render_chunk(const Problem& p, int cb, int cam0, int k0, const Workspace& ws, float* images,
                   cudaStream_t s) {
   if constexpr (KC <= 4) {
-    k_blend_render2<KC><<<cb * p.tiles, kThreads2, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,
+    k_blend_render2<KC><<<cb * p.tiles, kGThreads, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,
                                                            p.width, p.height, p.tiles_x, p.tiles, ws.payload, p.K,
                                                            k0, cam0, images);
   } else {
@@ -1036,7 +1031,7 @@ bool launch_blend_refine(const Problem& p, int cb, int cam0, const void* targets
   if (p.K > 3) return false;
   const int64_t stride = p.L == 0 ? 0 : p.n * (int64_t)p.acc_stride;
 #define ICGS_REF(KC)                                                                                         \
-  k_blend_refine2<KC><<<cb * p.tiles, kThreads2, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,     \
+  k_blend_refine2<KC><<<cb * p.tiles, kGThreads, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,     \
                                                           p.width, p.height, p.tiles_x, p.tiles, targets, dtype, \
                                                           p.K, cam0, ws.payload, ws.acc, p.acc_stride, stride,   \
                                                           ws.status)
@@ -1056,7 +1051,7 @@ void launch_blend_adjoint(const Problem& p, int cb, int cam0, const void* target
                                                          p.width, p.height, p.tiles_x, p.tiles, targets,     \
                                                          dtype, ws.payload, p.K, cam0, grad_targets, go)
 #define ICGS_ADJ2(KC)                                                                                        \
-  k_blend_adjoint2<KC><<<cb * p.tiles, kThreads2, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,  \
+  k_blend_adjoint2<KC><<<cb * p.tiles, kGThreads, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,  \
                                                            p.width, p.height, p.tiles_x, p.tiles, targets,     \
                                                            dtype, ws.payload, p.K, cam0, grad_targets, go)
   if (p.K == 1) ICGS_ADJ2(1);
