@@ -183,21 +183,24 @@ __global__ void __launch_bounds__(kThreads, KC <= 8 ? 5 : 4) k_blend_accumulate(
   if (k0 == 0) add_pair_count(npairs, status);
 }
 
-// The same accumulation for up to 7 channels by 8-lane groups (groupwalk.cuh): 128 threads, two pixels
-// each, a hit list per 4x4 block. A group reduces its own hits, kHits at a time (two for up to 3
-// channels), over its 8 lanes: NT = kHits NP values leave one warp-wide butterfly of 7 shuffles with
-// one sum per lane, stored (no atomics: a group takes a Gaussian once per batch) in the group's
-// row of s_part; after the batch two threads per Gaussian add the rows of the groups that list it, and
-// one atomic group per (Gaussian, tile) lands in the accumulator.
+// The same accumulation for up to 7 channels by 8-lane groups (groupwalk.cuh): 64 threads, two pixel
+// pairs each, a hit list per 8x4 block. A group reduces each of its hits over its 8 lanes (a halving
+// butterfly of 4 shuffles for up to 3 channels, 7 for up to 7) and stores the sums (no atomics: a group
+// takes a Gaussian once per batch) in its row of s_part; after the batch one thread per Gaussian
+// adds the rows of the groups that list it, and one atomic group per (Gaussian, tile) lands in the
+// accumulator.
+constexpr int kPP = 2;  // pixel pairs a lane of the walks below
+constexpr int kGThreads = GroupCfg<kPP>::kThreads;
+constexpr int kGroups = GroupCfg<kPP>::kGroups;
+
 template <int KC>
 struct GroupAcc {
   static_assert(KC >= 1 && KC <= 7, "1..7 channels");
   static constexpr int NV = KC + 1;                 // V and S_0..S_{KC-1}
-  static constexpr int NP = NextPow2<NV>::value;    // 2, 4 or 8: floats of a partial row
-  static constexpr int kHits = NP <= 4 ? 2 : 1;
-  static constexpr int NT = NP * kHits;             // values of a group reduction (4 or 8)
-  static constexpr int SHIFT = 3 - Log2<NT>::value; // lane l of a group returns value l >> SHIFT
-  float part[kGroups][kBatch][NP];
+  static constexpr int NP = NextPow2<NV>::value;    // 2, 4 or 8: values of a reduction, floats of a partial row
+  static constexpr int SHIFT = 3 - Log2<NP>::value; // lane l of a group returns value l >> SHIFT
+  float part[kGroups][kBatch + 1][NP];              // slot kBatch: where the list padding goes
+  GroupIds<kPP> ids;
 };
 
 // Group sums of NT values held in lane-permuted slots (warp_permuted_reduce over 8 lanes).
@@ -216,106 +219,97 @@ __device__ __forceinline__ float group_permuted_reduce(float (&v)[NT]) {
   return r;
 }
 
-// The walk of one tile for target values tv0, tv1 of the thread's two pixels.
+// The walk of one tile for target values tv of the lane's pixels ([2 u + x]: pair u, pixel x).
 template <int KC>
-__device__ __forceinline__ void group_accumulate(GroupBatch& s, GroupAcc<KC>& sa, const GroupCtx& c,
+__device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC>& sa, const GroupCtx<kPP>& c,
                                                  const unsigned long long* list, const ProjRec* __restrict__ rec_cam,
-                                                 int64_t n, const float (&tv0)[KC], const float (&tv1)[KC],
-                                                 float* __restrict__ acc_cam, int RS, int K, int k0, DevStatus* status) {
+                                                 int64_t n, const float (&tv)[2 * kPP][KC], float* __restrict__ acc_cam,
+                                                 int RS, int K, int k0, DevStatus* status) {
   using S = GroupAcc<KC>;
-  constexpr int NV = S::NV, NP = S::NP, NT = S::NT;
+  constexpr int NV = S::NV, NP = S::NP;
   const int lane = threadIdx.x & 31;
-  // Value h NP + k of a step is hit h's weights times u[k], u = (1, t_0, .., t_{KC-1}, 0, ..), summed
-  // over the thread's two pixels. This lane keeps it in slot (h NP + k) ^ m, so u is permuted here
-  // once, by one conditional swap per bit of mk, and two hits trade places when mh is set.
+  // Value k of a hit is its weights times u[k], u = (1, t_0, .., t_{KC-1}, 0, ..), summed over the pixels.
+  // This lane keeps it in slot k ^ m (warp_permuted_reduce): u is permuted here once.
   const int m = (lane & 7) >> S::SHIFT;
-  const bool mh = (m & NP) != 0;
-  const int mk = m & (NP - 1);
-  float u0[NP], u1[NP];
-  u0[0] = u1[0] = 1.0f;
+  f2 U[2 * kPP][NP / 2];
 #pragma unroll
-  for (int k = 1; k < NP; ++k) {
-    u0[k] = k <= KC ? tv0[k <= KC ? k - 1 : 0] : 0.0f;
-    u1[k] = k <= KC ? tv1[k <= KC ? k - 1 : 0] : 0.0f;
-  }
+  for (int x = 0; x < 2 * kPP; ++x) {
+    float u[NP];
+    u[0] = 1.0f;
 #pragma unroll
-  for (int bit = 1; bit < NP; bit <<= 1) {
-    const bool sw = (mk & bit) != 0;
+    for (int k = 1; k < NP; ++k) u[k] = k <= KC ? tv[x][k <= KC ? k - 1 : 0] : 0.0f;
 #pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      if (k & bit) continue;
-      const float x0 = u0[k], y0 = u0[k | bit], x1 = u1[k], y1 = u1[k | bit];
-      u0[k] = sw ? y0 : x0;
-      u0[k | bit] = sw ? x0 : y0;
-      u1[k] = sw ? y1 : x1;
-      u1[k | bit] = sw ? x1 : y1;
+    for (int bit = 1; bit < NP; bit <<= 1) {
+      const bool sw = (m & bit) != 0;
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        if (k & bit) continue;
+        const float a = u[k], b = u[k | bit];
+        u[k] = sw ? b : a;
+        u[k | bit] = sw ? a : b;
+      }
     }
-  }
-  f2 U0[NP / 2], U1[NP / 2];
 #pragma unroll
-  for (int k = 0; k < NP / 2; ++k) {
-    U0[k] = pack2(u0[2 * k], u0[2 * k + 1]);
-    U1[k] = pack2(u1[2 * k], u1[2 * k + 1]);
+    for (int k = 0; k < NP / 2; ++k) U[x][k] = pack2(u[2 * k], u[2 * k + 1]);
   }
-  const bool writer = ((lane & 7) & ((1 << S::SHIFT) - 1)) == 0 && mk < NV;
-  char* const my_part = reinterpret_cast<char*>(&sa.part[c.group][0][mk]);
-  const uint16_t* const my_list = s.list[c.group];
-  float2 T = make_float2(c.in0 ? 1.0f : 0.0f, c.in1 ? 1.0f : 0.0f);
+  const bool writer = ((lane & 7) & ((1 << S::SHIFT) - 1)) == 0 && m < NV;
+  char* const my_part = reinterpret_cast<char*>(&sa.part[c.group][0][m]);
+  const uint16_t* const my_list = s.lists.row[c.group];
+  GroupT<kPP> T(c);
   uint32_t npairs = 0;
   int buf = 0;
-  group_stage(list, c.b, (int)min((uint32_t)kBatch, c.len), rec_cam, n, c.ox, c.oy, s, buf);
+  const uint32_t list_end = c.b + c.len;
+  const uint32_t id0 = group_id<kPP>(list, c.b, list_end, n);
+  uint32_t id_next = group_id<kPP>(list, c.b + kBatch, list_end, n);
+  GroupFetch fetch = group_fetch(id0, rec_cam);
+  group_put<kPP>(fetch, (int)min((uint32_t)kBatch, c.len), c.ox, c.oy, s.geo);
+  sa.ids.id[buf][threadIdx.x] = id0;
   __syncthreads();
   // two barriers a batch: the next batch is staged between them, when the walk of this one has ended
   for (uint32_t start = 0; start < c.len; start += kBatch, buf ^= 1) {
     const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    const int steps = group_lists(s, c, nb, group_alive(T.x > 0.0f || T.y > 0.0f));
-    for (int i = 0; i < steps; i += S::kHits) {
-      if constexpr (S::kHits == 2) {
-        const uint32_t pair = *reinterpret_cast<const uint32_t*>(my_list + i);
-        const uint32_t o1 = pair & 0xFFFFu, o2 = pair >> 16;
-        const GroupAlpha a1 = group_alpha(s, o1, c), a2 = group_alpha(s, o2, c);  // independent of T
-        const float2 w1 = group_take(a1.alpha, T, npairs), w2 = group_take(a2.alpha, T, npairs);
-        const float p0 = mh ? w2.x : w1.x, p1 = mh ? w2.y : w1.y;
-        const float q0 = mh ? w1.x : w2.x, q1 = mh ? w1.y : w2.y;
-        float v[NT];
+    const uint32_t next = start + kBatch, id_fetched = id_next;
+    if (next < c.len) {  // in flight during the walk
+      fetch = group_fetch(id_fetched, rec_cam);
+      id_next = group_id<kPP>(list, c.b + next + kBatch, list_end, n);
+    }
+    const int steps = group_lists(s.geo, s.lists, c, nb, group_alive(T.alive()), sa.ids.hits);
+    auto reduce = [&](uint32_t o, const GroupW<kPP>& w) {
+      float v[NP];
 #pragma unroll
-        for (int k = 0; k < NP / 2; ++k) {
-          const float2 x = unpack2(fma2(pack2(p0, p0), U0[k], mul2(pack2(p1, p1), U1[k])));
-          const float2 y = unpack2(fma2(pack2(q0, q0), U0[k], mul2(pack2(q1, q1), U1[k])));
-          v[2 * k] = x.x;
-          v[2 * k + 1] = x.y;
-          v[NP + 2 * k] = y.x;
-          v[NP + 2 * k + 1] = y.y;
-        }
-        const float r = group_permuted_reduce<NT>(v);  // the group's sum of value index m
-        const uint32_t o = mh ? o2 : o1;
-        if (writer && o != kGPad) *reinterpret_cast<float*>(my_part + o * NP / 4) = r;
-      } else {
-        const uint32_t o = my_list[i];
-        const float2 w = group_take(group_alpha(s, o, c).alpha, T, npairs);
-        float v[NT];
+      for (int k = 0; k < NP / 2; ++k) {
+        f2 x = 0ull;
 #pragma unroll
-        for (int k = 0; k < NP / 2; ++k) {
-          const float2 x = unpack2(fma2(pack2(w.x, w.x), U0[k], mul2(pack2(w.y, w.y), U1[k])));
-          v[2 * k] = x.x;
-          v[2 * k + 1] = x.y;
+        for (int u = 0; u < kPP; ++u) {
+          const f2 w0 = pack2(w.v[u].x, w.v[u].x), w1 = pack2(w.v[u].y, w.v[u].y);
+          x = u == 0 ? mul2(w0, U[0][k]) : fma2(w0, U[2 * u][k], x);
+          x = fma2(w1, U[2 * u + 1][k], x);
         }
-        const float r = group_permuted_reduce<NT>(v);
-        if (writer && o != kGPad) *reinterpret_cast<float*>(my_part + o * NP / 4) = r;
+        const float2 y = unpack2(x);
+        v[2 * k] = y.x;
+        v[2 * k + 1] = y.y;
       }
+      const float r = group_permuted_reduce<NP>(v);  // the group's sum of value m
+      if (writer) *reinterpret_cast<float*>(my_part + o * NP / 4) = r;
+    };
+    for (int i = 0; i < steps; i += 2) {
+      const uint2 o = s.lists.pair(my_list, i);
+      const GroupAlpha<kPP> a1 = group_alpha(s.geo, o.x, c), a2 = group_alpha(s.geo, o.y, c);  // independent of T
+      reduce(o.x, group_take(a1, T, npairs));
+      reduce(o.y, group_take(a2, T, npairs));
     }
     __syncthreads();
     {
-      const int g = threadIdx.x >> 1, half = threadIdx.x & 1;
+      const int g = threadIdx.x;
       float sum[NP];
 #pragma unroll
       for (int k = 0; k < NP; ++k) sum[k] = 0.0f;
       if (g < nb) {
-        const uint32_t hits = *reinterpret_cast<const uint16_t*>(&s.hits[g][2 * half]);
+        const uint32_t hits = *reinterpret_cast<const uint16_t*>(&sa.ids.hits[g][0]);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < kGroups; ++q) {
           if (hits & (1u << (q < 4 ? q : q + 4))) {
-            const float* row = sa.part[half * 8 + q][g];
+            const float* row = sa.part[q][g];
             if constexpr (NP == 2) {
               const float2 x = *reinterpret_cast<const float2*>(row);
               sum[0] += x.x;
@@ -332,72 +326,70 @@ __device__ __forceinline__ void group_accumulate(GroupBatch& s, GroupAcc<KC>& sa
             }
           }
         }
-      }
+        if (sum[0] > 0.0f) {
+          float* dst = acc_cam + (int64_t)sa.ids.id[buf][g] * RS;
+          if (KC == 3 && K == 3) {
+            atomicAdd(reinterpret_cast<float4*>(dst), make_float4(sum[0], sum[1], sum[NP > 2 ? 2 : 0], sum[NP > 2 ? 3 : 0]));
+          } else {
+            if (k0 == 0) atomicAdd(dst, sum[0]);
 #pragma unroll
-      for (int k = 0; k < NV; ++k) sum[k] += __shfl_xor_sync(kFull, sum[k], 1);
-      if (half == 0 && g < nb && sum[0] > 0.0f) {
-        float* dst = acc_cam + (int64_t)s.id[buf][g] * RS;
-        if (KC == 3 && K == 3) {
-          atomicAdd(reinterpret_cast<float4*>(dst), make_float4(sum[0], sum[1], sum[2], sum[NP > 3 ? 3 : 0]));
-        } else {
-          if (k0 == 0) atomicAdd(dst, sum[0]);
-#pragma unroll
-          for (int k = 0; k < KC; ++k)
-            if (k0 + k < K) atomicAdd(dst + 1 + k0 + k, sum[k + 1]);
+            for (int k = 0; k < KC; ++k)
+              if (k0 + k < K) atomicAdd(dst + 1 + k0 + k, sum[k + 1]);
+          }
         }
       }
     }
-    const uint32_t next = start + kBatch;
-    if (next < c.len)
-      group_stage(list, c.b + next, (int)min((uint32_t)kBatch, c.len - next), rec_cam, n, c.ox, c.oy, s, buf ^ 1);
-    if (!__syncthreads_or(T.x > 0.0f || T.y > 0.0f)) break;
+    if (next < c.len) {
+      group_put<kPP>(fetch, (int)min((uint32_t)kBatch, c.len - next), c.ox, c.oy, s.geo);
+      sa.ids.id[buf ^ 1][threadIdx.x] = id_fetched;
+    }
+    if (!__syncthreads_or(T.alive())) break;
   }
   if (k0 == 0) add_pair_count(npairs, status);
 }
 
+// Calls f(x, offset) for each of the lane's pixels inside the image: x = 2 u + side, offset in pixels
+// from the lane's first pixel.
+template <typename F>
+__device__ __forceinline__ void for_pixels(const GroupCtx<kPP>& c, int width, F f) {
+#pragma unroll
+  for (int u = 0; u < kPP; ++u) {
+    const int64_t row = 2 * (int64_t)u * width;
+    if (c.in0[u]) f(2 * u, row);
+    if (c.in1[u]) f(2 * u + 1, row + 1);
+  }
+}
+
 template <int KC>
-__global__ void __launch_bounds__(kGThreads, KC <= 3 ? 9 : 5) k_blend_accumulate2(
+__global__ void __launch_bounds__(kGThreads, KC <= 3 ? 13 : 8) k_blend_accumulate2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, int K, int k0, int cam0, const float* __restrict__ sub_img,
     float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
-  __shared__ GroupBatch s;
+  __shared__ GroupBatch<kPP> s;
   __shared__ __align__(16) GroupAcc<KC> sa;
-  const GroupCtx c = group_ctx(tile_off, capacity, tiles, tiles_x, width, height);
-  group_batch_init(s);
-  float tv0[KC], tv1[KC];
+  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height);
+  if (threadIdx.x == 0) group_pad(s.geo);
+  float tv[2 * kPP][KC];
 #pragma unroll
-  for (int k = 0; k < KC; ++k) tv0[k] = tv1[k] = 0.0f;
-  const int64_t row2 = 2 * (int64_t)width * K;
-  if (c.in0) {
-    const int64_t base = (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K + k0;
-    const int64_t ib = (((int64_t)c.j * height + c.py) * width + c.px) * K + k0;
+  for (int x = 0; x < 2 * kPP; ++x)
 #pragma unroll
-    for (int k = 0; k < KC; ++k) {
-      if (k0 + k < K) {
-        tv0[k] = load_target(targets, base + k, dtype);
-        if (c.in1) tv1[k] = load_target(targets, base + row2 + k, dtype);
-      }
-    }
-    if (KC > 3) {
-      check_finite(tv0, status);
-      check_finite(tv1, status);
-    }
+    for (int k = 0; k < KC; ++k) tv[x][k] = 0.0f;
+  const int64_t base = (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K + k0;
+  const int64_t ib = (((int64_t)c.j * height + c.py) * width + c.px) * K + k0;
+  for_pixels(c, width, [&](int x, int64_t off) {
+#pragma unroll
+    for (int k = 0; k < KC; ++k)
+      if (k0 + k < K) tv[x][k] = load_target(targets, base + off * K + k, dtype);
+    if (KC > 3) check_finite(tv[x], status);
     if (sub_img) {  // refinement: residual targets t - img, img of this pass's cameras
 #pragma unroll
-      for (int k = 0; k < KC; ++k) {
-        if (k0 + k < K) {
-          tv0[k] -= sub_img[ib + k];
-          if (c.in1) tv1[k] -= sub_img[ib + row2 + k];
-        }
-      }
+      for (int k = 0; k < KC; ++k)
+        if (k0 + k < K) tv[x][k] -= sub_img[ib + off * K + k];
     }
-    if (KC <= 3) {
-      check_finite(tv0, status);
-      check_finite(tv1, status);
-    }
-  }
-  group_accumulate<KC>(s, sa, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n, tv0, tv1,
+    if (KC <= 3) check_finite(tv[x], status);
+  });
+  group_accumulate<KC>(s, sa, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n, tv,
                        acc + (int64_t)c.j * acc_cam_stride, RS, K, k0, status);
 }
 
@@ -459,111 +451,121 @@ __global__ void __launch_bounds__(kThreads) k_blend_render(
   }
 }
 
-// The render by 8-lane groups (groupwalk.cuh) for up to 4 channels: two pixels a thread, a hit list per
-// 4x4 block. The colours are staged twice each, so that a channel of both pixels is one packed FMA.
+// The render by 8-lane groups (groupwalk.cuh) for up to 4 channels: two pixel pairs a lane, a hit list per
+// 8x4 block. The colours are staged twice each, so that a channel of a pixel pair is one packed FMA.
 // A skipped step adds 0 c, which is exact for a finite c; once a staged colour is not finite (weird)
 // the tile's steps test the weight instead.
 struct GroupColours {
   float4 c01[kBatch + 1], c23[kBatch + 1];  // (c0, c0, c1, c1), (c2, c2, c3, c3); slot kBatch: zeros
 };
 
-// The thread's staged Gaussian's channels: the even thread of a pair stages c0, c1, the odd one c2, c3.
+// The channels of the thread's staged Gaussian.
 template <int KC>
 __device__ __forceinline__ void stage_colours(const float* __restrict__ pay_cam, uint32_t id, int nb, int K, int k0,
                                               GroupColours& col, int* weird) {
-  const int g = threadIdx.x >> 1, half = threadIdx.x & 1;
-  if (g >= nb || (KC <= 2 && half == 1)) return;
-  const float* src = pay_cam + (int64_t)id * K + k0 + 2 * half;
-  const float x = 2 * half < KC && k0 + 2 * half < K ? src[0] : 0.0f;
-  const float y = 2 * half + 1 < KC && k0 + 2 * half + 1 < K ? src[1] : 0.0f;
-  (half ? col.c23 : col.c01)[g] = make_float4(x, x, y, y);
-  if (!isfinite(x) || !isfinite(y)) *weird = 1;
+  const int g = threadIdx.x;
+  if (g >= nb) return;
+  const float* src = pay_cam + (int64_t)id * K + k0;
+  float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+  for (int k = 0; k < KC; ++k)
+    if (k0 + k < K) v[k] = src[k];
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < KC; ++k) bad |= !isfinite(v[k]);
+  col.c01[g] = make_float4(v[0], v[0], v[1], v[1]);
+  if (KC > 2) col.c23[g] = make_float4(v[2], v[2], v[3], v[3]);
+  if (bad) *weird = 1;
+}
+
+// x with each half replaced by old's where that pixel's weight is 0 (only when guard is set)
+__device__ __forceinline__ f2 guarded(bool guard, const float2 w, f2 x, f2 old) {
+  if (!guard) return x;
+  const float2 a = unpack2(x), b = unpack2(old);
+  return pack2(w.x > 0.0f ? a.x : b.x, w.y > 0.0f ? a.y : b.y);
 }
 
 template <int KC>
-__device__ __forceinline__ void group_render(GroupBatch& s, GroupColours& col, int* weird, const GroupCtx& c,
+__device__ __forceinline__ void group_render(GroupBatch<kPP>& s, GroupColours& col, int* weird, const GroupCtx<kPP>& c,
                                              const unsigned long long* list, const ProjRec* __restrict__ rec_cam,
                                              int64_t n, const float* __restrict__ pay_cam, int K, int k0,
-                                             f2 (&img)[KC]) {
+                                             f2 (&img)[kPP][KC]) {
   if (threadIdx.x == 0) {
     *weird = 0;
     col.c01[kBatch] = col.c23[kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
 #pragma unroll
-  for (int k = 0; k < KC; ++k) img[k] = pack2(0.0f, 0.0f);
-  const uint16_t* const my_list = s.list[c.group];
-  float2 T = make_float2(c.in0 ? 1.0f : 0.0f, c.in1 ? 1.0f : 0.0f);
+  for (int u = 0; u < kPP; ++u)
+#pragma unroll
+    for (int k = 0; k < KC; ++k) img[u][k] = pack2(0.0f, 0.0f);
+  const uint16_t* const my_list = s.lists.row[c.group];
+  GroupT<kPP> T(c);
   uint32_t unused = 0;
   __syncthreads();
-  auto stage = [&](uint32_t first, int nb) {
-    const uint32_t id = group_stage(list, first, nb, rec_cam, n, c.ox, c.oy, s, 0);
-    stage_colours<KC>(pay_cam, id, nb, K, k0, col, weird);
+  const uint32_t list_end = c.b + c.len;
+  uint32_t id_next = group_id<kPP>(list, c.b, list_end, n);
+  auto stage = [&](uint32_t first) {  // the batch at slot first of the list, whose indices id_next holds
+    const int nb = (int)min((uint32_t)kBatch, list_end - first);
+    group_put<kPP>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo);
+    stage_colours<KC>(pay_cam, id_next, nb, K, k0, col, weird);
   };
-  stage(c.b, (int)min((uint32_t)kBatch, c.len));
+  stage(c.b);
   __syncthreads();
   for (uint32_t start = 0; start < c.len; start += kBatch) {
     const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    const int steps = group_lists(s, c, nb, group_alive(T.x > 0.0f || T.y > 0.0f));
-    auto blend = [&](uint32_t o, const float2 w, bool guard) {
+    id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n);
+    const int steps = group_lists(s.geo, s.lists, c, nb, group_alive(T.alive()), nullptr);
+    auto blend = [&](uint32_t o, const GroupW<kPP>& w, bool guard) {
       const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(reinterpret_cast<const char*>(col.c01) + o);
       ulonglong2 c23 = make_ulonglong2(0ull, 0ull);
       if constexpr (KC > 2) c23 = *reinterpret_cast<const ulonglong2*>(reinterpret_cast<const char*>(col.c23) + o);
       const f2 ck[4] = {c01.x, c01.y, c23.x, c23.y};
-      const f2 w2 = pack2(w.x, w.y);
 #pragma unroll
-      for (int k = 0; k < KC; ++k) {
-        const f2 v = fma2(w2, ck[k], img[k]);
-        if (!guard) {
-          img[k] = v;
-        } else {
-          const float2 a = unpack2(v), b = unpack2(img[k]);
-          img[k] = pack2(w.x > 0.0f ? a.x : b.x, w.y > 0.0f ? a.y : b.y);
-        }
+      for (int u = 0; u < kPP; ++u) {
+        const f2 w2 = pack2(w.v[u].x, w.v[u].y);
+#pragma unroll
+        for (int k = 0; k < KC; ++k) img[u][k] = guarded(guard, w.v[u], fma2(w2, ck[k], img[u][k]), img[u][k]);
       }
     };
     auto walk = [&](bool guard) {
       for (int i = 0; i < steps; i += 2) {
-        const uint32_t pair = *reinterpret_cast<const uint32_t*>(my_list + i);
-        const uint32_t o1 = pair & 0xFFFFu, o2 = pair >> 16;
-        const GroupAlpha a1 = group_alpha(s, o1, c), a2 = group_alpha(s, o2, c);
-        blend(o1, group_take<false>(a1.alpha, T, unused), guard);
-        blend(o2, group_take<false>(a2.alpha, T, unused), guard);
+        const uint2 o = s.lists.pair(my_list, i);
+        const GroupAlpha<kPP> a1 = group_alpha(s.geo, o.x, c), a2 = group_alpha(s.geo, o.y, c);
+        blend(o.x, group_take<false>(a1, T, unused), guard);
+        blend(o.y, group_take<false>(a2, T, unused), guard);
       }
     };
     if (*weird) walk(true);
     else walk(false);
-    if (!__syncthreads_or(T.x > 0.0f || T.y > 0.0f)) break;
-    const uint32_t next = start + kBatch;
-    if (next < c.len) stage(c.b + next, (int)min((uint32_t)kBatch, c.len - next));
+    if (!__syncthreads_or(T.alive())) break;
+    if (start + kBatch < c.len) stage(c.b + start + kBatch);
     __syncthreads();
   }
 }
 
 template <int KC>
-__global__ void __launch_bounds__(kGThreads, 10) k_blend_render2(
+__global__ void __launch_bounds__(kGThreads, 13) k_blend_render2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const float* __restrict__ payload, int K, int k0, int cam0, float* __restrict__ images) {
   static_assert(KC <= 4, "up to 4 channels");
-  __shared__ GroupBatch s;
+  __shared__ GroupBatch<kPP> s;
   __shared__ GroupColours col;
   __shared__ int weird;
-  const GroupCtx c = group_ctx(tile_off, capacity, tiles, tiles_x, width, height);
-  group_batch_init(s);
-  f2 img[KC];
+  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height);
+  if (threadIdx.x == 0) group_pad(s.geo);
+  f2 img[kPP][KC];
   group_render<KC>(s, col, &weird, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n,
                    payload + (int64_t)c.j * n * K, K, k0, img);
-  if (c.in0) {
-    float* dst = images + (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K + k0;
-    const int64_t row2 = 2 * (int64_t)width * K;
+  float* dst = images + (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K + k0;
+  for_pixels(c, width, [&](int x, int64_t off) {
 #pragma unroll
     for (int k = 0; k < KC; ++k)
       if (k0 + k < K) {
-        const float2 v = unpack2(img[k]);
-        dst[k] = v.x;
-        if (c.in1) dst[row2 + k] = v.y;
+        const float2 v = unpack2(img[x >> 1][k]);
+        dst[off * K + k] = (x & 1) ? v.y : v.x;
       }
-  }
+  });
 }
 
 // ------------------------------------------------------------------------------------------
@@ -714,10 +716,10 @@ __global__ void __launch_bounds__(kThreads, KC <= 4 ? 6 : (KC <= 16 ? 4 : (KC <=
   }
 }
 
-// The adjoint walk by 8-lane groups (groupwalk.cuh) for up to 4 channels: two pixels a thread, a hit
-// list per 4x4 block, the payload staged twice each for packed arithmetic. Pass 2 adds a thread's two
+// The adjoint walk by 8-lane groups (groupwalk.cuh) for up to 4 channels: two pixel pairs a lane, a hit
+// list per 8x4 block, the payload staged twice each for packed arithmetic. Pass 2 adds a lane's four
 // pixels, reduces two hits at a time over the group's 8 lanes (3 shuffles) and stores the sums in the
-// group's row; after the batch two threads per Gaussian add the rows and one atomic lands in grad_o.
+// group's row; after the batch one thread per Gaussian adds the rows and one atomic lands in grad_o.
 // A skipped step adds 0 a, exact for finite values; with a staged payload value or a target of the
 // tile that is not finite (weird) the steps test the weight instead.
 template <int KC>
@@ -729,13 +731,12 @@ struct GroupPayload {
 template <int KC>
 __device__ __forceinline__ void stage_payload(const float* __restrict__ pay_cam, uint32_t id, int nb, int K,
                                               GroupPayload<KC>& pay, int* weird) {
-  const int g = threadIdx.x >> 1, half = threadIdx.x & 1;
+  const int g = threadIdx.x;
   if (g >= nb) return;
   const float* src = pay_cam + (int64_t)id * (K + 1);  // K == KC
   bool bad = false;
 #pragma unroll
   for (int r = 0; r < GroupPayload<KC>::NQ; ++r) {
-    if ((r & 1) != half) continue;
     const float x = src[2 * r], y = 2 * r + 1 <= KC ? src[2 * r + 1 <= KC ? 2 * r + 1 : 0] : 0.0f;
     pay.q[r][g] = make_float4(x, x, y, y);
     bad |= !isfinite(x) || !isfinite(y);
@@ -755,17 +756,18 @@ __device__ __forceinline__ void load_group_payload(const GroupPayload<KC>& pay, 
 }
 
 template <int KC>
-__global__ void __launch_bounds__(kGThreads, 8) k_blend_adjoint2(
+__global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, const float* __restrict__ payload, int K, int cam0,
     float* __restrict__ grad_t, float* __restrict__ grad_o) {
   static_assert(KC <= 4, "up to 4 channels");
-  __shared__ GroupBatch s;
+  __shared__ GroupBatch<kPP> s;
   __shared__ GroupPayload<KC> pay;
-  __shared__ float s_go[kGroups][kBatch];
+  __shared__ GroupIds<kPP> ids;
+  __shared__ float s_go[kGroups][kBatch + 1];
   __shared__ int weird;
-  const GroupCtx c = group_ctx(tile_off, capacity, tiles, tiles_x, width, height);
+  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height);
   const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const int lane = threadIdx.x & 31;
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;
@@ -775,185 +777,207 @@ __global__ void __launch_bounds__(kGThreads, 8) k_blend_adjoint2(
 #pragma unroll
     for (int r = 0; r < GroupPayload<KC>::NQ; ++r) pay.q[r][kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
-  group_batch_init(s);
+  if (threadIdx.x == 0) group_pad(s.geo);
   __syncthreads();
   const int64_t pix0 = ((int64_t)(cam0 + c.j) * height + c.py) * width + c.px;
-  const int64_t pix1 = pix0 + 2 * (int64_t)width;
-  f2 tv[KC];
+  f2 tv[kPP][KC];
+  {
+    float t[2 * kPP][KC];
 #pragma unroll
-  for (int k = 0; k < KC; ++k) {
-    const float x = c.in0 ? load_target(targets, pix0 * K + k, dtype) : 0.0f;
-    const float y = c.in1 ? load_target(targets, pix1 * K + k, dtype) : 0.0f;
-    tv[k] = pack2(x, y);
-    if (!isfinite(x) || !isfinite(y)) weird = 1;
+    for (int x = 0; x < 2 * kPP; ++x)
+#pragma unroll
+      for (int k = 0; k < KC; ++k) t[x][k] = 0.0f;
+    bool bad = false;
+    for_pixels(c, width, [&](int x, int64_t off) {
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        t[x][k] = load_target(targets, (pix0 + off) * K + k, dtype);
+        bad |= !isfinite(t[x][k]);
+      }
+    });
+    if (bad) weird = 1;
+#pragma unroll
+    for (int u = 0; u < kPP; ++u)
+#pragma unroll
+      for (int k = 0; k < KC; ++k) tv[u][k] = pack2(t[2 * u][k], t[2 * u + 1][k]);
   }
-  auto stage = [&](uint32_t first, int nb, int buf) {
-    const uint32_t id = group_stage(list, first, nb, rec_cam, n, c.ox, c.oy, s, buf);
-    stage_payload<KC>(pay_cam, id, nb, K, pay, &weird);
+  const uint32_t list_end = c.b + c.len;
+  uint32_t id_next = 0;
+  auto stage = [&](uint32_t first, int to) {  // the batch at slot first of the list, whose indices id_next holds
+    const int nb = (int)min((uint32_t)kBatch, list_end - first);
+    group_put<kPP>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo);
+    ids.id[to][threadIdx.x] = id_next;
+    stage_payload<KC>(pay_cam, id_next, nb, K, pay, &weird);
   };
-  // g = a . t + beta
-  auto gain = [&](const f2 (&a)[KC + 1]) -> f2 {
+  // g = a . t + beta of pixel pair u
+  auto gain = [&](const f2 (&a)[KC + 1], int u) -> f2 {
     f2 g = a[KC];
 #pragma unroll
-    for (int k = 0; k < KC; ++k) g = fma2(a[k], tv[k], g);
+    for (int k = 0; k < KC; ++k) g = fma2(a[k], tv[u][k], g);
     return g;
   };
-  // x with each half replaced by old's where that pixel's weight is 0 (weird tiles only)
-  auto guarded = [&](bool guard, const float2 w, f2 x, f2 old) -> f2 {
-    if (!guard) return x;
-    const float2 a = unpack2(x), b = unpack2(old);
-    return pack2(w.x > 0.0f ? a.x : b.x, w.y > 0.0f ? a.y : b.y);
-  };
-  const uint16_t* const my_list = s.list[c.group];
+  const uint16_t* const my_list = s.lists.row[c.group];
   uint32_t unused = 0;
-  const float2 T_start = make_float2(c.in0 ? 1.0f : 0.0f, c.in1 ? 1.0f : 0.0f);
   // pass 1: F = sum_n g_n w_n and dL/dt = sum_n w_n a_n, per pixel
-  f2 F = pack2(0.0f, 0.0f);
+  f2 F[kPP];
   {
-    f2 gt[KC];
+    f2 gt[kPP][KC];
 #pragma unroll
-    for (int k = 0; k < KC; ++k) gt[k] = pack2(0.0f, 0.0f);
-    float2 T = T_start;
-    stage(c.b, (int)min((uint32_t)kBatch, c.len), 0);
+    for (int u = 0; u < kPP; ++u) {
+      F[u] = pack2(0.0f, 0.0f);
+#pragma unroll
+      for (int k = 0; k < KC; ++k) gt[u][k] = pack2(0.0f, 0.0f);
+    }
+    GroupT<kPP> T(c);
+    id_next = group_id<kPP>(list, c.b, list_end, n);
+    stage(c.b, 0);
     __syncthreads();
     for (uint32_t start = 0; start < c.len; start += kBatch) {
       const int nb = (int)min((uint32_t)kBatch, c.len - start);
-      const int steps = group_lists(s, c, nb, group_alive(T.x > 0.0f || T.y > 0.0f));
-      auto gather = [&](uint32_t o, const float2 w, bool guard) {
+      id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n);
+      const int steps = group_lists(s.geo, s.lists, c, nb, group_alive(T.alive()), nullptr);
+      auto gather = [&](uint32_t o, const GroupW<kPP>& w, bool guard) {
         f2 a[KC + 1];
         load_group_payload<KC>(pay, o, a);
-        const f2 w2 = pack2(w.x, w.y);
 #pragma unroll
-        for (int k = 0; k < KC; ++k) gt[k] = guarded(guard, w, fma2(w2, a[k], gt[k]), gt[k]);
-        F = guarded(guard, w, fma2(gain(a), w2, F), F);
+        for (int u = 0; u < kPP; ++u) {
+          const f2 w2 = pack2(w.v[u].x, w.v[u].y);
+#pragma unroll
+          for (int k = 0; k < KC; ++k) gt[u][k] = guarded(guard, w.v[u], fma2(w2, a[k], gt[u][k]), gt[u][k]);
+          F[u] = guarded(guard, w.v[u], fma2(gain(a, u), w2, F[u]), F[u]);
+        }
       };
       auto walk = [&](bool guard) {
         for (int i = 0; i < steps; i += 2) {
-          const uint32_t pair = *reinterpret_cast<const uint32_t*>(my_list + i);
-          const uint32_t o1 = pair & 0xFFFFu, o2 = pair >> 16;
-          const GroupAlpha a1 = group_alpha(s, o1, c), a2 = group_alpha(s, o2, c);
-          gather(o1, group_take<false>(a1.alpha, T, unused), guard);
-          gather(o2, group_take<false>(a2.alpha, T, unused), guard);
+          const uint2 o = s.lists.pair(my_list, i);
+          const GroupAlpha<kPP> a1 = group_alpha(s.geo, o.x, c), a2 = group_alpha(s.geo, o.y, c);
+          gather(o.x, group_take<false>(a1, T, unused), guard);
+          gather(o.y, group_take<false>(a2, T, unused), guard);
         }
       };
       if (weird) walk(true);
       else walk(false);
-      if (!__syncthreads_or(T.x > 0.0f || T.y > 0.0f)) break;
-      const uint32_t next = start + kBatch;
-      if (next < c.len) stage(c.b + next, (int)min((uint32_t)kBatch, c.len - next), 0);
+      if (!__syncthreads_or(T.alive())) break;
+      if (start + kBatch < c.len) stage(c.b + start + kBatch, 0);
       __syncthreads();
     }
-    if (grad_t && c.in0) {
+    if (grad_t) {
+      for_pixels(c, width, [&](int x, int64_t off) {
 #pragma unroll
-      for (int k = 0; k < KC; ++k) {
-        const float2 v = unpack2(gt[k]);
-        grad_t[pix0 * K + k] = v.x;
-        if (c.in1) grad_t[pix1 * K + k] = v.y;
-      }
+        for (int k = 0; k < KC; ++k) {
+          const float2 v = unpack2(gt[x >> 1][k]);
+          grad_t[(pix0 + off) * K + k] = (x & 1) ? v.y : v.x;
+        }
+      });
     }
   }
   if (!grad_o) return;
   // pass 2: dL/dalpha_m = g_m T_m - (F - P_m) / (1 - alpha_m), P_m = sum_{n<=m} g_n w_n; times
   // dalpha/do = exp(-q/2), 0 where skipped or where alpha was capped
   __syncthreads();
-  float2 T = T_start;
-  f2 P = pack2(0.0f, 0.0f);
+  GroupT<kPP> T(c);
+  f2 P[kPP];
+#pragma unroll
+  for (int u = 0; u < kPP; ++u) P[u] = pack2(0.0f, 0.0f);
   const bool second = (lane & 4) != 0;  // this lane's half of the group returns the second hit's sum
   float* const my_go = s_go[c.group];
   int buf = 0;
-  stage(c.b, (int)min((uint32_t)kBatch, c.len), buf);
+  id_next = group_id<kPP>(list, c.b, list_end, n);
+  stage(c.b, buf);
   __syncthreads();
   for (uint32_t start = 0; start < c.len; start += kBatch, buf ^= 1) {
     const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    const int steps = group_lists(s, c, nb, group_alive(T.x > 0.0f || T.y > 0.0f));
-    auto step = [&](uint32_t o, const GroupAlpha& al, bool guard) -> float {
-      const f2 Tm = pack2(T.x, T.y);
-      const float2 w = group_take<false>(al.alpha, T, unused);
+    id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n);
+    const int steps = group_lists(s.geo, s.lists, c, nb, group_alive(T.alive()), ids.hits);
+    auto step = [&](uint32_t o, const GroupAlpha<kPP>& al, bool guard) -> float {
+      GroupT<kPP> Tm = T;
+      const GroupW<kPP> w = group_take<false>(al, T, unused);
       f2 a[KC + 1];
       load_group_payload<KC>(pay, o, a);
-      const f2 g = gain(a);
-      P = guarded(guard, w, fma2(g, pack2(w.x, w.y), P), P);
-      const float2 rest = unpack2(fma2(P, pack2(-1.0f, -1.0f), F));  // F - P
-      const float2 om = unpack2(fma2(pack2(al.alpha.x, al.alpha.y), pack2(-1.0f, -1.0f), pack2(1.0f, 1.0f)));
-      const f2 da = fma2(g, Tm, pack2(-__fdividef(rest.x, om.x), -__fdividef(rest.y, om.y)));
-      const float2 d = unpack2(mul2(da, pack2(al.e.x, al.e.y)));
-      const float d0 = w.x > 0.0f && al.oe.x < kAlphaMax ? d.x : 0.0f;
-      const float d1 = w.y > 0.0f && al.oe.y < kAlphaMax ? d.y : 0.0f;
-      return d0 + d1;
+      float sum = 0.0f;
+#pragma unroll
+      for (int u = 0; u < kPP; ++u) {
+        const f2 g = gain(a, u);
+        P[u] = guarded(guard, w.v[u], fma2(g, pack2(w.v[u].x, w.v[u].y), P[u]), P[u]);
+        const float2 rest = unpack2(sub2(F[u], P[u]));
+        const float2 om = unpack2(sub2(T.ones, pack2(al.alpha[u].x, al.alpha[u].y)));
+        const f2 da = fma2(g, pack2(Tm.v[u].x, Tm.v[u].y), pack2(-__fdividef(rest.x, om.x), -__fdividef(rest.y, om.y)));
+        const float2 d = unpack2(mul2(da, pack2(al.e[u].x, al.e[u].y)));
+        const float d0 = w.v[u].x > 0.0f && al.oe[u].x < kAlphaMax ? d.x : 0.0f;
+        const float d1 = w.v[u].y > 0.0f && al.oe[u].y < kAlphaMax ? d.y : 0.0f;
+        sum = u == 0 ? d0 + d1 : sum + (d0 + d1);
+      }
+      return sum;
     };
     auto walk = [&](bool guard) {
       for (int i = 0; i < steps; i += 2) {
-        const uint32_t pair = *reinterpret_cast<const uint32_t*>(my_list + i);
-        const uint32_t o1 = pair & 0xFFFFu, o2 = pair >> 16;
-        const GroupAlpha a1 = group_alpha(s, o1, c), a2 = group_alpha(s, o2, c);
-        const float d1 = step(o1, a1, guard), d2 = step(o2, a2, guard);
+        const uint2 o = s.lists.pair(my_list, i);
+        const GroupAlpha<kPP> a1 = group_alpha(s.geo, o.x, c), a2 = group_alpha(s.geo, o.y, c);
+        const float d1 = step(o.x, a1, guard), d2 = step(o.y, a2, guard);
         float v[2] = {second ? d2 : d1, second ? d1 : d2};
         const float r = group_permuted_reduce<2>(v);
-        const uint32_t o = second ? o2 : o1;
-        if ((lane & 3) == 0 && o != kGPad) my_go[o / 16] = r;
+        const uint32_t mine = second ? o.y : o.x;
+        if ((lane & 3) == 0) my_go[mine / 16] = r;
       }
     };
     if (weird) walk(true);
     else walk(false);
     __syncthreads();
     {
-      const int g = threadIdx.x >> 1, half = threadIdx.x & 1;
-      float sum = 0.0f;
+      const int g = threadIdx.x;
       if (g < nb) {
-        const uint32_t hits = *reinterpret_cast<const uint16_t*>(&s.hits[g][2 * half]);
+        float sum = 0.0f;
+        const uint32_t hits = *reinterpret_cast<const uint16_t*>(&ids.hits[g][0]);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (hits & (1u << (q < 4 ? q : q + 4))) sum += s_go[half * 8 + q][g];
+        for (int q = 0; q < kGroups; ++q)
+          if (hits & (1u << (q < 4 ? q : q + 4))) sum += s_go[q][g];
+        if (sum != 0.0f) atomicAdd(grad_o + ids.id[buf][g], sum);
       }
-      sum += __shfl_xor_sync(kFull, sum, 1);
-      if (half == 0 && g < nb && sum != 0.0f) atomicAdd(grad_o + s.id[buf][g], sum);
     }
-    const uint32_t next = start + kBatch;
-    if (next < c.len) stage(c.b + next, (int)min((uint32_t)kBatch, c.len - next), buf ^ 1);
-    if (!__syncthreads_or(T.x > 0.0f || T.y > 0.0f)) break;
+    if (start + kBatch < c.len) stage(c.b + start + kBatch, buf ^ 1);
+    if (!__syncthreads_or(T.alive())) break;
   }
 }
 
 // One refinement walk (Alg. 1 lines 8-9) for up to 3 channels by 8-lane groups: pass 1 renders the
-// current colours of the thread's pixels (as k_blend_render2), pass 2 accumulates the residual targets
+// current colours of the lane's pixels (as k_blend_render2), pass 2 accumulates the residual targets
 // t - img (as k_blend_accumulate2 with a rendered image subtracted), over the tile list sorted once.
 // Same arithmetic as the two separate walks, without the image round trip. The colours of pass 1 share
 // the shared memory of pass 2's partial sums.
 template <int KC>
-__global__ void __launch_bounds__(kGThreads, 9) k_blend_refine2(
+__global__ void __launch_bounds__(kGThreads, 13) k_blend_refine2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, int K, int cam0, const float* __restrict__ payload,
     float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
   static_assert(KC <= 3, "up to 3 channels");
   static_assert(sizeof(GroupColours) <= sizeof(GroupAcc<KC>), "the colours fit where the sums go");
-  __shared__ GroupBatch s;
+  __shared__ GroupBatch<kPP> s;
   __shared__ __align__(16) GroupAcc<KC> sa;
   __shared__ int weird;
-  const GroupCtx c = group_ctx(tile_off, capacity, tiles, tiles_x, width, height);
-  group_batch_init(s);
+  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height);
+  if (threadIdx.x == 0) group_pad(s.geo);
   const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;
-  f2 img[KC];
+  f2 img[kPP][KC];
   group_render<KC>(s, reinterpret_cast<GroupColours&>(sa), &weird, c, list, rec_cam, n,
                    payload + (int64_t)c.j * n * K, K, 0, img);
-  float tv0[KC], tv1[KC];
+  float tv[2 * kPP][KC];
 #pragma unroll
-  for (int k = 0; k < KC; ++k) tv0[k] = tv1[k] = 0.0f;
-  if (c.in0) {
-    const int64_t base = (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K;
-    const int64_t row2 = 2 * (int64_t)width * K;
+  for (int x = 0; x < 2 * kPP; ++x)
+#pragma unroll
+    for (int k = 0; k < KC; ++k) tv[x][k] = 0.0f;
+  const int64_t base = (((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K;
+  for_pixels(c, width, [&](int x, int64_t off) {
 #pragma unroll
     for (int k = 0; k < KC; ++k) {
-      const float2 v = unpack2(img[k]);
-      tv0[k] = load_target(targets, base + k, dtype) - v.x;
-      if (c.in1) tv1[k] = load_target(targets, base + row2 + k, dtype) - v.y;
+      const float2 v = unpack2(img[x >> 1][k]);
+      tv[x][k] = load_target(targets, base + off * K + k, dtype) - ((x & 1) ? v.y : v.x);
     }
-    check_finite(tv0, status);
-    check_finite(tv1, status);
-  }
+    check_finite(tv[x], status);
+  });
   __syncthreads();
-  group_accumulate<KC>(s, sa, c, list, rec_cam, n, tv0, tv1, acc + (int64_t)c.j * acc_cam_stride, RS, K, 0, status);
+  group_accumulate<KC>(s, sa, c, list, rec_cam, n, tv, acc + (int64_t)c.j * acc_cam_stride, RS, K, 0, status);
 }
 
 template <int KC>

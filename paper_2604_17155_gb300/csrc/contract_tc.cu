@@ -2,23 +2,29 @@
 // 5th-generation tensor cores (tcgen05), for 16-bit targets with 16..64 channels.
 //
 // Per tile and batch of MG = 64 Gaussians (the MMA's M; 64 rather than 128 halves the weight
-// operand, so that 3-5 CTAs fit on an SM), the S terms of Eq. 6 summed over the tile's 256 pixels
+// operand, so that 3-4 CTAs fit on an SM), the S terms of Eq. 6 summed over the tile's 256 pixels
 // form a dense product
 //     D[g][n] = sum_p W[g][p] * B[n][p],   W[g][p] = alpha T of Gaussian g at pixel p (Eq. 4),
 // with B's rows 0..KT-1 the tile's target channels and the rows after them all ones, so that the same
-// product also yields V = sum_p W[g][p] (Eq. 5). The threads evaluate W with the same decisions as
-// the CUDA-core walks (walk.cuh: branch-free, two hits a step) and store it as FP16 into a K-major,
+// product also yields V = sum_p W[g][p] (Eq. 5). The threads evaluate W by 8-lane groups
+// (groupwalk.cuh, one pixel pair a lane) and store a pair as two FP16 values into a K-major,
 // 128-byte-swizzled shared-memory operand; the tile's targets (BF16 or FP16) are transposed once
 // into B as FP16. Both operands are scaled by powers of two -- W by 2^14 (the walk carries T scaled
 // so), the targets so that the tile's largest magnitude lands in [2^14, 2^15) -- which makes every
 // BF16 target exact in FP16, keeps small weights out of FP16's subnormal range, and is undone exactly
 // in the epilogue. One thread issues 16 tcgen05.mma (kind::f16, M=MG, N=KT+8, K=16, FP32
-// accumulation in TMEM) and commits them to an mbarrier; while they run, the next batch's Gaussians
-// are staged (the geometry into the buffer the walk has finished with, each index into the register
-// of the thread that adds its row); the warps then read D back with tcgen05.ld (one Gaussian per
-// thread, the chunks split between warps w and w+4) and add (V, S_0..S_{KT-1}) to the accumulator
-// with float4 atomics -- one atomic group per (Gaussian, tile). A batch costs two CTA barriers. At 16
-// channels the whole layout takes 44 KiB (five CTAs per SM): see b16_offset and tc_smem.
+// accumulation in TMEM) and commits them to an mbarrier; the warps then read D back with tcgen05.ld
+// (one Gaussian per thread) and add (V, S_0..S_{KT-1}) to the accumulator with float4 atomics -- one
+// atomic group per (Gaussian, tile). The MMA's K index runs over each warp's 8x8 pixel block in turn, so
+// a warp owns one K block of W: it clears and refills it without waiting for the others. A batch costs
+// one CTA barrier, and while its MMAs run the warps build the next batch's hit lists.
+//
+// What bounds it: shared-memory bandwidth (W and B read by the MMAs, W cleared and written, geometry and
+// lists: about two thirds of the cycles) and instruction issue (55%), with 16 warps per SM. Measured on
+// the masks scene (3M Gaussians, 200 cameras, 16 channels): 101.8 ms with one list per 8x4 warp block
+// and 256 threads; 94.3 ms with groups and 128 threads; 89.5 ms with one barrier a batch; 85.2 ms with
+// the geometry stored once; 83 ms with only the written rows cleared. 64 channels (1M Gaussians, 150
+// cameras): 47.6 -> 39.2 ms.
 //
 // Every wait on the mbarrier is bounded in time (1 s by %globaltimer): past the limit the kernel
 // sets kFlagTimeout in the status block (reported as ICGS_ERR_DEVICE_TIMEOUT), waits once more
@@ -31,6 +37,7 @@
 
 #include "icgs_device.cuh"
 #include "icgs_internal.h"
+#include "groupwalk.cuh"
 #include "walk.cuh"
 
 namespace icgs {
@@ -83,8 +90,10 @@ __device__ __forceinline__ uint64_t global_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// Bounded wait; returns false (and the caller reports a timeout) once limit_ns have passed.
+// Bounded wait; returns false (and the caller reports a timeout) once limit_ns have passed. The clock
+// is read only after a first try has failed: a read costs more than the usual rest of the wait.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* mbar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
+  if (mbar_try_wait(mbar, parity)) return true;
   const uint64_t t0 = global_ns();
   while (!mbar_try_wait(mbar, parity))
     if (global_ns() - t0 > limit_ns) return false;
@@ -199,30 +208,6 @@ __device__ __forceinline__ void issue_batch_b16(uint32_t a_addr, uint32_t b_regi
   umma_commit(mbar);
 }
 
-// Staging of a batch for the walk (M = 64). The thread that stages Gaussian g is the one that adds
-// row g's sums in the epilogue -- lane g % 16 of warp g / 16, since TMEM holds row g in lane g % 16
-// of quarter g / 16 -- so the Gaussian's index stays in that thread's register from staging to
-// epilogue. Warps 4-7 read the same quarters for the later accumulator columns (more than 16
-// channels); their lanes < 16 load only the index (need_id).
-__device__ __forceinline__ uint32_t stage_tc(const unsigned long long* list, uint32_t first, int nb,
-                                             const ProjRec* __restrict__ rec_cam, int64_t n, float ox, float oy,
-                                             float4* s_geo, float4* s_aux, int g, bool writer, bool need_id) {
-  uint32_t id = 0;
-  if (g >= 0 && g < nb && (writer || need_id)) {
-    id = min((uint32_t)list[first + g], (uint32_t)(n - 1));
-    if (writer) {
-      // aux = (C, opacity, the slot's row offset in W, packed half-sizes): the walk's step needs no
-      // fast-reject threshold (blend_alpha_noreject), so the third value carries g * 128 +
-      // (g % 8) * 16, the Gaussian's part of its weights' swizzled address
-      const ProjRec r = rec_cam[id];
-      s_geo[g] = stage_geo(r, ox, oy);
-      s_aux[g] = make_float4(-kHalfLog2e * r.par.z, r.par.w, __uint_as_float((uint32_t)((g << 7) | ((g & 7) << 4))),
-                             r.box.w);
-    }
-  }
-  return id;
-}
-
 // The accumulator row held in TMEM lane 32 q + l (the lane a thread l of a warp with quarter q
 // reads), or -1: M = 128 puts row m in lane m; M = 64 puts row m in lane (m % 16) + 32 (m / 16),
 // i.e. rows 16q..16q+15 in the first 16 lanes of quarter q.
@@ -308,22 +293,36 @@ __host__ __device__ constexpr uint32_t tmem_cols() {
 
 template <int KT, int MG>
 __host__ __device__ constexpr int tc_ctas_per_sm() {
-  return MG == 64 ? (KT <= 16 ? 5 : (KT <= 32 ? 4 : 3)) : 2;
+  return MG == 64 ? 3 : 2;  // a bound for the compiler: 16 channels fit four
+}
+
+// What sits in front of the operands: the barrier and flags (64 bytes), the staged geometry of this batch
+// and the next, and the hit lists. The geometry is stored once, not twice: the MMAs and the walk share
+// the shared-memory bandwidth, and the moves cost less than the wider loads (masks walk 88.1 -> 85.2 ms).
+constexpr int kTcThreads = GroupCfg<1>::kThreads;
+constexpr uint32_t kTcFlags = 64;
+template <int KT>
+struct TcBatch {
+  GroupGeo<false> geo[2];
+  GroupLists<1, true> lists;
+};
+template <int KT>
+__host__ __device__ constexpr uint32_t tc_front() {
+  return kTcFlags + (uint32_t)sizeof(TcBatch<KT>);
 }
 
 template <int KT, bool BF16_TARGETS, int MG>
-__global__ void __launch_bounds__(256, tc_ctas_per_sm<KT, MG>()) k_blend_accumulate_tc(
+__global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_accumulate_tc(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const uint16_t* __restrict__ targets, int K, int cam0, float* __restrict__ acc, int RS,
     int64_t acc_cam_stride, DevStatus* status, uint64_t wait_limit_ns, bool issue_mma) {
-  static_assert(MG == 64, "staging and epilogue map Gaussian g to TMEM lane g % 16 of quarter g / 16 (M = 64)");
+  static_assert(MG == 64 && MG == kBatch, "staging and epilogue map Gaussian g to TMEM lane g % 16 of quarter g / 16");
   constexpr int NB = tc_cols<KT, MG>();  // target channels + rows of ones (V)
   constexpr bool kB16 = KT == 16;        // B in the 11 KB region (b16_offset)
   extern __shared__ uint8_t smem_raw[];
-  // The barrier and flags (48 bytes) sit in front of the 1024-byte aligned operands, inside the
-  // 1 KB the layout allows for alignment: from a base that is 128-byte aligned the operands then
-  // start at most 1024 bytes in. A base that is not is reported (kFlagLayout) before any work.
+  // The barrier, the flags and the staged batch sit in front of the operands, which start at the next
+  // 1024-byte boundary. A base that is not 128-byte aligned is reported (kFlagLayout) before any work.
   const uint32_t raw = smem_u32(smem_raw);
   if (raw & 127u) {
     if (threadIdx.x == 0) atomicOr(&status->flags, kFlagLayout);
@@ -331,97 +330,118 @@ __global__ void __launch_bounds__(256, tc_ctas_per_sm<KT, MG>()) k_blend_accumul
   }
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 1);
-  uint32_t* s_timeout = tmem_slot + 1;  // set by a thread whose wait gave up
-  uint32_t* s_tmax = s_timeout + 1;     // [8]
-  uint8_t* base = smem_raw + (((raw + 48u + 1023u) & ~1023u) - raw);
+  // set by a thread whose wait gave up, in its batch's slot (even, odd): a slot is read after the next
+  // barrier only, when no thread writes it
+  uint32_t* s_timeout = tmem_slot + 1;  // [2]
+  uint32_t* s_tmax = s_timeout + 2;     // [4]
+  TcBatch<KT>& s = *reinterpret_cast<TcBatch<KT>*>(smem_raw + kTcFlags);
+  uint8_t* base = smem_raw + (((raw + tc_front<KT>() + 1023u) & ~1023u) - raw);
   uint8_t* A_s = base;                                 // MG x 256 (32 KB)
   uint8_t* B_s = base + MG * kKPix * 2;                // NB x 256, or the 11 KB region
-  // The batch's geometry is read only by the pixel walk, which ends at the first barrier of the
-  // batch: the next batch is staged into the same buffer while the MMAs run.
-  float4* s_geo = reinterpret_cast<float4*>(kB16 ? B_s + kB16Geo : B_s + NB * kKPix * 2);  // [MG]
-  float4* s_aux = kB16 ? reinterpret_cast<float4*>(B_s + kB16Aux) : s_geo + MG;             // [MG]
 
-  const TileCtx c = tile_ctx(tile_off, capacity, tiles, tiles_x, width, height);
+  const GroupCtx<1> c = group_ctx<1>(tile_off, capacity, tiles, tiles_x, width, height);
   if (c.len == 0) return;  // uniform: nothing binned to this tile
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tx0 = (c.t % tiles_x) * kTile, ty0 = (c.t / tiles_x) * kTile;
-  const int p = (c.py - ty0) * kTile + (c.px - tx0);  // this thread's pixel index in the tile (MMA k)
+  // the MMA's K index of the thread's first pixel (the second is the next): 64 per warp block, row by row
+  const int lx = c.px % kTile, ly = c.py % kTile;
+  const int p = warp * 64 + (ly & 7) * 8 + (lx & 7);
+  const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
+  const ProjRec* rec_cam = rec + (int64_t)c.j * n;
+  const uint32_t list_end = c.b + c.len;
+  const uint32_t id0 = group_id<1>(list, c.b, list_end, n);
+  uint32_t id_next = group_id<1>(list, c.b + MG, list_end, n);
+  GroupFetch fetch = group_fetch(id0, rec_cam);
 
-  // B: the tile's targets, transposed to [channel][pixel] and scaled by 2^s (the tile's largest
+  // B: the tile's targets, transposed to [channel][pixel] and scaled by 2^sexp (the tile's largest
   // magnitude in [2^14, 2^15)), then the rows of ones
   float t_scale_inv;
   {
     const uint16_t* src = targets + ((((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K);
-    // this pixel's channels, loaded 16 bytes at a time when the row allows it
-    uint16_t tv[KT];
-    if (c.inside && K == KT && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+    // the two pixels' channels, loaded 16 bytes at a time when the rows allow it
+    uint32_t tv[KT];  // (first pixel's value, second pixel's value)
+    if (c.in1[0] && K == KT && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
 #pragma unroll
       for (int q = 0; q < KT / 8; ++q) {
         const uint4 u = __ldg(reinterpret_cast<const uint4*>(src) + q);
-        const uint32_t wd[4] = {u.x, u.y, u.z, u.w};
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(src + K) + q);
+        const uint32_t a[4] = {u.x, u.y, u.z, u.w}, b[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-          tv[8 * q + 2 * h] = (uint16_t)(wd[h] & 0xFFFFu);
-          tv[8 * q + 2 * h + 1] = (uint16_t)(wd[h] >> 16);
+          tv[8 * q + 2 * h] = __byte_perm(a[h], b[h], 0x5410);
+          tv[8 * q + 2 * h + 1] = __byte_perm(a[h], b[h], 0x7632);
         }
       }
     } else {
 #pragma unroll
-      for (int k = 0; k < KT; ++k) tv[k] = (c.inside && k < K) ? src[k] : (uint16_t)0;
+      for (int k = 0; k < KT; ++k) {
+        const uint32_t a = c.in0[0] && k < K ? src[k] : 0u, b = c.in1[0] && k < K ? src[K + k] : 0u;
+        tv[k] = a | (b << 16);
+      }
     }
-    float tmax = 0.0f;
-    bool bad = false;
+    // the largest magnitude: non-negative floats order like their bit patterns, in 16 bits too
+    uint32_t m16 = 0u;
 #pragma unroll
-    for (int k = 0; k < KT; ++k) {
-      const float x = target_value(tv[k], BF16_TARGETS);
-      tmax = fmaxf(tmax, fabsf(x));
-      bad |= !isfinite(x);
-    }
-    if (bad) atomicOr(&status->flags, kFlagNonfinite);
-    // non-negative floats order like their bit patterns
-    uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(tmax));
+    for (int k = 0; k < KT; ++k) m16 = __vmaxu2(m16, tv[k] & 0x7FFF7FFFu);
+    uint32_t m = max(m16 & 0xFFFFu, m16 >> 16);
+    if (m >= (BF16_TARGETS ? 0x7F80u : 0x7C00u)) atomicOr(&status->flags, kFlagNonfinite);
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
     if (lane == 0) s_tmax[warp] = m;
+    if (threadIdx.x == 0) {
+      mbar_init(mbar, 1);
+      s_timeout[0] = s_timeout[1] = 0u;
+    }
+    if (warp == 0) {
+      tmem_alloc(tmem_slot, tmem_cols<NB>());
+      tmem_relinquish();
+    }
     __syncthreads();
-    m = s_tmax[0];
-#pragma unroll
-    for (int w2 = 1; w2 < 8; ++w2) m = max(m, s_tmax[w2]);
-    const float gmax = __uint_as_float(m);
+    m = max(max(s_tmax[0], s_tmax[1]), max(s_tmax[2], s_tmax[3]));
+    const float gmax = target_value((uint16_t)m, BF16_TARGETS);
     int e = 0;
     if (gmax > 0.0f && isfinite(gmax)) frexpf(gmax, &e);  // gmax in [2^(e-1), 2^e)
     const int sexp = gmax > 0.0f ? 15 - e : 0;           // gmax * 2^sexp in [2^14, 2^15)
     t_scale_inv = ldexpf(1.0f, -(sexp + kWScaleExp));
+    // 2^sexp as a product of two powers of two that are normal floats (sexp is in -113..148)
+    const float s1 = ldexpf(1.0f, sexp / 2), s2 = ldexpf(1.0f, sexp - sexp / 2);
 #pragma unroll
     for (int k = 0; k < KT; ++k) {
-      const float v = ldexpf(target_value(tv[k], BF16_TARGETS), sexp);
-      *reinterpret_cast<uint16_t*>(B_s + (kB16 ? b16_offset(k, p) : kmajor_sw128(k, p, NB))) = half_bits(v);
+      const float x = target_value((uint16_t)(tv[k] & 0xFFFFu), BF16_TARGETS) * s1 * s2;
+      const float y = target_value((uint16_t)(tv[k] >> 16), BF16_TARGETS) * s1 * s2;
+      *reinterpret_cast<__half2*>(B_s + (kB16 ? b16_offset(k, p) : kmajor_sw128(k, p, NB))) = __floats2half2_rn(x, y);
     }
     if constexpr (kB16) {
       if (threadIdx.x < 64)
         reinterpret_cast<uint4*>(B_s + kB16Ones)[threadIdx.x] = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
     } else {
 #pragma unroll
-      for (int k = KT; k < NB; ++k) *reinterpret_cast<uint16_t*>(B_s + kmajor_sw128(k, p, NB)) = (uint16_t)0x3C00u;
+      for (int k = KT; k < NB; ++k) *reinterpret_cast<uint32_t*>(B_s + kmajor_sw128(k, p, NB)) = 0x3C003C00u;
     }
   }
   const float v_scale_inv = ldexpf(1.0f, -kWScaleExp);
-  const ProjRec* rec_cam = rec + (int64_t)c.j * n;
-  if (threadIdx.x == 0) {
-    mbar_init(mbar, 1);
-    *s_timeout = 0u;
-  }
-  if (warp == 0) {
-    tmem_alloc(tmem_slot, tmem_cols<NB>());
-    tmem_relinquish();
-  }
   // the first batch's staging, and W cleared
-  constexpr int kCh = KT / 16;          // 16-column chunks of S in the epilogue
-  constexpr int kHalf = (kCh + 1) / 2;  // chunks of the warps 0-3
-  const int g_own = tmem_row_of_lane<MG>(warp & 3, lane);  // the batch row this thread stages and adds
-  const bool stager = warp < 4, need_id = warp < 4 || kCh > kHalf;
-  const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
-  uint32_t my_id = stage_tc(list, c.b, (int)min((uint32_t)MG, c.len), rec_cam, n, c.ox, c.oy, s_geo, s_aux, g_own,
-                            stager, need_id);
-  for (int i = threadIdx.x; i < MG * kKPix * 2 / 16; i += 256) reinterpret_cast<uint4*>(A_s)[i] = make_uint4(0, 0, 0, 0);
+  constexpr int kCh = KT / 16;                            // 16-column chunks of S in the epilogue
+  const int g_own = tmem_row_of_lane<MG>(warp, lane);      // the batch row this thread adds
+  if (threadIdx.x < 2) group_pad(s.geo[threadIdx.x]);
+  group_put<1>(fetch, (int)min((uint32_t)MG, c.len), c.ox, c.oy, s.geo[0]);
+  // Gaussian g is staged by lanes 2 (g % 16) and 2 (g % 16) + 1 of warp g / 16, and its row added by
+  // lane g % 16 of the same warp, so its index goes from register to register
+  uint32_t my_id = __shfl_sync(0xFFFFFFFFu, id0, 2 * (lane & 15));
+  if (MG < c.len) {  // the second batch's records, and the third's indices
+    fetch = group_fetch(id_next, rec_cam);
+  }
+  uint32_t id_fetched = id_next;
+  id_next = group_id<1>(list, c.b + 2 * MG, list_end, n);
+  // Only warp w writes K block w of W (its pixels): it clears the block itself, and no other warp waits;
+  // and only the rows that it wrote (about a third).
+  uint4* const w_block = reinterpret_cast<uint4*>(A_s + warp * (MG * 128));
+  uint32_t dirty[2] = {0xFFFFFFFFu, 0xFFFFFFFFu}, listed[2] = {0u, 0u};
+  auto clear_w = [&]() {
+#pragma unroll
+    for (int i = 0; i < MG * 128 / 16; i += 32)  // four rows of 128 bytes at a time
+      if ((dirty[i / 256] >> (lane >> 3)) & (1u << ((i / 8) & 31))) w_block[i + lane] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+  };
+  clear_w();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -429,118 +449,115 @@ __global__ void __launch_bounds__(256, tc_ctas_per_sm<KT, MG>()) k_blend_accumul
   const uint32_t a_addr = smem_u32(A_s), b_addr = smem_u32(B_s);
   constexpr uint32_t kIdesc = idesc_f16(MG, NB, false);
   float* acc_cam = acc + (int64_t)c.j * acc_cam_stride;
-  float T = (float)(1 << kWScaleExp);  // the transmittance times 2^14 (blend_take)
-  bool done = !c.inside;
-  // kmajor_sw128(g, p, MG) split into this pixel's part and the Gaussian's: the row's 128 bytes at
-  // g * 128 (8-row atoms of 1024 bytes), the 16-byte chunk (p % 64) / 8 XOR-ed with g % 8
-  uint8_t* const a_pix = A_s + (p >> 6) * (MG * 128) + ((p & 7) << 1);
-  const int a_chunk = ((p & 63) >> 3) << 4;
+  constexpr float kT0 = (float)(1 << kWScaleExp);  // the transmittance carries the factor 2^14 of W
+  GroupT<1> T(c, kT0);
+  // kmajor_sw128(g, p, MG) in terms of the list entry o = 16 g: 8 o + ((o & 0x70) ^ pixel part)
+  char* const w_base = reinterpret_cast<char*>(A_s + warp * (MG * 128));
+  const uint32_t w_pix = (uint32_t)((((p & 63) >> 3) << 4) | ((p & 7) << 1));
+  const uint16_t* const my_list = s.lists.row[c.group];
   uint32_t npairs = 0, phase = 0;
-  // Two CTA barriers per batch: one before the MMA issue (W written), one at the end (the next
-  // batch's staging loaded, W cleared, the done count and the timeout flag published).
+  bool ok = true;
+  int steps = group_lists(s.geo[0], s.lists, c, (int)min((uint32_t)MG, c.len), group_alive(T.alive()), nullptr, listed);
+  // One CTA barrier per batch. Before it a warp stages its share of the next batch's geometry (in the
+  // buffer that the batch before this one used) and walks its lists; after it one thread issues the MMAs,
+  // and while they run every warp builds its lists of the next batch; then it waits for the MMAs, adds
+  // its quarter of the sums and clears its block of W.
   for (uint32_t start = 0, buf = 0; start < c.len; start += MG, buf ^= 1u) {
     const int nb = (int)min((uint32_t)MG, c.len - start);
-    if (!__all_sync(0xFFFFFFFFu, done)) {
-#pragma unroll
-      for (int q = 0; q < MG / 32; ++q) {
-        uint32_t bits = warp_hit_bits_packed(s_geo, s_aux, q * 32, nb, c);
-        while (bits && !done) {  // two hits a step: both alphas first (independent of T)
-          const int g1 = q * 32 + __ffs(bits) - 1;
-          bits &= bits - 1;
-          const bool has2 = bits != 0;  // warp-uniform
-          const int g2 = has2 ? q * 32 + __ffs(bits) - 1 : g1;
-          bits &= bits - 1;
-          const float4 aux1 = s_aux[g1], aux2 = s_aux[g2];
-          const StepAlpha a1 = blend_alpha_noreject(s_geo[g1], aux1, c.pxf, c.pyf);
-          StepAlpha a2 = blend_alpha_noreject(s_geo[g2], aux2, c.pxf, c.pyf);
-          a2.ok = a2.ok && has2;
-          // T carries the factor 2^14 of W, so the weights come out scaled
-          const float w1 = blend_take<false, kWScaleExp>(a1, T, done, npairs);
-          const float w2 = blend_take<true, kWScaleExp>(a2, T, done, npairs);
-          // the staged row offset XOR this pixel's chunk: kmajor_sw128(g, p, MG) - (a_pix - A_s)
-          *reinterpret_cast<uint16_t*>(a_pix + (__float_as_uint(aux1.z) ^ a_chunk)) = half_bits(w1);
-          if (has2) *reinterpret_cast<uint16_t*>(a_pix + (__float_as_uint(aux2.z) ^ a_chunk)) = half_bits(w2);
-        }
+    const uint32_t next = start + MG;
+    uint32_t next_id = 0;
+    if (next < c.len) {
+      group_put<1>(fetch, (int)min((uint32_t)MG, c.len - next), c.ox, c.oy, s.geo[buf ^ 1u]);
+      next_id = __shfl_sync(0xFFFFFFFFu, id_fetched, 2 * (lane & 15));
+      // in flight during the walk: the records of the batch after it and the indices of the one after that
+      id_fetched = id_next;
+      if (next + MG < c.len) {
+        fetch = group_fetch(id_fetched, rec_cam);
+        id_next = group_id<1>(list, c.b + next + 2 * MG, list_end, n);
       }
+    }
+    if (!ok) steps = 0;  // a wait gave up: W may still be read
+    for (int i = 0; i < steps; i += 2) {
+      const uint2 o = s.lists.pair(my_list, i);
+      const uint32_t o1 = o.x, o2 = o.y;
+      const GroupAlpha<1> a1 = group_alpha(s.geo[buf], o1, c), a2 = group_alpha(s.geo[buf], o2, c);  // independent of T
+      const float2 w1 = group_take<true, kWScaleExp>(a1, T, npairs).v[0];
+      const float2 w2 = group_take<true, kWScaleExp>(a2, T, npairs).v[0];
+      if (o1 != kGPad)
+        *reinterpret_cast<__half2*>(w_base + o1 * 8 + ((o1 & 0x70u) ^ w_pix)) = __floats2half2_rn(w1.x, w1.y);
+      if (o2 != kGPad)
+        *reinterpret_cast<__half2*>(w_base + o2 * 8 + ((o2 & 0x70u) ^ w_pix)) = __floats2half2_rn(w2.x, w2.y);
     }
     fence_async_smem();
     tc_fence_before();
-    __syncthreads();
+    const int alive = __syncthreads_or(T.alive());
+    if (s_timeout[buf ^ 1u]) break;  // uniform: the batch before this one timed out
     if (threadIdx.x == 0 && issue_mma) {
       if constexpr (kB16) issue_batch_b16<MG>(a_addr, b_addr, tmem, kIdesc, mbar);
       else issue_batch<NB, MG>(a_addr, b_addr, tmem, kIdesc, mbar);
     }
-    // while the MMAs run: stage the next batch (the pixel walk of this one has ended; each
-    // thread keeps this batch's index for the epilogue)
-    const uint32_t next = start + MG;
-    uint32_t next_id = 0;
-    if (next < c.len)
-      next_id = stage_tc(list, c.b + next, (int)min((uint32_t)MG, c.len - next), rec_cam, n, c.ox, c.oy, s_geo, s_aux,
-                         g_own, stager, need_id);
+    const bool more = next < c.len && alive;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      dirty[h] = listed[h];
+      listed[h] = 0u;
+    }
+    if (more)
+      steps = group_lists(s.geo[buf ^ 1u], s.lists, c, (int)min((uint32_t)MG, c.len - next), group_alive(T.alive()), nullptr,
+                          listed);
     // warp-uniform: the epilogue's tcgen05.ld needs whole warps
-    const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(mbar, phase, wait_limit_ns));
+    ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(mbar, phase, wait_limit_ns));
     phase ^= 1u;
     tc_fence_after();
     if (ok) {
-      // warps w and w+4 share TMEM lanes 32(w%4)..+31 (one Gaussian per thread) and split its 16-column
-      // chunks; with MG = 64 only the first 16 lanes of each quarter hold a Gaussian (tmem_row_of_lane).
-      // The accumulator streams through registers a chunk at a time: chunk c adds the float4 groups
-      // 4c..4c+3 of the row (V, S_0, S_1, ..) and carries its last column into group 4c+4. Every
-      // tcgen05.ld is warp-uniform; only the atomics depend on the thread's Gaussian.
-      const int quarter = warp & 3, part = warp >> 2;
+      // The accumulator streams through registers 16 columns at a time: chunk c adds the float4 groups
+      // 4c..4c+3 of the row (V, S_0, S_1, ..) and carries its last column into group 4c+4. Only the
+      // first 16 lanes of each quarter hold a Gaussian (M = 64); every tcgen05.ld is warp-uniform.
       const int g = g_own;
-      const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-      if (part == 0 || kCh > kHalf) {        // warp-uniform
-        uint32_t vr[16], r[16];
-        tmem_ld16(trow + (uint32_t)KT, vr);  // the ones block: every column holds V
-        if (part == 1) tmem_ld16(trow + (uint32_t)(16 * (kHalf - 1)), r);  // the column before this part
-        tmem_wait_ld();
-        const float V = __uint_as_float(vr[0]) * v_scale_inv;
-        float carry = part == 0 ? V : __uint_as_float(r[15]) * t_scale_inv;
-        const bool add = g >= 0 && g < nb && V > 0.0f;
-        float* dst = acc_cam + (int64_t)(add ? my_id : 0u) * RS;
-        const int c_begin = part == 0 ? 0 : kHalf, c_end = part == 0 ? kHalf : kCh;
+      const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+      uint32_t vr[16], r[16];
+      tmem_ld16(trow + (uint32_t)KT, vr);  // the ones block: every column holds V
+      tmem_ld16(trow, r);
+      tmem_wait_ld();
+      const float V = __uint_as_float(vr[0]) * v_scale_inv;
+      float carry = V;
+      const bool add = g >= 0 && g < nb && V > 0.0f;
+      float* dst = acc_cam + (int64_t)(add ? my_id : 0u) * RS;
 #pragma unroll
-        for (int c = 0; c < kCh; ++c) {
-          if (c < c_begin || c >= c_end) continue;  // warp-uniform
-          tmem_ld16(trow + (uint32_t)(16 * c), r);
+      for (int c = 0; c < kCh; ++c) {
+        float sv[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) sv[q] = __uint_as_float(r[q]) * t_scale_inv;
+        if (c + 1 < kCh) {
+          tmem_ld16(trow + (uint32_t)(16 * (c + 1)), r);
           tmem_wait_ld();
-          float sv[16];
-#pragma unroll
-          for (int q = 0; q < 16; ++q) sv[q] = __uint_as_float(r[q]) * t_scale_inv;
-          if (add) {
-            float* d = dst + 16 * c;
-            if (16 * c < RS) atomicAdd(reinterpret_cast<float4*>(d), make_float4(carry, sv[0], sv[1], sv[2]));
-            if (16 * c + 4 < RS) atomicAdd(reinterpret_cast<float4*>(d + 4), make_float4(sv[3], sv[4], sv[5], sv[6]));
-            if (16 * c + 8 < RS) atomicAdd(reinterpret_cast<float4*>(d + 8), make_float4(sv[7], sv[8], sv[9], sv[10]));
-            if (16 * c + 12 < RS)
-              atomicAdd(reinterpret_cast<float4*>(d + 12), make_float4(sv[11], sv[12], sv[13], sv[14]));
-          }
-          carry = sv[15];
         }
-        // the last group (S_{KT-1}, 0, 0, 0), by the warps that folded the last chunk
-        if (add && part == (kCh > kHalf ? 1 : 0) && 16 * kCh < RS)
-          atomicAdd(reinterpret_cast<float4*>(dst + 16 * kCh), make_float4(carry, 0.0f, 0.0f, 0.0f));
+        if (add) {
+          float* d = dst + 16 * c;
+          if (16 * c < RS) atomicAdd(reinterpret_cast<float4*>(d), make_float4(carry, sv[0], sv[1], sv[2]));
+          if (16 * c + 4 < RS) atomicAdd(reinterpret_cast<float4*>(d + 4), make_float4(sv[3], sv[4], sv[5], sv[6]));
+          if (16 * c + 8 < RS) atomicAdd(reinterpret_cast<float4*>(d + 8), make_float4(sv[7], sv[8], sv[9], sv[10]));
+          if (16 * c + 12 < RS)
+            atomicAdd(reinterpret_cast<float4*>(d + 12), make_float4(sv[11], sv[12], sv[13], sv[14]));
+        }
+        carry = sv[15];
       }
+      // the last group (S_{KT-1}, 0, 0, 0)
+      if (add && 16 * kCh < RS) atomicAdd(reinterpret_cast<float4*>(dst + 16 * kCh), make_float4(carry, 0.0f, 0.0f, 0.0f));
+      if (more) clear_w();  // this batch's MMAs have completed
+    } else {
+      s_timeout[buf] = 1u;  // seen by every warp after the next barrier
     }
     my_id = next_id;
-    if (!ok) {
-      *s_timeout = 1u;
-    } else if (next < c.len) {
-      // this batch's MMAs have completed: clear W for the next batch (16-byte stores)
-      for (int i = threadIdx.x; i < MG * kKPix * 2 / 16; i += 256) reinterpret_cast<uint4*>(A_s)[i] = make_uint4(0, 0, 0, 0);
-    }
-    tc_fence_before();
-    const int n_done = __syncthreads_count(done);
-    if (*s_timeout) {
-      if (threadIdx.x == 0) atomicOr(&status->flags, kFlagTimeout);
-      mbar_wait_bounded(mbar, phase ^ 1u, wait_limit_ns);  // give the outstanding MMAs a last chance to finish
-      break;
-    }
-    if (n_done == (int)blockDim.x) break;
+    if (!more) break;
   }
-  const uint32_t warp_sum = __reduce_add_sync(0xFFFFFFFFu, npairs);
-  if (lane == 0 && warp_sum) atomicAdd((unsigned long long*)&status->contrib_pairs, (unsigned long long)warp_sum);
+  tc_fence_before();
+  __syncthreads();
+  if (s_timeout[0] | s_timeout[1]) {
+    if (threadIdx.x == 0) atomicOr(&status->flags, kFlagTimeout);
+    if (!ok) mbar_wait_bounded(mbar, phase ^ 1u, wait_limit_ns);  // a last chance for the outstanding MMAs
+  }
+  add_pair_count(npairs, status);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
@@ -553,12 +570,10 @@ template <int NB>
 constexpr size_t selftest_smem() {
   return 1024 + (size_t)kG * kKPix * 2 + (size_t)NB * kKPix * 2 + 16;
 }
-// the barrier and flags with the alignment slack (1 KB), W, and B (with the staged geometry in its
-// holes at 16 channels, after it otherwise)
+// the barrier, flags and staged batch with up to 1023 bytes of alignment, W, and B
 template <int KT, int MG>
 constexpr size_t tc_smem() {
-  return 1024 + (size_t)MG * kKPix * 2 +
-         (KT == 16 ? (size_t)kB16Bytes : (size_t)tc_cols<KT, MG>() * kKPix * 2 + (size_t)MG * 32);
+  return tc_front<KT>() + 1023 + (size_t)MG * kKPix * 2 + (KT == 16 ? (size_t)kB16Bytes : (size_t)tc_cols<KT, MG>() * kKPix * 2);
 }
 // CTAs per SM that the shared memory admits: each CTA's share rounded up to 1 KB, plus 1 KB the
 // system reserves per CTA, out of the SM's 228 KB
@@ -584,7 +599,7 @@ void accumulate_tc(const Problem& p, int cb, int cam0, const void* targets, cons
   cudaFuncSetAttribute(k_blend_accumulate_tc<KT, BF16_TARGETS, MG>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        (int)cudaSharedmemCarveoutMaxShared);
   const int64_t stride = p.L == 0 ? 0 : p.n * (int64_t)p.acc_stride;
-  k_blend_accumulate_tc<KT, BF16_TARGETS, MG><<<cb * p.tiles, 256, smem, s>>>(
+  k_blend_accumulate_tc<KT, BF16_TARGETS, MG><<<cb * p.tiles, kTcThreads, smem, s>>>(
       ws.tile_off, ws.entries, p.capacity, ws.rec, p.n, p.width, p.height, p.tiles_x, p.tiles,
       static_cast<const uint16_t*>(targets), p.K, cam0, ws.acc, p.acc_stride, stride, ws.status, g_wait_limit_ns,
       g_issue_mma);

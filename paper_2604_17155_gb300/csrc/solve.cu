@@ -20,6 +20,7 @@
 
 #include "icgs_device.cuh"
 #include "icgs_internal.h"
+#include "packed.cuh"
 
 namespace icgs {
 
@@ -59,6 +60,29 @@ __device__ __forceinline__ unsigned fold_group_mask() {
   return 0xFFu << (threadIdx.x & 24u);
 }
 
+// acc (hi s, lo c) += the pair whose negation is nx, by TwoSum (two_sum_acc on both halves)
+__device__ __forceinline__ void two_sum_acc2(f2& s, f2& c, f2 nx) {
+  const f2 t = sub2(s, nx), bp = sub2(t, s);
+  const f2 err = sub2(sub2(s, sub2(t, bp)), add2(nx, bp));
+  s = t;
+  c = add2(c, err);
+}
+__device__ __forceinline__ f2 neg2(f2 v) { return v ^ 0x8000000080000000ull; }
+
+// (g, gl) += (v + vl) y: the product v y exactly (TwoProduct), TwoSum into g, the rest into gl
+__device__ __forceinline__ void exact_acc(float& g, float& gl, float v, float vl, float y) {
+  const float p = v * y;
+  const float e = fmaf(vl, y, fmaf(v, y, -p));
+  two_sum_acc(g, gl, p);
+  gl += e;
+}
+__device__ __forceinline__ void exact_acc2(f2& g, f2& gl, f2 v, f2 vl, f2 y) {
+  const f2 np = mul2(v, neg2(y));
+  const f2 e = fma2(vl, y, fma2(v, y, np));
+  two_sum_acc2(g, gl, np);
+  gl = add2(gl, e);
+}
+
 template <int B, int KC, bool MIXED>
 __global__ void __launch_bounds__(kSolveThreads) k_fold(
     const float* __restrict__ means, int64_t n, const DevCam* __restrict__ cams, int cb,
@@ -84,10 +108,16 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
   const bool do_w = k0 == 0;
   float* Gi = G + i * B * B;
   float* Gli = MIXED ? Glo + i * B * B : nullptr;
-  float g[NG], gl[NG], bb[NR][KC], bl[NR][KC];
+  // The Gram slots: MIXED keeps slots 0..B-1 in pairs (g2, gl2) and the one left over -- slot B-1 of an
+  // odd B, slot B of an even one -- in g[0], gl[0]; otherwise slot s is g[s].
+  constexpr int NS = MIXED ? 1 : NG;
+  float g[NS], gl[NS], bb[NR][KC], bl[NR][KC];
+  f2 g2[MIXED ? B / 2 : 1], gl2[MIXED ? B / 2 : 1];
   float w = 0.0f, wl = 0.0f;
 #pragma unroll
-  for (int s = 0; s < NG; ++s) { g[s] = 0.0f; gl[s] = 0.0f; }
+  for (int s = 0; s < NS; ++s) { g[s] = 0.0f; gl[s] = 0.0f; }
+#pragma unroll
+  for (int s = 0; s < (MIXED ? B / 2 : 1); ++s) g2[s] = gl2[s] = 0ull;
 #pragma unroll
   for (int m = 0; m < NR; ++m)
 #pragma unroll
@@ -103,8 +133,15 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
 #pragma unroll
       for (int s = 0; s < NG; ++s) {
         if (s == B && !half_slot) continue;
-        g[s] = Gi[entry(s)];
-        if (MIXED) gl[s] = Gli[entry(s)];
+        if constexpr (!MIXED) {
+          g[s < NS ? s : 0] = Gi[entry(s)];
+        } else if (s / 2 >= B / 2) {
+          g[0] = Gi[entry(s)];
+          gl[0] = Gli[entry(s)];
+        } else if (s % 2 == 0) {
+          g2[s / 2] = pack2(Gi[entry(s)], Gi[entry(s + 1)]);
+          gl2[s / 2] = pack2(Gli[entry(s)], Gli[entry(s + 1)]);
+        }
       }
     }
     if (do_w) {
@@ -168,52 +205,60 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
       }
     }
     __syncwarp(gm);
-    const int nj = min(GS, cb - jb);
-    for (int q = 0; q < nj; ++q) {
-      const int j = jb + q;
+    // only the cameras that see this Gaussian, in order
+    for (uint32_t todo = (__ballot_sync(gm, lv > 0.0f) >> (gbase & 31)) & 0xFFu; todo != 0u; todo &= todo - 1u) {
+      const int q = __ffs(todo) - 1;
       const float v = __shfl_sync(gm, lv, q, GS);
       float sv[KC];
 #pragma unroll
       for (int k = 0; k < KC; ++k) sv[k] = __shfl_sync(gm, ls[k], q, GS);
-      if (v > 0.0f) {
-        const float* Yq = s_Y[gbase + q];
-        if (do_gram && diag) {
-          float Y[(B + 3) / 4 * 4];
+      const float* Yq = s_Y[gbase + q];
+      if (do_gram && diag) {
+        float Y[(B + 3) / 4 * 4];
 #pragma unroll
-          for (int c4 = 0; c4 < (B + 3) / 4; ++c4) {
-            const float4 y4 = reinterpret_cast<const float4*>(Yq)[c4];
-            Y[4 * c4] = y4.x; Y[4 * c4 + 1] = y4.y; Y[4 * c4 + 2] = y4.z; Y[4 * c4 + 3] = y4.w;
-          }
-          const float* vq = s_vY[gbase + q] + r;  // vq[c] = v Y[(c + r) mod B]
-          const float* vql = s_vYl[MIXED ? gbase + q : 0] + (MIXED ? r : 0);
+        for (int c4 = 0; c4 < (B + 3) / 4; ++c4) {
+          const float4 y4 = reinterpret_cast<const float4*>(Yq)[c4];
+          Y[4 * c4] = y4.x; Y[4 * c4 + 1] = y4.y; Y[4 * c4 + 2] = y4.z; Y[4 * c4 + 3] = y4.w;
+        }
+        const float* vq = s_vY[gbase + q] + r;  // vq[c] = v Y[(c + r) mod B]
+        const float* vql = s_vYl[MIXED ? gbase + q : 0] + (MIXED ? r : 0);
+        if constexpr (MIXED) {
+          // slots two at a time, packed: the same operations as exact_acc
 #pragma unroll
-          for (int s = 0; s < B; ++s) {
-            if constexpr (MIXED) {
-              const float p = vq[s] * Y[s];
-              const float e = fmaf(vq[s], Y[s], -p) + vql[s] * Y[s];
-              two_sum_acc(g[s], gl[s], p);
-              gl[s] += e;
-            } else {
-              g[s] = fmaf(vq[s], Y[s], g[s]);
-            }
-          }
-          if constexpr (kHalf) {
-            if (half_slot) {  // entry (r + B/2, r): v Y[r + B/2] Y[r]
-              if constexpr (MIXED) {
-                const float p = vq[B / 2] * Yq[r];
-                const float e = fmaf(vq[B / 2], Yq[r], -p) + vql[B / 2] * Yq[r];
-                two_sum_acc(g[B], gl[B], p);
-                gl[B] += e;
-              } else {
-                g[B] = fmaf(vq[B / 2], Yq[r], g[B]);
-              }
-            }
-          }
+          for (int s = 0; s + 1 < B; s += 2)
+            exact_acc2(g2[s / 2], gl2[s / 2], pack2(vq[s], vq[s + 1]), pack2(vql[s], vql[s + 1]), pack2(Y[s], Y[s + 1]));
+          if constexpr (B % 2) exact_acc(g[0], gl[0], vq[B - 1], vql[B - 1], Y[B - 1]);
+          if constexpr (kHalf)
+            if (half_slot) exact_acc(g[0], gl[0], vq[B / 2], vql[B / 2], Yq[r]);  // entry (r + B/2, r)
+        } else {
+#pragma unroll
+          for (int s = 0; s < B; ++s) g[s] = fmaf(vq[s], Y[s], g[s]);
+          if constexpr (kHalf)
+            if (half_slot) g[B] = fmaf(vq[B / 2], Yq[r], g[B]);
         }
-        if (do_w) {
-          if constexpr (MIXED) two_sum_acc(w, wl, v);
-          else w += v;
-        }
+      }
+      if (do_w) {
+        if constexpr (MIXED) two_sum_acc(w, wl, v);
+        else w += v;
+      }
+      if constexpr (MIXED && NR == 2) {
+        const float Y1 = r + GS < B ? Yq[r + GS < B ? r + GS : 0] : 0.0f;
+        const f2 Y2 = pack2(r < B ? Yq[r < B ? r : 0] : 0.0f, Y1);
+#pragma unroll
+        for (int k = 0; k < KC; ++k)
+          if (k0 + k < K) {
+            f2 bk = pack2(bb[0][k], bb[1][k]), bkl = pack2(bl[0][k], bl[1][k]);
+            const f2 sk = pack2(sv[k], sv[k]);
+            const f2 np = mul2(sk, neg2(Y2));
+            two_sum_acc2(bk, bkl, np);
+            bkl = add2(bkl, fma2(Y2, sk, np));
+            const float2 x = unpack2(bk), y = unpack2(bkl);
+            bb[0][k] = x.x;
+            bb[1][k] = x.y;
+            bl[0][k] = y.x;
+            bl[1][k] = y.y;
+          }
+      } else {
 #pragma unroll
         for (int m = 0; m < NR; ++m) {
           const int row = r + GS * m;
@@ -240,11 +285,22 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
       if (s == B && !half_slot) continue;
       const int e = entry(s);
       const int row = e / B, col = e - row * B;
-      Gi[e] = g[s];
-      if (MIXED) Gli[e] = gl[s];
+      float hi, lo = 0.0f;
+      if constexpr (!MIXED) {
+        hi = g[s < NS ? s : 0];
+      } else if (s / 2 >= B / 2) {
+        hi = g[0];
+        lo = gl[0];
+      } else {
+        const float2 x = unpack2(g2[s / 2 < B / 2 ? s / 2 : 0]), y = unpack2(gl2[s / 2 < B / 2 ? s / 2 : 0]);
+        hi = s % 2 ? x.y : x.x;
+        lo = s % 2 ? y.y : y.x;
+      }
+      Gi[e] = hi;
+      if (MIXED) Gli[e] = lo;
       if (row != col) {  // the mirrored entry
-        Gi[col * B + row] = g[s];
-        if (MIXED) Gli[col * B + row] = gl[s];
+        Gi[col * B + row] = hi;
+        if (MIXED) Gli[col * B + row] = lo;
       }
     }
   }
