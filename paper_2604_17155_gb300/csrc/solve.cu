@@ -46,18 +46,43 @@ __device__ __forceinline__ F group_sum(F v) {
 // ------------------------------------------------------------------------------------------
 // fold
 // ------------------------------------------------------------------------------------------
-// One 8-lane group per Gaussian. G is symmetric, so the group forms only its B (B + 1) / 2 unique
-// unique entries only, by wrapped diagonals: lane r accumulates diagonal r, the entries
-// ((c + r) mod B, c) for c = 0..B-1, and for even B also the entry (r + B/2, r) of the half
-// diagonal B/2. Diagonals 0..ceil(B/2)-1 and that half diagonal hold every unordered pair {row, col}
-// exactly once. Per camera the column factor Y[c] is a compile-time index (a broadcast float4
-// load) and the row factor v Y[(c + r) mod B] is read from a doubled copy of the v Y row at the
-// lane's own offset r, so an entry costs one FMA. b rows r, r + 8 belong to lane r. G is written
-// out in full (both triangles), row-major like the sums of the single-camera-group layout.
+// One 8-lane group per Gaussian, the cameras that see it one at a time. G is symmetric and is formed by
+// wrapped diagonals of 2x2 blocks: with NB = ceil(B/2) block rows (index Bp = 2 NB; an odd B has a zero
+// last basis function), lane l < NB takes rows 2l, 2l + 1 against the columns 2l .. 2l + 2 NC - 1 (mod Bp),
+// that is NC whole block diagonals; an even NB leaves half of block diagonal NB/2, of which the lane takes
+// one pair. Every unordered pair of indices comes up once (but for the two orders of (2l, 2l + 1)). The
+// layout is chosen for shared-memory reads, which bounded the fold (82% of the wavefront rate with one
+// wrapped diagonal a lane, 36 loads a camera): a lane reads its two rows of v Y, one window of Y and the row,
+// eight loads for 18 entries, and the products are packed two at a time (packed.cuh). b rows 2l, 2l + 1
+// belong to lane l. MIXED: every product is exact in float-float (v Y_r split by an FMA, then each entry's
+// product split again) and every addition a TwoSum into the running (hi, lo) pair, so G, b and w are the
+// sums of the float32 basis to about 2^-44 relative -- the same basis the adjoint's payload uses.
+// G is kept in the order that the lanes write it, [pair][lane][2] per Gaussian
+// (gram_floats of them, gram_pos of an entry), so that a warp writes whole sectors: as full rows, mirrored
+// entries included, the 72 scattered stores a lane cost more than the sums of 20 cameras.
 constexpr int kFoldGroup = 8;
 
-__device__ __forceinline__ unsigned fold_group_mask() {
-  return 0xFFu << (threadIdx.x & 24u);
+__host__ __device__ constexpr int gram_floats(int B) {
+  const int NB = (B + 1) / 2, NC = (NB + 1) / 2;
+  return (2 * NC + (NB % 2 == 0 ? 1 : 0)) * NB * 2;
+}
+// The place of entry (r, c) = (c, r) in a Gaussian's block.
+__host__ __device__ inline int gram_pos(int r, int c, int B) {
+  const int NB = (B + 1) / 2, NC = (NB + 1) / 2;
+  if (r / 2 == c / 2 && r > c) {  // inside a diagonal block the upper entry is kept
+    const int t = r;
+    r = c;
+    c = t;
+  }
+  const int br = r / 2, bc = c / 2;
+  const int d = bc >= br ? bc - br : bc - br + NB;
+  if (d < NC) return (((r & 1) * NC + d) * NB + br) * 2 + (c & 1);
+  if (NB - d < NC) return (((c & 1) * NC + NB - d) * NB + bc) * 2 + (r & 1);
+  // the half diagonal: the row with even index in the lower block against the upper block's columns belongs
+  // to the lower block's lane, the other to the upper block's
+  const int e = br < bc ? r & 1 : c & 1, f = br < bc ? c & 1 : r & 1;
+  const int lo = br < bc ? br : bc, hi = br < bc ? bc : br;
+  return (2 * NC * NB + (e == 0 ? lo : hi)) * 2 + f;
 }
 
 // acc (hi s, lo c) += the pair whose negation is nx, by TwoSum (two_sum_acc on both halves)
@@ -67,17 +92,13 @@ __device__ __forceinline__ void two_sum_acc2(f2& s, f2& c, f2 nx) {
   s = t;
   c = add2(c, err);
 }
+// the signs flipped on the ALU: the FMA pipe is the fold's bound
 __device__ __forceinline__ f2 neg2(f2 v) { return v ^ 0x8000000080000000ull; }
 
-// (g, gl) += (v + vl) y: the product v y exactly (TwoProduct), TwoSum into g, the rest into gl
-__device__ __forceinline__ void exact_acc(float& g, float& gl, float v, float vl, float y) {
-  const float p = v * y;
-  const float e = fmaf(vl, y, fmaf(v, y, -p));
-  two_sum_acc(g, gl, p);
-  gl += e;
-}
-__device__ __forceinline__ void exact_acc2(f2& g, f2& gl, f2 v, f2 vl, f2 y) {
-  const f2 np = mul2(v, neg2(y));
+// (g, gl) += (v + vl) y for pairs, ny = -y: the product v y exactly (TwoProduct), TwoSum into g, the rest
+// into gl
+__device__ __forceinline__ void exact_acc2(f2& g, f2& gl, f2 v, f2 vl, f2 y, f2 ny) {
+  const f2 np = mul2(v, ny);
   const f2 e = fma2(vl, y, fma2(v, y, np));
   two_sum_acc2(g, gl, np);
   gl = add2(gl, e);
@@ -90,58 +111,56 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
     float* __restrict__ Glo, float* __restrict__ bvec, float* __restrict__ blo,
     float* __restrict__ wsum, float* __restrict__ wlo) {
   constexpr int GS = kFoldGroup;
-  constexpr int ND = (B + 1) / 2;              // full wrapped diagonals (lanes 0..ND-1)
-  constexpr bool kHalf = (B % 2) == 0;         // even B: lanes 0..B/2-1 also take one entry of diagonal B/2
-  constexpr int NG = B + (kHalf ? 1 : 0);      // Gram slots of a lane
-  constexpr int NR = (B + GS - 1) / GS;        // b rows of a lane: r, r + 8
-  constexpr int kYStride = (B + 3) / 4 * 4 + 4;
-  constexpr int kVStride = 2 * B + 1;          // odd: the four groups' rows fall in distinct banks
-  static_assert(ND <= GS, "one diagonal per lane");
+  constexpr int NB = (B + 1) / 2, Bp = 2 * NB;
+  constexpr int NC = (NB + 1) / 2;             // column pairs of a lane's window
+  constexpr bool kExtra = NB % 2 == 0;         // an even NB: one more pair, of block diagonal NB/2
+  constexpr int NG = 2 * NC + (kExtra ? 1 : 0);  // pairs: row 0's, row 1's, the extra one
+  constexpr int kWin = 2 * (NB - 1) + 2 * NC;  // values of Y stored, wrapped around
+  // row stride of 2 mod 4 words: rows 8 apart (the groups' rows of one camera) fall 16 banks apart
+  constexpr int kYStride = (kWin + 5) / 4 * 4 - 2 >= kWin ? (kWin + 5) / 4 * 4 - 2 : (kWin + 5) / 4 * 4 + 2;
+  constexpr int kSW = (KC + 1 + 3) / 4 * 4;    // V and the channels of a camera's row
+  static_assert(NB <= GS, "one block row per lane");
+  static_assert(kYStride % 4 == 2 && kYStride >= kWin, "bank layout");
   __shared__ __align__(16) float s_Y[kSolveThreads][kYStride];
-  __shared__ float s_vY[kSolveThreads][kVStride];
-  __shared__ float s_vYl[MIXED ? kSolveThreads : 1][MIXED ? kVStride : 1];  // lo parts of v Y (MIXED)
-  const int64_t i = (blockIdx.x * (int64_t)kSolveThreads + threadIdx.x) / GS;
+  // v Y of rows 2l, 2l + 1 and, MIXED, its lo parts; one more slot a row keeps the rows' banks apart
+  __shared__ float4 s_vY[kSolveThreads][NB + 1];
+  __shared__ __align__(16) float s_row[kSolveThreads][kSW];
+  const int64_t i_own = (blockIdx.x * (int64_t)kSolveThreads + threadIdx.x) / GS;
   const int r = threadIdx.x % GS;
-  if (i >= n) return;  // whole groups exit together
-  const bool diag = r < ND;
+  // Groups past the end repeat the last Gaussian without writing: the warp's vote and barriers below
+  // name all its lanes (with a mask per group, the groups ran one after the other).
+  const bool valid = i_own < n;
+  const int64_t i = valid ? i_own : n - 1;
+  const int l2 = r < NB ? 2 * r : 0;          // first row of the lane (lanes past NB compute and drop)
+  const bool owner = r < NB;
+  // The extra pair: row 2l against the columns 2l + NB, 2l + NB + 1 (lanes l < NB/2), or rows 2l, 2l + 1
+  // against the column (2l + NB + 1) mod Bp (the other lanes): v Y of the lane's own rows, Y at x0, x1.
+  const bool x_cols = r < NB / 2;
+  const int x0 = x_cols ? l2 + NB : (l2 + NB + 1) % Bp, x1 = x_cols ? x0 + 1 : x0;
   const bool do_gram = k0 == 0 && want_gram;  // G (skipped by refinement, whose Gram is fixed)
   const bool do_w = k0 == 0;
-  float* Gi = G + i * B * B;
-  float* Gli = MIXED ? Glo + i * B * B : nullptr;
-  // The Gram slots: MIXED keeps slots 0..B-1 in pairs (g2, gl2) and the one left over -- slot B-1 of an
-  // odd B, slot B of an even one -- in g[0], gl[0]; otherwise slot s is g[s].
-  constexpr int NS = MIXED ? 1 : NG;
-  float g[NS], gl[NS], bb[NR][KC], bl[NR][KC];
-  f2 g2[MIXED ? B / 2 : 1], gl2[MIXED ? B / 2 : 1];
+  static_assert(gram_floats(B) == NG * NB * 2, "layout");
+  // the lane's pairs: s at Gi[s NB], lanes past NB none
+  f2* Gi = reinterpret_cast<f2*>(G + i * gram_floats(B)) + (owner ? r : 0);
+  f2* Gli = MIXED ? reinterpret_cast<f2*>(Glo + i * gram_floats(B)) + (owner ? r : 0) : nullptr;
+  f2 g[NG], gl[MIXED ? NG : 1], bb[KC], bl[MIXED ? KC : 1];
   float w = 0.0f, wl = 0.0f;
 #pragma unroll
-  for (int s = 0; s < NS; ++s) { g[s] = 0.0f; gl[s] = 0.0f; }
+  for (int s = 0; s < NG; ++s) {
+    g[s] = 0ull;
+    if (MIXED) gl[s] = 0ull;
+  }
 #pragma unroll
-  for (int s = 0; s < (MIXED ? B / 2 : 1); ++s) g2[s] = gl2[s] = 0ull;
-#pragma unroll
-  for (int m = 0; m < NR; ++m)
-#pragma unroll
-    for (int k = 0; k < KC; ++k) { bb[m][k] = 0.0f; bl[m][k] = 0.0f; }
-  // slot s < B: entry ((s + r) mod B, s); slot B (even B): entry (r + B/2, r)
-  auto entry = [&](int s) -> int {
-    if (s < B) { const int row = s + r < B ? s + r : s + r - B; return row * B + s; }
-    return (r + B / 2) * B + r;
-  };
-  const bool half_slot = kHalf && r < B / 2;
+  for (int k = 0; k < KC; ++k) {
+    bb[k] = 0ull;
+    if (MIXED) bl[k] = 0ull;
+  }
   if (!first) {
-    if (do_gram && diag) {
+    if (do_gram) {
 #pragma unroll
       for (int s = 0; s < NG; ++s) {
-        if (s == B && !half_slot) continue;
-        if constexpr (!MIXED) {
-          g[s < NS ? s : 0] = Gi[entry(s)];
-        } else if (s / 2 >= B / 2) {
-          g[0] = Gi[entry(s)];
-          gl[0] = Gli[entry(s)];
-        } else if (s % 2 == 0) {
-          g2[s / 2] = pack2(Gi[entry(s)], Gi[entry(s + 1)]);
-          gl2[s / 2] = pack2(Gli[entry(s)], Gli[entry(s + 1)]);
-        }
+        g[s] = Gi[s * NB];
+        if (MIXED) gl[s] = Gli[s * NB];
       }
     }
     if (do_w) {
@@ -149,159 +168,141 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
       if (MIXED) wl = wlo[i];
     }
 #pragma unroll
-    for (int m = 0; m < NR; ++m) {
-      const int row = r + GS * m;
-      if (row < B) {
+    for (int k = 0; k < KC; ++k) {
+      float x[2] = {0.0f, 0.0f}, y[2] = {0.0f, 0.0f};
 #pragma unroll
-        for (int k = 0; k < KC; ++k)
-          if (k0 + k < K) {
-            bb[m][k] = bvec[(i * B + row) * K + k0 + k];
-            if (MIXED) bl[m][k] = blo[(i * B + row) * K + k0 + k];
-          }
-      }
+      for (int h = 0; h < 2; ++h)
+        if (owner && l2 + h < B && k0 + k < K) {
+          x[h] = bvec[(i * B + l2 + h) * K + k0 + k];
+          if (MIXED) y[h] = blo[(i * B + l2 + h) * K + k0 + k];
+        }
+      bb[k] = pack2(x[0], x[1]);
+      if (MIXED) bl[k] = pack2(y[0], y[1]);
     }
   }
   const float mu[3] = {means[3 * i], means[3 * i + 1], means[3 * i + 2]};
   const int64_t stride = n * (int64_t)RS;
-  // MIXED: every product is exact in float-float (v Y_r split by an FMA, then each entry's product
-  // split again) and every addition a TwoSum into the running (hi, lo) pair, so G, b and w are the
-  // sums of the float32 basis to about 2^-44 relative -- the same basis the adjoint's payload uses
-  const unsigned gm = fold_group_mask();
   const int gbase = threadIdx.x & ~(GS - 1);
-  // 8 cameras at a time: lane q loads camera jb + q's row (V, S), evaluates its basis Y into s_Y
-  // and v Y (twice) into s_vY; the group shares V, S by shuffles and reads the rows back
-  for (int jb = 0; jb < cb; jb += GS) {
-    float lv = 0.0f, ls[KC];
+  const bool row4 = KC == 3 && K == 3;  // a row is one float4 (V, S_0, S_1, S_2)
+  // 8 cameras at a time: lane q loads camera jb + q's row (V, S) -- a block ahead -- and writes its basis Y,
+  // v Y and the row to shared memory for the group
+  float nv = 0.0f, ns[KC];
+  auto load_row = [&](int j) {
+    nv = 0.0f;
 #pragma unroll
-    for (int k = 0; k < KC; ++k) ls[k] = 0.0f;
-    if (jb + r < cb) {
-      const float* a = acc + (int64_t)(jb + r) * stride + i * RS;
-      lv = a[0];
+    for (int k = 0; k < KC; ++k) ns[k] = 0.0f;
+    if (j >= cb) return;
+    const float* a = acc + (int64_t)j * stride + i * RS;
+    if (row4) {
+      const float4 x = *reinterpret_cast<const float4*>(a);
+      nv = x.x;
+      ns[0] = x.y;
+      ns[KC > 1 ? 1 : 0] = x.z;
+      ns[KC > 2 ? 2 : 0] = x.w;
+    } else {
+      nv = a[0];
 #pragma unroll
       for (int k = 0; k < KC; ++k)
-        if (k0 + k < K) ls[k] = a[1 + k0 + k];
+        if (k0 + k < K) ns[k] = a[1 + k0 + k];
     }
+  };
+  load_row(r);
+  for (int jb = 0; jb < cb; jb += GS) {
+    const float lv = nv;
+    float ls[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) ls[k] = ns[k];
+    load_row(jb + GS + r);
     if (lv > 0.0f) {
       const float3 d = view_dir(mu, cams[jb + r]);
-      float Yl[kYStride];
+      float Yl[Bp];
+      if (B < Bp) Yl[Bp - 1] = 0.0f;
       sh_basis<B>(d.x, d.y, d.z, Yl);
 #pragma unroll
-      for (int c4 = 0; c4 < (B + 3) / 4; ++c4)
-        reinterpret_cast<float4*>(s_Y[threadIdx.x])[c4] =
-            make_float4(Yl[4 * c4], 4 * c4 + 1 < B ? Yl[4 * c4 + 1] : 0.0f, 4 * c4 + 2 < B ? Yl[4 * c4 + 2] : 0.0f,
-                        4 * c4 + 3 < B ? Yl[4 * c4 + 3] : 0.0f);
+      for (int c = 0; c < kWin; c += 2)
+        *reinterpret_cast<float2*>(&s_Y[threadIdx.x][c]) = make_float2(Yl[c % Bp], Yl[(c + 1) % Bp]);
       if (do_gram) {
 #pragma unroll
-        for (int c = 0; c < B; ++c) {
-          const float vy = lv * Yl[c];
-          s_vY[threadIdx.x][c] = vy;
-          s_vY[threadIdx.x][c + B] = vy;
-          if constexpr (MIXED) {
-            const float vyl = fmaf(lv, Yl[c], -vy);
-            s_vYl[threadIdx.x][c] = vyl;
-            s_vYl[threadIdx.x][c + B] = vyl;
-          }
+        for (int c = 0; c < NB; ++c) {
+          const float v0 = lv * Yl[2 * c], v1 = lv * Yl[2 * c + 1];
+          s_vY[threadIdx.x][c] = make_float4(v0, v1, MIXED ? fmaf(lv, Yl[2 * c], -v0) : 0.0f,
+                                             MIXED ? fmaf(lv, Yl[2 * c + 1], -v1) : 0.0f);
         }
       }
+      float row[kSW];
+#pragma unroll
+      for (int k = 0; k < kSW; ++k) row[k] = k == 0 ? lv : (k <= KC ? ls[k <= KC && k > 0 ? k - 1 : 0] : 0.0f);
+#pragma unroll
+      for (int k = 0; k < kSW; k += 4)
+        *reinterpret_cast<float4*>(&s_row[threadIdx.x][k]) = make_float4(row[k], row[k + 1], row[k + 2], row[k + 3]);
     }
-    __syncwarp(gm);
+    __syncwarp();
     // only the cameras that see this Gaussian, in order
-    for (uint32_t todo = (__ballot_sync(gm, lv > 0.0f) >> (gbase & 31)) & 0xFFu; todo != 0u; todo &= todo - 1u) {
+    for (uint32_t todo = (__ballot_sync(0xFFFFFFFFu, lv > 0.0f) >> (gbase & 31)) & 0xFFu; todo != 0u; todo &= todo - 1u) {
       const int q = __ffs(todo) - 1;
-      const float v = __shfl_sync(gm, lv, q, GS);
-      float sv[KC];
+      const int at = gbase + q;
+      float row[kSW];
 #pragma unroll
-      for (int k = 0; k < KC; ++k) sv[k] = __shfl_sync(gm, ls[k], q, GS);
-      const float* Yq = s_Y[gbase + q];
-      if (do_gram && diag) {
-        float Y[(B + 3) / 4 * 4];
-#pragma unroll
-        for (int c4 = 0; c4 < (B + 3) / 4; ++c4) {
-          const float4 y4 = reinterpret_cast<const float4*>(Yq)[c4];
-          Y[4 * c4] = y4.x; Y[4 * c4 + 1] = y4.y; Y[4 * c4 + 2] = y4.z; Y[4 * c4 + 3] = y4.w;
-        }
-        const float* vq = s_vY[gbase + q] + r;  // vq[c] = v Y[(c + r) mod B]
-        const float* vql = s_vYl[MIXED ? gbase + q : 0] + (MIXED ? r : 0);
+      for (int k = 0; k < kSW; k += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(&s_row[at][k]);
+        row[k] = x.x;
+        row[k + 1] = x.y;
+        row[k + 2] = x.z;
+        row[k + 3] = x.w;
+      }
+      const float v = row[0];
+      const float* Yq = s_Y[at];
+      const f2 Y0 = *reinterpret_cast<const f2*>(Yq + l2);
+      const f2 nY0 = MIXED ? neg2(Y0) : 0ull;
+      if (do_gram) {
+        const float4 vr = s_vY[at][l2 / 2];
+        const f2 v0 = pack2(vr.x, vr.x), v1 = pack2(vr.y, vr.y);
+        const f2 xv = pack2(vr.x, x_cols ? vr.x : vr.y), xy = pack2(Yq[x0], Yq[x1]);
         if constexpr (MIXED) {
-          // slots two at a time, packed: the same operations as exact_acc
+          const f2 l0 = pack2(vr.z, vr.z), l1 = pack2(vr.w, vr.w);
 #pragma unroll
-          for (int s = 0; s + 1 < B; s += 2)
-            exact_acc2(g2[s / 2], gl2[s / 2], pack2(vq[s], vq[s + 1]), pack2(vql[s], vql[s + 1]), pack2(Y[s], Y[s + 1]));
-          if constexpr (B % 2) exact_acc(g[0], gl[0], vq[B - 1], vql[B - 1], Y[B - 1]);
-          if constexpr (kHalf)
-            if (half_slot) exact_acc(g[0], gl[0], vq[B / 2], vql[B / 2], Yq[r]);  // entry (r + B/2, r)
+          for (int c = 0; c < NC; ++c) {
+            const f2 y = c == 0 ? Y0 : *reinterpret_cast<const f2*>(Yq + l2 + 2 * c);
+            const f2 ny = c == 0 ? nY0 : neg2(y);
+            exact_acc2(g[c], gl[c], v0, l0, y, ny);
+            exact_acc2(g[NC + c], gl[NC + c], v1, l1, y, ny);
+          }
+          if constexpr (kExtra)
+            exact_acc2(g[2 * NC], gl[2 * NC], xv, pack2(vr.z, x_cols ? vr.z : vr.w), xy, neg2(xy));
         } else {
 #pragma unroll
-          for (int s = 0; s < B; ++s) g[s] = fmaf(vq[s], Y[s], g[s]);
-          if constexpr (kHalf)
-            if (half_slot) g[B] = fmaf(vq[B / 2], Yq[r], g[B]);
+          for (int c = 0; c < NC; ++c) {
+            const f2 y = c == 0 ? Y0 : *reinterpret_cast<const f2*>(Yq + l2 + 2 * c);
+            g[c] = fma2(v0, y, g[c]);
+            g[NC + c] = fma2(v1, y, g[NC + c]);
+          }
+          if constexpr (kExtra) g[2 * NC] = fma2(xv, xy, g[2 * NC]);
         }
       }
       if (do_w) {
         if constexpr (MIXED) two_sum_acc(w, wl, v);
         else w += v;
       }
-      if constexpr (MIXED && NR == 2) {
-        const float Y1 = r + GS < B ? Yq[r + GS < B ? r + GS : 0] : 0.0f;
-        const f2 Y2 = pack2(r < B ? Yq[r < B ? r : 0] : 0.0f, Y1);
 #pragma unroll
-        for (int k = 0; k < KC; ++k)
-          if (k0 + k < K) {
-            f2 bk = pack2(bb[0][k], bb[1][k]), bkl = pack2(bl[0][k], bl[1][k]);
-            const f2 sk = pack2(sv[k], sv[k]);
-            const f2 np = mul2(sk, neg2(Y2));
-            two_sum_acc2(bk, bkl, np);
-            bkl = add2(bkl, fma2(Y2, sk, np));
-            const float2 x = unpack2(bk), y = unpack2(bkl);
-            bb[0][k] = x.x;
-            bb[1][k] = x.y;
-            bl[0][k] = y.x;
-            bl[1][k] = y.y;
-          }
-      } else {
-#pragma unroll
-        for (int m = 0; m < NR; ++m) {
-          const int row = r + GS * m;
-          const float Yr = row < B ? Yq[row] : 0.0f;
-#pragma unroll
-          for (int k = 0; k < KC; ++k)
-            if (k0 + k < K) {
-              if constexpr (MIXED) {
-                const float p = Yr * sv[k];
-                two_sum_acc(bb[m][k], bl[m][k], p);
-                bl[m][k] += fmaf(Yr, sv[k], -p);
-              } else {
-                bb[m][k] = fmaf(Yr, sv[k], bb[m][k]);
-              }
-            }
+      for (int k = 0; k < KC; ++k) {  // channels past K add exact zeros
+        const f2 sk = pack2(row[k + 1], row[k + 1]);
+        if constexpr (MIXED) {
+          const f2 np = mul2(sk, nY0);
+          two_sum_acc2(bb[k], bl[k], np);
+          bl[k] = add2(bl[k], fma2(Y0, sk, np));
+        } else {
+          bb[k] = fma2(Y0, sk, bb[k]);
         }
       }
     }
-    __syncwarp(gm);
+    __syncwarp();
   }
-  if (do_gram && diag) {
+  if (!valid) return;
+  if (do_gram && owner) {
 #pragma unroll
     for (int s = 0; s < NG; ++s) {
-      if (s == B && !half_slot) continue;
-      const int e = entry(s);
-      const int row = e / B, col = e - row * B;
-      float hi, lo = 0.0f;
-      if constexpr (!MIXED) {
-        hi = g[s < NS ? s : 0];
-      } else if (s / 2 >= B / 2) {
-        hi = g[0];
-        lo = gl[0];
-      } else {
-        const float2 x = unpack2(g2[s / 2 < B / 2 ? s / 2 : 0]), y = unpack2(gl2[s / 2 < B / 2 ? s / 2 : 0]);
-        hi = s % 2 ? x.y : x.x;
-        lo = s % 2 ? y.y : y.x;
-      }
-      Gi[e] = hi;
-      if (MIXED) Gli[e] = lo;
-      if (row != col) {  // the mirrored entry
-        Gi[col * B + row] = hi;
-        if (MIXED) Gli[col * B + row] = lo;
-      }
+      Gi[s * NB] = g[s];
+      if (MIXED) Gli[s * NB] = gl[s];
     }
   }
   if (do_w && r == 0) {
@@ -309,16 +310,14 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
     if (MIXED) wlo[i] = wl;
   }
 #pragma unroll
-  for (int m = 0; m < NR; ++m) {
-    const int row = r + GS * m;
-    if (row < B) {
+  for (int k = 0; k < KC; ++k) {
+    const float2 x = unpack2(bb[k]), y = MIXED ? unpack2(bl[MIXED ? k : 0]) : make_float2(0.0f, 0.0f);
 #pragma unroll
-      for (int k = 0; k < KC; ++k)
-        if (k0 + k < K) {
-          bvec[(i * B + row) * K + k0 + k] = bb[m][k];
-          if (MIXED) blo[(i * B + row) * K + k0 + k] = bl[m][k];
-        }
-    }
+    for (int h = 0; h < 2; ++h)
+      if (owner && l2 + h < B && k0 + k < K) {
+        bvec[(i * B + l2 + h) * K + k0 + k] = h ? x.y : x.x;
+        if (MIXED) blo[(i * B + l2 + h) * K + k0 + k] = h ? y.y : y.x;
+      }
   }
 }
 
@@ -532,41 +531,71 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
     DevStatus* status, const float* __restrict__ acc, int RS, int n_acc_cams,
     const DevCam* __restrict__ cams, const float* __restrict__ means) {
   __shared__ float s_Y[MIXED ? kSolveThreads : 1][B + 1];  // per lane: basis of its camera (re-fold)
-  __shared__ float s_L[(kSolveThreads / kGroup) * B * (B + 1)];  // per group: the rows of L
+  constexpr int NGr = kSolveThreads / kGroup, GF = gram_floats(B), R3 = solve_record_floats(B);
+  __shared__ float s_L[NGr * B * (B + 1)];  // per group: the rows of L
+  // Per group the fold's block of G (its hi, then its lo parts), read as it lies in memory, and the record
+  // before it is written out as it lies; s_pos[r][c] = the place of entry (r, c) in the block.
+  __shared__ __align__(16) float s_G[NGr][MIXED ? 2 : 1][GF];
+  __shared__ __align__(16) float s_rec[NGr][R3];
+  __shared__ __align__(16) uint8_t s_pos[B][16];
+  for (int e = threadIdx.x; e < B * B; e += kSolveThreads) s_pos[e / B][e % B] = (uint8_t)gram_pos(e / B, e % B, B);
+  __syncthreads();
   const int64_t i = (blockIdx.x * (int64_t)kSolveThreads + threadIdx.x) / kGroup;
   const int r = threadIdx.x % kGroup;
   if (i >= n) return;
+  const int grp = threadIdx.x / kGroup;
   const bool row = r < B;
   float w = wsum[i];
   const float lam_r = row ? lam[r] : 0.0f;
   constexpr int P = B * (B + 1) / 2;
   float* rec = chol ? chol + i * solve_record_floats(B) : nullptr;
   if (!(w > 0.0f)) {
-    if (row) {
+    if (row)
       for (int k = 0; k < K; ++k) coeffs[(i * B + r) * K + k] = 0.0f;
-      if (rec)
-        for (int c = 0; c <= r; ++c) {  // no register array
-          const int e = r * (r + 1) / 2 + c;
-          rec[e] = 0.0f;
-          rec[P + e] = 0.0f;
-          rec[2 * P + e] = 0.0f;
-        }
-    }
+    if (rec)
+      for (int e = r; e < R3; e += kGroup) rec[e] = 0.0f;
     if (r == 0 && status_out) status_out[i] = kGaussUnseen;
     return;
   }
+  static_assert(GF % 4 == 0, "blocks are read 16 bytes at a time");
+#pragma unroll
+  for (int e = 0; e < GF / 4; e += kGroup)
+    if (e + r < GF / 4) {
+      reinterpret_cast<float4*>(s_G[grp][0])[e + r] = reinterpret_cast<const float4*>(G + i * GF)[e + r];
+      if (MIXED) reinterpret_cast<float4*>(s_G[grp][MIXED ? 1 : 0])[e + r] = reinterpret_cast<const float4*>(Glo + i * GF)[e + r];
+    }
+  __syncwarp(group_mask());
+  uint32_t pos[4] = {0u, 0u, 0u, 0u};  // the places of this lane's row, a byte each
+  if (row) {
+    const uint4 u = *reinterpret_cast<const uint4*>(s_pos[r]);
+    pos[0] = u.x;
+    pos[1] = u.y;
+    pos[2] = u.z;
+    pos[3] = u.w;
+  }
+  auto gram = [&](int part, int c) -> float { return row ? s_G[grp][part][(pos[c / 4] >> (8 * (c % 4))) & 0xFFu] : 0.0f; };
+  // writes the record out, once it is complete in s_rec
+  float* const rec_s = s_rec[grp];
+  auto write_record = [&]() {
+    __syncwarp(group_mask());
+    if (R3 % 4 == 0 && (reinterpret_cast<uintptr_t>(chol) & 15u) == 0) {
+      for (int e = r; e < R3 / 4; e += kGroup) reinterpret_cast<float4*>(rec)[e] = reinterpret_cast<const float4*>(rec_s)[e];
+    } else {
+      for (int e = r; e < R3; e += kGroup) rec[e] = rec_s[e];
+    }
+  };
   float a[B];
 #pragma unroll
   for (int c = 0; c < B; ++c) {
-    a[c] = row ? G[(i * B + r) * B + c] : 0.0f;
+    a[c] = gram(0, c);
     if (c == r) a[c] += w * lam_r;
   }
   if (!MIXED && rec && row) {  // PLAIN: A in FP32 (no compensation term)
 #pragma unroll
     for (int c = 0; c < B; ++c)
       if (c <= r) {
-        rec[P + r * (r + 1) / 2 + c] = a[c];
-        rec[2 * P + r * (r + 1) / 2 + c] = 0.0f;
+        rec_s[P + r * (r + 1) / 2 + c] = a[c];
+        rec_s[2 * P + r * (r + 1) / 2 + c] = 0.0f;
       }
   }
   float minratio = group_cholesky<B, float>(a, r);
@@ -603,8 +632,8 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
       wl = wlo[i];
 #pragma unroll
       for (int c = 0; c < B; ++c) {
-        ghi[c] = row ? G[(i * B + r) * B + c] : 0.0f;
-        glo[c] = row ? Glo[(i * B + r) * B + c] : 0.0f;
+        ghi[c] = gram(0, c);
+        glo[c] = gram(MIXED ? 1 : 0, c);
       }
     }
   }
@@ -618,8 +647,8 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
           two_sum_acc(hi, lo, p);
           lo += fmaf(w, lam_r, -p) + wl * lam_r;
         }
-        rec[P + r * (r + 1) / 2 + c] = hi;
-        rec[2 * P + r * (r + 1) / 2 + c] = lo;
+        rec_s[P + r * (r + 1) / 2 + c] = hi;
+        rec_s[2 * P + r * (r + 1) / 2 + c] = lo;
       }
   }
   const bool fp64 = MIXED && !(minratio >= (refold ? cond_tau * kRefoldFp64Scale : cond_tau));
@@ -674,10 +703,11 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
       for (int q = 0; q < NR; ++q)
         if (row && k0 + q < K) coeffs[(i * B + r) * K + k0 + q] = x[q];
     }
-    if (chol && row) {
+    if (rec) {
 #pragma unroll
       for (int c = 0; c < B; ++c)
-        if (c <= r) chol[i * solve_record_floats(B) + r * (r + 1) / 2 + c] = a[c];
+        if (row && c <= r) rec_s[r * (r + 1) / 2 + c] = a[c];
+      write_record();
     }
     if (r == 0 && status_out) status_out[i] = kGaussOk;
     return;
@@ -717,10 +747,11 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
       if (row) coeffs[(i * B + r) * K + k0 + q] = (float)x;
     }
   }
-  if (chol && row) {
+  if (rec) {
 #pragma unroll
     for (int c = 0; c < B; ++c)
-      if (c <= r) chol[i * solve_record_floats(B) + r * (r + 1) / 2 + c] = (float)ad[c];
+      if (row && c <= r) rec_s[r * (r + 1) / 2 + c] = (float)ad[c];
+    write_record();
   }
   if (r == 0) {
     if (status_out) status_out[i] = kGaussFp64;
@@ -1085,10 +1116,6 @@ __device__ __forceinline__ void packed_rc(int k, int B, int& r, int& c) {
   }
   c = r + k;
 }
-__device__ __forceinline__ int packed_index(int r, int c, int B) {  // r <= c
-  return r * B - r * (r - 1) / 2 + (c - r);
-}
-
 __global__ void k_export_packed(int64_t n, int B, int K, const float* __restrict__ G, const float* __restrict__ Glo,
                                 const float* __restrict__ b, const float* __restrict__ blo,
                                 const float* __restrict__ w, const float* __restrict__ wlo, double* __restrict__ out) {
@@ -1101,7 +1128,7 @@ __global__ void k_export_packed(int64_t n, int B, int K, const float* __restrict
     if (k < P) {
       int r, c;
       packed_rc(k, B, r, c);
-      const int64_t idx = (i * B + r) * B + c;
+      const int64_t idx = i * gram_floats(B) + gram_pos(r, c, B);
       v = (double)G[idx] + (Glo ? (double)Glo[idx] : 0.0);
     } else if (k < P + B * K) {
       const int64_t idx = i * B * K + (k - P);
@@ -1132,20 +1159,22 @@ __device__ __forceinline__ void split_double(double x, float& hi, float& lo) {
 __global__ void k_import_packed(int64_t n, int B, int K, const double* __restrict__ in, float* __restrict__ G,
                                 float* __restrict__ Glo, float* __restrict__ b, float* __restrict__ blo,
                                 float* __restrict__ w, float* __restrict__ wlo) {
-  const int P = B * (B + 1) / 2, R = P + B * K + 1, E = B * B + B * K + 1;
+  const int P = B * (B + 1) / 2, R = P + B * K + 1, E = R;
   const int64_t total = n * (int64_t)E, stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += stride) {
     const int64_t i = e / E;
     const int k = (int)(e - i * E);
     const double* row = in + i * R;
     float hi, lo;
-    if (k < B * B) {
-      const int r = k / B, c = k - r * B;
-      split_double(row[r <= c ? packed_index(r, c, B) : packed_index(c, r, B)], hi, lo);
-      G[i * B * B + k] = hi;
-      if (Glo) Glo[i * B * B + k] = lo;
-    } else if (k < B * B + B * K) {
-      const int kk = k - B * B;
+    if (k < P) {
+      int r, c;
+      packed_rc(k, B, r, c);
+      split_double(row[k], hi, lo);
+      const int64_t idx = i * gram_floats(B) + gram_pos(r, c, B);
+      G[idx] = hi;
+      if (Glo) Glo[idx] = lo;
+    } else if (k < P + B * K) {
+      const int kk = k - P;
       split_double(row[P + kk], hi, lo);
       b[i * B * K + kk] = hi;
       if (blo) blo[i * B * K + kk] = lo;
