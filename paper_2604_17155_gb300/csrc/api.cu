@@ -259,8 +259,12 @@ struct UploadBatch {
 };
 static_assert(sizeof(UploadBatch) + 2 * sizeof(void*) <= 32000, "kernel parameter space");
 
-__global__ void k_upload(const UploadBatch batch, DevCam* __restrict__ dst, float* __restrict__ lam_dst) {
+// status: zeroed when given (the first batch of a call)
+__global__ void k_upload(const UploadBatch batch, DevCam* __restrict__ dst, float* __restrict__ lam_dst,
+                         DevStatus* __restrict__ status) {
   const int t = threadIdx.x;
+  static_assert(sizeof(DevStatus) % 4 == 0 && sizeof(DevStatus) / 4 <= kUploadCams, "a word per thread");
+  if (status && t < (int)(sizeof(DevStatus) / 4)) reinterpret_cast<uint32_t*>(status)[t] = 0u;
   if (t < batch.count) dst[t] = batch.cams[t];
   if (t < batch.n_lam) lam_dst[t] = batch.lam[t];
 }
@@ -269,7 +273,6 @@ icgs_status upload_common(const Problem& p, const icgs_cameras* cams, const floa
                           const Workspace& ws, cudaStream_t s) {
   const std::vector<DevCam> dc = build_cams(cams);
   g_launches = 0;
-  ICGS_TRY_CUDA(cudaMemsetAsync(ws.status, 0, sizeof(DevStatus), s));
   UploadBatch batch;
   for (size_t j0 = 0; j0 < dc.size(); j0 += kUploadCams) {
     std::memset(&batch, 0, sizeof batch);
@@ -279,7 +282,7 @@ icgs_status upload_common(const Problem& p, const icgs_cameras* cams, const floa
       batch.n_lam = p.B;
       std::memcpy(batch.lam, lam_host, sizeof(float) * (size_t)p.B);
     }
-    k_upload<<<1, kUploadCams, 0, s>>>(batch, ws.cams + j0, ws.lam);
+    k_upload<<<1, kUploadCams, 0, s>>>(batch, ws.cams + j0, ws.lam, j0 == 0 ? ws.status : nullptr);
     ICGS_TRY_CUDA(cudaGetLastError());
     icgs::note_launches(1);
   }
@@ -292,8 +295,8 @@ icgs_status upload_common(const Problem& p, const icgs_cameras* cams, const floa
 icgs_status bin_pass(const Problem& p, const icgs_scene* sc, int cb, bool first, const Workspace& wp, cudaStream_t s) {
   const int64_t ct = (int64_t)cb * p.tiles;
   if (first) launch_spatial_order(p, sc->means, sc->scales, sc->quats, sc->opacity, wp, s);
-  ICGS_TRY_CUDA(cudaMemsetAsync(wp.tile_off, 0, sizeof(uint32_t) * (size_t)(ct + 1), s));
-  ICGS_TRY_CUDA(cudaMemsetAsync(wp.tile_cur, 0, sizeof(uint32_t) * (size_t)ct, s));
+  // the counts and the cursors, which follow them in the workspace
+  ICGS_TRY_CUDA(cudaMemsetAsync(wp.tile_off, 0, (size_t)(reinterpret_cast<char*>(wp.tile_cur + ct) - reinterpret_cast<char*>(wp.tile_off)), s));
   launch_project(p, sc->means, sc->scales, sc->quats, sc->opacity, cb, wp, s);
   g_timer.mark(kProject, s);
   launch_scan(p, cb, wp, s);
@@ -856,8 +859,13 @@ icgs_status icgs_solve(int64_t n, int32_t sh_degree, int32_t channels, const dou
   const Workspace ws = carve_solve(static_cast<char*>(workspace), p);
   if (p.n == 0) return ICGS_OK;
   g_launches = 0;
-  ICGS_TRY_CUDA(cudaMemsetAsync(ws.status, 0, sizeof(DevStatus), s));
-  ICGS_TRY_CUDA(cudaMemcpyAsync(ws.lam, lam, sizeof(float) * p.B, cudaMemcpyHostToDevice, s));
+  UploadBatch batch;
+  std::memset(&batch, 0, sizeof batch);
+  batch.n_lam = p.B;
+  std::memcpy(batch.lam, lam, sizeof(float) * (size_t)p.B);
+  k_upload<<<1, kUploadCams, 0, s>>>(batch, nullptr, ws.lam, ws.status);
+  ICGS_TRY_CUDA(cudaGetLastError());
+  icgs::note_launches(1);
   g_timer.begin(s);
   launch_import_normal(p, ws, sums, s);
   // the per-camera sums are not available here: no exact re-fold, FP64 below cond_tau
