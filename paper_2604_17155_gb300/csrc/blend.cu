@@ -259,10 +259,10 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
   uint32_t npairs = 0;
   int buf = 0;
   const uint32_t list_end = c.b + c.len;
-  const uint32_t id0 = group_id<kPP>(list, c.b, list_end, n);
-  uint32_t id_next = group_id<kPP>(list, c.b + kBatch, list_end, n);
+  const uint32_t id0 = group_id<kPP>(list, c.b, list_end, n, threadIdx.x);
+  uint32_t id_next = group_id<kPP>(list, c.b + kBatch, list_end, n, threadIdx.x);
   GroupFetch fetch = group_fetch(id0, rec_cam);
-  group_put<kPP>(fetch, (int)min((uint32_t)kBatch, c.len), c.ox, c.oy, s.geo);
+  group_put<kPP>(fetch, (int)min((uint32_t)kBatch, c.len), c.ox, c.oy, s.geo, s.lim, threadIdx.x);
   sa.ids.id[buf][threadIdx.x] = id0;
   __syncthreads();
   // two barriers a batch: the next batch is staged between them, when the walk of this one has ended
@@ -271,9 +271,9 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
     const uint32_t next = start + kBatch, id_fetched = id_next;
     if (next < c.len) {  // in flight during the walk
       fetch = group_fetch(id_fetched, rec_cam);
-      id_next = group_id<kPP>(list, c.b + next + kBatch, list_end, n);
+      id_next = group_id<kPP>(list, c.b + next + kBatch, list_end, n, threadIdx.x);
     }
-    const int steps = group_lists(s.geo, s.lists, c, nb, group_alive(T.alive()), sa.ids.hits);
+    const int steps = group_lists(s.geo, s.lim, s.lists, c, nb, group_alive(T.alive()), threadIdx.x, sa.ids.hits);
     auto reduce = [&](uint32_t o, const GroupW<kPP>& w) {
       float v[NP];
 #pragma unroll
@@ -340,7 +340,7 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
       }
     }
     if (next < c.len) {
-      group_put<kPP>(fetch, (int)min((uint32_t)kBatch, c.len - next), c.ox, c.oy, s.geo);
+      group_put<kPP>(fetch, (int)min((uint32_t)kBatch, c.len - next), c.ox, c.oy, s.geo, s.lim, threadIdx.x);
       sa.ids.id[buf ^ 1][threadIdx.x] = id_fetched;
     }
     if (!__syncthreads_or(T.alive())) break;
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 13 : 8) k_blend_accumulat
     float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
   __shared__ GroupBatch<kPP> s;
   __shared__ __align__(16) GroupAcc<KC> sa;
-  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height);
+  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
   if (threadIdx.x == 0) group_pad(s.geo);
   float tv[2 * kPP][KC];
 #pragma unroll
@@ -503,18 +503,18 @@ __device__ __forceinline__ void group_render(GroupBatch<kPP>& s, GroupColours& c
   uint32_t unused = 0;
   __syncthreads();
   const uint32_t list_end = c.b + c.len;
-  uint32_t id_next = group_id<kPP>(list, c.b, list_end, n);
+  uint32_t id_next = group_id<kPP>(list, c.b, list_end, n, threadIdx.x);
   auto stage = [&](uint32_t first) {  // the batch at slot first of the list, whose indices id_next holds
     const int nb = (int)min((uint32_t)kBatch, list_end - first);
-    group_put<kPP>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo);
+    group_put<kPP>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo, s.lim, threadIdx.x);
     stage_colours<KC>(pay_cam, id_next, nb, K, k0, col, weird);
   };
   stage(c.b);
   __syncthreads();
   for (uint32_t start = 0; start < c.len; start += kBatch) {
     const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n);
-    const int steps = group_lists(s.geo, s.lists, c, nb, group_alive(T.alive()), nullptr);
+    id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n, threadIdx.x);
+    const int steps = group_lists(s.geo, s.lim, s.lists, c, nb, group_alive(T.alive()), threadIdx.x, nullptr);
     auto blend = [&](uint32_t o, const GroupW<kPP>& w, bool guard) {
       const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(reinterpret_cast<const char*>(col.c01) + o);
       ulonglong2 c23 = make_ulonglong2(0ull, 0ull);
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(kGThreads, 13) k_blend_render2(
   __shared__ GroupBatch<kPP> s;
   __shared__ GroupColours col;
   __shared__ int weird;
-  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height);
+  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
   if (threadIdx.x == 0) group_pad(s.geo);
   f2 img[kPP][KC];
   group_render<KC>(s, col, &weird, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n,
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
   __shared__ GroupIds<kPP> ids;
   __shared__ float s_go[kGroups][kBatch + 1];
   __shared__ int weird;
-  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height);
+  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
   const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const int lane = threadIdx.x & 31;
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
   uint32_t id_next = 0;
   auto stage = [&](uint32_t first, int to) {  // the batch at slot first of the list, whose indices id_next holds
     const int nb = (int)min((uint32_t)kBatch, list_end - first);
-    group_put<kPP>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo);
+    group_put<kPP>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo, s.lim, threadIdx.x);
     ids.id[to][threadIdx.x] = id_next;
     stage_payload<KC>(pay_cam, id_next, nb, K, pay, &weird);
   };
@@ -829,13 +829,13 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
       for (int k = 0; k < KC; ++k) gt[u][k] = pack2(0.0f, 0.0f);
     }
     GroupT<kPP> T(c);
-    id_next = group_id<kPP>(list, c.b, list_end, n);
+    id_next = group_id<kPP>(list, c.b, list_end, n, threadIdx.x);
     stage(c.b, 0);
     __syncthreads();
     for (uint32_t start = 0; start < c.len; start += kBatch) {
       const int nb = (int)min((uint32_t)kBatch, c.len - start);
-      id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n);
-      const int steps = group_lists(s.geo, s.lists, c, nb, group_alive(T.alive()), nullptr);
+      id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n, threadIdx.x);
+      const int steps = group_lists(s.geo, s.lim, s.lists, c, nb, group_alive(T.alive()), threadIdx.x, nullptr);
       auto gather = [&](uint32_t o, const GroupW<kPP>& w, bool guard) {
         f2 a[KC + 1];
         load_group_payload<KC>(pay, o, a);
@@ -882,13 +882,13 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
   const bool second = (lane & 4) != 0;  // this lane's half of the group returns the second hit's sum
   float* const my_go = s_go[c.group];
   int buf = 0;
-  id_next = group_id<kPP>(list, c.b, list_end, n);
+  id_next = group_id<kPP>(list, c.b, list_end, n, threadIdx.x);
   stage(c.b, buf);
   __syncthreads();
   for (uint32_t start = 0; start < c.len; start += kBatch, buf ^= 1) {
     const int nb = (int)min((uint32_t)kBatch, c.len - start);
-    id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n);
-    const int steps = group_lists(s.geo, s.lists, c, nb, group_alive(T.alive()), ids.hits);
+    id_next = group_id<kPP>(list, c.b + start + kBatch, list_end, n, threadIdx.x);
+    const int steps = group_lists(s.geo, s.lim, s.lists, c, nb, group_alive(T.alive()), threadIdx.x, ids.hits);
     auto step = [&](uint32_t o, const GroupAlpha<kPP>& al, bool guard) -> float {
       GroupT<kPP> Tm = T;
       const GroupW<kPP> w = group_take<false>(al, T, unused);
@@ -955,7 +955,7 @@ __global__ void __launch_bounds__(kGThreads, 13) k_blend_refine2(
   __shared__ GroupBatch<kPP> s;
   __shared__ __align__(16) GroupAcc<KC> sa;
   __shared__ int weird;
-  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height);
+  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
   if (threadIdx.x == 0) group_pad(s.geo);
   const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;

@@ -70,6 +70,17 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// Named barriers of some of the CTA's warps (barrier 0 is __syncthreads): wait with, or only announce, the
+// count threads that take part.
+template <int ID, int COUNT>
+__device__ __forceinline__ void bar_sync() {
+  asm volatile("barrier.cta.sync %0, %1;" ::"n"(ID), "n"(COUNT) : "memory");
+}
+template <int ID, int COUNT>
+__device__ __forceinline__ void bar_arrive() {
+  asm volatile("barrier.cta.arrive %0, %1;" ::"n"(ID), "n"(COUNT) : "memory");
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -123,6 +134,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
+}
+// One column.
+__device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
+  uint32_t r;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+  return r;
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -293,23 +310,26 @@ __host__ __device__ constexpr uint32_t tmem_cols() {
 
 template <int KT, int MG>
 __host__ __device__ constexpr int tc_ctas_per_sm() {
-  return MG == 64 ? 3 : 2;  // a bound for the compiler: 16 channels fit four
+  return MG == 64 ? (KT <= 16 ? 4 : 3) : 2;
 }
 
-// What sits in front of the operands: the barrier and flags (64 bytes), the staged geometry of this batch
-// and the next, and the hit lists. The geometry is stored once, not twice: the MMAs and the walk share
-// the shared-memory bandwidth, and the moves cost less than the wider loads (masks walk 88.1 -> 85.2 ms).
-constexpr int kTcThreads = GroupCfg<1>::kThreads;
-constexpr uint32_t kTcFlags = 64;
-template <int KT>
+// What sits in front of the operands: the barrier and flags, the staged geometry and the hit lists of two
+// batches. The geometry is stored once, not twice: the MMAs and the walk share the shared-memory
+// bandwidth, and the moves cost less than the wider loads (masks walk 88.1 -> 85.2 ms).
+constexpr int kTcWalkers = GroupCfg<1>::kThreads;  // warps 0-3
+constexpr int kTcThreads = 2 * kTcWalkers;         // and the helpers, warps 4-7
 struct TcBatch {
+  uint64_t mbar;
+  uint32_t tmem_slot;
+  uint32_t timeout[2];   // set by a thread whose wait gave up, by the parity of the batch
+  uint32_t tmax[8];
+  uint32_t alive[2][4];  // by parity and walker warp: groups with a pixel that has not stopped
+  uint32_t counts[2][kBatch / 4];  // list lengths by parity and group
   GroupGeo<false> geo[2];
-  GroupLists<1, true> lists;
+  float2 lim[kBatch];
+  GroupLists<1, true> lists[2];
 };
-template <int KT>
-__host__ __device__ constexpr uint32_t tc_front() {
-  return kTcFlags + (uint32_t)sizeof(TcBatch<KT>);
-}
+constexpr uint32_t kTcFront = (sizeof(TcBatch) + 15) / 16 * 16;
 
 template <int KT, bool BF16_TARGETS, int MG>
 __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_accumulate_tc(
@@ -321,47 +341,53 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
   constexpr int NB = tc_cols<KT, MG>();  // target channels + rows of ones (V)
   constexpr bool kB16 = KT == 16;        // B in the 11 KB region (b16_offset)
   extern __shared__ uint8_t smem_raw[];
-  // The barrier, the flags and the staged batch sit in front of the operands, which start at the next
+  // The barrier, the flags and the staged batches sit in front of the operands, which start at the next
   // 1024-byte boundary. A base that is not 128-byte aligned is reported (kFlagLayout) before any work.
   const uint32_t raw = smem_u32(smem_raw);
   if (raw & 127u) {
     if (threadIdx.x == 0) atomicOr(&status->flags, kFlagLayout);
     return;
   }
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 1);
-  // set by a thread whose wait gave up, in its batch's slot (even, odd): a slot is read after the next
-  // barrier only, when no thread writes it
-  uint32_t* s_timeout = tmem_slot + 1;  // [2]
-  uint32_t* s_tmax = s_timeout + 2;     // [4]
-  TcBatch<KT>& s = *reinterpret_cast<TcBatch<KT>*>(smem_raw + kTcFlags);
-  uint8_t* base = smem_raw + (((raw + tc_front<KT>() + 1023u) & ~1023u) - raw);
+  TcBatch& s = *reinterpret_cast<TcBatch*>(smem_raw);
+  uint8_t* base = smem_raw + (((raw + kTcFront + 1023u) & ~1023u) - raw);
   uint8_t* A_s = base;                                 // MG x 256 (32 KB)
   uint8_t* B_s = base + MG * kKPix * 2;                // NB x 256, or the 11 KB region
 
-  const GroupCtx<1> c = group_ctx<1>(tile_off, capacity, tiles, tiles_x, width, height);
+  // Walkers and helpers are numbered alike: tid, and warp 0-3 by K block and TMEM quarter.
+  const bool walker = threadIdx.x < kTcWalkers;
+  const int tid = threadIdx.x & (kTcWalkers - 1);
+  const GroupCtx<1> c = group_ctx<1>(tile_off, capacity, tiles, tiles_x, width, height, tid);
   if (c.len == 0) return;  // uniform: nothing binned to this tile
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tid >> 5, lane = tid & 31;
   // the MMA's K index of the thread's first pixel (the second is the next): 64 per warp block, row by row
-  const int lx = c.px % kTile, ly = c.py % kTile;
-  const int p = warp * 64 + (ly & 7) * 8 + (lx & 7);
+  const int p = warp * 64 + ((c.py % kTile) & 7) * 8 + ((c.px % kTile) & 7);
   const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;
   const uint32_t list_end = c.b + c.len;
-  const uint32_t id0 = group_id<1>(list, c.b, list_end, n);
-  uint32_t id_next = group_id<1>(list, c.b + MG, list_end, n);
-  GroupFetch fetch = group_fetch(id0, rec_cam);
+  // helpers: the indices of the first four batches and the records of the first
+  uint32_t id0 = 0, id1 = 0, id2 = 0, id3 = 0;
+  GroupFetch fetch = {make_float4(0.0f, 0.0f, 0.0f, 0.0f), make_float4(0.0f, 0.0f, 0.0f, 0.0f)};
+  if (!walker) {
+    id0 = group_id<1>(list, c.b, list_end, n, tid);
+    id1 = group_id<1>(list, c.b + MG, list_end, n, tid);
+    id2 = group_id<1>(list, c.b + 2 * MG, list_end, n, tid);
+    id3 = group_id<1>(list, c.b + 3 * MG, list_end, n, tid);
+    fetch = group_fetch(id0, rec_cam);
+  }
 
   // B: the tile's targets, transposed to [channel][pixel] and scaled by 2^sexp (the tile's largest
-  // magnitude in [2^14, 2^15)), then the rows of ones
+  // magnitude in [2^14, 2^15)), then the rows of ones. A walker takes the first half of its pixels'
+  // channels, the helper of the same number the second.
   float t_scale_inv;
   {
-    const uint16_t* src = targets + ((((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K);
+    constexpr int KH = KT / 2;
+    const int kh = walker ? 0 : KH;
+    const uint16_t* src = targets + ((((int64_t)(cam0 + c.j) * height + c.py) * width + c.px) * K) + kh;
     // the two pixels' channels, loaded 16 bytes at a time when the rows allow it
-    uint32_t tv[KT];  // (first pixel's value, second pixel's value)
+    uint32_t tv[KH];  // (first pixel's value, second pixel's value)
     if (c.in1[0] && K == KT && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
 #pragma unroll
-      for (int q = 0; q < KT / 8; ++q) {
+      for (int q = 0; q < KH / 8; ++q) {
         const uint4 u = __ldg(reinterpret_cast<const uint4*>(src) + q);
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(src + K) + q);
         const uint32_t a[4] = {u.x, u.y, u.z, u.w}, b[4] = {v.x, v.y, v.z, v.w};
@@ -373,29 +399,31 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
       }
     } else {
 #pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        const uint32_t a = c.in0[0] && k < K ? src[k] : 0u, b = c.in1[0] && k < K ? src[K + k] : 0u;
+      for (int k = 0; k < KH; ++k) {
+        const uint32_t a = c.in0[0] && kh + k < K ? src[k] : 0u, b = c.in1[0] && kh + k < K ? src[K + k] : 0u;
         tv[k] = a | (b << 16);
       }
     }
     // the largest magnitude: non-negative floats order like their bit patterns, in 16 bits too
     uint32_t m16 = 0u;
 #pragma unroll
-    for (int k = 0; k < KT; ++k) m16 = __vmaxu2(m16, tv[k] & 0x7FFF7FFFu);
+    for (int k = 0; k < KH; ++k) m16 = __vmaxu2(m16, tv[k] & 0x7FFF7FFFu);
     uint32_t m = max(m16 & 0xFFFFu, m16 >> 16);
     if (m >= (BF16_TARGETS ? 0x7F80u : 0x7C00u)) atomicOr(&status->flags, kFlagNonfinite);
     m = __reduce_max_sync(0xFFFFFFFFu, m);
-    if (lane == 0) s_tmax[warp] = m;
+    if (lane == 0) s.tmax[threadIdx.x >> 5] = m;
     if (threadIdx.x == 0) {
-      mbar_init(mbar, 1);
-      s_timeout[0] = s_timeout[1] = 0u;
+      mbar_init(&s.mbar, 1);
+      s.timeout[0] = s.timeout[1] = 0u;
     }
-    if (warp == 0) {
-      tmem_alloc(tmem_slot, tmem_cols<NB>());
+    if (threadIdx.x < 32) {
+      tmem_alloc(&s.tmem_slot, tmem_cols<NB>());
       tmem_relinquish();
     }
     __syncthreads();
-    m = max(max(s_tmax[0], s_tmax[1]), max(s_tmax[2], s_tmax[3]));
+    m = s.tmax[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) m = max(m, s.tmax[w]);
     const float gmax = target_value((uint16_t)m, BF16_TARGETS);
     int e = 0;
     if (gmax > 0.0f && isfinite(gmax)) frexpf(gmax, &e);  // gmax in [2^(e-1), 2^e)
@@ -404,163 +432,188 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
     // 2^sexp as a product of two powers of two that are normal floats (sexp is in -113..148)
     const float s1 = ldexpf(1.0f, sexp / 2), s2 = ldexpf(1.0f, sexp - sexp / 2);
 #pragma unroll
-    for (int k = 0; k < KT; ++k) {
+    for (int k = 0; k < KH; ++k) {
       const float x = target_value((uint16_t)(tv[k] & 0xFFFFu), BF16_TARGETS) * s1 * s2;
       const float y = target_value((uint16_t)(tv[k] >> 16), BF16_TARGETS) * s1 * s2;
-      *reinterpret_cast<__half2*>(B_s + (kB16 ? b16_offset(k, p) : kmajor_sw128(k, p, NB))) = __floats2half2_rn(x, y);
+      *reinterpret_cast<__half2*>(B_s + (kB16 ? b16_offset(kh + k, p) : kmajor_sw128(kh + k, p, NB))) = __floats2half2_rn(x, y);
     }
     if constexpr (kB16) {
       if (threadIdx.x < 64)
         reinterpret_cast<uint4*>(B_s + kB16Ones)[threadIdx.x] = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
-    } else {
+    } else if (walker) {
 #pragma unroll
       for (int k = KT; k < NB; ++k) *reinterpret_cast<uint32_t*>(B_s + kmajor_sw128(k, p, NB)) = 0x3C003C00u;
     }
   }
   const float v_scale_inv = ldexpf(1.0f, -kWScaleExp);
-  // the first batch's staging, and W cleared
-  constexpr int kCh = KT / 16;                            // 16-column chunks of S in the epilogue
-  const int g_own = tmem_row_of_lane<MG>(warp, lane);      // the batch row this thread adds
-  if (threadIdx.x < 2) group_pad(s.geo[threadIdx.x]);
-  group_put<1>(fetch, (int)min((uint32_t)MG, c.len), c.ox, c.oy, s.geo[0]);
-  // Gaussian g is staged by lanes 2 (g % 16) and 2 (g % 16) + 1 of warp g / 16, and its row added by
-  // lane g % 16 of the same warp, so its index goes from register to register
-  uint32_t my_id = __shfl_sync(0xFFFFFFFFu, id0, 2 * (lane & 15));
-  if (MG < c.len) {  // the second batch's records, and the third's indices
-    fetch = group_fetch(id_next, rec_cam);
-  }
-  uint32_t id_fetched = id_next;
-  id_next = group_id<1>(list, c.b + 2 * MG, list_end, n);
-  // Only warp w writes K block w of W (its pixels): it clears the block itself, and no other warp waits;
-  // and only the rows that it wrote (about a third).
+  constexpr float kT0 = (float)(1 << kWScaleExp);  // the transmittance carries the factor 2^14 of W
+  GroupT<1> T(c, kT0);
+  uint32_t npairs = 0, phase = 0;
+  bool ok = true;
+  const int n_first = (int)min((uint32_t)MG, c.len);
   uint4* const w_block = reinterpret_cast<uint4*>(A_s + warp * (MG * 128));
-  uint32_t dirty[2] = {0xFFFFFFFFu, 0xFFFFFFFFu}, listed[2] = {0u, 0u};
-  auto clear_w = [&]() {
+  uint32_t listed0[2] = {0u, 0u}, listed1[2] = {0u, 0u};  // rows of W that the walk of this batch / the next writes
+  if (!walker) {
+    if (tid < 2) group_pad(s.geo[tid]);
+    // the first two batches' geometry and lists, and W cleared (block w by helper warp w)
+    group_put<1>(fetch, n_first, c.ox, c.oy, s.geo[0], s.lim, tid);
+    fetch = group_fetch(id1, rec_cam);
 #pragma unroll
-    for (int i = 0; i < MG * 128 / 16; i += 32)  // four rows of 128 bytes at a time
-      if ((dirty[i / 256] >> (lane >> 3)) & (1u << ((i / 8) & 31))) w_block[i + lane] = make_uint4(0, 0, 0, 0);
-    __syncwarp();
-  };
-  clear_w();
+    for (int i = 0; i < MG * 128 / 16; i += 32) w_block[i + lane] = make_uint4(0, 0, 0, 0);
+    bar_sync<2, kTcWalkers>();
+    group_lists(s.geo[0], s.lim, s.lists[0], c, n_first, 0xFu, tid, nullptr, listed0, s.counts[0]);
+    if (MG < c.len) {
+      const int n_second = (int)min((uint32_t)MG, c.len - MG);
+      bar_sync<2, kTcWalkers>();  // lim has been read
+      group_put<1>(fetch, n_second, c.ox, c.oy, s.geo[1], s.lim, tid);
+      fetch = group_fetch(id2, rec_cam);
+      bar_sync<2, kTcWalkers>();
+      group_lists(s.geo[1], s.lim, s.lists[1], c, n_second, 0xFu, tid, nullptr, listed1, s.counts[1]);
+    }
+  }
+  fence_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t a_addr = smem_u32(A_s), b_addr = smem_u32(B_s);
-  constexpr uint32_t kIdesc = idesc_f16(MG, NB, false);
-  float* acc_cam = acc + (int64_t)c.j * acc_cam_stride;
-  constexpr float kT0 = (float)(1 << kWScaleExp);  // the transmittance carries the factor 2^14 of W
-  GroupT<1> T(c, kT0);
-  // kmajor_sw128(g, p, MG) in terms of the list entry o = 16 g: 8 o + ((o & 0x70) ^ pixel part)
-  char* const w_base = reinterpret_cast<char*>(A_s + warp * (MG * 128));
-  const uint32_t w_pix = (uint32_t)((((p & 63) >> 3) << 4) | ((p & 7) << 1));
-  const uint16_t* const my_list = s.lists.row[c.group];
-  uint32_t npairs = 0, phase = 0;
-  bool ok = true;
-  int steps = group_lists(s.geo[0], s.lists, c, (int)min((uint32_t)MG, c.len), group_alive(T.alive()), nullptr, listed);
-  // One CTA barrier per batch. Before it a warp stages its share of the next batch's geometry (in the
-  // buffer that the batch before this one used) and walks its lists; after it one thread issues the MMAs,
-  // and while they run every warp builds its lists of the next batch; then it waits for the MMAs, adds
-  // its quarter of the sums and clears its block of W.
-  for (uint32_t start = 0, buf = 0; start < c.len; start += MG, buf ^= 1u) {
-    const int nb = (int)min((uint32_t)MG, c.len - start);
-    const uint32_t next = start + MG;
-    uint32_t next_id = 0;
-    if (next < c.len) {
-      group_put<1>(fetch, (int)min((uint32_t)MG, c.len - next), c.ox, c.oy, s.geo[buf ^ 1u]);
-      next_id = __shfl_sync(0xFFFFFFFFu, id_fetched, 2 * (lane & 15));
-      // in flight during the walk: the records of the batch after it and the indices of the one after that
-      id_fetched = id_next;
-      if (next + MG < c.len) {
-        fetch = group_fetch(id_fetched, rec_cam);
-        id_next = group_id<1>(list, c.b + next + 2 * MG, list_end, n);
+  const uint32_t tmem = s.tmem_slot;
+
+  // Whether a batch follows the one of parity buf that starts at start, from what every walker warp wrote
+  // before the CTA barrier.
+  auto more_after = [&](uint32_t start, uint32_t buf) -> bool {
+    return start + MG < c.len && (s.alive[buf][0] | s.alive[buf][1] | s.alive[buf][2] | s.alive[buf][3]) != 0u;
+  };
+
+  if (walker) {
+    // Walk the lists of a batch into W, hand W to the tensor cores, wait until it is clear again.
+    const uint32_t a_addr = smem_u32(A_s), b_addr = smem_u32(B_s);
+    constexpr uint32_t kIdesc = idesc_f16(MG, NB, false);
+    // kmajor_sw128(g, p, MG) in terms of the list entry o = 16 g: 8 o + ((o & 0x70) ^ pixel part)
+    char* const w_base = reinterpret_cast<char*>(A_s + warp * (MG * 128));
+    const uint32_t w_pix = (uint32_t)((((p & 63) >> 3) << 4) | ((p & 7) << 1));
+    for (uint32_t start = 0, buf = 0;; start += MG, buf ^= 1u) {
+      // lists may still name groups whose pixels have all stopped since they were built
+      const bool live = (group_alive(T.alive()) >> (lane >> 3)) & 1u;
+      const int steps = (int)__reduce_max_sync(0xFFFFFFFFu, live ? s.counts[buf][c.group] : 0u);
+      const GroupGeo<false>& geo = s.geo[buf];
+      const uint16_t* const my_list = s.lists[buf].row[c.group];
+      for (int i = 0; i < steps; i += 2) {
+        const uint2 o = GroupLists<1, true>::pair(my_list, i);
+        const uint32_t o1 = o.x, o2 = o.y;
+        const GroupAlpha<1> a1 = group_alpha(geo, o1, c), a2 = group_alpha(geo, o2, c);  // independent of T
+        const float2 w1 = group_take<true, kWScaleExp>(a1, T, npairs).v[0];
+        const float2 w2 = group_take<true, kWScaleExp>(a2, T, npairs).v[0];
+        if (o1 != kGPad)
+          *reinterpret_cast<__half2*>(w_base + o1 * 8 + ((o1 & 0x70u) ^ w_pix)) = __floats2half2_rn(w1.x, w1.y);
+        if (o2 != kGPad)
+          *reinterpret_cast<__half2*>(w_base + o2 * 8 + ((o2 & 0x70u) ^ w_pix)) = __floats2half2_rn(w2.x, w2.y);
       }
+      const uint32_t alive = group_alive(T.alive());
+      if (lane == 0) s.alive[buf][warp] = alive;
+      fence_async_smem();
+      tc_fence_before();
+      bar_sync<1, kTcWalkers>();  // W is written
+      if (warp == 0) {
+        if (start > 0) bar_sync<3, kTcWalkers + 32>();  // the helpers have read the last batch's sums
+        if (lane == 0 && issue_mma) {
+          if constexpr (kB16) issue_batch_b16<MG>(a_addr, b_addr, tmem, kIdesc, &s.mbar);
+          else issue_batch<NB, MG>(a_addr, b_addr, tmem, kIdesc, &s.mbar);
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+      if (s.timeout[buf] || !more_after(start, buf)) break;
     }
-    if (!ok) steps = 0;  // a wait gave up: W may still be read
-    for (int i = 0; i < steps; i += 2) {
-      const uint2 o = s.lists.pair(my_list, i);
-      const uint32_t o1 = o.x, o2 = o.y;
-      const GroupAlpha<1> a1 = group_alpha(s.geo[buf], o1, c), a2 = group_alpha(s.geo[buf], o2, c);  // independent of T
-      const float2 w1 = group_take<true, kWScaleExp>(a1, T, npairs).v[0];
-      const float2 w2 = group_take<true, kWScaleExp>(a2, T, npairs).v[0];
-      if (o1 != kGPad)
-        *reinterpret_cast<__half2*>(w_base + o1 * 8 + ((o1 & 0x70u) ^ w_pix)) = __floats2half2_rn(w1.x, w1.y);
-      if (o2 != kGPad)
-        *reinterpret_cast<__half2*>(w_base + o2 * 8 + ((o2 & 0x70u) ^ w_pix)) = __floats2half2_rn(w2.x, w2.y);
-    }
-    fence_async_smem();
-    tc_fence_before();
-    const int alive = __syncthreads_or(T.alive());
-    if (s_timeout[buf ^ 1u]) break;  // uniform: the batch before this one timed out
-    if (threadIdx.x == 0 && issue_mma) {
-      if constexpr (kB16) issue_batch_b16<MG>(a_addr, b_addr, tmem, kIdesc, mbar);
-      else issue_batch<NB, MG>(a_addr, b_addr, tmem, kIdesc, mbar);
-    }
-    const bool more = next < c.len && alive;
+  } else {
+    // Wait for a batch's MMAs, clear W, and then, beside the next batch's walk, add the sums and prepare the
+    // geometry and lists of the batch after it.
+    constexpr int kCh = KT / 16;                            // 16-column chunks of S
+    const int g_own = tmem_row_of_lane<MG>(warp, lane);      // the batch row this thread adds
+    float* acc_cam = acc + (int64_t)c.j * acc_cam_stride;
+    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+    for (uint32_t start = 0, buf = 0;; start += MG, buf ^= 1u) {
+      // warp-uniform: tcgen05.ld needs whole warps
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(&s.mbar, phase, wait_limit_ns));
+      phase ^= 1u;
+      tc_fence_after();
+      if (ok) {  // the rows that the walk wrote (about a third), four of 128 bytes at a time
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      dirty[h] = listed[h];
-      listed[h] = 0u;
-    }
-    if (more)
-      steps = group_lists(s.geo[buf ^ 1u], s.lists, c, (int)min((uint32_t)MG, c.len - next), group_alive(T.alive()), nullptr,
-                          listed);
-    // warp-uniform: the epilogue's tcgen05.ld needs whole warps
-    ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(mbar, phase, wait_limit_ns));
-    phase ^= 1u;
-    tc_fence_after();
-    if (ok) {
-      // The accumulator streams through registers 16 columns at a time: chunk c adds the float4 groups
-      // 4c..4c+3 of the row (V, S_0, S_1, ..) and carries its last column into group 4c+4. Only the
+        for (int i = 0; i < MG * 128 / 16; i += 32)
+          if ((listed0[i / 256] >> (lane >> 3)) & (1u << ((i / 8) & 31))) w_block[i + lane] = make_uint4(0, 0, 0, 0);
+        fence_async_smem();
+      } else {
+        s.timeout[buf] = 1u;
+      }
+      __syncthreads();
+      if (s.timeout[buf]) break;
+      const bool more = more_after(start, buf);
+      // The accumulator streams through registers 16 columns at a time: chunk q adds the float4 groups
+      // 4q..4q+3 of the row (V, S_0, S_1, ..) and carries its last column into group 4q+4. Only the
       // first 16 lanes of each quarter hold a Gaussian (M = 64); every tcgen05.ld is warp-uniform.
-      const int g = g_own;
-      const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-      uint32_t vr[16], r[16];
-      tmem_ld16(trow + (uint32_t)KT, vr);  // the ones block: every column holds V
+      const int nb = (int)min((uint32_t)MG, c.len - start);
+      const uint32_t my_id = __shfl_sync(0xFFFFFFFFu, id0, 2 * (lane & 15));
+      uint32_t r[16];
+      const uint32_t vr = tmem_ld1(trow + (uint32_t)KT);  // the ones block: every column holds V
       tmem_ld16(trow, r);
       tmem_wait_ld();
-      const float V = __uint_as_float(vr[0]) * v_scale_inv;
+      const float V = __uint_as_float(vr) * v_scale_inv;
       float carry = V;
-      const bool add = g >= 0 && g < nb && V > 0.0f;
+      const bool add = g_own >= 0 && g_own < nb && V > 0.0f;
       float* dst = acc_cam + (int64_t)(add ? my_id : 0u) * RS;
 #pragma unroll
-      for (int c = 0; c < kCh; ++c) {
+      for (int q = 0; q < kCh; ++q) {
         float sv[16];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) sv[q] = __uint_as_float(r[q]) * t_scale_inv;
-        if (c + 1 < kCh) {
-          tmem_ld16(trow + (uint32_t)(16 * (c + 1)), r);
+        for (int h = 0; h < 16; ++h) sv[h] = __uint_as_float(r[h]) * t_scale_inv;
+        if (q + 1 < kCh) {
+          tmem_ld16(trow + (uint32_t)(16 * (q + 1)), r);
           tmem_wait_ld();
         }
+        if (q + 1 >= kCh && more) {  // every column is in registers: the next batch's MMAs may write
+          tc_fence_before();
+          bar_arrive<3, kTcWalkers + 32>();
+        }
         if (add) {
-          float* d = dst + 16 * c;
-          if (16 * c < RS) atomicAdd(reinterpret_cast<float4*>(d), make_float4(carry, sv[0], sv[1], sv[2]));
-          if (16 * c + 4 < RS) atomicAdd(reinterpret_cast<float4*>(d + 4), make_float4(sv[3], sv[4], sv[5], sv[6]));
-          if (16 * c + 8 < RS) atomicAdd(reinterpret_cast<float4*>(d + 8), make_float4(sv[7], sv[8], sv[9], sv[10]));
-          if (16 * c + 12 < RS)
+          float* d = dst + 16 * q;
+          if (16 * q < RS) atomicAdd(reinterpret_cast<float4*>(d), make_float4(carry, sv[0], sv[1], sv[2]));
+          if (16 * q + 4 < RS) atomicAdd(reinterpret_cast<float4*>(d + 4), make_float4(sv[3], sv[4], sv[5], sv[6]));
+          if (16 * q + 8 < RS) atomicAdd(reinterpret_cast<float4*>(d + 8), make_float4(sv[7], sv[8], sv[9], sv[10]));
+          if (16 * q + 12 < RS)
             atomicAdd(reinterpret_cast<float4*>(d + 12), make_float4(sv[11], sv[12], sv[13], sv[14]));
         }
         carry = sv[15];
+        __syncwarp();
       }
       // the last group (S_{KT-1}, 0, 0, 0)
       if (add && 16 * kCh < RS) atomicAdd(reinterpret_cast<float4*>(dst + 16 * kCh), make_float4(carry, 0.0f, 0.0f, 0.0f));
-      if (more) clear_w();  // this batch's MMAs have completed
-    } else {
-      s_timeout[buf] = 1u;  // seen by every warp after the next barrier
+      if (!more) break;
+      listed0[0] = listed1[0];
+      listed0[1] = listed1[1];
+      listed1[0] = listed1[1] = 0u;
+      const uint32_t after = start + 2 * MG;  // the batch that takes this one's buffers
+      if (after < c.len) {
+        const int na = (int)min((uint32_t)MG, c.len - after);
+        group_put<1>(fetch, na, c.ox, c.oy, s.geo[buf], s.lim, tid);
+        fetch = group_fetch(id3, rec_cam);
+        const uint32_t alive = s.alive[buf][warp];
+        bar_sync<2, kTcWalkers>();
+        group_lists(s.geo[buf], s.lim, s.lists[buf], c, na, alive, tid, nullptr, listed1, s.counts[buf]);
+      }
+      id0 = id1;
+      id1 = id2;
+      id2 = id3;
+      id3 = group_id<1>(list, c.b + start + 4 * MG, list_end, n, tid);
     }
-    my_id = next_id;
-    if (!more) break;
   }
   tc_fence_before();
   __syncthreads();
-  if (s_timeout[0] | s_timeout[1]) {
+  if (s.timeout[0] | s.timeout[1]) {
     if (threadIdx.x == 0) atomicOr(&status->flags, kFlagTimeout);
-    if (!ok) mbar_wait_bounded(mbar, phase ^ 1u, wait_limit_ns);  // a last chance for the outstanding MMAs
+    if (!ok) mbar_wait_bounded(&s.mbar, phase ^ 1u, wait_limit_ns);  // a last chance for the outstanding MMAs
   }
-  add_pair_count(npairs, status);
+  if (walker) add_pair_count(npairs, status);
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (threadIdx.x < 32) {
     tc_fence_after();
     tmem_dealloc(tmem, tmem_cols<NB>());
   }
@@ -573,7 +626,7 @@ constexpr size_t selftest_smem() {
 // the barrier, flags and staged batch with up to 1023 bytes of alignment, W, and B
 template <int KT, int MG>
 constexpr size_t tc_smem() {
-  return tc_front<KT>() + 1023 + (size_t)MG * kKPix * 2 + (KT == 16 ? (size_t)kB16Bytes : (size_t)tc_cols<KT, MG>() * kKPix * 2);
+  return kTcFront + 1023 + (size_t)MG * kKPix * 2 + (KT == 16 ? (size_t)kB16Bytes : (size_t)tc_cols<KT, MG>() * kKPix * 2);
 }
 // CTAs per SM that the shared memory admits: each CTA's share rounded up to 1 KB, plus 1 KB the
 // system reserves per CTA, out of the SM's 228 KB

@@ -51,7 +51,8 @@ struct GroupCfg {
   static constexpr float kHalfX = PP == 2 ? 3.5f : 1.5f, kHalfY = 1.5f;  // pixel centres off the block's centre
 };
 
-// A lane's pixels: (px, py), (px + 1, py) and, with PP = 2, (px, py + 2), (px + 1, py + 2).
+// The walk's threads are numbered tid = 0 .. GroupCfg::kThreads - 1, which a kernel with other warps beside
+// them passes on. A lane's pixels: (px, py), (px + 1, py) and, with PP = 2, (px, py + 2), (px + 1, py + 2).
 template <int PP>
 struct GroupCtx {
   int j, t, px, py;         // camera, tile, first pixel
@@ -65,13 +66,13 @@ struct GroupCtx {
 
 template <int PP>
 __device__ __forceinline__ GroupCtx<PP> group_ctx(const uint32_t* __restrict__ tile_off, uint32_t capacity, int tiles,
-                                                  int tiles_x, int width, int height) {
+                                                  int tiles_x, int width, int height, int tid) {
   GroupCtx<PP> c;
   const int bid = blockIdx.x;
   c.j = bid / tiles;
   c.t = bid - c.j * tiles;
   const int tyi = c.t / tiles_x, txi = c.t - tyi * tiles_x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tid >> 5, lane = tid & 31;
   const int gq = lane >> 3, l = lane & 7;
   const int bx = PP == 2 ? 0 : (warp & 1) * 8, by = PP == 2 ? warp * 8 : (warp >> 1) * 8;
   const int lx = bx + (gq & 1) * 4 * PP + (PP == 2 ? l & 3 : l & 1) * 2;
@@ -118,7 +119,8 @@ struct GroupT {
 // The geometry of a batch of kBatch Gaussians as the groups read it (slot kBatch: the padding). The means
 // are negated, so that the offset pixel - mean is one packed addition. With DUP every value is stored
 // twice, so that a packed operand is read and not assembled (three 16-byte loads a step); without, a
-// step takes a 16-byte and an 8-byte load and six moves, for half the shared memory.
+// step takes a 16-byte and an 8-byte load and six moves, for half the shared memory. What only the list
+// test reads is apart: lim = (E_lim, packed half-sizes of the support box) per Gaussian.
 struct GroupOperands {
   f2 nx, ny, A, Bc, C, o;
 };
@@ -127,7 +129,6 @@ struct GroupGeo;
 template <>
 struct GroupGeo<true> {
   float4 xy[kBatch + 1], ab[kBatch + 1], co[kBatch + 1];  // (-mx, -mx, -my, -my), (A, A, Bc, Bc), (C, C, o, o)
-  float2 lim[kBatch];                                     // (E_lim, packed half-sizes of the support box)
   __device__ __forceinline__ void put_mean(int g, float nx, float ny, float A, float Bc) {
     xy[g] = make_float4(nx, nx, ny, ny);
     ab[g] = make_float4(A, A, Bc, Bc);
@@ -144,7 +145,6 @@ template <>
 struct GroupGeo<false> {
   float4 xyab[kBatch + 1];  // (-mx, -my, A, Bc)
   float2 co[kBatch + 1];    // (C, o)
-  float2 lim[kBatch];
   __device__ __forceinline__ void put_mean(int g, float nx, float ny, float A, float Bc) { xyab[g] = make_float4(nx, ny, A, Bc); }
   __device__ __forceinline__ void put_rest(int g, float C, float o) { co[g] = make_float2(C, o); }
   __device__ __forceinline__ GroupOperands at(uint32_t off) const {
@@ -155,11 +155,11 @@ struct GroupGeo<false> {
 };
 
 // The groups' hit lists of a batch: byte offsets (16 per Gaussian) into the geometry, or with BYTES the
-// slots themselves, which saves a KB where shared memory decides the CTAs per SM. Row strides of 144 /
-// 80 bytes put four groups' rows in distinct banks.
+// slots themselves, which saves a KB where shared memory decides the CTAs per SM. A row stride of 144
+// bytes puts four groups' rows in distinct banks.
 template <int PP, bool BYTES = false>
 struct GroupLists {
-  static constexpr int kStride = BYTES ? 80 : 72;  // entries of a row
+  static constexpr int kStride = BYTES ? 64 : 72;  // entries of a row
   uint16_t row[GroupCfg<PP>::kGroups][kStride / (BYTES ? 2 : 1)];
 
   // the byte offsets of entries i, i + 1 (i even) of a group's row
@@ -178,6 +178,7 @@ struct GroupLists {
 template <int PP>
 struct GroupBatch {
   GroupGeo<true> geo;
+  float2 lim[kBatch];
   GroupLists<PP> lists;
 };
 
@@ -211,16 +212,17 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // the odd one (C, opacity) and what the list test reads). In three parts, so that the two dependent
 // loads are off the path: a batch's indices are loaded two batches ahead, its records one batch ahead.
 template <int PP>
-__device__ __forceinline__ int group_slot() {
-  return PP == 2 ? (int)threadIdx.x : (int)(threadIdx.x >> 1);
+__device__ __forceinline__ int group_slot(int tid) {
+  return PP == 2 ? tid : tid >> 1;
 }
 struct GroupFetch {
   float4 box, par;
 };
 // The index of the thread's Gaussian of the batch that starts at slot first; 0 past the list's end.
 template <int PP>
-__device__ __forceinline__ uint32_t group_id(const unsigned long long* list, uint32_t first, uint32_t end, int64_t n) {
-  const uint32_t at = first + (uint32_t)group_slot<PP>();
+__device__ __forceinline__ uint32_t group_id(const unsigned long long* list, uint32_t first, uint32_t end, int64_t n,
+                                             int tid) {
+  const uint32_t at = first + (uint32_t)group_slot<PP>(tid);
   return at < end ? min((uint32_t)list[at], (uint32_t)(n - 1)) : 0u;
 }
 __device__ __forceinline__ GroupFetch group_fetch(uint32_t id, const ProjRec* __restrict__ rec_cam) {
@@ -233,23 +235,24 @@ __device__ __forceinline__ GroupFetch group_fetch(uint32_t id, const ProjRec* __
 // of itself and 7.2e-5; the approximate logarithm and roots are within 2^-20, and the square is
 // widened by 1e-5.
 template <int PP, bool DUP>
-__device__ __forceinline__ void group_put(const GroupFetch& f, int nb, float ox, float oy, GroupGeo<DUP>& geo) {
-  const int g = group_slot<PP>();
+__device__ __forceinline__ void group_put(const GroupFetch& f, int nb, float ox, float oy, GroupGeo<DUP>& geo,
+                                          float2* lim, int tid) {
+  const int g = group_slot<PP>(tid);
   if (g >= nb) return;
   const float A = -kHalfLog2e * f.par.x, Bc = -2.0f * kHalfLog2e * f.par.y, C = -kHalfLog2e * f.par.z;
-  if (PP == 2 || (threadIdx.x & 1) == 0) {
+  if (PP == 2 || (tid & 1) == 0) {
     const float2 lo = unpack_half2(f.box.z);
     const float mx = __fadd_rn(__fsub_rn(f.box.x, ox), __fmul_rn(lo.x, kMeanLoScaleInv));
     const float my = __fadd_rn(__fsub_rn(f.box.y, oy), __fmul_rn(lo.y, kMeanLoScaleInv));
     geo.put_mean(g, -mx, -my, A, Bc);
   }
-  if (PP == 2 || (threadIdx.x & 1) == 1) {
+  if (PP == 2 || (tid & 1) == 1) {
     constexpr float hx = GroupCfg<PP>::kHalfX, hy = GroupCfg<PP>::kHalfY;
     const float thr = fmaf(fmaxf(lg2_approx(255.0f * f.par.w), 0.0f), 1.0001f, 7.2e-5f);
     const float corner = fmaf(hx * hx, fabsf(A), fmaf(hy * hy, fabsf(C), hx * hy * fabsf(Bc)));
     const float reach = sqrt_approx(thr) + sqrt_approx(corner);
     geo.put_rest(g, C, f.par.w);
-    geo.lim[g] = make_float2(-1.00001f * reach * reach, f.box.w);
+    lim[g] = make_float2(-1.00001f * reach * reach, f.box.w);
   }
 }
 
@@ -263,12 +266,14 @@ __device__ __forceinline__ void group_put(const GroupFetch& f, int nb, float ox,
 // the instructions. The margin for rounding is 2e-5 of |A dx^2| + |C dy^2|, which bounds half the sum of
 // the three terms' magnitudes (the conic is positive definite); E itself is a few 2^-24 of those off.
 // alive: bit q set while group q has a pixel that has not stopped. hits: the per-Gaussian masks, when
-// wanted. any: the Gaussians that some group of the warp lists (two words, ORed into), when wanted.
+// wanted. any: the Gaussians that some group of the warp lists (two words, ORed into), counts: the
+// tile's list lengths by group, when wanted.
 template <int PP, bool DUP, bool BYTES>
-__device__ __forceinline__ int group_lists(const GroupGeo<DUP>& geo, GroupLists<PP, BYTES>& lists, const GroupCtx<PP>& c,
-                                           int nb, uint32_t alive, uint8_t (*hits)[GroupCfg<PP>::kWarps],
-                                           uint32_t* any = nullptr) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__device__ __forceinline__ int group_lists(const GroupGeo<DUP>& geo, const float2* lim_of, GroupLists<PP, BYTES>& lists,
+                                           const GroupCtx<PP>& c, int nb, uint32_t alive, int tid,
+                                           uint8_t (*hits)[GroupCfg<PP>::kWarps], uint32_t* any = nullptr,
+                                           uint32_t* counts = nullptr) {
+  const int warp = tid >> 5, lane = tid & 31;
   constexpr int kStride = GroupLists<PP, BYTES>::kStride;
   constexpr float wx = 4.0f * PP;  // block width
   uint16_t* const rows = lists.row[warp * 4];
@@ -279,8 +284,10 @@ __device__ __forceinline__ int group_lists(const GroupGeo<DUP>& geo, GroupLists<
   for (int i = 0; i < kRowStores; i += 32)
     if (i + lane < kRowStores) reinterpret_cast<uint4*>(rows)[i + lane] = make_uint4(kPad, kPad, kPad, kPad);
   __syncwarp();
-  int cnt[4] = {0, 0, 0, 0};
-  const uint32_t lt = (1u << lane) - 1u;
+  // Lane (q, j) writes the entries of group q whose Gaussians lie in the j-th four of each 32.
+  const int gq = lane >> 3, j4 = (lane & 7) * 4;
+  uint16_t* const my_row = reinterpret_cast<uint16_t*>(reinterpret_cast<char*>(rows) + gq * kStride * (BYTES ? 1 : 2));
+  int cnt = 0;
 #pragma unroll
   for (int half = 0; half < kBatch / 32; ++half) {
     if (half * 32 >= nb) break;  // uniform
@@ -288,8 +295,8 @@ __device__ __forceinline__ int group_lists(const GroupGeo<DUP>& geo, GroupLists<
     bool h[4] = {false, false, false, false};
     if (g < nb) {
       const GroupOperands op = geo.at((uint32_t)g * 16u);
-      const float2 lim = geo.lim[g], half = unpack_half2(lim.y);
-      const float hx = half.x + GroupCfg<PP>::kHalfX, hy = half.y + GroupCfg<PP>::kHalfY;
+      const float2 lim = lim_of[g], half2 = unpack_half2(lim.y);
+      const float hx = half2.x + GroupCfg<PP>::kHalfX, hy = half2.y + GroupCfg<PP>::kHalfY;
       const f2 dx = add2(pack2(c.bx + 0.5f * wx, c.bx + 1.5f * wx), op.nx);
       const f2 ax = mul2(mul2(op.A, dx), dx), bx = mul2(op.Bc, dx);
       const float2 dxs = unpack2(dx);
@@ -304,25 +311,35 @@ __device__ __forceinline__ int group_lists(const GroupGeo<DUP>& geo, GroupLists<
         h[2 * v] = e.x >= lim.x && in_x[0] && in_y;
         h[2 * v + 1] = e.y >= lim.x && in_x[1] && in_y;
       }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) h[q] = h[q] && ((alive >> q) & 1u);
-      if (hits) hits[g][warp] = (uint8_t)((h[0] ? 1 : 0) | (h[1] ? 2 : 0) | (h[2] ? 4 : 0) | (h[3] ? 8 : 0));
     }
+    uint32_t m[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t m = __ballot_sync(kFull, h[q]);
-      const int at = q * kStride + cnt[q] + __popc(m & lt);
+    for (int q = 0; q < 4; ++q) m[q] = __ballot_sync(kFull, h[q] && ((alive >> q) & 1u));
+    if (hits && g < nb) {
+      uint32_t byte = 0u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) byte |= ((m[q] >> lane) & 1u) << q;
+      hits[g][warp] = (uint8_t)byte;
+    }
+    if (any) any[half] |= (m[0] | m[1]) | (m[2] | m[3]);
+    const uint32_t mine = gq < 2 ? (gq == 0 ? m[0] : m[1]) : (gq == 2 ? m[2] : m[3]);
+    int at = cnt + __popc(mine & ((1u << j4) - 1u));
+    const uint32_t four = mine >> j4;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const bool in = (four >> b) & 1u;
       if constexpr (BYTES) {
-        if (h[q]) reinterpret_cast<uint8_t*>(rows)[at] = (uint8_t)g;
+        if (in) reinterpret_cast<uint8_t*>(my_row)[at] = (uint8_t)(half * 32 + j4 + b);
       } else {
-        if (h[q]) rows[at] = (uint16_t)(g * 16);
+        if (in) my_row[at] = (uint16_t)((half * 32 + j4 + b) * 16);
       }
-      cnt[q] += __popc(m);
-      if (any) any[half] |= m;
+      at += in ? 1 : 0;
     }
+    cnt += __popc(mine);
   }
+  if (counts && (lane & 7) == 0) counts[warp * 4 + gq] = (uint32_t)cnt;
   __syncwarp();
-  return max(max(cnt[0], cnt[1]), max(cnt[2], cnt[3]));
+  return __reduce_max_sync(kFull, cnt);
 }
 
 // Which of the warp's groups still have a pixel that has not stopped (bit q for group q).
