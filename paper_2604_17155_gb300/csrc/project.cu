@@ -196,8 +196,15 @@ __device__ __forceinline__ int4 project_pair(const float4 mo, const float4 sq, c
 // CTA zeroes and flushes one histogram bin per tile, so large tile grids take more Gaussians a
 // thread, which spreads that per-CTA cost; smaller ones take fewer, which keeps more CTAs in flight.
 // Measured choices: the projection 8 / 32 and the scatter 4 / 16 Gaussians a thread below / from
-// 4,096 tiles.
+// 4,096 tiles, and fewer, down to one, while that leaves under kFullGrid CTAs (a thousand Gaussians on eight
+// cameras were 8 CTAs, scatter 18.9 us; 50,000 on one camera of 6,700 tiles 7 CTAs, call 435 us against 188).
 constexpr int kBigTileGrid = 4096;
+constexpr int kFullGrid = 4 * 152;
+inline int hist_chunk(int64_t n, int cb, int tiles, int small, int big) {
+  int pt = tiles >= kBigTileGrid ? big : small;
+  while (pt > 1 && ((n + 256 * pt - 1) / (256 * pt)) * cb < kFullGrid) pt >>= 1;
+  return pt;
+}
 __host__ __device__ constexpr int hist_per_cta(int per_thread) { return 256 * per_thread; }
 constexpr int kHistTiles = 12288;             // largest tile grid the shared-memory histograms take
 
@@ -299,7 +306,7 @@ __global__ void __launch_bounds__(256) k_scatter_hist(
   __syncthreads();
   // The rectangles are read kGroup at a time (all loads in flight before the first is used), and
   // the per-tile reservations kFlush tiles at a time, so that global round trips overlap.
-  constexpr int kGroup = 4, kFlush = 8;
+  constexpr int kGroup = PT < 4 ? PT : 4, kFlush = 8;
   static_assert(PT % kGroup == 0, "whole groups of rectangles");
   const int64_t i0 = (int64_t)blockIdx.x * hist_per_cta(PT);
   const uint4* rect_j = rect + (int64_t)j * n;
@@ -620,10 +627,11 @@ void launch_project(const Problem& p, const float* means, const float* scales, c
                     const float* opac, int cb, const Workspace& ws, cudaStream_t s) {
   if (p.tiles <= kHistTiles) {
     const size_t smem = sizeof(uint32_t) * (size_t)p.tiles;
-    const bool big = p.tiles >= kBigTileGrid;
-    auto kern = big ? k_project_hist<32> : k_project_hist<8>;
+    const int pt = hist_chunk(p.n, cb, p.tiles, 8, 32);
+    auto kern = pt == 1 ? k_project_hist<1> : pt == 2 ? k_project_hist<2> : pt == 4 ? k_project_hist<4>
+              : pt == 8 ? k_project_hist<8> : pt == 16 ? k_project_hist<16> : k_project_hist<32>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int per_cta = hist_per_cta(big ? 32 : 8);
+    const int per_cta = hist_per_cta(pt);
     const int64_t chunks = (p.n + per_cta - 1) / per_cta;
     // cameras per launch so that the 1-D grid stays below 2^31 CTAs
     const int per = (int)std::min<int64_t>(cb, std::max<int64_t>(1, 0x7FFFFFFF / std::max<int64_t>(chunks, 1)));
@@ -694,10 +702,11 @@ void launch_spatial_order(const Problem& p, const float* means, const float* sca
 void launch_scatter(const Problem& p, int cb, const Workspace& ws, cudaStream_t s) {
   if (p.tiles <= kHistTiles) {
     const size_t smem = 2 * sizeof(uint32_t) * (size_t)p.tiles;
-    const bool big = p.tiles >= kBigTileGrid;
-    auto kern = big ? k_scatter_hist<16> : k_scatter_hist<4>;
+    const int pt = hist_chunk(p.n, cb, p.tiles, 4, 16);
+    auto kern = pt == 1 ? k_scatter_hist<1> : pt == 2 ? k_scatter_hist<2> : pt == 4 ? k_scatter_hist<4>
+              : pt == 8 ? k_scatter_hist<8> : k_scatter_hist<16>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int per_cta = hist_per_cta(big ? 16 : 4);
+    const int per_cta = hist_per_cta(pt);
     dim3 grid((unsigned)((p.n + per_cta - 1) / per_cta), (unsigned)cb);
     kern<<<grid, 256, smem, s>>>(p.n, ws.rect, ws.order, p.tiles_x, p.tiles, ws.tile_off, ws.tile_cur, ws.entries,
                                  p.capacity, ws.status);
