@@ -1050,14 +1050,20 @@ int payload_group(int B, int K, int arrays) {
   return G;
 }
 
+// Whether the fold and the solve take the channels three at a time rather than four: where that needs no more
+// rounds, and so carries fewer zero channels (RGB, three RGB sets).
+bool three_channels(int K) { return (K + 2) / 3 <= (K + 3) / 4; }
+
 template <int B, bool MIXED>
 void fold_b(const Problem& p, const float* means, int cb, const Workspace& ws, bool first, bool want_gram,
             cudaStream_t s) {
   const unsigned grid = (unsigned)((p.n * kFoldGroup + kSolveThreads - 1) / kSolveThreads);
-  if (p.K == 3) {  // RGB: one launch of three channels (no zero fourth channel)
-    k_fold<B, 3, MIXED><<<grid, kSolveThreads, 0, s>>>(means, p.n, ws.cams, cb, ws.acc, p.K, p.acc_stride, 0, first,
-                                                        want_gram, ws.G, ws.Glo, ws.bvec, ws.blo, ws.wsum, ws.wlo);
-    note_launches(1);
+  if (three_channels(p.K)) {
+    for (int k0 = 0; k0 < p.K; k0 += 3) {
+      k_fold<B, 3, MIXED><<<grid, kSolveThreads, 0, s>>>(means, p.n, ws.cams, cb, ws.acc, p.K, p.acc_stride, k0, first,
+                                                          want_gram, ws.G, ws.Glo, ws.bvec, ws.blo, ws.wsum, ws.wlo);
+      note_launches(1);
+    }
     return;
   }
   for (int k0 = 0; k0 < p.K; k0 += 4) {
@@ -1071,7 +1077,7 @@ template <int B, bool MIXED>
 void solve_b(const Problem& p, const float* lam_dev, const Workspace& ws, float* coeffs, uint8_t* st,
              float* chol, const float* means, int n_acc_cams, cudaStream_t s) {
   const unsigned grid = (unsigned)((p.n * kGroup + kSolveThreads - 1) / kSolveThreads);
-  if (p.K == 3)
+  if (three_channels(p.K))
     k_solve<B, MIXED, 3><<<grid, kSolveThreads, 0, s>>>(p.n, p.K, ws.G, ws.Glo, ws.bvec, ws.blo, ws.wsum, ws.wlo,
                                                          lam_dev, p.cond_tau, p.refold_tau, coeffs, st, chol,
                                                          ws.status, ws.acc,
