@@ -5,8 +5,8 @@
 // operand, so that 3-4 CTAs fit on an SM), the S terms of Eq. 6 summed over the tile's 256 pixels
 // form a dense product
 //     D[g][n] = sum_p W[g][p] * B[n][p],   W[g][p] = alpha T of Gaussian g at pixel p (Eq. 4),
-// with B's rows 0..KT-1 the tile's target channels and the rows after them all ones, so that the same
-// product also yields V = sum_p W[g][p] (Eq. 5). The threads evaluate W by 8-lane groups
+// with B's row 0 all ones, so that the same product also yields V = sum_p W[g][p] (Eq. 5), and rows 1..KT
+// the tile's target channels. The threads evaluate W by 8-lane groups
 // (groupwalk.cuh, one pixel pair a lane) and store a pair as two FP16 values into a K-major,
 // 128-byte-swizzled shared-memory operand; the tile's targets (BF16 or FP16) are transposed once
 // into B as FP16. Both operands are scaled by powers of two -- W by 2^14 (the walk carries T scaled
@@ -135,11 +135,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
-// One column.
-__device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
-  uint32_t r;
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
-  return r;
+// 8 consecutive columns of 16 TMEM lanes by the whole warp, as an accumulator fragment: thread t gets columns
+// 2 (t % 4), + 1 of lane t / 4 in r[0], r[1] and of lane t / 4 + 8 in r[2], r[3].
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -186,40 +188,6 @@ __device__ __forceinline__ void issue_batch(uint32_t a_addr, uint32_t b_addr, ui
     const int kb = ks >> 2, kk = ks & 3;
     const uint64_t ad = desc_kmajor_sw128(a_addr + kb * (MG * 128) + kk * 32);
     const uint64_t bd = desc_kmajor_sw128(b_addr + kb * (NB * 128) + kk * 32);
-    umma_f16(d_tmem, ad, bd, idesc, ks > 0 ? 1u : 0u);
-  }
-  umma_commit(mbar);
-}
-
-// ---- B of the 16-channel walk in 11 KB ---------------------------------------------------------
-// B is [24 x 256]: 16 target rows (two 8-row atoms per K block of 64 pixels) and 8 rows of ones. An
-// MMA reads its three atoms at start, start + SBO and start + 2 SBO, and every MMA has its own
-// descriptor, so each K block kb gets its own stride s_kb (in KB) and puts its two target atoms at
-// 2 s_kb and s_kb KB below one shared atom of ones. With s = 1, 3, 4, 5 the eight target atoms and
-// the ones occupy KB 0, 2, 4-10 of an 11 KB region (ones at KB 10); KB 1 and 3 hold the staged
-// geometry. The ones' values do not depend on the pixel, so every K block may read the same atom.
-__host__ __device__ constexpr int b16_stride_kb(int kb) { return kb == 0 ? 1 : kb + 2; }
-constexpr uint32_t kB16Ones = 10 * 1024;  // offset of the ones atom in the region
-constexpr uint32_t kB16Bytes = 11 * 1024;
-constexpr uint32_t kB16Geo = 1 * 1024, kB16Aux = 3 * 1024;  // the holes
-
-// byte offset of B[channel k][pixel p] (k < 16) in the region
-__device__ __forceinline__ uint32_t b16_offset(int k, int p) {
-  const int kb = p >> 6, s = b16_stride_kb(kb);
-  const uint32_t atom = kB16Ones - (uint32_t)((k < 8 ? 2 : 1) * s) * 1024u;
-  return atom + (uint32_t)((k & 7) * 128 + ((((p & 63) >> 3) ^ (k & 7)) << 4) + ((p & 7) << 1));
-}
-
-// The 16 MMAs of one batch of the 16-channel walk (N = 24: columns 0-15 the targets, 16-23 V).
-template <int MG>
-__device__ __forceinline__ void issue_batch_b16(uint32_t a_addr, uint32_t b_region, uint32_t d_tmem, uint32_t idesc,
-                                                uint64_t* mbar) {
-  tc_fence_after();
-#pragma unroll
-  for (int ks = 0; ks < kKPix / 16; ++ks) {
-    const int kb = ks >> 2, kk = ks & 3, sk = b16_stride_kb(kb);
-    const uint64_t ad = desc_kmajor_sw128(a_addr + kb * (MG * 128) + kk * 32);
-    const uint64_t bd = desc_kmajor_sw128(b_region + kB16Ones - (uint32_t)(2 * sk) * 1024u + kk * 32, (uint32_t)sk * 1024u);
     umma_f16(d_tmem, ad, bd, idesc, ks > 0 ? 1u : 0u);
   }
   umma_commit(mbar);
@@ -294,13 +262,12 @@ __global__ void __launch_bounds__(256) k_tc_selftest(const uint16_t* __restrict_
 }
 
 // ---- the accumulate walk with the tensor-core contraction --------------------------------------
-// MG: Gaussians per batch, the MMA M (128, or 64 for up to 32 channels: half the weight operand, so
-// that more CTAs fit on an SM). TMEM columns: the accumulator width rounded up to a power of two.
-// Columns of B and of the accumulator: the KT target channels, then rows of ones that yield V (16
-// for M = 128, whose N must be a multiple of 16; 8 for M = 64, which allows multiples of 8).
-template <int KT, int MG>
+// MG: Gaussians per batch, the MMA M. TMEM columns: the accumulator width rounded up to a power of two.
+// Columns of B and of the accumulator: V, the KT target channels and zeros to a multiple of 8 (an M of 64
+// takes N in steps of 8).
+template <int KT>
 __host__ __device__ constexpr int tc_cols() {
-  return KT + (MG == 64 ? 8 : 16);
+  return KT + 8;
 }
 
 template <int NB>
@@ -338,8 +305,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
     const uint16_t* __restrict__ targets, int K, int cam0, float* __restrict__ acc, int RS,
     int64_t acc_cam_stride, DevStatus* status, uint64_t wait_limit_ns, bool issue_mma) {
   static_assert(MG == 64 && MG == kBatch, "staging and epilogue map Gaussian g to TMEM lane g % 16 of quarter g / 16");
-  constexpr int NB = tc_cols<KT, MG>();  // target channels + rows of ones (V)
-  constexpr bool kB16 = KT == 16;        // B in the 11 KB region (b16_offset)
+  constexpr int NB = tc_cols<KT>();  // the row of ones (V), the target channels, rows of zeros
   extern __shared__ uint8_t smem_raw[];
   // The barrier, the flags and the staged batches sit in front of the operands, which start at the next
   // 1024-byte boundary. A base that is not 128-byte aligned is reported (kFlagLayout) before any work.
@@ -351,7 +317,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
   TcBatch& s = *reinterpret_cast<TcBatch*>(smem_raw);
   uint8_t* base = smem_raw + (((raw + kTcFront + 1023u) & ~1023u) - raw);
   uint8_t* A_s = base;                                 // MG x 256 (32 KB)
-  uint8_t* B_s = base + MG * kKPix * 2;                // NB x 256, or the 11 KB region
+  uint8_t* B_s = base + MG * kKPix * 2;                // NB x 256
 
   // Walkers and helpers are numbered alike: tid, and warp 0-3 by K block and TMEM quarter.
   const bool walker = threadIdx.x < kTcWalkers;
@@ -376,8 +342,9 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
   }
 
   // B: the tile's targets, transposed to [channel][pixel] and scaled by 2^sexp (the tile's largest
-  // magnitude in [2^14, 2^15)), then the rows of ones. A walker takes the first half of its pixels'
-  // channels, the helper of the same number the second.
+  // magnitude in [2^14, 2^15)) in rows 1..KT, below a row of ones, so that D's columns lie as the accumulator
+  // row (V, S_0, S_1, ..) does; the rows left are zero. A walker takes the first half of its pixels' channels,
+  // the helper of the same number the second.
   float t_scale_inv;
   {
     constexpr int KH = KT / 2;
@@ -435,15 +402,12 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
     for (int k = 0; k < KH; ++k) {
       const float x = target_value((uint16_t)(tv[k] & 0xFFFFu), BF16_TARGETS) * s1 * s2;
       const float y = target_value((uint16_t)(tv[k] >> 16), BF16_TARGETS) * s1 * s2;
-      *reinterpret_cast<__half2*>(B_s + (kB16 ? b16_offset(kh + k, p) : kmajor_sw128(kh + k, p, NB))) = __floats2half2_rn(x, y);
+      *reinterpret_cast<__half2*>(B_s + kmajor_sw128(1 + kh + k, p, NB)) = __floats2half2_rn(x, y);
     }
-    if constexpr (kB16) {
-      if (threadIdx.x < 64)
-        reinterpret_cast<uint4*>(B_s + kB16Ones)[threadIdx.x] = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
-    } else if (walker) {
+    if (walker) *reinterpret_cast<uint32_t*>(B_s + kmajor_sw128(0, p, NB)) = 0x3C003C00u;
+    else
 #pragma unroll
-      for (int k = KT; k < NB; ++k) *reinterpret_cast<uint32_t*>(B_s + kmajor_sw128(k, p, NB)) = 0x3C003C00u;
-    }
+      for (int k = KT + 1; k < NB; ++k) *reinterpret_cast<uint32_t*>(B_s + kmajor_sw128(k, p, NB)) = 0u;
   }
   const float v_scale_inv = ldexpf(1.0f, -kWScaleExp);
   constexpr float kT0 = (float)(1 << kWScaleExp);  // the transmittance carries the factor 2^14 of W
@@ -515,8 +479,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
       if (warp == 0) {
         if (start > 0) bar_sync<3, kTcWalkers + 32>();  // the helpers have read the last batch's sums
         if (lane == 0 && issue_mma) {
-          if constexpr (kB16) issue_batch_b16<MG>(a_addr, b_addr, tmem, kIdesc, &s.mbar);
-          else issue_batch<NB, MG>(a_addr, b_addr, tmem, kIdesc, &s.mbar);
+          issue_batch<NB, MG>(a_addr, b_addr, tmem, kIdesc, &s.mbar);
         }
         __syncwarp();
       }
@@ -526,8 +489,8 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
   } else {
     // Wait for a batch's MMAs, clear W, and then, beside the next batch's walk, add the sums and prepare the
     // geometry and lists of the batch after it.
-    constexpr int kCh = KT / 16;                            // 16-column chunks of S
-    const int g_own = tmem_row_of_lane<MG>(warp, lane);      // the batch row this thread adds
+    constexpr int kBlocks = KT / 8 + 1;                      // 8-column blocks of (V, S)
+    const int ra = lane >> 2, rb = ra + 8, q2 = 2 * (lane & 3);  // the rows and columns of the thread's fragment
     float* acc_cam = acc + (int64_t)c.j * acc_cam_stride;
     const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
     for (uint32_t start = 0, buf = 0;; start += MG, buf ^= 1u) {
@@ -546,45 +509,47 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
       __syncthreads();
       if (s.timeout[buf]) break;
       const bool more = more_after(start, buf);
-      // The accumulator streams through registers 16 columns at a time: chunk q adds the float4 groups
-      // 4q..4q+3 of the row (V, S_0, S_1, ..) and carries its last column into group 4q+4. Only the
-      // first 16 lanes of each quarter hold a Gaussian (M = 64); every tcgen05.ld is warp-uniform.
+      // The sums stream through registers 8 columns at a time as accumulator fragments: four neighbouring
+      // threads hold 32 consecutive bytes of a row, so an instruction's 8-byte atomics fall in whole sectors
+      // of 8 rows (with a row per thread, 16-byte atomics touched 16 rows: the 64-channel walk at 1600 x 1060,
+      // 8 views, took 39.1 ms, now 36.7; the 16-channel one, a third of the sectors, is unchanged at 80.4).
       const int nb = (int)min((uint32_t)MG, c.len - start);
-      const uint32_t my_id = __shfl_sync(0xFFFFFFFFu, id0, 2 * (lane & 15));
-      uint32_t r[16];
-      const uint32_t vr = tmem_ld1(trow + (uint32_t)KT);  // the ones block: every column holds V
-      tmem_ld16(trow, r);
-      tmem_wait_ld();
-      const float V = __uint_as_float(vr) * v_scale_inv;
-      float carry = V;
-      const bool add = g_own >= 0 && g_own < nb && V > 0.0f;
-      float* dst = acc_cam + (int64_t)(add ? my_id : 0u) * RS;
+      const uint32_t id_a = __shfl_sync(0xFFFFFFFFu, id0, 2 * ra), id_b = __shfl_sync(0xFFFFFFFFu, id0, 2 * rb);
+      float* const dst_a = acc_cam + (int64_t)id_a * RS + q2;
+      float* const dst_b = acc_cam + (int64_t)id_b * RS + q2;
+      bool add_a = false, add_b = false;
 #pragma unroll
-      for (int q = 0; q < kCh; ++q) {
-        float sv[16];
+      for (int q = 0; q < kBlocks; q += 4) {
+        uint32_t r[16];
 #pragma unroll
-        for (int h = 0; h < 16; ++h) sv[h] = __uint_as_float(r[h]) * t_scale_inv;
-        if (q + 1 < kCh) {
-          tmem_ld16(trow + (uint32_t)(16 * (q + 1)), r);
-          tmem_wait_ld();
-        }
-        if (q + 1 >= kCh && more) {  // every column is in registers: the next batch's MMAs may write
+        for (int h = 0; h < 4; ++h)
+          if (q + h < kBlocks) tmem_ld_frag(trow + (uint32_t)(8 * (q + h)), r + 4 * h);
+        tmem_wait_ld();
+        if (q + 4 >= kBlocks && more) {  // every column is in registers: the next batch's MMAs may write
           tc_fence_before();
           bar_arrive<3, kTcWalkers + 32>();
         }
-        if (add) {
-          float* d = dst + 16 * q;
-          if (16 * q < RS) atomicAdd(reinterpret_cast<float4*>(d), make_float4(carry, sv[0], sv[1], sv[2]));
-          if (16 * q + 4 < RS) atomicAdd(reinterpret_cast<float4*>(d + 4), make_float4(sv[3], sv[4], sv[5], sv[6]));
-          if (16 * q + 8 < RS) atomicAdd(reinterpret_cast<float4*>(d + 8), make_float4(sv[7], sv[8], sv[9], sv[10]));
-          if (16 * q + 12 < RS)
-            atomicAdd(reinterpret_cast<float4*>(d + 12), make_float4(sv[11], sv[12], sv[13], sv[14]));
+        if (q == 0) {  // V, column 0: a row that nothing reached is left alone
+          const float va = __uint_as_float(__shfl_sync(0xFFFFFFFFu, r[0], lane & 28));
+          const float vb = __uint_as_float(__shfl_sync(0xFFFFFFFFu, r[2], lane & 28));
+          add_a = 16 * warp + ra < nb && va > 0.0f;
+          add_b = 16 * warp + rb < nb && vb > 0.0f;
         }
-        carry = sv[15];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          if (q + h >= kBlocks) continue;
+          const int col = 8 * (q + h);
+          const float s0 = q + h == 0 && q2 == 0 ? v_scale_inv : t_scale_inv;
+          const bool in = col + q2 < RS;  // RS is even
+          if (add_a && in)
+            atomicAdd(reinterpret_cast<float2*>(dst_a + col),
+                      make_float2(__uint_as_float(r[4 * h]) * s0, __uint_as_float(r[4 * h + 1]) * t_scale_inv));
+          if (add_b && in)
+            atomicAdd(reinterpret_cast<float2*>(dst_b + col),
+                      make_float2(__uint_as_float(r[4 * h + 2]) * s0, __uint_as_float(r[4 * h + 3]) * t_scale_inv));
+        }
         __syncwarp();
       }
-      // the last group (S_{KT-1}, 0, 0, 0)
-      if (add && 16 * kCh < RS) atomicAdd(reinterpret_cast<float4*>(dst + 16 * kCh), make_float4(carry, 0.0f, 0.0f, 0.0f));
       if (!more) break;
       listed0[0] = listed1[0];
       listed0[1] = listed1[1];
@@ -626,7 +591,7 @@ constexpr size_t selftest_smem() {
 // the barrier, flags and staged batch with up to 1023 bytes of alignment, W, and B
 template <int KT, int MG>
 constexpr size_t tc_smem() {
-  return kTcFront + 1023 + (size_t)MG * kKPix * 2 + (KT == 16 ? (size_t)kB16Bytes : (size_t)tc_cols<KT, MG>() * kKPix * 2);
+  return kTcFront + 1023 + (size_t)MG * kKPix * 2 + (size_t)tc_cols<KT>() * kKPix * 2;
 }
 // CTAs per SM that the shared memory admits: each CTA's share rounded up to 1 KB, plus 1 KB the
 // system reserves per CTA, out of the SM's 228 KB
