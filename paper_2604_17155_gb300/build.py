@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libicgs.so")
 SOURCES = ["api.cu", "project.cu", "tilesort.cu", "blend.cu", "contract_tc.cu", "solve.cu", "noalloc.cu"]
-HEADERS = ["icgs_internal.h", "icgs_device.cuh", "walk.cuh", "groupwalk.cuh", "packed.cuh", "radix.cuh"]
+HEADERS = ["icgs_internal.h", "icgs_device.cuh", "walk.cuh", "groupwalk.cuh", "packed.cuh", "bucket.cuh", "radix.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

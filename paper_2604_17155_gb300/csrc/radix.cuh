@@ -1,6 +1,7 @@
 // radix.cuh -- depth order of one tile list in shared memory by a stable LSD radix sort (the "depth
-// ordered list" of Eq. 2): by one warp (lists that fit its two buffers, no CTA barrier) or by
-// one CTA of 256 threads (longer lists).
+// ordered list" of Eq. 2), for the lists whose depths crowd into few values (the others are bucket
+// sorted, bucket.cuh): by one warp (lists that fit its two buffers, no CTA barrier) or by one CTA of
+// 256 threads (longer lists).
 //
 // A key is (float32 depth bits << 32) | Gaussian index. Depths are positive and finite, so their
 // bit patterns order like the depths, and keys are unique. The sort takes 8-bit digits of
@@ -180,10 +181,10 @@ __device__ __forceinline__ bool warp_fix_ties(unsigned long long* r, int n) {
 
 // Sorts the n (1 < n <= 65535) keys at g with one warp; a and b are its two shared buffers of at
 // least n keys, ws.match must be zero (it is again on return). Returns the buffer (a or b) that
-// holds the sorted keys; WRITE also writes them back to g.
-template <bool WRITE>
-__device__ __forceinline__ const unsigned long long* warp_sort_keys(unsigned long long* g, int n, unsigned long long* a,
-                                                                    unsigned long long* b, WarpScratch& ws) {
+// holds the sorted keys.
+__device__ __forceinline__ const unsigned long long* warp_sort_keys(const unsigned long long* g, int n,
+                                                                    unsigned long long* a, unsigned long long* b,
+                                                                    WarpScratch& ws) {
   const int lane = threadIdx.x & 31;
   // every key of the list in flight at once (asynchronous 8-byte copies into a), then one wait
   for (int pos = lane; pos < n; pos += 32) {
@@ -215,21 +216,12 @@ __device__ __forceinline__ const unsigned long long* warp_sort_keys(unsigned lon
     warp_passes(a, b, n, np, cur, n_hi, 0, lmin, hmin, ws);
     const unsigned long long* r = np & 1 ? b : a;
     bool t = false;
-    for (int pos = lane; pos < n; pos += 32) {  // write out; a tie means another sort and write
-      const unsigned long long k = r[pos];
-      if (WRITE) g[pos] = k;
-      t |= pos > 0 && key_word(k, true) == key_word(r[pos - 1], true);
-    }
+    for (int pos = lane + 1; pos < n; pos += 32) t |= key_word(r[pos], true) == key_word(r[pos - 1], true);
     tie = __any_sync(kFull, t);
   }
   if (tie && n_hi > 0) {  // uniform over the warp: try the runs of equal depths by transposition
     unsigned long long* r = np & 1 ? b : a;
-    if (warp_fix_ties(r, n)) {
-      if (WRITE)
-        for (int pos = lane; pos < n; pos += 32) g[pos] = r[pos];
-      __syncwarp();
-      return r;
-    }
+    if (warp_fix_ties(r, n)) return r;
   }
   if (tie) {  // uniform over the warp: index order first, then depth order again
     const unsigned long long* r = np & 1 ? b : a;
@@ -239,19 +231,9 @@ __device__ __forceinline__ const unsigned long long* warp_sort_keys(unsigned lon
     __syncwarp();
     warp_scan(ws.count[cur], 0u);
     warp_passes(a, b, n, np, cur, n_lo + n_hi, n_lo, lmin, hmin, ws);
-    if (WRITE) {
-      const unsigned long long* o = np & 1 ? b : a;
-      for (int pos = lane; pos < n; pos += 32) g[pos] = o[pos];
-    }
   }
   __syncwarp();
   return np & 1 ? b : a;
-}
-
-// Sorts the n (1 < n <= 65535) keys at g in place with one warp (warp_sort_keys, written back).
-__device__ __forceinline__ void warp_sort(unsigned long long* g, int n, unsigned long long* a, unsigned long long* b,
-                                          WarpScratch& ws) {
-  warp_sort_keys<true>(g, n, a, b, ws);
 }
 
 // ---------------------------------------------------------------------------------------------

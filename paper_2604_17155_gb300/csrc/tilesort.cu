@@ -2,17 +2,23 @@
 //
 // After binning, each tile owns a contiguous slot range of 64-bit keys (float32 depth bits << 32 |
 // Gaussian index); the keys are unique, so sorting them ascending gives depth order with ties in
-// index order. Every sort here is the stable LSD radix sort of radix.cuh, in shared memory, and
-// every list of a pass is sorted before the walks read it: lists of up to kWarpSortCap keys by a
-// persistent kernel in which each warp sorts one tile at a time (k_sort_tiles, no CTA barrier);
-// longer lists are queued. Lists of up to kMidCap keys go to two warps each (k_sort_pairs: a warp
-// sort per half, then one merge-path merge); longer ones to one CTA each (k_sort_queued: up to
-// kSortCap keys by the block radix sort at once, longer lists as sorted runs of kSortCap keys
-// followed by merge-path merges between the slot range and a scratch range of the same place).
+// index order, and every list of a pass is sorted before the walks read it. A list is bucket sorted
+// (bucket.cuh) in shared memory by a team sized to it: lists of up to kWarpSortCap keys by one warp
+// each of a persistent kernel (k_sort_tiles, no CTA barrier), which queues the others; up to kMidCap
+// keys by a CTA of four warps (k_sort_mid); longer ones, in runs of kSortCap keys that are merged,
+// by a CTA of eight (k_sort_queued). A list whose depths crowd takes the stable LSD radix sort of
+// radix.cuh in the queue's kernels instead.
+//
+// Latency of shared-memory atomics and loads bounds these kernels, so passes over the keys and warps
+// in flight count: with three or four radix passes a list, the sort of 1.1e9 keys in 1.3 million lists
+// (200 views of 1600 x 1060) took 16.5 ms, with one bucket pass 9.4 (its keys read and written once at
+// the copy rate: 2.6); 5.4e7 keys in 250,000 lists 0.88 -> 0.50 ms. Teams: lists of 1025..2048 keys
+// by two warps with 32 keys a thread (159 registers, 12 warps an SM) gave 10.5 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
+#include "bucket.cuh"
 #include "icgs_internal.h"
 #include "radix.cuh"
 
@@ -24,11 +30,14 @@ constexpr int kSortThreads = radix::kThreads;  // CTA of the queued sort
 constexpr int kWarpSortCap = 1024;             // longest list a warp sorts alone
 constexpr int kWarpSortWarps = 4;              // warps per CTA of k_sort_tiles
 constexpr int kWarpSortChunk = 4;              // most tiles a warp claims per work-counter increment
-constexpr int kMidCap = 2 * kWarpSortCap;       // queued lists up to this length: two warps each (k_sort_pairs)
+constexpr int kMidCap = 2 * kWarpSortCap;       // queued lists up to this length: k_sort_mid
+constexpr int kMidThreads = 128;               // its CTA
+
+constexpr int kWarpBins = 2048;                 // bins of a warp's bucket sort: two a key of its longest list
 
 struct WarpSortSmem {
-  unsigned long long a[kWarpSortCap], b[kWarpSortCap];
-  radix::WarpScratch sc;
+  unsigned long long keys[kWarpSortCap];
+  bucket::Bins<1, kWarpBins> bins;
 };
 
 __device__ __forceinline__ void tile_range(const uint32_t* tile_off, int t, uint32_t capacity,
@@ -42,17 +51,17 @@ __device__ __forceinline__ void tile_range(const uint32_t* tile_off, int t, uint
 __device__ __forceinline__ int merge_path(const unsigned long long* A, int na, const unsigned long long* B,
                                           int nb, int d);
 
-// Every tile list of the pass, by warps that claim chunk tiles at a time from the work counter: lists of up to kWarpSortCap keys are sorted in place by the claiming warp, longer ones
-// queued for k_sort_queued.
-__global__ void __launch_bounds__(32 * kWarpSortWarps) k_sort_tiles(const uint32_t* __restrict__ tile_off,
+// Every tile list of the pass, by warps that claim chunk tiles at a time from the work counter: lists of up
+// to kWarpSortCap keys are bucket sorted in place by the claiming warp, longer and crowded ones queued. 16
+// warps an SM, by shared memory (12 KB each) and registers (32 keys a lane): CTAs of three warps fit 18,
+// but at 96 registers that spill (large scene 10.7 ms against 10.5).
+__global__ void __launch_bounds__(32 * kWarpSortWarps, 4) k_sort_tiles(const uint32_t* __restrict__ tile_off,
                                                                     unsigned long long* __restrict__ entries,
                                                                     uint32_t capacity, int ntiles, int chunk,
                                                                     uint32_t* __restrict__ queue, DevStatus* status) {
   extern __shared__ __align__(16) unsigned long long s_dyn[];  // kWarpSortWarps x WarpSortSmem
   WarpSortSmem& m = reinterpret_cast<WarpSortSmem*>(s_dyn)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  for (int i = lane; i < radix::kBins; i += 32) m.sc.match[i] = 0u;
-  __syncwarp();
   while (true) {
     uint32_t t0 = 0;
     if (lane == 0) t0 = atomicAdd(&status->sort_next, (uint32_t)chunk);
@@ -73,14 +82,14 @@ __global__ void __launch_bounds__(32 * kWarpSortWarps) k_sort_tiles(const uint32
       tile_range(tile_off, t, capacity, b, e);
       const int n = (int)(e - b);
       if (n <= 1) continue;
-      if (n > kWarpSortCap) {  // queued: up to kMidCap keys from the front, longer lists from the back
+      bool done = false;
+      if (n <= kWarpSortCap) done = bucket::sort_list<1, kWarpSortCap / 32>(entries + b, n, m.keys, m.bins);
+      if (!done) {  // queued: up to kMidCap keys from the front, longer lists from the back
         if (lane == 0) {
           if (n <= kMidCap) queue[atomicAdd(&status->big_tiles, 1u)] = (uint32_t)t;
           else queue[ntiles - 1 - (int)atomicAdd(&status->long_tiles, 1u)] = (uint32_t)t;
         }
-        continue;
       }
-      radix::warp_sort(entries + b, n, m.a, m.b, m.sc);
     }
   }
 }
@@ -114,42 +123,51 @@ __device__ __forceinline__ void merge_runs(const unsigned long long* A, int na, 
   }
 }
 
-// Sorts the queued lists of 1025..kMidCap keys (queue[0, big_tiles)), a grid-stride loop with two
-// warps per list: warp w sorts one half (at most kWarpSortCap keys) with the warp radix sort in its
-// part of two shared pools, the halves are gathered into the first pool, and a merge-path merge
-// (every thread an equal share of the outputs) writes the list back to its slot range.
-__global__ void __launch_bounds__(64) k_sort_pairs(const uint32_t* __restrict__ tile_off,
-                                                   unsigned long long* __restrict__ entries, uint32_t capacity,
-                                                   const uint32_t* __restrict__ queue, const DevStatus* status) {
+// Sorts the queued lists of up to kMidCap keys (queue[0, big_tiles)), a grid-stride loop with a CTA per list:
+// those of more than kWarpSortCap keys by a bucket sort of the CTA. The crowded ones, and the shorter lists
+// that a warp's bucket sort refused, by two warps: warp w sorts one half (at most kWarpSortCap keys) with the
+// warp radix sort in its part of two shared pools, the halves are gathered into the first pool, and a
+// merge-path merge (every thread an equal share of the outputs) writes the list back to its slot range.
+__global__ void __launch_bounds__(kMidThreads, 6) k_sort_mid(const uint32_t* __restrict__ tile_off,
+                                                             unsigned long long* __restrict__ entries, uint32_t capacity,
+                                                             const uint32_t* __restrict__ queue,
+                                                             const DevStatus* status) {
   extern __shared__ __align__(16) unsigned long long s_dyn[];  // pools P0, P1 of 2 x kWarpSortCap keys, scratch
   unsigned long long* P0 = s_dyn;
   unsigned long long* P1 = s_dyn + 2 * kWarpSortCap;
-  radix::WarpScratch& sc = reinterpret_cast<radix::WarpScratch*>(P1 + 2 * kWarpSortCap)[threadIdx.x >> 5];
   __shared__ int s_len[2];
+  using MidBins = bucket::Bins<kMidThreads / 32, 2 * kMidCap / (kMidThreads / 32)>;
+  MidBins& bins = *reinterpret_cast<MidBins*>(P1);
+  static_assert(sizeof(MidBins) <= 2 * kWarpSortCap * sizeof(unsigned long long), "bins in P1");
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int i = lane; i < radix::kBins; i += 32) sc.match[i] = 0u;
-  __syncwarp();
+  radix::WarpScratch& sc = reinterpret_cast<radix::WarpScratch*>(P1 + 2 * kWarpSortCap)[w & 1];
+  if (w < 2)
+    for (int i = lane; i < radix::kBins; i += 32) sc.match[i] = 0u;
   const uint32_t count = status->big_tiles;
   for (uint32_t q = blockIdx.x; q < count; q += gridDim.x) {
     uint32_t b, e;
     tile_range(tile_off, queue[q], capacity, b, e);
     const int n = (int)(e - b);
-    const int h = (n + 1) / 2;
-    const int lo = min(n, w * h), len = min(h, n - lo);
-    unsigned long long* a = P0 + w * kWarpSortCap;
-    unsigned long long* bb = P1 + w * kWarpSortCap;
-    if (len > 1) {
-      const unsigned long long* run = radix::warp_sort_keys<false>(entries + b + lo, len, a, bb, sc);
-      if (run != a) {  // gather the half into the first pool
-        for (int pos = lane; pos < len; pos += 32) a[pos] = run[pos];
-        __syncwarp();
+    if (n > kWarpSortCap && bucket::sort_list<kMidThreads / 32, kMidCap / kMidThreads>(entries + b, n, P0, bins)) continue;  // uniform
+    if (w < 2) {
+      __syncwarp();
+      const int h = (n + 1) / 2;
+      const int lo = min(n, w * h), len = min(h, n - lo);
+      unsigned long long* a = P0 + w * kWarpSortCap;
+      unsigned long long* bb = P1 + w * kWarpSortCap;
+      if (len > 1) {
+        const unsigned long long* run = radix::warp_sort_keys(entries + b + lo, len, a, bb, sc);
+        if (run != a) {  // gather the half into the first pool
+          for (int pos = lane; pos < len; pos += 32) a[pos] = run[pos];
+          __syncwarp();
+        }
+      } else if (len == 1 && lane == 0) {
+        a[0] = entries[b + lo];
       }
-    } else if (len == 1 && lane == 0) {
-      a[0] = entries[b + lo];
+      if (lane == 0) s_len[w] = max(0, len);
     }
-    if (lane == 0) s_len[w] = max(0, len);
     __syncthreads();
-    merge_runs<64>(P0, s_len[0], P0 + kWarpSortCap, s_len[1], entries + b, threadIdx.x);
+    merge_runs<kMidThreads>(P0, s_len[0], P0 + kWarpSortCap, s_len[1], entries + b, threadIdx.x);
     __syncthreads();
   }
 }
@@ -164,17 +182,21 @@ __device__ __forceinline__ void block_sort_list(unsigned long long* g, int m, un
 }
 
 // Sorts the queued lists of more than kMidCap keys (the last long_tiles entries of the queue) in
-// place, a grid-stride loop. A list of up to kSortCap keys is sorted at once by the block radix
-// sort; a longer one as runs of kSortCap keys, then pairwise merge-path merges ping-ponging between
-// its slot range and the same range of the scratch array.
+// place, a grid-stride loop with a CTA per list: in runs of up to kSortCap keys, each by a bucket sort or, when
+// crowded, by the block radix sort; a longer list then by pairwise merge-path merges ping-ponging between its
+// slot range and the same range of the scratch array. (A bucket sort of 2 kSortCap keys in both buffers at
+// once spilled its 32 keys a thread and was slower, 1.06 ms a pass against 0.65.)
 __global__ void __launch_bounds__(kSortThreads, 2) k_sort_queued(const uint32_t* __restrict__ tile_off,
                                                                  unsigned long long* __restrict__ entries,
                                                                  unsigned long long* __restrict__ scratch,
                                                                  uint32_t capacity, const uint32_t* __restrict__ queue,
                                                                  int ntiles, const DevStatus* status) {
-  constexpr int CAP = kSortCap;
+  constexpr int CAP = kSortCap, kWarps = kSortThreads / 32;
+  using QueueBins = bucket::Bins<kWarps, 2 * CAP / kWarps>;
+  static_assert(sizeof(QueueBins) <= CAP * sizeof(unsigned long long), "bins in the second buffer");
   extern __shared__ __align__(16) unsigned long long s_dyn[];  // 2 x CAP keys
   __shared__ radix::BlockScratch sc;
+  QueueBins& bins = *reinterpret_cast<QueueBins*>(s_dyn + CAP);
   for (int i = threadIdx.x; i < radix::kWarps * radix::kBins; i += kSortThreads) sc.match[i] = 0u;
   __syncthreads();
   const uint32_t count = status->long_tiles;
@@ -184,7 +206,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort_queued(const uint32_t*
     const int n = (int)(e - b);
     for (int r0 = 0; r0 < n; r0 += CAP) {  // sorted runs (the whole list when it fits)
       const int m = min(CAP, n - r0);
-      if (m > 1) block_sort_list(entries + b + r0, m, s_dyn, s_dyn + CAP, sc);
+      if (m > 1 && !bucket::sort_list<kWarps, CAP / kSortThreads>(entries + b + r0, m, s_dyn, bins))
+        block_sort_list(entries + b + r0, m, s_dyn, s_dyn + CAP, sc);
     }
     if (n <= CAP) continue;  // uniform
     unsigned long long* src = entries + b;
@@ -227,7 +250,7 @@ int sm_count() {
 
 }  // namespace
 
-// Orders every tile list of the pass: the warp-per-list kernel, then the queued long lists. The queue
+// Orders every tile list of the pass: the warp-per-list kernel, then the queued lists. The queue
 // counters of the status block are zero (the scan of the pass's counts empties them).
 void launch_tile_sort(const Problem& p, int cb, const Workspace& ws, cudaStream_t s) {
   const int ntiles = cb * p.tiles;
@@ -245,10 +268,10 @@ void launch_tile_sort(const Problem& p, int cb, const Workspace& ws, cudaStream_
   unsigned long long* entries = reinterpret_cast<unsigned long long*>(ws.entries);
   unsigned long long* scratch = reinterpret_cast<unsigned long long*>(ws.entries_tmp);
   const int psmem = 2 * (2 * kWarpSortCap * (int)sizeof(unsigned long long) + (int)sizeof(radix::WarpScratch));
-  cudaFuncSetAttribute(k_sort_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem);
+  cudaFuncSetAttribute(k_sort_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, psmem);
   int per_sm2 = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, k_sort_pairs, 64, psmem);
-  k_sort_pairs<<<sms * (per_sm2 > 0 ? per_sm2 : 1), 64, psmem, s>>>(ws.tile_off, entries, p.capacity, ws.big_list,
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, k_sort_mid, kMidThreads, psmem);
+  k_sort_mid<<<sms * (per_sm2 > 0 ? per_sm2 : 1), kMidThreads, psmem, s>>>(ws.tile_off, entries, p.capacity, ws.big_list,
                                                                     ws.status);
   const int qsmem = 2 * kSortCap * (int)sizeof(unsigned long long);
   cudaFuncSetAttribute(k_sort_queued, cudaFuncAttributeMaxDynamicSharedMemorySize, qsmem);
