@@ -65,8 +65,8 @@ SPECS = {
 # source files hash to the value it was captured with; after any change it is null until
 # re-captured.
 KERNEL_SOURCES = {
-    "cuda-core": ["blend.cu", "walk.cuh", "icgs_device.cuh", "icgs_internal.h"],
-    "tensor-core": ["contract_tc.cu", "walk.cuh", "icgs_device.cuh", "icgs_internal.h"],
+    "cuda-core": ["blend.cu", "groupwalk.cuh", "packed.cuh", "walk.cuh", "icgs_device.cuh", "icgs_internal.h"],
+    "tensor-core": ["contract_tc.cu", "groupwalk.cuh", "packed.cuh", "walk.cuh", "icgs_device.cuh", "icgs_internal.h"],
 }
 MEASURED_TRAFFIC = {
     # relight, 100 cameras: one full-size launch captured
@@ -409,7 +409,7 @@ def walk_roofline(name, kind, K, L, blend_ms, stats, target_bytes, n, n_cams, ti
                 "traffic_unit": "bytes per scene (DRAM read + write, ncu)", "peak_source": pk["source"],
                 "tensor_view": tensor, "alu_view": alu}
     else:
-        kname = f"k_blend_accumulate2<{K}>" if K <= 3 else f"k_blend_accumulate<{min(K, 16)}>"
+        kname = f"k_blend_accumulate2<{K if K <= 3 else 7}>" if K <= 7 else f"k_blend_accumulate<{15 if K <= 15 else 16}>"
         roof = {"kernel": kname, "bound": "alu", "achieved": alu["achieved_tflops"], "peak": alu["peak_tflops"],
                 "unit": "TFLOP/s", "frac": alu["frac"], "traffic": traffic,
                 "traffic_unit": "bytes per scene (DRAM read + write, ncu)", "peak_source": alu["peak_source"],

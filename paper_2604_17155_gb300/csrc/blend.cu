@@ -1,24 +1,27 @@
-// blend.cu -- the per-tile front-to-back walks (Eq. 2, Eq. 4-6), one CTA per 16x16 screen tile:
-// 256 threads with one pixel each, or (the kernels named ...2, for up to 3 or 4 channels) 128
-// threads with two pixels each.
+// blend.cu -- the per-tile front-to-back walks (Eq. 2, Eq. 4-6), one CTA per 16x16 screen tile.
 //
 //   k_blend_accumulate  colorize: for every (pixel, Gaussian) blend weight w = alpha T (Eq. 4)
-//   (2: <= 3 channels)  accumulate V = sum w (Eq. 5) and S_k = sum w t_k (Eq. 6 numerator). The
-//                       tile's pixels are reduced per Gaussian inside each warp (a halving
-//                       butterfly that leaves value v's warp sum in lane v * 32/NP) and across
-//                       warps with shared-memory atomics; then ONE global atomic group per
-//                       (Gaussian, tile) lands in the per-(camera, Gaussian) accumulator.
+//   (2: <= 7 channels)  accumulate V = sum w (Eq. 5) and S_k = sum w t_k (Eq. 6 numerator), reduced
+//                       over the tile's pixels; then ONE global atomic group per (Gaussian, tile)
+//                       lands in the per-(camera, Gaussian) accumulator.
 //   k_blend_render      render: img_k = sum w C_k (Eq. 1-3) with C from the payload.
 //   (2: <= 4 channels)
 //   k_blend_adjoint     gradient: dL/dt_k = sum w a_k and, per Gaussian, dL/do = sum over pixels of
 //   (2: <= 4 channels)  (g T - sum_{n>m} g_n w_n / (1-alpha)) * alpha/o with g = beta + a . t.
+//   k_blend_refine2     refinement: render and accumulation of the residuals in one kernel (<= 3 channels).
 //
-// Warp w of a CTA covers the 8x4 pixel block ((w&1)*8, (w>>1)*4) of the tile (8x8 blocks at
-// ((w&1)*8, (w>>1)*8) in the two-pixel walks). A warp skips a Gaussian whose padded support box
-// misses its block (a warp-uniform ballot; the accumulate and adjoint walks then also test the
-// ellipse against the block), and skips a whole batch once all its pixels stopped. Every walk
-// takes its decisions through blend_step(), written with explicit round-to-nearest intrinsics, so
-// all walks take the same threshold decisions for the same inputs.
+// The kernels named ...2 walk by 8-lane groups (groupwalk.cuh): 64 threads with four pixels each, every
+// group its own hit list over its 8x4 pixel block, pixel pairs in packed FP32. They issue in about 78% of
+// the cycles, with the ALU and FMA pipes at 55-60%; what is left is the list's own waste (a warp's four
+// groups run to the longest of their lists, 1.08 of their mean). Against one list a warp and two pixels
+// a thread, at 800 x 800: accumulating 100 views 9.3 -> 5.8 ms, rendering them 9.0 -> 4.3, the adjoint
+// of 40 views 6.5 -> 3.7.
+//
+// The others (more channels, whose per-pixel values and sums fill the registers) have 256 threads with one
+// pixel each: warp w covers the 8x4 block ((w&1)*8, (w>>1)*4), skips a Gaussian whose padded support box
+// misses its block (a ballot; the accumulate walk then also tests the ellipse), and skips a whole batch
+// once all its pixels stopped. Sums go over a warp by a halving butterfly that leaves value v's sum in
+// lane v * 32/NP, and over warps with shared-memory atomics.
 #include <cuda_runtime.h>
 
 #include "icgs_device.cuh"
@@ -76,7 +79,7 @@ __global__ void __launch_bounds__(kThreads, KC <= 8 ? 5 : 4) k_blend_accumulate(
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, int K, int k0, int cam0, const float* __restrict__ sub_img,
     float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
-  static_assert(KC >= 4, "up to 3 channels take the two-pixel walk");
+  static_assert(KC >= 8, "up to 7 channels take the group walk");
   constexpr int NV = KC + 1;                      // V and S_0..S_{KC-1}
   // 16 channels reduce V on its own, so that the sums fill a 16-value reduction instead of a
   // 32-value one padded with 15 zeros; otherwise V is value 0 of the reduction.
@@ -148,7 +151,7 @@ __global__ void __launch_bounds__(kThreads, KC <= 8 ? 5 : 4) k_blend_accumulate(
         while (bits) {  // only the Gaussians whose box touches this warp's block, in depth order
           const int g = half * 32 + __ffs(bits) - 1;
           bits &= bits - 1;
-          const float w = blend_weight<true>(s_geo[g], s_aux[g], c.pxf, c.pyf, T, done, npairs);
+          const float w = blend_weight(s_geo[g], s_aux[g], c.pxf, c.pyf, T, done, npairs);
           if (__any_sync(kFull, w > 0.0f)) {
             float v[NP];
 #pragma unroll
@@ -1017,7 +1020,8 @@ void render_chunk(const Problem& p, int cb, int cam0, int k0, const Workspace& w
 
 // Channels are processed in chunks of at most 16 per walk; the chunk width is the smallest
 // instantiated width that covers the remaining channels (1+KC values are reduced per Gaussian,
-// padded to a power of two).
+// padded to a power of two: 2, 4 and 8 in the group walk, 16 and, V apart, 16 in the other). The group
+// walk holds four pixels' values and the sums of a thread in registers, up to 7 channels.
 void launch_blend_accumulate(const Problem& p, int cb, int cam0, const void* targets, int dtype,
                              const float* sub_img, const Workspace& ws, cudaStream_t s) {
   if (!sub_img && tc_accumulate_applies(p, dtype)) {

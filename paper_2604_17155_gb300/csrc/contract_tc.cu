@@ -6,25 +6,26 @@
 // form a dense product
 //     D[g][n] = sum_p W[g][p] * B[n][p],   W[g][p] = alpha T of Gaussian g at pixel p (Eq. 4),
 // with B's row 0 all ones, so that the same product also yields V = sum_p W[g][p] (Eq. 5), and rows 1..KT
-// the tile's target channels. The threads evaluate W by 8-lane groups
-// (groupwalk.cuh, one pixel pair a lane) and store a pair as two FP16 values into a K-major,
-// 128-byte-swizzled shared-memory operand; the tile's targets (BF16 or FP16) are transposed once
-// into B as FP16. Both operands are scaled by powers of two -- W by 2^14 (the walk carries T scaled
+// the tile's target channels. Four walker warps evaluate W by 8-lane groups (groupwalk.cuh, one
+// pixel pair a lane) and store a pair as two FP16 values into a K-major, 128-byte-swizzled
+// shared-memory operand; the tile's targets (BF16 or FP16) are transposed once into B as FP16. Both operands are scaled by powers of two -- W by 2^14 (the walk carries T scaled
 // so), the targets so that the tile's largest magnitude lands in [2^14, 2^15) -- which makes every
 // BF16 target exact in FP16, keeps small weights out of FP16's subnormal range, and is undone exactly
 // in the epilogue. One thread issues 16 tcgen05.mma (kind::f16, M=MG, N=KT+8, K=16, FP32
-// accumulation in TMEM) and commits them to an mbarrier; the warps then read D back with tcgen05.ld
-// (one Gaussian per thread) and add (V, S_0..S_{KT-1}) to the accumulator with float4 atomics -- one
-// atomic group per (Gaussian, tile). The MMA's K index runs over each warp's 8x8 pixel block in turn, so
-// a warp owns one K block of W: it clears and refills it without waiting for the others. A batch costs
-// one CTA barrier, and while its MMAs run the warps build the next batch's hit lists.
+// accumulation in TMEM) and commits them to an mbarrier. Four helper warps, one per K block of W and TMEM
+// quarter, wait for them, clear the rows of W that were written, read D back with tcgen05.ld and add
+// (V, S_0..S_{KT-1}) to the accumulator -- one atomic group per (Gaussian, tile) -- and stage the records
+// and hit lists of the batch after next, all beside the walkers' next batch. The MMA's K index runs over
+// each warp's 8x8 pixel block in turn, so a warp owns one K block of W. A batch costs one CTA barrier.
 //
-// What bounds it: shared-memory bandwidth (W and B read by the MMAs, W cleared and written, geometry and
-// lists: about two thirds of the cycles) and instruction issue (55%), with 16 warps per SM. Measured on
-// the masks scene (3M Gaussians, 200 cameras, 16 channels): 101.8 ms with one list per 8x4 warp block
-// and 256 threads; 94.3 ms with groups and 128 threads; 89.5 ms with one barrier a batch; 85.2 ms with
-// the geometry stored once; 83 ms with only the written rows cleared. 64 channels (1M Gaussians, 150
-// cameras): 47.6 -> 39.2 ms.
+// What bounds it: instruction issue (about 70% of the cycles, with 31 warps per SM) and shared-memory
+// bandwidth (about 56%: W and B read by the MMAs, W cleared and written, geometry and lists), then the
+// wait for a batch's MMAs and sums. Measured on the masks scene (3M Gaussians, 200 cameras, 16 channels):
+// 101.8 ms with one list per 8x4 warp block and 256 threads; 94.3 with groups and 128 threads; 89.5 with
+// one barrier a batch; 85.2 with the geometry stored once; 83 with only the written rows cleared; 80.4
+// with the helper warps. 64 channels (1M Gaussians, 150 cameras): 47.6 -> 39.1, and 36.7 with the sums as
+// fragments. Of the 80.4, the atomics take 1.5 and three quarters of the MMAs 6. Tried and slower:
+// batches of 48 (84.8 against 81.9), alpha one pixel at a time (83.6 against 81.2).
 //
 // Every wait on the mbarrier is bounded in time (1 s by %globaltimer): past the limit the kernel
 // sets kFlagTimeout in the status block (reported as ICGS_ERR_DEVICE_TIMEOUT), waits once more
@@ -511,8 +512,8 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
       const bool more = more_after(start, buf);
       // The sums stream through registers 8 columns at a time as accumulator fragments: four neighbouring
       // threads hold 32 consecutive bytes of a row, so an instruction's 8-byte atomics fall in whole sectors
-      // of 8 rows (with a row per thread, 16-byte atomics touched 16 rows: the 64-channel walk at 1600 x 1060,
-      // 8 views, took 39.1 ms, now 36.7; the 16-channel one, a third of the sectors, is unchanged at 80.4).
+      // of 8 rows (with a row per thread, 16-byte atomics touched 16 rows: the 64-channel walk took
+      // 39.1 ms, now 36.7; the 16-channel one, with a third of the sectors, is unchanged at 80.4).
       const int nb = (int)min((uint32_t)MG, c.len - start);
       const uint32_t id_a = __shfl_sync(0xFFFFFFFFu, id0, 2 * ra), id_b = __shfl_sync(0xFFFFFFFFu, id0, 2 * rb);
       float* const dst_a = acc_cam + (int64_t)id_a * RS + q2;

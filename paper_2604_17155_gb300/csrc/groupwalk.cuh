@@ -2,8 +2,8 @@
 // channels and the tensor-core walk of contract_tc.cu: a depth-ordered hit list of its own for every
 // small pixel block, and packed two-pixel arithmetic.
 //
-// What bounds these walks is instruction issue (80-85% of the cycles issued) with shared-memory reads
-// close behind, so the layout is chosen for instructions per contributing (pixel, Gaussian) pair:
+// What bounds these walks is instruction issue (70-80% of the cycles issued) with shared-memory reads
+// or the FP32 pipes close behind, so the layout is chosen for instructions per contributing (pixel, Gaussian) pair:
 //   - The 8 lanes of a group own one block of 4 rows: 8x4 pixels with PP = 2 pixel pairs a lane (64
 //     threads a tile), 4x4 with PP = 1 (128 threads). A warp's four groups step through their own lists
 //     side by side, so a warp takes as many steps as its longest list has entries. Measured on the relight

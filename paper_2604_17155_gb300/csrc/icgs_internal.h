@@ -11,7 +11,6 @@
 namespace icgs {
 
 constexpr int kTile = 16;            // screen tiles are 16x16 pixels; one CTA of 256 threads each
-constexpr int kTilePixels = kTile * kTile;
 constexpr int kMaxSH = 16;           // (L+1)^2 for L = 3
 // A payload CTA stages at least one Gaussian's (L+1)^2 x K coefficients in 48 KB of shared memory.
 constexpr int kMaxPayloadRow = 12287;

@@ -19,8 +19,8 @@
 //
 // Binning is a counting sort: k_project_hist counts instances per tile, an exclusive scan turns
 // counts into offsets, and k_scatter_hist writes (depth key << 32 | index) into each tile's slot
-// range. Both work on CTAs of 2048 Gaussians of one camera that count in a shared-memory
-// histogram of the camera's tiles, so a global atomic is issued per (CTA, touched tile) rather
+// range. Both work on CTAs of up to 8192 Gaussians of one camera (fewer while that leaves SMs
+// idle) that count in a shared-memory histogram of the camera's tiles, so a global atomic is issued per (CTA, touched tile) rather
 // than per instance. The order inside a tile is fixed later by the per-tile sort.
 #include <cuda_runtime.h>
 

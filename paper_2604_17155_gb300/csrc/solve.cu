@@ -1,8 +1,8 @@
 // solve.cu -- the normal equations and the batched regularised solve (Eq. 12-14, Alg. 1 lines 5-6).
 //
 //   k_fold          G_i += sum_j V_ij Y_ij Y_ij^T, b_i += sum_j Y_ij S_ij^T, w_i += sum_j V_ij over the
-//                   cameras of one pass (L > 0). One 8-lane group per Gaussian: lane r forms wrapped
-//                   diagonal r of the symmetric G_i and rows r, r + 8 of b_i. MIXED forms every
+//                   cameras of one pass (L > 0). One 8-lane group per Gaussian: lane l forms rows 2l, 2l + 1
+//                   of the symmetric G_i in wrapped 2x2 blocks, and of b_i. MIXED forms every
 //                   product exactly (TwoProduct) and keeps a TwoSum compensation term per entry.
 //   k_solve         A_i = G_i + w_i Lambda; Cholesky with the rows in registers of the group (pivots
 //                   and columns exchanged by shuffles); forward and back substitution per channel.

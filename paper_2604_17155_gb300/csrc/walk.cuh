@@ -1,6 +1,6 @@
-// walk.cuh -- the per-pixel front-to-back step shared by every tile walk (Eq. 2, Eq. 4): the CUDA-core
-// accumulate / render / adjoint kernels and the tensor-core accumulate kernel all take their
-// threshold decisions through these functions, so they agree for the same inputs.
+// walk.cuh -- the per-pixel front-to-back step (Eq. 2, Eq. 4) and the staging of the walks with one pixel a
+// thread, a CTA of 256 per tile (blend.cu's kernels for many channels). The walks by 8-lane groups take the
+// same threshold decisions with the same rounding (groupwalk.cuh), so all walks agree for the same inputs.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -27,11 +27,7 @@ struct TileCtx {
   uint32_t b, len;
 };
 
-// ROWS = 1: CTAs of 256 threads, warp w covers the 8x4 block ((w&1)*8, (w>>1)*4) with one pixel
-// per lane. ROWS = 2: CTAs of 128 threads, warp w covers the 8x8 block ((w&1)*8, (w>>1)*8) and lane
-// l the two pixels (l&7, l>>3) and (l&7, (l>>3) + 4) of it; px, py, pyf and inside then describe
-// the first of the two (the second is 4 rows below).
-template <int ROWS = 1>
+// Warp w covers the 8x4 block ((w&1)*8, (w>>1)*4) with one pixel per lane.
 __device__ __forceinline__ TileCtx tile_ctx(const uint32_t* tile_off, uint32_t capacity, int tiles,
                                             int tiles_x, int width, int height) {
   TileCtx c;
@@ -41,7 +37,7 @@ __device__ __forceinline__ TileCtx tile_ctx(const uint32_t* tile_off, uint32_t c
   const int tyi = c.t / tiles_x, txi = c.t - tyi * tiles_x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ox = txi * kTile, oy = tyi * kTile;
-  const int bx = (warp & 1) * 8, by = (warp >> 1) * 4 * ROWS;  // warp block, tile-relative
+  const int bx = (warp & 1) * 8, by = (warp >> 1) * 4;  // warp block, tile-relative
   c.px = ox + bx + (lane & 7);
   c.py = oy + by + (lane >> 3);
   c.inside = c.px < width && c.py < height;
@@ -52,7 +48,7 @@ __device__ __forceinline__ TileCtx tile_ctx(const uint32_t* tile_off, uint32_t c
   c.wx0 = (float)bx + 0.5f;
   c.wx1 = (float)bx + 7.5f;
   c.wy0 = (float)by + 0.5f;
-  c.wy1 = (float)(by + 4 * ROWS) - 0.5f;
+  c.wy1 = (float)(by + 4) - 0.5f;
   const uint32_t b = min(tile_off[bid], capacity);
   uint32_t e = min(tile_off[bid + 1], capacity);
   if (e < b) e = b;
@@ -125,7 +121,7 @@ __device__ __forceinline__ bool ellipse_reaches_block(const float4 geo, const fl
 // Gaussian base + i (< nb) touches the warp's pixel block: its box, and with ELLIPSE also its
 // ellipse. One Gaussian per lane, one ballot; iterating the set bits in ascending order keeps the
 // depth order. The ellipse test removes about 15% of the box hits of an 8x8 block; it pays in the
-// issue-bound accumulate walks and costs latency in the tensor-core walk, so each walk chooses.
+// issue-bound accumulate walk, so each walk chooses.
 template <bool ELLIPSE = false>
 __device__ __forceinline__ uint32_t warp_hit_bits(const float4* s_geo, const float4* s_aux, const float2* s_half,
                                                   int base, int nb, const TileCtx& c) {
@@ -169,12 +165,8 @@ __device__ __forceinline__ float blend_step(const float4 geo, const float4 aux, 
 // blend_step without branches, for walks that only need w: the same decisions (the fast reject,
 // alpha >= 1/255, the stop when T (1 - alpha) < 1e-4) taken as predicates on values that every
 // lane computes, so a warp whose lanes disagree does not split. blend_alpha is the part that does
-// not depend on T; blend_take applies one alpha to the pixel's transmittance and returns w (0 if
-// skipped), counting a taken step in npairs. With LIVE a pixel already done takes nothing (for walks
-// that call it on every pixel). With TEXP the walk carries T scaled by 2^TEXP (from 2^TEXP down), so
-// that w comes out scaled by 2^TEXP too; the stop compares with the threshold scaled the same way.
-// Scaling by a power of two commutes with rounding for these normal values, so the decisions and
-// the scaled weights are exactly those of the unscaled step.
+// not depend on T; blend_weight applies it to the pixel's transmittance and returns w (0 if skipped,
+// or if the pixel is done), counting a taken step in npairs.
 struct StepAlpha {
   float alpha;
   bool ok;  // past the fast reject and alpha >= 1/255
@@ -185,35 +177,18 @@ __device__ __forceinline__ StepAlpha blend_alpha(const float4 geo, const float4 
   const float alpha = fminf(kAlphaMax, __fmul_rn(aux.y, ex2_approx(E)));
   return {alpha, E >= aux.z && alpha >= kAlphaMin};
 }
-// blend_alpha without the fast reject, for walks that compute alpha for every step anyway: the
-// reject only ever drops steps whose alpha is below 1/255 (E < E_thr implies o 2^E < 1/255 by its
-// margin), so alpha >= 1/255 alone takes the same decisions. Alpha is clamped by a select, which
-// keeps a NaN product NaN so that it fails the test, as it failed the reject. aux.z is not read.
-__device__ __forceinline__ StepAlpha blend_alpha_noreject(const float4 geo, const float4 aux, float pxf, float pyf) {
-  const float dx = __fsub_rn(pxf, geo.x), dy = __fsub_rn(pyf, geo.y);
-  const float E = __fmaf_rn(__fmaf_rn(geo.z, dx, __fmul_rn(geo.w, dy)), dx, __fmul_rn(__fmul_rn(aux.x, dy), dy));
-  const float oe = __fmul_rn(aux.y, ex2_approx(E));
-  const float alpha = oe > kAlphaMax ? kAlphaMax : oe;
-  return {alpha, alpha >= kAlphaMin};
-}
-
-template <bool LIVE = false, int TEXP = 0>
-__device__ __forceinline__ float blend_take(const StepAlpha a, float& T, bool& done, uint32_t& npairs) {
-  constexpr float kTMinScaled = kTMin * (float)(1 << TEXP);
+__device__ __forceinline__ float blend_weight(const float4 geo, const float4 aux, float pxf, float pyf, float& T,
+                                              bool& done, uint32_t& npairs) {
+  const StepAlpha a = blend_alpha(geo, aux, pxf, pyf);
   const float tT = __fmul_rn(T, __fsub_rn(1.0f, a.alpha));
-  const bool take = (!LIVE || !done) && a.ok;
-  const bool stop = take && tT < kTMinScaled;
+  const bool take = !done && a.ok;
+  const bool stop = take && tT < kTMin;
   const bool keep = take && !stop;
   npairs += keep ? 1u : 0u;
   const float w = keep ? __fmul_rn(a.alpha, T) : 0.0f;
   T = keep ? tT : T;
   done = done || stop;
   return w;
-}
-template <bool LIVE = false>
-__device__ __forceinline__ float blend_weight(const float4 geo, const float4 aux, float pxf, float pyf, float& T,
-                                              bool& done, uint32_t& npairs) {
-  return blend_take<LIVE>(blend_alpha(geo, aux, pxf, pyf), T, done, npairs);
 }
 
 // Slot ranges are only fully written when the pass fit its capacity; an overflowed pass (reported
@@ -250,31 +225,6 @@ __device__ __forceinline__ void load_batch(const unsigned long long* list, uint3
     s_aux[threadIdx.x] = aux;
     s_half[threadIdx.x] = unpack_half2(r.box.w);
   }
-}
-
-// load_batch without the separate half-size array: the ballot reads the half-sizes from aux.w
-// (warp_hit_bits_packed).
-__device__ __forceinline__ void load_batch_packed(const unsigned long long* list, uint32_t first, int nb,
-                                                  const ProjRec* __restrict__ rec_cam, int64_t n, float ox, float oy,
-                                                  float4* s_geo, float4* s_aux, uint32_t* s_id) {
-  if ((int)threadIdx.x < nb) {
-    const uint32_t id = min((uint32_t)list[first + threadIdx.x], (uint32_t)(n - 1));
-    const ProjRec r = rec_cam[id];
-    float4 geo, aux;
-    stage_record(r, ox, oy, geo, aux);
-    s_id[threadIdx.x] = id;
-    s_geo[threadIdx.x] = geo;
-    s_aux[threadIdx.x] = aux;
-  }
-}
-
-// warp_hit_bits (box test only) for batches staged by load_batch_packed.
-__device__ __forceinline__ uint32_t warp_hit_bits_packed(const float4* s_geo, const float4* s_aux, int base, int nb,
-                                                         const TileCtx& c) {
-  const int g = base + (int)(threadIdx.x & 31);
-  bool h = false;
-  if (g < nb) h = warp_hits(s_geo[g], unpack_half2(s_aux[g].w), c);
-  return __ballot_sync(kFull, h);
 }
 
 // Flags a non-finite target value in the status block (the call then fails with
