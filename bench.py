@@ -70,12 +70,12 @@ KERNEL_SOURCES = {
 }
 MEASURED_TRAFFIC = {
     # relight, 100 cameras: one full-size launch captured
-    ("relight", "cuda-core"): {"bytes_per_scene": 2141550080 + 288479744, "source_sha": "6a638ba3bc449478"},
+    ("relight", "cuda-core"): {"bytes_per_scene": 2144945408 + 287176448, "source_sha": "77cffe489d388dfc"},
     # features: a 10-camera launch captured and scaled by 150/10 cameras (the targets, the per-camera
     # tile lists and the per-camera accumulator re-streaming all grow with the camera count)
-    ("features", "tensor-core"): {"bytes_per_scene": 15 * (3270310656 + 1473606912), "source_sha": "912af52a3bb4b57b"},
+    ("features", "tensor-core"): {"bytes_per_scene": 15 * (3285446656 + 1462439424), "source_sha": "8161746af9376fff"},
     # segmentation masks: a 4-camera launch captured and scaled by 200/4 cameras (as above)
-    ("segmentation", "tensor-core"): {"bytes_per_scene": 50 * (1781086720 + 501826560), "source_sha": "912af52a3bb4b57b"},
+    ("segmentation", "tensor-core"): {"bytes_per_scene": 50 * (1813982976 + 502541312), "source_sha": "8161746af9376fff"},
 }
 
 
