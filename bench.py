@@ -398,7 +398,7 @@ def walk_roofline(name, kind, K, L, blend_ms, stats, target_bytes, n, n_cams, ti
         # (survey 8(d)). The tensor view counts the dense MMA work issued: one
         # [64 x 256] x [256 x (K + 8)] product per batch of 64 Gaussians of a tile list.
         batches = inst / 64.0 + n_cams * tiles
-        kpad = 16 if K <= 16 else (32 if K <= 32 else 64)
+        kpad = next(w for w in (16, 24, 32, 48, 64) if K <= w)
         mma_flops = batches * 2 * 64 * 256 * (kpad + 8)
         tensor = {"issued_mma_flops": mma_flops, "achieved_tflops": mma_flops / sec / 1e12,
                   "peak_tflops": pk["bf16_tflops"], "frac": mma_flops / sec / 1e12 / pk["bf16_tflops"],

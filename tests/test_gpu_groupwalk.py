@@ -36,10 +36,11 @@ def _gpu(icgs, sc, cams):
 
 
 # FP32: every width of the group walk's sums (2, 4 and 8 values), then the first of the other walk and a
-# second chunk of 1 and of 7 channels. 16 bits: the tensor-core operand's widths 16, 32 and 64, whole and padded.
+# second chunk of 1 and of 7 channels. 16 bits: the tensor-core operand's widths 16, 24, 32, 48 and 64, whole and
+# padded.
 @pytest.mark.parametrize("K,dtype", [(1, "f32"), (2, "f32"), (3, "f32"), (4, "f32"), (7, "f32"), (8, "f32"),
-                                     (17, "f32"), (23, "f32"), (16, "bf16"), (17, "f16"), (21, "f16"), (32, "bf16"),
-                                     (33, "f16"), (63, "bf16"), (64, "f16")])
+                                     (17, "f32"), (23, "f32"), (16, "bf16"), (17, "f16"), (21, "f16"), (24, "bf16"), (25, "f16"),
+                                     (32, "bf16"), (33, "f16"), (48, "bf16"), (49, "f16"), (63, "bf16"), (64, "f16")])
 def test_accumulate_widths(icgs, K, dtype):
     sc, cams = _scene(6000, 401, 6, 77, 51)
     rng = np.random.default_rng(402 + K)
