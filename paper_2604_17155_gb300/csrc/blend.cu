@@ -11,11 +11,11 @@
 //   k_blend_refine2     refinement: render and accumulation of the residuals in one kernel (<= 3 channels).
 //
 // The kernels named ...2 walk by 8-lane groups (groupwalk.cuh): 64 threads with four pixels each, every
-// group its own hit list over its 8x4 pixel block, pixel pairs in packed FP32. They issue in about 78% of
-// the cycles, with the ALU and FMA pipes at 55-60%; what is left is the list's own waste (a warp's four
-// groups run to the longest of their lists, 1.08 of their mean). Against one list a warp and two pixels
-// a thread, at 800 x 800: accumulating 100 views 9.3 -> 5.8 ms, rendering them 9.0 -> 4.3, the adjoint
-// of 40 views 6.5 -> 3.7.
+// group its own hit list over its 8x4 or 4x8 pixel block, pixel pairs in packed FP32. They issue in about
+// 75% of the cycles, with the ALU and FMA pipes at 50-65%; what is left is the list's own waste (a warp's
+// four groups run to the longest of their lists, 1.08 of their mean). Against one list a warp and two
+// pixels a thread, at 800 x 800: accumulating 100 views 9.3 -> 6.1 ms, rendering them 9.0 -> 4.3, the
+// adjoint of 40 views 6.5 -> 3.7.
 //
 // The others (more channels, whose per-pixel values and sums fill the registers) have 256 threads with one
 // pixel each: warp w covers the 8x4 block ((w&1)*8, (w>>1)*4), skips a Gaussian whose padded support box
@@ -196,13 +196,22 @@ constexpr int kPP = 2;  // pixel pairs a lane of the walks below
 constexpr int kGThreads = GroupCfg<kPP>::kThreads;
 constexpr int kGroups = GroupCfg<kPP>::kGroups;
 
+// V decides, through the pivots of the solve, which Gaussians are solved in FP64, so its sum over a pixel
+// block keeps one order, that of a halving over the block's rows and then its columns (rows 4 apart, 2, 1,
+// columns 4 apart, 2, 1): over 8x8 blocks up to three channels, over 8x4 blocks with more. The groups have
+// the shape with which the levels fall inside a lane, inside a group and, last, between two groups:
+// TALL 4x8 blocks keep V as the sums of their four columns, which two groups' columns 4 apart then join. (With V
+// a sum of each group like the others the accumulation of 100 views took 5.8 ms, but a handful of three
+// million Gaussians at the limit changed between the FP32 and the FP64 solve.) The rows of a block's sums
+// are what fills the shared memory: 10 CTAs an SM.
 template <int KC>
 struct GroupAcc {
   static_assert(KC >= 1 && KC <= 7, "1..7 channels");
-  static constexpr int NV = KC + 1;                 // V and S_0..S_{KC-1}
-  static constexpr int NP = NextPow2<NV>::value;    // 2, 4 or 8: values of a reduction, floats of a partial row
-  static constexpr int SHIFT = 3 - Log2<NP>::value; // lane l of a group returns value l >> SHIFT
-  float part[kGroups][kBatch + 1][NP];              // slot kBatch: where the list padding goes
+  static constexpr bool kTall = KC <= 3;
+  static constexpr int NP = kTall ? (KC == 3 ? 4 : 2) : 8;  // values of a reduction: kTall S alone, else V and S
+  static constexpr int SHIFT = 3 - Log2<NP>::value;         // lane l of a group returns value l >> SHIFT
+  static constexpr int kRow = 8;                            // floats of a row: kTall V by columns, then S
+  float part[kGroups][kBatch + 1][kRow];                    // slot kBatch: where the list padding goes
   GroupIds<kPP> ids;
 };
 
@@ -224,23 +233,25 @@ __device__ __forceinline__ float group_permuted_reduce(float (&v)[NT]) {
 
 // The walk of one tile for target values tv of the lane's pixels ([2 u + x]: pair u, pixel x).
 template <int KC>
-__device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC>& sa, const GroupCtx<kPP>& c,
+__device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC>& sa,
+                                                 const GroupCtx<kPP, GroupAcc<KC>::kTall>& c,
                                                  const unsigned long long* list, const ProjRec* __restrict__ rec_cam,
                                                  int64_t n, const float (&tv)[2 * kPP][KC], float* __restrict__ acc_cam,
                                                  int RS, int K, int k0, DevStatus* status) {
   using S = GroupAcc<KC>;
-  constexpr int NV = S::NV, NP = S::NP;
+  constexpr bool kTall = S::kTall;
+  constexpr int NP = S::NP, k1 = kTall ? 0 : 1;  // S_0 is value k1
   const int lane = threadIdx.x & 31;
-  // Value k of a hit is its weights times u[k], u = (1, t_0, .., t_{KC-1}, 0, ..), summed over the pixels.
+  // Value k of a hit is its weights times u[k], u = (t_0, .., t_{KC-1}, 0, ..) with, not kTall, a place for V
+  // first, summed over the pixels.
   // This lane keeps it in slot k ^ m (warp_permuted_reduce): u is permuted here once.
   const int m = (lane & 7) >> S::SHIFT;
   f2 U[2 * kPP][NP / 2];
 #pragma unroll
   for (int x = 0; x < 2 * kPP; ++x) {
     float u[NP];
-    u[0] = 1.0f;
 #pragma unroll
-    for (int k = 1; k < NP; ++k) u[k] = k <= KC ? tv[x][k <= KC ? k - 1 : 0] : 0.0f;
+    for (int k = 0; k < NP; ++k) u[k] = k >= k1 && k < k1 + KC ? tv[x][k >= k1 && k < k1 + KC ? k - k1 : 0] : 0.0f;
 #pragma unroll
     for (int bit = 1; bit < NP; bit <<= 1) {
       const bool sw = (m & bit) != 0;
@@ -255,8 +266,13 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
 #pragma unroll
     for (int k = 0; k < NP / 2; ++k) U[x][k] = pack2(u[2 * k], u[2 * k + 1]);
   }
-  const bool writer = ((lane & 7) & ((1 << S::SHIFT) - 1)) == 0 && m < NV;
-  char* const my_part = reinterpret_cast<char*>(&sa.part[c.group][0][m]);
+  // The lane's place in a row: kTall, lanes 1, 2, 6, 7 the columns of V that they end up with (2, 0, 1, 3) and
+  // lanes 0, 3, 4 sums of the value that they return; else lane l value l, V in place of value 0.
+  const int l = lane & 7;
+  const bool has_v = kTall ? l == 1 || l == 2 || l == 6 || l == 7 : l == 0;
+  const bool writer = kTall ? has_v || (l == 0 || l == 4 || (l == 3 && KC == 3)) : m < 1 + KC;
+  const int my_col = !kTall ? m : (has_v ? 2 * (l & 1) + (l >> 2) : 4 + m);
+  char* const my_part = reinterpret_cast<char*>(&sa.part[c.group][0][my_col]);
   const uint16_t* const my_list = s.lists.row[c.group];
   GroupT<kPP> T(c);
   uint32_t npairs = 0;
@@ -265,7 +281,7 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
   const uint32_t id0 = group_id<kPP>(list, c.b, list_end, n, threadIdx.x);
   uint32_t id_next = group_id<kPP>(list, c.b + kBatch, list_end, n, threadIdx.x);
   GroupFetch fetch = group_fetch(id0, rec_cam);
-  group_put<kPP>(fetch, (int)min((uint32_t)kBatch, c.len), c.ox, c.oy, s.geo, s.lim, threadIdx.x);
+  group_put<kPP, kTall>(fetch, (int)min((uint32_t)kBatch, c.len), c.ox, c.oy, s.geo, s.lim, threadIdx.x);
   sa.ids.id[buf][threadIdx.x] = id0;
   __syncthreads();
   // two barriers a batch: the next batch is staged between them, when the walk of this one has ended
@@ -293,7 +309,16 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
         v[2 * k + 1] = y.y;
       }
       const float r = group_permuted_reduce<NP>(v);  // the group's sum of value m
-      if (writer) *reinterpret_cast<float*>(my_part + o * NP / 4) = r;
+      // V: the lane's rows, then the rows of the lanes (kTall two levels), each lane keeping one of its columns
+      const float2 t = unpack2(add2(pack2(w.v[0].x, w.v[0].y), pack2(w.v[1].x, w.v[1].y)));
+      const bool odd = (lane & 4) != 0;
+      float V = (odd ? t.y : t.x) + __shfl_xor_sync(kFull, odd ? t.x : t.y, 4);
+      V += __shfl_xor_sync(kFull, V, 2);
+      if (!kTall) {  // the columns: 4 apart (above), 2, 1
+        V += __shfl_xor_sync(kFull, V, 1);
+        V += __shfl_xor_sync(kFull, V, 4);
+      }
+      if (writer) *reinterpret_cast<float*>(my_part + o * (S::kRow / 4)) = has_v ? V : r;
     };
     for (int i = 0; i < steps; i += 2) {
       const uint2 o = s.lists.pair(my_list, i);
@@ -304,22 +329,36 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
     __syncthreads();
     {
       const int g = threadIdx.x;
-      float sum[NP];
+      float sum[8];  // V, S_0, ..
 #pragma unroll
-      for (int k = 0; k < NP; ++k) sum[k] = 0.0f;
+      for (int k = 0; k < 8; ++k) sum[k] = 0.0f;
       if (g < nb) {
         const uint32_t hits = *reinterpret_cast<const uint16_t*>(&sa.ids.hits[g][0]);
+        if constexpr (kTall) {
 #pragma unroll
-        for (int q = 0; q < kGroups; ++q) {
-          if (hits & (1u << (q < 4 ? q : q + 4))) {
-            const float* row = sa.part[q][g];
-            if constexpr (NP == 2) {
-              const float2 x = *reinterpret_cast<const float2*>(row);
-              sum[0] += x.x;
-              sum[1] += x.y;
-            } else {
+          for (int q = 0; q < kGroups; q += 2) {  // an 8x8 block
+            const uint32_t both = (hits >> (q < 4 ? q : q + 4)) & 3u;
+            if (both == 0u) continue;
+            float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+            if (both & 1u) {
+              a = *reinterpret_cast<const float4*>(sa.part[q][g]);
 #pragma unroll
-              for (int k = 0; k < NP; k += 4) {
+              for (int k = 0; k < KC; ++k) sum[1 + k] += sa.part[q][g][4 + k];
+            }
+            if (both & 2u) {
+              b = *reinterpret_cast<const float4*>(sa.part[q + 1][g]);
+#pragma unroll
+              for (int k = 0; k < KC; ++k) sum[1 + k] += sa.part[q + 1][g][4 + k];
+            }
+            sum[0] += ((a.x + b.x) + (a.z + b.z)) + ((a.y + b.y) + (a.w + b.w));
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < kGroups; ++q) {
+            if (hits & (1u << (q < 4 ? q : q + 4))) {
+              const float* row = sa.part[q][g];
+#pragma unroll
+              for (int k = 0; k < 8; k += 4) {
                 const float4 x = *reinterpret_cast<const float4*>(row + k);
                 sum[k] += x.x;
                 sum[k + 1] += x.y;
@@ -332,7 +371,7 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
         if (sum[0] > 0.0f) {
           float* dst = acc_cam + (int64_t)sa.ids.id[buf][g] * RS;
           if (KC == 3 && K == 3) {
-            atomicAdd(reinterpret_cast<float4*>(dst), make_float4(sum[0], sum[1], sum[NP > 2 ? 2 : 0], sum[NP > 2 ? 3 : 0]));
+            atomicAdd(reinterpret_cast<float4*>(dst), make_float4(sum[0], sum[1], sum[2], sum[3]));
           } else {
             if (k0 == 0) atomicAdd(dst, sum[0]);
 #pragma unroll
@@ -343,7 +382,7 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
       }
     }
     if (next < c.len) {
-      group_put<kPP>(fetch, (int)min((uint32_t)kBatch, c.len - next), c.ox, c.oy, s.geo, s.lim, threadIdx.x);
+      group_put<kPP, kTall>(fetch, (int)min((uint32_t)kBatch, c.len - next), c.ox, c.oy, s.geo, s.lim, threadIdx.x);
       sa.ids.id[buf ^ 1][threadIdx.x] = id_fetched;
     }
     if (!__syncthreads_or(T.alive())) break;
@@ -353,25 +392,25 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
 
 // Calls f(x, offset) for each of the lane's pixels inside the image: x = 2 u + side, offset in pixels
 // from the lane's first pixel.
-template <typename F>
-__device__ __forceinline__ void for_pixels(const GroupCtx<kPP>& c, int width, F f) {
+template <bool TALL, typename F>
+__device__ __forceinline__ void for_pixels(const GroupCtx<kPP, TALL>& c, int width, F f) {
 #pragma unroll
   for (int u = 0; u < kPP; ++u) {
-    const int64_t row = 2 * (int64_t)u * width;
+    const int64_t row = (int64_t)(GroupShape<kPP, TALL>::kRowStep * u) * width;
     if (c.in0[u]) f(2 * u, row);
     if (c.in1[u]) f(2 * u + 1, row + 1);
   }
 }
 
 template <int KC>
-__global__ void __launch_bounds__(kGThreads, KC <= 3 ? 13 : 8) k_blend_accumulate2(
+__global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_accumulate2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, int K, int k0, int cam0, const float* __restrict__ sub_img,
     float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
   __shared__ GroupBatch<kPP> s;
   __shared__ __align__(16) GroupAcc<KC> sa;
-  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
+  const auto c = group_ctx<kPP, GroupAcc<KC>::kTall>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
   if (threadIdx.x == 0) group_pad(s.geo);
   float tv[2 * kPP][KC];
 #pragma unroll
@@ -488,8 +527,8 @@ __device__ __forceinline__ f2 guarded(bool guard, const float2 w, f2 x, f2 old) 
   return pack2(w.x > 0.0f ? a.x : b.x, w.y > 0.0f ? a.y : b.y);
 }
 
-template <int KC>
-__device__ __forceinline__ void group_render(GroupBatch<kPP>& s, GroupColours& col, int* weird, const GroupCtx<kPP>& c,
+template <int KC, bool TALL>
+__device__ __forceinline__ void group_render(GroupBatch<kPP>& s, GroupColours& col, int* weird, const GroupCtx<kPP, TALL>& c,
                                              const unsigned long long* list, const ProjRec* __restrict__ rec_cam,
                                              int64_t n, const float* __restrict__ pay_cam, int K, int k0,
                                              f2 (&img)[kPP][KC]) {
@@ -509,7 +548,7 @@ __device__ __forceinline__ void group_render(GroupBatch<kPP>& s, GroupColours& c
   uint32_t id_next = group_id<kPP>(list, c.b, list_end, n, threadIdx.x);
   auto stage = [&](uint32_t first) {  // the batch at slot first of the list, whose indices id_next holds
     const int nb = (int)min((uint32_t)kBatch, list_end - first);
-    group_put<kPP>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo, s.lim, threadIdx.x);
+    group_put<kPP, TALL>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo, s.lim, threadIdx.x);
     stage_colours<KC>(pay_cam, id_next, nb, K, k0, col, weird);
   };
   stage(c.b);
@@ -948,7 +987,7 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
 // Same arithmetic as the two separate walks, without the image round trip. The colours of pass 1 share
 // the shared memory of pass 2's partial sums.
 template <int KC>
-__global__ void __launch_bounds__(kGThreads, 13) k_blend_refine2(
+__global__ void __launch_bounds__(kGThreads, 10) k_blend_refine2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, int K, int cam0, const float* __restrict__ payload,
@@ -958,7 +997,7 @@ __global__ void __launch_bounds__(kGThreads, 13) k_blend_refine2(
   __shared__ GroupBatch<kPP> s;
   __shared__ __align__(16) GroupAcc<KC> sa;
   __shared__ int weird;
-  const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
+  const auto c = group_ctx<kPP, GroupAcc<KC>::kTall>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
   if (threadIdx.x == 0) group_pad(s.geo);
   const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;

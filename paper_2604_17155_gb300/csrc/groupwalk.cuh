@@ -4,8 +4,8 @@
 //
 // What bounds these walks is instruction issue (70-80% of the cycles issued) with shared-memory reads
 // or the FP32 pipes close behind, so the layout is chosen for instructions per contributing (pixel, Gaussian) pair:
-//   - The 8 lanes of a group own one block of 4 rows: 8x4 pixels with PP = 2 pixel pairs a lane (64
-//     threads a tile), 4x4 with PP = 1 (128 threads). A warp's four groups step through their own lists
+//   - The 8 lanes of a group own one block: 8x4 or 4x8 pixels with PP = 2 pixel pairs a lane (64 threads a
+//     tile), 4x4 with PP = 1 (128 threads). A warp's four groups step through their own lists
 //     side by side, so a warp takes as many steps as its longest list has entries. Measured on the relight
 //     scene, per (Gaussian, tile) instance: 1.69 steps of 64 pixels with one list per 8x8 warp block, 1.25
 //     with 4x4 groups, 0.81 steps of 128 pixels with 8x4 groups. PP = 2 halves what a step costs besides
@@ -48,13 +48,23 @@ template <int PP>
 struct GroupCfg {
   static_assert(PP == 1 || PP == 2, "one or two pixel pairs a lane");
   static constexpr int kThreads = 128 / PP, kWarps = 4 / PP, kGroups = 16 / PP;
-  static constexpr float kHalfX = PP == 2 ? 3.5f : 1.5f, kHalfY = 1.5f;  // pixel centres off the block's centre
+};
+
+// A group's block of pixels: 4x4 with PP = 1, 8x4 with PP = 2 or, TALL, 4x8. A lane's pixels: (px, py),
+// (px + 1, py) and, with PP = 2, the same kRowStep rows below.
+template <int PP, bool TALL>
+struct GroupShape {
+  static_assert(PP == 2 || !TALL, "4x8 blocks have two pixel pairs a lane");
+  static constexpr float kHalfX = PP == 2 && !TALL ? 3.5f : 1.5f;  // pixel centres off the block's centre
+  static constexpr float kHalfY = TALL ? 3.5f : 1.5f;
+  static constexpr int kRowStep = TALL ? 4 : 2;
 };
 
 // The walk's threads are numbered tid = 0 .. GroupCfg::kThreads - 1, which a kernel with other warps beside
-// them passes on. A lane's pixels: (px, py), (px + 1, py) and, with PP = 2, (px, py + 2), (px + 1, py + 2).
-template <int PP>
+// them passes on.
+template <int PP, bool TALL = false>
 struct GroupCtx {
+  using Shape = GroupShape<PP, TALL>;
   int j, t, px, py;         // camera, tile, first pixel
   bool in0[PP], in1[PP];    // the pixels inside the image
   float ox, oy;             // tile origin in image pixels
@@ -64,10 +74,11 @@ struct GroupCtx {
   uint32_t b, len;
 };
 
-template <int PP>
-__device__ __forceinline__ GroupCtx<PP> group_ctx(const uint32_t* __restrict__ tile_off, uint32_t capacity, int tiles,
+template <int PP, bool TALL = false>
+__device__ __forceinline__ GroupCtx<PP, TALL> group_ctx(const uint32_t* __restrict__ tile_off, uint32_t capacity, int tiles,
                                                   int tiles_x, int width, int height, int tid) {
-  GroupCtx<PP> c;
+  GroupCtx<PP, TALL> c;
+  constexpr int kStep = GroupShape<PP, TALL>::kRowStep;
   const int bid = blockIdx.x;
   c.j = bid / tiles;
   c.t = bid - c.j * tiles;
@@ -75,8 +86,8 @@ __device__ __forceinline__ GroupCtx<PP> group_ctx(const uint32_t* __restrict__ t
   const int warp = tid >> 5, lane = tid & 31;
   const int gq = lane >> 3, l = lane & 7;
   const int bx = PP == 2 ? 0 : (warp & 1) * 8, by = PP == 2 ? warp * 8 : (warp >> 1) * 8;
-  const int lx = bx + (gq & 1) * 4 * PP + (PP == 2 ? l & 3 : l & 1) * 2;
-  const int ly = by + (gq >> 1) * 4 + (PP == 2 ? l >> 2 : l >> 1);
+  const int lx = TALL ? bx + gq * 4 + (l & 1) * 2 : bx + (gq & 1) * 4 * PP + (PP == 2 ? l & 3 : l & 1) * 2;
+  const int ly = TALL ? by + (l >> 1) : by + (gq >> 1) * 4 + (PP == 2 ? l >> 2 : l >> 1);
   c.group = warp * 4 + gq;
   c.px = txi * kTile + lx;
   c.py = tyi * kTile + ly;
@@ -85,9 +96,9 @@ __device__ __forceinline__ GroupCtx<PP> group_ctx(const uint32_t* __restrict__ t
   c.x2 = pack2((float)lx + 0.5f, (float)lx + 1.5f);
 #pragma unroll
   for (int u = 0; u < PP; ++u) {
-    c.in0[u] = c.px < width && c.py + 2 * u < height;
-    c.in1[u] = c.px + 1 < width && c.py + 2 * u < height;
-    c.y2[u] = pack2((float)(ly + 2 * u) + 0.5f, (float)(ly + 2 * u) + 0.5f);
+    c.in0[u] = c.px < width && c.py + kStep * u < height;
+    c.in1[u] = c.px + 1 < width && c.py + kStep * u < height;
+    c.y2[u] = pack2((float)(ly + kStep * u) + 0.5f, (float)(ly + kStep * u) + 0.5f);
   }
   c.bx = (float)bx;
   c.by = (float)by;
@@ -104,7 +115,8 @@ template <int PP>
 struct GroupT {
   float2 v[PP];
   f2 ones;
-  __device__ __forceinline__ GroupT(const GroupCtx<PP>& c, float one = 1.0f) : ones(opaque_ones()) {
+  template <bool TALL>
+  __device__ __forceinline__ GroupT(const GroupCtx<PP, TALL>& c, float one = 1.0f) : ones(opaque_ones()) {
 #pragma unroll
     for (int u = 0; u < PP; ++u) v[u] = make_float2(c.in0[u] ? one : 0.0f, c.in1[u] ? one : 0.0f);
   }
@@ -234,7 +246,7 @@ __device__ __forceinline__ GroupFetch group_fetch(uint32_t id, const ProjRec* __
 // E_lim is explained at group_lists. -E_thr = log2(255 o) (o >= 1/255 in every list), widened by 1e-4
 // of itself and 7.2e-5; the approximate logarithm and roots are within 2^-20, and the square is
 // widened by 1e-5.
-template <int PP, bool DUP>
+template <int PP, bool TALL = false, bool DUP>
 __device__ __forceinline__ void group_put(const GroupFetch& f, int nb, float ox, float oy, GroupGeo<DUP>& geo,
                                           float2* lim, int tid) {
   const int g = group_slot<PP>(tid);
@@ -247,7 +259,7 @@ __device__ __forceinline__ void group_put(const GroupFetch& f, int nb, float ox,
     geo.put_mean(g, -mx, -my, A, Bc);
   }
   if (PP == 2 || (tid & 1) == 1) {
-    constexpr float hx = GroupCfg<PP>::kHalfX, hy = GroupCfg<PP>::kHalfY;
+    constexpr float hx = GroupShape<PP, TALL>::kHalfX, hy = GroupShape<PP, TALL>::kHalfY;
     const float thr = fmaf(fmaxf(lg2_approx(255.0f * f.par.w), 0.0f), 1.0001f, 7.2e-5f);
     const float corner = fmaf(hx * hx, fabsf(A), fmaf(hy * hy, fabsf(C), hx * hy * fabsf(Bc)));
     const float reach = sqrt_approx(thr) + sqrt_approx(corner);
@@ -268,14 +280,14 @@ __device__ __forceinline__ void group_put(const GroupFetch& f, int nb, float ox,
 // alive: bit q set while group q has a pixel that has not stopped. hits: the per-Gaussian masks, when
 // wanted. any: the Gaussians that some group of the warp lists (two words, ORed into), counts: the
 // tile's list lengths by group, when wanted.
-template <int PP, bool DUP, bool BYTES>
+template <int PP, bool TALL, bool DUP, bool BYTES>
 __device__ __forceinline__ int group_lists(const GroupGeo<DUP>& geo, const float2* lim_of, GroupLists<PP, BYTES>& lists,
-                                           const GroupCtx<PP>& c, int nb, uint32_t alive, int tid,
+                                           const GroupCtx<PP, TALL>& c, int nb, uint32_t alive, int tid,
                                            uint8_t (*hits)[GroupCfg<PP>::kWarps], uint32_t* any = nullptr,
                                            uint32_t* counts = nullptr) {
   const int warp = tid >> 5, lane = tid & 31;
   constexpr int kStride = GroupLists<PP, BYTES>::kStride;
-  constexpr float wx = 4.0f * PP;  // block width
+  constexpr float wx = TALL ? 4.0f : 4.0f * PP;  // block width
   uint16_t* const rows = lists.row[warp * 4];
   // pad every entry first, by 16-byte stores
   constexpr uint32_t kPad = BYTES ? (uint32_t)kBatch * 0x01010101u : kGPad | (kGPad << 16);
@@ -296,20 +308,20 @@ __device__ __forceinline__ int group_lists(const GroupGeo<DUP>& geo, const float
     if (g < nb) {
       const GroupOperands op = geo.at((uint32_t)g * 16u);
       const float2 lim = lim_of[g], half2 = unpack_half2(lim.y);
-      const float hx = half2.x + GroupCfg<PP>::kHalfX, hy = half2.y + GroupCfg<PP>::kHalfY;
-      const f2 dx = add2(pack2(c.bx + 0.5f * wx, c.bx + 1.5f * wx), op.nx);
-      const f2 ax = mul2(mul2(op.A, dx), dx), bx = mul2(op.Bc, dx);
-      const float2 dxs = unpack2(dx);
-      const bool in_x[2] = {fabsf(dxs.x) <= hx, fabsf(dxs.y) <= hx};
+      const float hx = half2.x + GroupShape<PP, TALL>::kHalfX, hy = half2.y + GroupShape<PP, TALL>::kHalfY;
+      // two blocks at a time, side by side: (0, 1) and (2, 3), below them or, TALL, to their right
 #pragma unroll
       for (int v = 0; v < 2; ++v) {
-        const float cy = c.by + (4.0f * (float)v + 2.0f);
+        const float cx = TALL ? c.bx + 8.0f * (float)v : c.bx, cy = TALL ? c.by + 4.0f : c.by + (4.0f * (float)v + 2.0f);
+        const f2 dx = add2(pack2(cx + 0.5f * wx, cx + 1.5f * wx), op.nx);
+        const f2 ax = mul2(mul2(op.A, dx), dx), bx = mul2(op.Bc, dx);
+        const float2 dxs = unpack2(dx);
         const f2 dy = add2(pack2(cy, cy), op.ny);
         const f2 sq = fma2(mul2(op.C, dy), dy, ax);
         const float2 e = unpack2(fma2(pack2(-2e-5f, -2e-5f), sq, fma2(bx, dy, sq)));
         const bool in_y = fabsf(unpack2(dy).x) <= hy;
-        h[2 * v] = e.x >= lim.x && in_x[0] && in_y;
-        h[2 * v + 1] = e.y >= lim.x && in_x[1] && in_y;
+        h[2 * v] = e.x >= lim.x && fabsf(dxs.x) <= hx && in_y;
+        h[2 * v + 1] = e.y >= lim.x && fabsf(dxs.y) <= hx && in_y;
       }
     }
     uint32_t m[4];
@@ -354,8 +366,9 @@ template <int PP>
 struct GroupAlpha {
   float2 alpha[PP], oe[PP], e[PP];
 };
-template <int PP, bool DUP>
-__device__ __forceinline__ GroupAlpha<PP> group_alpha(const GroupGeo<DUP>& geo, uint32_t off, const GroupCtx<PP>& c) {
+template <int PP, bool TALL, bool DUP>
+__device__ __forceinline__ GroupAlpha<PP> group_alpha(const GroupGeo<DUP>& geo, uint32_t off,
+                                                      const GroupCtx<PP, TALL>& c) {
   const GroupOperands q = geo.at(off);
   const f2 dx = add2(c.x2, q.nx);
   GroupAlpha<PP> r;

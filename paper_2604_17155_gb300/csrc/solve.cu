@@ -52,8 +52,11 @@ __device__ __forceinline__ F group_sum(F v) {
 // that is NC whole block diagonals; an even NB leaves half of block diagonal NB/2, of which the lane takes
 // one pair. Every unordered pair of indices comes up once (but for the two orders of (2l, 2l + 1)). The
 // layout is chosen for shared-memory reads, which bounded the fold (82% of the wavefront rate with one
-// wrapped diagonal a lane, 36 loads a camera): a lane reads its two rows of v Y, one window of Y and the row,
-// eight loads for 18 entries, and the products are packed two at a time (packed.cuh). b rows 2l, 2l + 1
+// wrapped diagonal a lane, 36 loads a camera): a lane reads its two rows of Y, one window of v Y and the row,
+// some ten loads for 18 entries, and the products are packed two at a time (packed.cuh). The pivots that decide
+// which Gaussians are solved in FP64 see the hi parts alone, so every entry {a, b} is formed with one fixed
+// association, v Y_b times Y_a with b after a on the shorter way round mod B (for a half way round b = a + B/2):
+// the window is of v Y, and the pairs for which block order and index order differ are put right. b rows 2l, 2l + 1
 // belong to lane l. MIXED: every product is exact in float-float (v Y_r split by an FMA, then each entry's
 // product split again) and every addition a TwoSum into the running (hi, lo) pair, so G, b and w are the
 // sums of the float32 basis to about 2^-44 relative -- the same basis the adjoint's payload uses.
@@ -78,11 +81,11 @@ __host__ __device__ inline int gram_pos(int r, int c, int B) {
   const int d = bc >= br ? bc - br : bc - br + NB;
   if (d < NC) return (((r & 1) * NC + d) * NB + br) * 2 + (c & 1);
   if (NB - d < NC) return (((c & 1) * NC + NB - d) * NB + bc) * 2 + (r & 1);
-  // the half diagonal: the row with even index in the lower block against the upper block's columns belongs
-  // to the lower block's lane, the other to the upper block's
-  const int e = br < bc ? r & 1 : c & 1, f = br < bc ? c & 1 : r & 1;
+  // the half diagonal: the upper block's even index against both of the lower block's is the lower block's
+  // lane's pair, its odd index the upper block's
   const int lo = br < bc ? br : bc, hi = br < bc ? bc : br;
-  return (2 * NC * NB + (e == 0 ? lo : hi)) * 2 + f;
+  const int plo = br < bc ? r & 1 : c & 1, phi = br < bc ? c & 1 : r & 1;
+  return (2 * NC * NB + (phi == 0 ? lo : hi)) * 2 + plo;
 }
 
 // acc (hi s, lo c) += the pair whose negation is nx, by TwoSum (two_sum_acc on both halves)
@@ -115,15 +118,12 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
   constexpr int NC = (NB + 1) / 2;             // column pairs of a lane's window
   constexpr bool kExtra = NB % 2 == 0;         // an even NB: one more pair, of block diagonal NB/2
   constexpr int NG = 2 * NC + (kExtra ? 1 : 0);  // pairs: row 0's, row 1's, the extra one
-  constexpr int kWin = 2 * (NB - 1) + 2 * NC;  // values of Y stored, wrapped around
-  // row stride of 2 mod 4 words: rows 8 apart (the groups' rows of one camera) fall 16 banks apart
-  constexpr int kYStride = (kWin + 5) / 4 * 4 - 2 >= kWin ? (kWin + 5) / 4 * 4 - 2 : (kWin + 5) / 4 * 4 + 2;
+  constexpr int kVStride = (NB - 1 + NC) | 1;  // pairs of v Y stored, wrapped around; odd: rows a bank quad apart
+  constexpr int kYStride = Bp % 4 == 2 ? Bp : Bp + 2;  // 2 mod 4: the groups' rows of a camera 16 banks apart
   constexpr int kSW = (KC + 1 + 3) / 4 * 4;    // V and the channels of a camera's row
   static_assert(NB <= GS, "one block row per lane");
-  static_assert(kYStride % 4 == 2 && kYStride >= kWin, "bank layout");
   __shared__ __align__(16) float s_Y[kSolveThreads][kYStride];
-  // v Y of rows 2l, 2l + 1 and, MIXED, its lo parts; one more slot a row keeps the rows' banks apart
-  __shared__ float4 s_vY[kSolveThreads][NB + 1];
+  __shared__ float4 s_vY[kSolveThreads][kVStride];  // v Y of columns 2c, 2c + 1 (mod Bp) and their lo parts
   __shared__ __align__(16) float s_row[kSolveThreads][kSW];
   const int64_t i_own = (blockIdx.x * (int64_t)kSolveThreads + threadIdx.x) / GS;
   const int r = threadIdx.x % GS;
@@ -133,10 +133,10 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
   const int64_t i = valid ? i_own : n - 1;
   const int l2 = r < NB ? 2 * r : 0;          // first row of the lane (lanes past NB compute and drop)
   const bool owner = r < NB;
-  // The extra pair: row 2l against the columns 2l + NB, 2l + NB + 1 (lanes l < NB/2), or rows 2l, 2l + 1
-  // against the column (2l + NB + 1) mod Bp (the other lanes): v Y of the lane's own rows, Y at x0, x1.
+  // The extra pair, of blocks l and l + NB/2: lanes l < NB/2 take column 2l + NB against their rows 2l, 2l + 1,
+  // the others the entries of column 2l + 1 with the rows 2l - NB, 2l - NB + 1.
   const bool x_cols = r < NB / 2;
-  const int x0 = x_cols ? l2 + NB : (l2 + NB + 1) % Bp, x1 = x_cols ? x0 + 1 : x0;
+  const int x_pair = owner ? (r + NB / 2) % NB : 0;  // the other block
   const bool do_gram = k0 == 0 && want_gram;  // G (skipped by refinement, whose Gram is fixed)
   const bool do_w = k0 == 0;
   static_assert(gram_floats(B) == NG * NB * 2, "layout");
@@ -219,14 +219,16 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
       if (B < Bp) Yl[Bp - 1] = 0.0f;
       sh_basis<B>(d.x, d.y, d.z, Yl);
 #pragma unroll
-      for (int c = 0; c < kWin; c += 2)
-        *reinterpret_cast<float2*>(&s_Y[threadIdx.x][c]) = make_float2(Yl[c % Bp], Yl[(c + 1) % Bp]);
+      for (int c = 0; c < Bp; c += 2)
+        *reinterpret_cast<float2*>(&s_Y[threadIdx.x][c]) = make_float2(Yl[c], Yl[c + 1]);
       if (do_gram) {
 #pragma unroll
         for (int c = 0; c < NB; ++c) {
           const float v0 = lv * Yl[2 * c], v1 = lv * Yl[2 * c + 1];
-          s_vY[threadIdx.x][c] = make_float4(v0, v1, MIXED ? fmaf(lv, Yl[2 * c], -v0) : 0.0f,
-                                             MIXED ? fmaf(lv, Yl[2 * c + 1], -v1) : 0.0f);
+          const float4 x = make_float4(v0, v1, MIXED ? fmaf(lv, Yl[2 * c], -v0) : 0.0f,
+                                       MIXED ? fmaf(lv, Yl[2 * c + 1], -v1) : 0.0f);
+          s_vY[threadIdx.x][c] = x;
+          if (c + NB < NB - 1 + NC) s_vY[threadIdx.x][c + NB] = x;
         }
       }
       float row[kSW];
@@ -255,28 +257,38 @@ __global__ void __launch_bounds__(kSolveThreads) k_fold(
       const f2 Y0 = *reinterpret_cast<const f2*>(Yq + l2);
       const f2 nY0 = MIXED ? neg2(Y0) : 0ull;
       if (do_gram) {
-        const float4 vr = s_vY[at][l2 / 2];
-        const f2 v0 = pack2(vr.x, vr.x), v1 = pack2(vr.y, vr.y);
-        const f2 xv = pack2(vr.x, x_cols ? vr.x : vr.y), xy = pack2(Yq[x0], Yq[x1]);
-        if constexpr (MIXED) {
-          const f2 l0 = pack2(vr.z, vr.z), l1 = pack2(vr.w, vr.w);
+        const float2 y0 = unpack2(Y0);
+        const f2 ya = pack2(y0.x, y0.x), yb = pack2(y0.y, y0.y);
+        const f2 nya = neg2(ya), nyb = neg2(yb);
+        float4 own;  // the column pair 2l, 2l + 1
 #pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            const f2 y = c == 0 ? Y0 : *reinterpret_cast<const f2*>(Yq + l2 + 2 * c);
-            const f2 ny = c == 0 ? nY0 : neg2(y);
-            exact_acc2(g[c], gl[c], v0, l0, y, ny);
-            exact_acc2(g[NC + c], gl[NC + c], v1, l1, y, ny);
+        for (int c = 0; c < NC; ++c) {
+          const float4 x = s_vY[at][l2 / 2 + c];
+          if (c == 0) own = x;
+          f2 v = pack2(x.x, x.y), vl = pack2(x.z, x.w), y = ya;
+          if (B == 9 && c == NC - 1) {  // {2l, 2l + 5}, five apart: v Y_2l Y_2l+5
+            if (r < 2) {
+              v = pack2(x.x, own.x);
+              vl = pack2(x.z, own.z);
+              y = pack2(y0.x, Yq[l2 + 5]);
+            }
           }
-          if constexpr (kExtra)
-            exact_acc2(g[2 * NC], gl[2 * NC], xv, pack2(vr.z, x_cols ? vr.z : vr.w), xy, neg2(xy));
-        } else {
-#pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            const f2 y = c == 0 ? Y0 : *reinterpret_cast<const f2*>(Yq + l2 + 2 * c);
-            g[c] = fma2(v0, y, g[c]);
-            g[NC + c] = fma2(v1, y, g[NC + c]);
+          const f2 ny = B == 9 && c == NC - 1 ? neg2(y) : nya;
+          if constexpr (MIXED) {
+            exact_acc2(g[c], gl[c], v, vl, y, ny);
+            exact_acc2(g[NC + c], gl[NC + c], pack2(x.x, x.y), pack2(x.z, x.w), yb, nyb);
+          } else {
+            g[c] = fma2(v, y, g[c]);
+            g[NC + c] = fma2(pack2(x.x, x.y), yb, g[NC + c]);
           }
-          if constexpr (kExtra) g[2 * NC] = fma2(xv, xy, g[2 * NC]);
+        }
+        if constexpr (kExtra) {
+          const float4 x = s_vY[at][x_pair];
+          const float yx = Yq[2 * x_pair + 1];
+          const f2 v = pack2(x.x, x_cols ? x.x : own.y), vl = pack2(x.z, x_cols ? x.z : own.w);
+          const f2 y = pack2(x_cols ? y0.x : y0.y, x_cols ? y0.y : yx);
+          if constexpr (MIXED) exact_acc2(g[2 * NC], gl[2 * NC], v, vl, y, neg2(y));
+          else g[2 * NC] = fma2(v, y, g[2 * NC]);
         }
       }
       if (do_w) {
