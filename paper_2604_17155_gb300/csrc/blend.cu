@@ -204,13 +204,15 @@ constexpr int kGroups = GroupCfg<kPP>::kGroups;
 // a sum of each group like the others the accumulation of 100 views took 5.8 ms, but a handful of three
 // million Gaussians at the limit changed between the FP32 and the FP64 solve.) The rows of a block's sums
 // are what fills the shared memory: 10 CTAs an SM.
-template <int KC>
+// Refinement, whose V decides nothing, sums it like S (not ORDERED): 8x4 blocks, rows of half the size.
+template <int KC, bool ORDERED = true>
 struct GroupAcc {
   static_assert(KC >= 1 && KC <= 7, "1..7 channels");
-  static constexpr bool kTall = KC <= 3;
-  static constexpr int NP = kTall ? (KC == 3 ? 4 : 2) : 8;  // values of a reduction: kTall S alone, else V and S
+  static constexpr bool kTall = ORDERED && KC <= 3;
+  // values of a reduction: kTall S alone, else V and S
+  static constexpr int NP = kTall ? (KC == 3 ? 4 : 2) : NextPow2<KC + 1>::value;
   static constexpr int SHIFT = 3 - Log2<NP>::value;         // lane l of a group returns value l >> SHIFT
-  static constexpr int kRow = 8;                            // floats of a row: kTall V by columns, then S
+  static constexpr int kRow = kTall ? 8 : NP;               // floats of a row: kTall V by columns, then S
   float part[kGroups][kBatch + 1][kRow];                    // slot kBatch: where the list padding goes
   GroupIds<kPP> ids;
 };
@@ -232,17 +234,17 @@ __device__ __forceinline__ float group_permuted_reduce(float (&v)[NT]) {
 }
 
 // The walk of one tile for target values tv of the lane's pixels ([2 u + x]: pair u, pixel x).
-template <int KC>
-__device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC>& sa,
-                                                 const GroupCtx<kPP, GroupAcc<KC>::kTall>& c,
+template <int KC, bool ORDERED>
+__device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC, ORDERED>& sa,
+                                                 const GroupCtx<kPP, GroupAcc<KC, ORDERED>::kTall>& c,
                                                  const unsigned long long* list, const ProjRec* __restrict__ rec_cam,
                                                  int64_t n, const float (&tv)[2 * kPP][KC], float* __restrict__ acc_cam,
                                                  int RS, int K, int k0, DevStatus* status) {
-  using S = GroupAcc<KC>;
+  using S = GroupAcc<KC, ORDERED>;
   constexpr bool kTall = S::kTall;
   constexpr int NP = S::NP, k1 = kTall ? 0 : 1;  // S_0 is value k1
   const int lane = threadIdx.x & 31;
-  // Value k of a hit is its weights times u[k], u = (t_0, .., t_{KC-1}, 0, ..) with, not kTall, a place for V
+  // Value k of a hit is its weights times u[k], u = (t_0, .., t_{KC-1}, 0, ..) with, not kTall, a 1 for V
   // first, summed over the pixels.
   // This lane keeps it in slot k ^ m (warp_permuted_reduce): u is permuted here once.
   const int m = (lane & 7) >> S::SHIFT;
@@ -251,7 +253,8 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
   for (int x = 0; x < 2 * kPP; ++x) {
     float u[NP];
 #pragma unroll
-    for (int k = 0; k < NP; ++k) u[k] = k >= k1 && k < k1 + KC ? tv[x][k >= k1 && k < k1 + KC ? k - k1 : 0] : 0.0f;
+    for (int k = 0; k < NP; ++k)
+      u[k] = k < k1 ? 1.0f : (k < k1 + KC ? tv[x][k >= k1 && k < k1 + KC ? k - k1 : 0] : 0.0f);
 #pragma unroll
     for (int bit = 1; bit < NP; bit <<= 1) {
       const bool sw = (m & bit) != 0;
@@ -267,10 +270,11 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
     for (int k = 0; k < NP / 2; ++k) U[x][k] = pack2(u[2 * k], u[2 * k + 1]);
   }
   // The lane's place in a row: kTall, lanes 1, 2, 6, 7 the columns of V that they end up with (2, 0, 1, 3) and
-  // lanes 0, 3, 4 sums of the value that they return; else lane l value l, V in place of value 0.
+  // lanes 0, 3, 4 sums of the value that they return; else the value they return, ORDERED V in place of value 0.
   const int l = lane & 7;
-  const bool has_v = kTall ? l == 1 || l == 2 || l == 6 || l == 7 : l == 0;
-  const bool writer = kTall ? has_v || (l == 0 || l == 4 || (l == 3 && KC == 3)) : m < 1 + KC;
+  const bool has_v = kTall ? l == 1 || l == 2 || l == 6 || l == 7 : ORDERED && l == 0;
+  const bool writer = kTall ? has_v || (l == 0 || l == 4 || (l == 3 && KC == 3))
+                            : (l & ((1 << S::SHIFT) - 1)) == 0 && m < 1 + KC;
   const int my_col = !kTall ? m : (has_v ? 2 * (l & 1) + (l >> 2) : 4 + m);
   char* const my_part = reinterpret_cast<char*>(&sa.part[c.group][0][my_col]);
   const uint16_t* const my_list = s.lists.row[c.group];
@@ -309,16 +313,18 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
         v[2 * k + 1] = y.y;
       }
       const float r = group_permuted_reduce<NP>(v);  // the group's sum of value m
-      // V: the lane's rows, then the rows of the lanes (kTall two levels), each lane keeping one of its columns
-      const float2 t = unpack2(add2(pack2(w.v[0].x, w.v[0].y), pack2(w.v[1].x, w.v[1].y)));
-      const bool odd = (lane & 4) != 0;
-      float V = (odd ? t.y : t.x) + __shfl_xor_sync(kFull, odd ? t.x : t.y, 4);
-      V += __shfl_xor_sync(kFull, V, 2);
-      if (!kTall) {  // the columns: 4 apart (above), 2, 1
-        V += __shfl_xor_sync(kFull, V, 1);
-        V += __shfl_xor_sync(kFull, V, 4);
+      float V = r;
+      if constexpr (ORDERED) {  // the lane's rows, then the rows of the lanes, each keeping one of its columns
+        const float2 t = unpack2(add2(pack2(w.v[0].x, w.v[0].y), pack2(w.v[1].x, w.v[1].y)));
+        const bool odd = (lane & 4) != 0;
+        V = (odd ? t.y : t.x) + __shfl_xor_sync(kFull, odd ? t.x : t.y, 4);
+        V += __shfl_xor_sync(kFull, V, 2);
+        if (!kTall) {  // the columns: 4 apart (above), 2, 1
+          V += __shfl_xor_sync(kFull, V, 1);
+          V += __shfl_xor_sync(kFull, V, 4);
+        }
       }
-      if (writer) *reinterpret_cast<float*>(my_part + o * (S::kRow / 4)) = has_v ? V : r;
+      if (writer) *reinterpret_cast<float*>(my_part + o * S::kRow / 4) = has_v ? V : r;
     };
     for (int i = 0; i < steps; i += 2) {
       const uint2 o = s.lists.pair(my_list, i);
@@ -357,13 +363,19 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
           for (int q = 0; q < kGroups; ++q) {
             if (hits & (1u << (q < 4 ? q : q + 4))) {
               const float* row = sa.part[q][g];
+              if constexpr (NP == 2) {
+                const float2 x = *reinterpret_cast<const float2*>(row);
+                sum[0] += x.x;
+                sum[1] += x.y;
+              } else {
 #pragma unroll
-              for (int k = 0; k < 8; k += 4) {
-                const float4 x = *reinterpret_cast<const float4*>(row + k);
-                sum[k] += x.x;
-                sum[k + 1] += x.y;
-                sum[k + 2] += x.z;
-                sum[k + 3] += x.w;
+                for (int k = 0; k < NP; k += 4) {
+                  const float4 x = *reinterpret_cast<const float4*>(row + k);
+                  sum[k] += x.x;
+                  sum[k + 1] += x.y;
+                  sum[k + 2] += x.z;
+                  sum[k + 3] += x.w;
+                }
               }
             }
           }
@@ -431,7 +443,7 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_accumulat
     }
     if (KC <= 3) check_finite(tv[x], status);
   });
-  group_accumulate<KC>(s, sa, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n, tv,
+  group_accumulate<KC, true>(s, sa, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n, tv,
                        acc + (int64_t)c.j * acc_cam_stride, RS, K, k0, status);
 }
 
@@ -987,17 +999,17 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
 // Same arithmetic as the two separate walks, without the image round trip. The colours of pass 1 share
 // the shared memory of pass 2's partial sums.
 template <int KC>
-__global__ void __launch_bounds__(kGThreads, 10) k_blend_refine2(
+__global__ void __launch_bounds__(kGThreads, 13) k_blend_refine2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, int K, int cam0, const float* __restrict__ payload,
     float* __restrict__ acc, int RS, int64_t acc_cam_stride, DevStatus* status) {
   static_assert(KC <= 3, "up to 3 channels");
-  static_assert(sizeof(GroupColours) <= sizeof(GroupAcc<KC>), "the colours fit where the sums go");
+  static_assert(sizeof(GroupColours) <= sizeof(GroupAcc<KC, false>), "the colours fit where the sums go");
   __shared__ GroupBatch<kPP> s;
-  __shared__ __align__(16) GroupAcc<KC> sa;
+  __shared__ __align__(16) GroupAcc<KC, false> sa;
   __shared__ int weird;
-  const auto c = group_ctx<kPP, GroupAcc<KC>::kTall>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
+  const auto c = group_ctx<kPP, GroupAcc<KC, false>::kTall>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
   if (threadIdx.x == 0) group_pad(s.geo);
   const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
   const ProjRec* rec_cam = rec + (int64_t)c.j * n;
@@ -1019,7 +1031,7 @@ __global__ void __launch_bounds__(kGThreads, 10) k_blend_refine2(
     check_finite(tv[x], status);
   });
   __syncthreads();
-  group_accumulate<KC>(s, sa, c, list, rec_cam, n, tv, acc + (int64_t)c.j * acc_cam_stride, RS, K, 0, status);
+  group_accumulate<KC, false>(s, sa, c, list, rec_cam, n, tv, acc + (int64_t)c.j * acc_cam_stride, RS, K, 0, status);
 }
 
 template <int KC>
