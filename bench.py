@@ -70,12 +70,12 @@ KERNEL_SOURCES = {
 }
 MEASURED_TRAFFIC = {
     # relight, 100 cameras: one full-size launch captured
-    ("relight", "cuda-core"): {"bytes_per_scene": 2144945408 + 287176448, "source_sha": "77cffe489d388dfc"},
+    ("relight", "cuda-core"): {"bytes_per_scene": 2146019072 + 288247040, "source_sha": "9100ec12c5109733"},
     # features: a 10-camera launch captured and scaled by 150/10 cameras (the targets, the per-camera
     # tile lists and the per-camera accumulator re-streaming all grow with the camera count)
-    ("features", "tensor-core"): {"bytes_per_scene": 15 * (3285446656 + 1462439424), "source_sha": "8161746af9376fff"},
+    ("features", "tensor-core"): {"bytes_per_scene": 15 * (3285384960 + 1462768384), "source_sha": "6027f9630ffe8186"},
     # segmentation masks: a 4-camera launch captured and scaled by 200/4 cameras (as above)
-    ("segmentation", "tensor-core"): {"bytes_per_scene": 50 * (1813982976 + 502541312), "source_sha": "8161746af9376fff"},
+    ("segmentation", "tensor-core"): {"bytes_per_scene": 50 * (1813298688 + 502618368), "source_sha": "6027f9630ffe8186"},
 }
 
 

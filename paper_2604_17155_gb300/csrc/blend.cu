@@ -11,8 +11,8 @@
 //   k_blend_refine2     refinement: render and accumulation of the residuals in one kernel (<= 3 channels).
 //
 // The kernels named ...2 walk by 8-lane groups (groupwalk.cuh): 64 threads with four pixels each, every
-// group its own hit list over its 8x4 or 4x8 pixel block, pixel pairs in packed FP32. They issue in about
-// 75% of the cycles, with the ALU and FMA pipes at 50-65%; what is left is the list's own waste (a warp's
+// group its own hit list over its 8x4 or 4x8 pixel block, pixel pairs in packed FP32. They issue in 72%
+// (accumulation) to 78% of the cycles, with the ALU and FMA pipes at 45-60%; what is left is the list's own waste (a warp's
 // four groups run to the longest of their lists, 1.08 of their mean). Against one list a warp and two
 // pixels a thread, at 800 x 800: accumulating 100 views 9.3 -> 6.1 ms, rendering them 9.0 -> 4.3, the
 // adjoint of 40 views 6.5 -> 3.7.
