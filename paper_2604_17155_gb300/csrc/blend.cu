@@ -774,28 +774,35 @@ __global__ void __launch_bounds__(kThreads, KC <= 4 ? 6 : (KC <= 16 ? 4 : (KC <=
 // list per 8x4 block, the payload staged twice each for packed arithmetic. Pass 2 adds a lane's four
 // pixels, reduces two hits at a time over the group's 8 lanes (3 shuffles) and stores the sums in the
 // group's row; after the batch one thread per Gaussian adds the rows and one atomic lands in grad_o.
-// A skipped step adds 0 a, exact for finite values; with a staged payload value or a target of the
-// tile that is not finite (weird) the steps test the weight instead.
+// A skipped step adds 0 a to dL/dt and 0 g to F and P, g = a . t + beta: exact while a and g are finite.
+// Once a staged payload could make g overflow at some pixel of the tile, or is not finite, or a target is not
+// (weird), the tile's steps test the weight instead.
 template <int KC>
 struct GroupPayload {
   static constexpr int NQ = (KC + 2) / 2;      // float4 rows of two doubled values: a_0.., beta
   float4 q[NQ][kBatch + 1];
 };
 
+// t_max: the largest magnitude of the tile's targets. |g| and every partial sum of it stay below
+// |beta| + t_max sum |a_k| (1 + 2^-21), so a bound below 2^126 rules an overflow out; a NaN, or an infinite
+// a or beta, fails the comparison too (t_max = 0 makes it NaN).
 template <int KC>
-__device__ __forceinline__ void stage_payload(const float* __restrict__ pay_cam, uint32_t id, int nb, int K,
+__device__ __forceinline__ void stage_payload(const float* __restrict__ pay_cam, uint32_t id, int nb, int K, float t_max,
                                               GroupPayload<KC>& pay, int* weird) {
   const int g = threadIdx.x;
   if (g >= nb) return;
   const float* src = pay_cam + (int64_t)id * (K + 1);  // K == KC
-  bool bad = false;
+  float sum_a = 0.0f, beta = 0.0f;
 #pragma unroll
   for (int r = 0; r < GroupPayload<KC>::NQ; ++r) {
     const float x = src[2 * r], y = 2 * r + 1 <= KC ? src[2 * r + 1 <= KC ? 2 * r + 1 : 0] : 0.0f;
     pay.q[r][g] = make_float4(x, x, y, y);
-    bad |= !isfinite(x) || !isfinite(y);
+    if (2 * r < KC) sum_a += fabsf(x);
+    else beta = x;
+    if (2 * r + 1 < KC) sum_a += fabsf(y);
+    else if (2 * r + 1 == KC) beta = y;
   }
-  if (bad) *weird = 1;
+  if (!(fmaf(t_max, sum_a, fabsf(beta)) < 0x1p126f)) *weird = 1;
 }
 
 // The staged payload of the Gaussian at byte offset o: a[0..KC-1], beta in a[KC].
@@ -820,6 +827,7 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
   __shared__ GroupPayload<KC> pay;
   __shared__ GroupIds<kPP> ids;
   __shared__ float s_go[kGroups][kBatch + 1];
+  __shared__ float s_tmax[kGThreads / 32];
   __shared__ int weird;
   const GroupCtx<kPP> c = group_ctx<kPP>(tile_off, capacity, tiles, tiles_x, width, height, threadIdx.x);
   const unsigned long long* list = reinterpret_cast<const unsigned long long*>(entries);
@@ -832,24 +840,29 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
     for (int r = 0; r < GroupPayload<KC>::NQ; ++r) pay.q[r][kBatch] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
   if (threadIdx.x == 0) group_pad(s.geo);
-  __syncthreads();
   const int64_t pix0 = ((int64_t)(cam0 + c.j) * height + c.py) * width + c.px;
   f2 tv[kPP][KC];
+  float t_max;
   {
     float t[2 * kPP][KC];
 #pragma unroll
     for (int x = 0; x < 2 * kPP; ++x)
 #pragma unroll
       for (int k = 0; k < KC; ++k) t[x][k] = 0.0f;
-    bool bad = false;
+    uint32_t m = 0u;  // non-negative floats order like their bit patterns, with infinity and NaN above
     for_pixels(c, width, [&](int x, int64_t off) {
 #pragma unroll
       for (int k = 0; k < KC; ++k) {
         t[x][k] = load_target(targets, (pix0 + off) * K + k, dtype);
-        bad |= !isfinite(t[x][k]);
+        m = max(m, __float_as_uint(fabsf(t[x][k])));
       }
     });
-    if (bad) weird = 1;
+    m = __reduce_max_sync(kFull, m);
+    if (lane == 0) s_tmax[threadIdx.x >> 5] = __uint_as_float(m);
+    __syncthreads();
+    t_max = __uint_as_float(max(__float_as_uint(s_tmax[0]), __float_as_uint(s_tmax[1])));
+    static_assert(kGThreads == 64, "two warps");
+    if (!(t_max < INFINITY)) weird = 1;
 #pragma unroll
     for (int u = 0; u < kPP; ++u)
 #pragma unroll
@@ -861,7 +874,7 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_adjoint2(
     const int nb = (int)min((uint32_t)kBatch, list_end - first);
     group_put<kPP>(group_fetch(id_next, rec_cam), nb, c.ox, c.oy, s.geo, s.lim, threadIdx.x);
     ids.id[to][threadIdx.x] = id_next;
-    stage_payload<KC>(pay_cam, id_next, nb, K, pay, &weird);
+    stage_payload<KC>(pay_cam, id_next, nb, K, t_max, pay, &weird);
   };
   // g = a . t + beta of pixel pair u
   auto gain = [&](const f2 (&a)[KC + 1], int u) -> f2 {
