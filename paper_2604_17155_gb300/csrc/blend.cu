@@ -233,8 +233,9 @@ __device__ __forceinline__ float group_permuted_reduce(float (&v)[NT]) {
   return r;
 }
 
-// The walk of one tile for target values tv of the lane's pixels ([2 u + x]: pair u, pixel x).
-template <int KC, bool ORDERED>
+// The walk of one tile for target values tv of the lane's pixels ([2 u + x]: pair u, pixel x). UNCHECKED: they
+// may be infinite or NaN without the call failing (residuals of more than three channels).
+template <int KC, bool ORDERED, bool UNCHECKED>
 __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC, ORDERED>& sa,
                                                  const GroupCtx<kPP, GroupAcc<KC, ORDERED>::kTall>& c,
                                                  const unsigned long long* list, const ProjRec* __restrict__ rec_cam,
@@ -368,6 +369,8 @@ __device__ __forceinline__ void group_accumulate(GroupBatch<kPP>& s, GroupAcc<KC
                 sum[0] += x.x;
                 sum[1] += x.y;
               } else {
+                // an infinite residual makes 0 t NaN: it stays with the Gaussians that have weight in its block
+                if (UNCHECKED && !(row[0] > 0.0f)) continue;
 #pragma unroll
                 for (int k = 0; k < NP; k += 4) {
                   const float4 x = *reinterpret_cast<const float4*>(row + k);
@@ -414,7 +417,7 @@ __device__ __forceinline__ void for_pixels(const GroupCtx<kPP, TALL>& c, int wid
   }
 }
 
-template <int KC>
+template <int KC, bool RESIDUAL>
 __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_accumulate2(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
@@ -436,15 +439,15 @@ __global__ void __launch_bounds__(kGThreads, KC <= 3 ? 10 : 8) k_blend_accumulat
     for (int k = 0; k < KC; ++k)
       if (k0 + k < K) tv[x][k] = load_target(targets, base + off * K + k, dtype);
     if (KC > 3) check_finite(tv[x], status);
-    if (sub_img) {  // refinement: residual targets t - img, img of this pass's cameras
+    if constexpr (RESIDUAL) {  // refinement: residual targets t - img, img of this pass's cameras
 #pragma unroll
       for (int k = 0; k < KC; ++k)
         if (k0 + k < K) tv[x][k] -= sub_img[ib + off * K + k];
     }
     if (KC <= 3) check_finite(tv[x], status);
   });
-  group_accumulate<KC, true>(s, sa, c, reinterpret_cast<const unsigned long long*>(entries), rec + (int64_t)c.j * n, n, tv,
-                       acc + (int64_t)c.j * acc_cam_stride, RS, K, k0, status);
+  group_accumulate<KC, true, RESIDUAL && (KC > 3)>(s, sa, c, reinterpret_cast<const unsigned long long*>(entries),
+                                                   rec + (int64_t)c.j * n, n, tv, acc + (int64_t)c.j * acc_cam_stride, RS, K, k0, status);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1044,7 +1047,7 @@ __global__ void __launch_bounds__(kGThreads, 13) k_blend_refine2(
     check_finite(tv[x], status);
   });
   __syncthreads();
-  group_accumulate<KC, false>(s, sa, c, list, rec_cam, n, tv, acc + (int64_t)c.j * acc_cam_stride, RS, K, 0, status);
+  group_accumulate<KC, false, false>(s, sa, c, list, rec_cam, n, tv, acc + (int64_t)c.j * acc_cam_stride, RS, K, 0, status);
 }
 
 template <int KC>
@@ -1052,10 +1055,10 @@ void accumulate_chunk(const Problem& p, int cb, int cam0, const void* targets, i
                       const float* sub_img, const Workspace& ws, cudaStream_t s) {
   const int64_t stride = p.L == 0 ? 0 : p.n * (int64_t)p.acc_stride;
   if constexpr (KC <= 7) {
-    k_blend_accumulate2<KC><<<cb * p.tiles, kGThreads, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,
-                                                               p.width, p.height, p.tiles_x, p.tiles, targets, dtype,
-                                                               p.K, k0, cam0, sub_img, ws.acc, p.acc_stride, stride,
-                                                               ws.status);
+    const auto kern = sub_img ? k_blend_accumulate2<KC, true> : k_blend_accumulate2<KC, false>;
+    kern<<<cb * p.tiles, kGThreads, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n, p.width, p.height,
+                                            p.tiles_x, p.tiles, targets, dtype, p.K, k0, cam0, sub_img, ws.acc,
+                                            p.acc_stride, stride, ws.status);
   } else {
     k_blend_accumulate<KC><<<cb * p.tiles, kThreads, 0, s>>>(ws.tile_off, ws.entries, p.capacity, ws.rec, p.n,
                                                               p.width, p.height, p.tiles_x, p.tiles, targets, dtype,
