@@ -1,6 +1,6 @@
 // radix.cuh -- depth order of one tile list in shared memory by a stable LSD radix sort (the "depth
-// ordered list" of Eq. 2), for the lists whose depths crowd into few values (the others are bucket
-// sorted, bucket.cuh): by one warp (lists that fit its two buffers, no CTA barrier) or by one CTA of
+// ordered list" of Eq. 2), for the lists that bucket.cuh's sorts refuse (whose keys crowd whatever
+// the splits): by one warp (lists that fit its two buffers, no CTA barrier) or by one CTA of
 // 256 threads (longer lists).
 //
 // A key is (float32 depth bits << 32) | Gaussian index. Depths are positive and finite, so their

@@ -6,8 +6,9 @@
 // (bucket.cuh) in shared memory by a team sized to it: lists of up to kWarpSortCap keys by one warp
 // each of a persistent kernel (k_sort_tiles, no CTA barrier), which queues the others; up to kMidCap
 // keys by a CTA of four warps (k_sort_mid); longer ones, in runs of kSortCap keys that are merged,
-// by a CTA of eight (k_sort_queued). A list whose depths crowd takes the stable LSD radix sort of
-// radix.cuh in the queue's kernels instead.
+// by a CTA of eight (k_sort_queued). A list in which many depths are equal, which the warp's or the CTA's sort
+// refuses, is split by its whole keys in the queue's kernels, and one that still crowds takes the stable LSD radix
+// sort of radix.cuh there.
 //
 // Latency of shared-memory atomics and loads bounds these kernels, so passes over the keys and warps
 // in flight count: with three or four radix passes a list, the sort of 1.1e9 keys in 1.3 million lists
@@ -124,10 +125,10 @@ __device__ __forceinline__ void merge_runs(const unsigned long long* A, int na, 
 }
 
 // Sorts the queued lists of up to kMidCap keys (queue[0, big_tiles)), a grid-stride loop with a CTA per list:
-// those of more than kWarpSortCap keys by a bucket sort of the CTA. The crowded ones, and the shorter lists
-// that a warp's bucket sort refused, by two warps: warp w sorts one half (at most kWarpSortCap keys) with the
-// warp radix sort in its part of two shared pools, the halves are gathered into the first pool, and a
-// merge-path merge (every thread an equal share of the outputs) writes the list back to its slot range.
+// those of more than kWarpSortCap keys by a bucket sort of the CTA; the crowded ones, and the shorter lists
+// that a warp's bucket sort refused, by splitting them. What remains by two warps: warp w sorts one half (at most
+// kWarpSortCap keys) with the warp radix sort in its part of two shared pools, the halves are gathered into the first
+// pool, and a merge-path merge (every thread an equal share of the outputs) writes the list back to its slot range.
 __global__ void __launch_bounds__(kMidThreads, 6) k_sort_mid(const uint32_t* __restrict__ tile_off,
                                                              unsigned long long* __restrict__ entries, uint32_t capacity,
                                                              const uint32_t* __restrict__ queue,
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kMidThreads, 6) k_sort_mid(const uint32_t* __r
     tile_range(tile_off, queue[q], capacity, b, e);
     const int n = (int)(e - b);
     if (n > kWarpSortCap && bucket::sort_list<kMidThreads / 32, kMidCap / kMidThreads>(entries + b, n, P0, bins)) continue;  // uniform
+    if (bucket::split_list<kMidThreads / 32, kMidCap / kMidThreads>(entries + b, n, P0, bins)) continue;  // uniform
     if (w < 2) {
       __syncwarp();
       const int h = (n + 1) / 2;
@@ -183,7 +185,7 @@ __device__ __forceinline__ void block_sort_list(unsigned long long* g, int m, un
 
 // Sorts the queued lists of more than kMidCap keys (the last long_tiles entries of the queue) in
 // place, a grid-stride loop with a CTA per list: in runs of up to kSortCap keys, each by a bucket sort or, when
-// crowded, by the block radix sort; a longer list then by pairwise merge-path merges ping-ponging between its
+// crowded, by splitting it or by the block radix sort; a longer list then by pairwise merge-path merges ping-ponging between its
 // slot range and the same range of the scratch array. (A bucket sort of 2 kSortCap keys in both buffers at
 // once spilled its 32 keys a thread and was slower, 1.06 ms a pass against 0.65.)
 __global__ void __launch_bounds__(kSortThreads, 2) k_sort_queued(const uint32_t* __restrict__ tile_off,
@@ -206,7 +208,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort_queued(const uint32_t*
     const int n = (int)(e - b);
     for (int r0 = 0; r0 < n; r0 += CAP) {  // sorted runs (the whole list when it fits)
       const int m = min(CAP, n - r0);
-      if (m > 1 && !bucket::sort_list<kWarps, CAP / kSortThreads>(entries + b + r0, m, s_dyn, bins))
+      if (m > 1 && !bucket::sort_list<kWarps, CAP / kSortThreads>(entries + b + r0, m, s_dyn, bins) &&
+          !bucket::split_list<kWarps, CAP / kSortThreads>(entries + b + r0, m, s_dyn, bins))
         block_sort_list(entries + b + r0, m, s_dyn, s_dyn + CAP, sc);
     }
     if (n <= CAP) continue;  // uniform
