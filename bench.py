@@ -409,7 +409,7 @@ def walk_roofline(name, kind, K, L, blend_ms, stats, target_bytes, n, n_cams, ti
                 "traffic_unit": "bytes per scene (DRAM read + write, ncu)", "peak_source": pk["source"],
                 "tensor_view": tensor, "alu_view": alu}
     else:
-        kname = f"k_blend_accumulate2<{K if K <= 3 else 7}>" if K <= 7 else f"k_blend_accumulate<{15 if K <= 15 else 16}>"
+        kname = f"k_blend_accumulate2<{K if K <= 3 else 7}, false>" if K <= 7 else f"k_blend_accumulate<{15 if K <= 15 else 16}>"
         roof = {"kernel": kname, "bound": "alu", "achieved": alu["achieved_tflops"], "peak": alu["peak_tflops"],
                 "unit": "TFLOP/s", "frac": alu["frac"], "traffic": traffic,
                 "traffic_unit": "bytes per scene (DRAM read + write, ncu)", "peak_source": alu["peak_source"],

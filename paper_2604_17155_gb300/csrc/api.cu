@@ -257,7 +257,7 @@ struct UploadBatch {
   int count;  // cameras in this batch
   int n_lam;  // lambda entries (first batch only)
 };
-static_assert(sizeof(UploadBatch) + 2 * sizeof(void*) <= 32000, "kernel parameter space");
+static_assert(sizeof(UploadBatch) + 3 * sizeof(void*) <= 32000, "kernel parameter space");
 
 // status: zeroed when given (the first batch of a call)
 __global__ void k_upload(const UploadBatch batch, DevCam* __restrict__ dst, float* __restrict__ lam_dst,

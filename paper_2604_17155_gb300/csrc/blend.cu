@@ -14,7 +14,7 @@
 // group its own hit list over its 8x4 or 4x8 pixel block, pixel pairs in packed FP32. They issue in 72%
 // (accumulation) to 78% of the cycles, with the ALU and FMA pipes at 45-60%; what is left is the list's own waste (a warp's
 // four groups run to the longest of their lists, 1.08 of their mean). Against one list a warp and two
-// pixels a thread, at 800 x 800: accumulating 100 views 9.3 -> 6.1 ms, rendering them 9.0 -> 4.3, the
+// pixels a thread, at 800 x 800: accumulating 100 views 9.3 -> 6.0 ms, rendering them 9.0 -> 4.2, the
 // adjoint of 40 views 6.5 -> 3.7.
 //
 // The others (more channels, whose per-pixel values and sums fill the registers) have 256 threads with one
@@ -693,10 +693,10 @@ __global__ void __launch_bounds__(kGThreads, 13) k_blend_render2(
 // ------------------------------------------------------------------------------------------
 // adjoint: dL/dt and dL/do. Payload per (camera, Gaussian) = (a_0..a_{K-1}, beta).
 // ------------------------------------------------------------------------------------------
-template <int KC, int NT = kThreads>
+template <int KC>
 __device__ __forceinline__ void load_payload(const float* __restrict__ pay_cam, int nb, int K, const uint32_t* s_id,
                                              float (*s_pay)[KC + 1]) {
-  for (int idx = threadIdx.x; idx < nb * (KC + 1); idx += NT) {
+  for (int idx = threadIdx.x; idx < nb * (KC + 1); idx += kThreads) {
     const int g = idx / (KC + 1), k = idx - g * (KC + 1);
     float v = 0.0f;
     if (k < KC) {
@@ -709,7 +709,7 @@ __device__ __forceinline__ void load_payload(const float* __restrict__ pay_cam, 
 }
 
 template <int KC>
-__global__ void __launch_bounds__(kThreads, KC <= 4 ? 6 : (KC <= 16 ? 4 : (KC <= 32 ? 2 : 1))) k_blend_adjoint(
+__global__ void __launch_bounds__(kThreads, KC <= 16 ? 4 : (KC <= 32 ? 2 : 1)) k_blend_adjoint(
     const uint32_t* __restrict__ tile_off, const uint64_t* __restrict__ entries, uint32_t capacity,
     const ProjRec* __restrict__ rec, int64_t n, int width, int height, int tiles_x, int tiles,
     const void* __restrict__ targets, int dtype, const float* __restrict__ payload, int K, int cam0,

@@ -18,14 +18,14 @@
 // and hit lists of the batch after next, all beside the walkers' next batch. The MMA's K index runs over
 // each warp's 8x8 pixel block in turn, so a warp owns one K block of W. A batch costs one CTA barrier.
 //
-// What bounds it: instruction issue (about 70% of the cycles, with 31 warps per SM) and shared-memory
-// bandwidth (about 56%: W and B read by the MMAs, W cleared and written, geometry and lists), then the
-// wait for a batch's MMAs and sums. Measured on the masks scene (3M Gaussians, 200 cameras, 16 channels):
-// 101.8 ms with one list per 8x4 warp block and 256 threads; 94.3 with groups and 128 threads; 89.5 with
-// one barrier a batch; 85.2 with the geometry stored once; 83 with only the written rows cleared; 80.4
-// with the helper warps. 64 channels (1M Gaussians, 150 cameras): 47.6 -> 39.1, and 36.7 with the sums as
-// fragments. Of the 80.4, the atomics take 1.5 and three quarters of the MMAs 6. Tried and slower:
-// batches of 48 (84.8 against 81.9), alpha one pixel at a time (83.6 against 81.2).
+// What bounds it: instruction issue (about 70% of the cycles, with 31 warps per SM; the ALU pipe 56%), then the wait
+// for a batch's MMAs and sums; shared memory takes 41% of its wavefronts besides the MMAs' own reads of W and B.
+// Measured at 16 channels (3M Gaussians, 200 views of 1600 x 1060), each step against the tree before it: 101.8 ms
+// with one list per 8x4 warp block and 256 threads; 94.3 with groups and 128 threads; 89.5 with one barrier a
+// batch; 85.2 with the geometry stored once; 83 with only the written rows cleared; 80.4 with the helper warps, and
+// 81.5 as it is now. 64 channels (1M Gaussians, 150 views): 47.6 -> 39.1, and 36.9 with the sums as fragments. Of the
+// 80.4, the atomics take 1.5 and three quarters of the MMAs 6. Tried and slower: batches of 48 (84.8 against
+// 81.9), alpha one pixel at a time (83.6 against 81.2).
 //
 // Every wait on the mbarrier is bounded in time (1 s by %globaltimer): past the limit the kernel
 // sets kFlagTimeout in the status block (reported as ICGS_ERR_DEVICE_TIMEOUT), waits once more
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kTcThreads, tc_ctas_per_sm<KT, MG>()) k_blend_
       // The sums stream through registers 8 columns at a time as accumulator fragments: four neighbouring
       // threads hold 32 consecutive bytes of a row, so an instruction's 8-byte atomics fall in whole sectors
       // of 8 rows (with a row per thread, 16-byte atomics touched 16 rows: the 64-channel walk took
-      // 39.1 ms, now 36.7; the 16-channel one, with a third of the sectors, is unchanged at 80.4).
+      // 39.1 ms, then 36.7; the 16-channel one, with a third of the sectors, 80.3 and 80.4).
       const int nb = (int)min((uint32_t)MG, c.len - start);
       const uint32_t id_a = __shfl_sync(0xFFFFFFFFu, id0, 2 * ra), id_b = __shfl_sync(0xFFFFFFFFu, id0, 2 * rb);
       float* const dst_a = acc_cam + (int64_t)id_a * RS + q2;

@@ -385,8 +385,9 @@ __device__ __forceinline__ GroupAlpha<PP> group_alpha(const GroupGeo<DUP>& geo, 
 
 // Applies the alphas to the pixels' transmittances and returns the weights (0 where skipped). A pixel
 // that stops gets T = 0, at which every later step stops again. COUNT: counts the steps taken in
-// npairs. TEXP: T carries a factor 2^TEXP, so that the weights come out scaled by it (walk.cuh,
-// blend_take).
+// npairs. TEXP: T carries a factor 2^TEXP (from 2^TEXP down), so that the weights come out scaled by it, and the
+// stop compares with the threshold scaled the same way: a power of two commutes with the roundings of these
+// normal values, so the decisions and the scaled weights are exactly those of the unscaled step.
 template <int PP>
 struct GroupW {
   float2 v[PP];

@@ -10,7 +10,7 @@
 
 namespace icgs {
 
-constexpr int kTile = 16;            // screen tiles are 16x16 pixels; one CTA of 256 threads each
+constexpr int kTile = 16;            // screen tiles are 16x16 pixels, a CTA each
 constexpr int kMaxSH = 16;           // (L+1)^2 for L = 3
 // A payload CTA stages at least one Gaussian's (L+1)^2 x K coefficients in 48 KB of shared memory.
 constexpr int kMaxPayloadRow = 12287;
@@ -83,8 +83,8 @@ struct Workspace {
   float4* packed = nullptr;        // [3 n] parameters by processing position (mean, o), (scale, qw), (qxyz, 0)
   float* payload = nullptr;        // [cb * n * (K+1)] per (camera, Gaussian) colour / adjoint terms
   float* acc = nullptr;            // [cb * n * RS] (L>0) or [n * RS] (L=0), RS = acc_stride
-  float* G = nullptr;              // [n * B * B] Gram rows, hi
-  float* Glo = nullptr;            // [n * B * B] compensation
+  float* G = nullptr;              // [n * B * B], of which n * gram_floats(B) as the fold writes them (solve.cu), hi
+  float* Glo = nullptr;            // the same, compensation
   float* bvec = nullptr;           // [n * B * K]
   float* blo = nullptr;            // [n * B * K]
   float* wsum = nullptr;           // [n]
@@ -133,6 +133,7 @@ void launch_spatial_order(const Problem& p, const float* means, const float* sca
                           const float* opac, const Workspace& ws, cudaStream_t s);
 void launch_scatter(const Problem& p, int cb, const Workspace& ws, cudaStream_t s);
 void launch_tile_sort(const Problem& p, int cb, const Workspace& ws, cudaStream_t s);
+int sm_count();  // of the current device
 // sub_img (nullable, float32 [cb,H,W,K] of this pass's cameras): accumulate t - img instead of t
 // (refinement); forces the CUDA-core walk.
 bool launch_blend_refine(const Problem& p, int cb, int cam0, const void* targets, int dtype, const Workspace& ws,

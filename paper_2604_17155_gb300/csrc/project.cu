@@ -196,13 +196,14 @@ __device__ __forceinline__ int4 project_pair(const float4 mo, const float4 sq, c
 // CTA zeroes and flushes one histogram bin per tile, so large tile grids take more Gaussians a
 // thread, which spreads that per-CTA cost; smaller ones take fewer, which keeps more CTAs in flight.
 // Measured choices: the projection 8 / 32 and the scatter 4 / 16 Gaussians a thread below / from
-// 4,096 tiles, and fewer, down to one, while that leaves under kFullGrid CTAs (a thousand Gaussians on eight
+// 4,096 tiles, and fewer, down to one, while that leaves under kFullGrid CTAs an SM (a thousand Gaussians on eight
 // cameras were 8 CTAs, scatter 18.9 us; 50,000 on one camera of 6,700 tiles 7 CTAs, call 435 us against 188).
 constexpr int kBigTileGrid = 4096;
-constexpr int kFullGrid = 4 * 152;
+constexpr int kFullGrid = 4;
 inline int hist_chunk(int64_t n, int cb, int tiles, int small, int big) {
+  const int64_t full = kFullGrid * (int64_t)sm_count();
   int pt = tiles >= kBigTileGrid ? big : small;
-  while (pt > 1 && ((n + 256 * pt - 1) / (256 * pt)) * cb < kFullGrid) pt >>= 1;
+  while (pt > 1 && ((n + 256 * pt - 1) / (256 * pt)) * cb < full) pt >>= 1;
   return pt;
 }
 __host__ __device__ constexpr int hist_per_cta(int per_thread) { return 256 * per_thread; }
@@ -695,7 +696,7 @@ void launch_spatial_order(const Problem& p, const float* means, const float* sca
   cudaMemsetAsync(ws.cell_off, 0, sizeof(uint32_t) * (size_t)(kCells + 1), s);
   cudaMemsetAsync(ws.cell_cur, 0, sizeof(uint32_t) * (size_t)kCells, s);
   const unsigned grid = (unsigned)((p.n + 255) / 256);
-  k_bounds<<<std::min(grid, 152u * 8u), 256, 0, s>>>(means, p.n, ws.cell_box);
+  k_bounds<<<std::min(grid, (unsigned)sm_count() * 8u), 256, 0, s>>>(means, p.n, ws.cell_box);
   k_cell_count<<<grid, 256, 0, s>>>(means, p.n, ws.cell_box, ws.cell_off);
   const int nblocks = (kCells + kScanBlock - 1) / kScanBlock;
   k_scan_reduce<<<nblocks, kScanBlock, 0, s>>>(ws.cell_off, kCells, ws.cell_tmp);

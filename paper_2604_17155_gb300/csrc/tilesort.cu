@@ -244,14 +244,14 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort_queued(const uint32_t*
   }
 }
 
+}  // namespace
+
 int sm_count() {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return sms > 0 ? sms : 1;
 }
-
-}  // namespace
 
 // Orders every tile list of the pass: the warp-per-list kernel, then the queued lists. The queue
 // counters of the status block are zero (the scan of the pass's counts empties them).
