@@ -92,3 +92,51 @@ def test_few_depths_not_slower_than_by_radix_passes(icgs, n, kind, radix):
     t = _best_ms(icgs, off, lists(lambda r: _words(kind, r, n)))
     print(f"{n} {kind} {t:.3f} ms, spread {spread:.3f}")
     assert t <= radix * spread
+
+
+def _nested(rng, n):
+    """Keys of one depth and neighbouring indices, but for one far index, one near depth and one far depth: the whole
+    key's range is so wide that every split finds the others in one bin."""
+    words = np.full(n, 0x40000000, np.uint64)
+    idx = 1000 + np.arange(n, dtype=np.uint64)
+    idx[n // 2] = 1 << 30
+    words[n // 3] += 1000
+    words[n // 4] += 1 << 28
+    return rng.permutation((words << np.uint64(32)) | idx)
+
+
+def _splits_refuse(keys, nb):
+    """Whether the splits of a list of keys in nb bins leave it crowded: the rule of bucket.cuh's split_list."""
+    n = len(keys)
+    d, i = (keys >> np.uint64(32)).astype(object), (keys & np.uint64(0xFFFFFFFF)).astype(object)
+    irange = max(i) - min(i) + 1
+    z = (d - min(d)) * irange + (i - min(i))
+    shift = max(0, (max(z)).bit_length() - 32)
+    x, low = z >> shift, z & ((1 << shift) - 1)
+    at = x * nb // (max(x) + 1)
+    for _ in range(3):
+        order, s0, new = np.unique(at), 0, np.zeros(n, object)
+        for b in order:
+            m = at == b
+            c2 = 2 * int(m.sum())
+            lo, hi = min(x[m]), max(x[m])
+            new[m] = 2 * s0 + ((x[m] - lo) * c2 // (hi - lo + 1) if hi > lo else (low[m] * c2) >> shift)
+            s0 += int(m.sum())
+        at = new
+        counts = np.unique(at, return_counts=True)[1]
+        if int((counts * (counts - 1) // 2).sum()) <= 32 * n:
+            return False
+    return True
+
+
+@pytest.mark.parametrize("n,bins", [(300, 4096), (1000, 4096), (1024, 4096), (1025, 4096), (2048, 4096), (2049, 8192),
+                                    (4096, 8192)])
+def test_what_the_splits_refuse_is_radix_sorted(icgs, n, bins):
+    rng = np.random.default_rng(n)
+    lists = [_nested(rng, n) for _ in range(5)] + [_nested(rng, n)[: n - 1] for _ in range(2)]
+    assert all(_splits_refuse(k, bins) for k in lists[:1])
+    off = np.concatenate([[0], np.cumsum([len(k) for k in lists])]).astype(np.int32)
+    keys = torch.tensor(np.concatenate(lists).view(np.int64), device="cuda")
+    icgs.sort_tile_lists(torch.tensor(off, device="cuda"), keys)
+    for k, got in zip(lists, np.split(keys.cpu().numpy().view(np.uint64), off[1:-1])):
+        assert np.array_equal(got, np.sort(k)), f"list of {len(k)} keys"
