@@ -70,12 +70,12 @@ KERNEL_SOURCES = {
 }
 MEASURED_TRAFFIC = {
     # relight, 100 cameras: one full-size launch captured
-    ("relight", "cuda-core"): {"bytes_per_scene": 2146019072 + 288247040, "source_sha": "9100ec12c5109733"},
+    ("relight", "cuda-core"): {"bytes_per_scene": 2144985344 + 287600896, "source_sha": "d833f628b2caca1f"},
     # features: a 10-camera launch captured and scaled by 150/10 cameras (the targets, the per-camera
     # tile lists and the per-camera accumulator re-streaming all grow with the camera count)
-    ("features", "tensor-core"): {"bytes_per_scene": 15 * (3285384960 + 1462768384), "source_sha": "6027f9630ffe8186"},
+    ("features", "tensor-core"): {"bytes_per_scene": 15 * (3285265152 + 1462657024), "source_sha": "4e799cc0d1a983c3"},
     # segmentation masks: a 4-camera launch captured and scaled by 200/4 cameras (as above)
-    ("segmentation", "tensor-core"): {"bytes_per_scene": 50 * (1813298688 + 502618368), "source_sha": "6027f9630ffe8186"},
+    ("segmentation", "tensor-core"): {"bytes_per_scene": 50 * (1813474560 + 502768896), "source_sha": "4e799cc0d1a983c3"},
 }
 
 

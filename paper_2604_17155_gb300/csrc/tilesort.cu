@@ -12,8 +12,8 @@
 //
 // Latency of shared-memory atomics and loads bounds these kernels, so passes over the keys and warps
 // in flight count: with three or four radix passes a list, the sort of 1.1e9 keys in 1.3 million lists
-// (200 views of 1600 x 1060) took 16.5 ms, with one bucket pass 9.4 (its keys read and written once at
-// the copy rate: 2.6); 5.4e7 keys in 250,000 lists 0.88 -> 0.50 ms. Teams: lists of 1025..2048 keys
+// (200 views of 1600 x 1060) took 16.5 ms, with one bucket pass 9.6 (its keys read and written once at
+// the copy rate: 2.6); 5.4e7 keys in 250,000 lists 0.88 -> 0.51 ms. Teams: lists of 1025..2048 keys
 // by two warps with 32 keys a thread (159 registers, 12 warps an SM) gave 10.5 ms.
 #include <cuda_runtime.h>
 
