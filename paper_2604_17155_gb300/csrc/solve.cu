@@ -476,7 +476,6 @@ __device__ __forceinline__ void exact_fold(const float* __restrict__ acc, int64_
                                            bool gram, int k0, int K, float (&gh)[B], float (&gl)[B], float& wh,
                                            float& wl, float (&bh)[4], float (&bl)[4], float (*s_Y)[B + 1]) {
   const unsigned gm = group_mask();
-  const int gbase = threadIdx.x & ~(kGroup - 1);
   const bool row = r < B;
   for (int jb = 0; jb < n_cams; jb += kGroup) {
     const int jq = jb + r;
@@ -490,7 +489,7 @@ __device__ __forceinline__ void exact_fold(const float* __restrict__ acc, int64_
     }
     if (vq > 0.0f) {
       const float3 d = view_dir(mu, cams[jq]);
-      sh_basis<B>(d.x, d.y, d.z, s_Y[threadIdx.x]);
+      sh_basis<B>(d.x, d.y, d.z, s_Y[r]);
     }
     __syncwarp(gm);
     const int nj = min(kGroup, n_cams - jb);
@@ -500,7 +499,7 @@ __device__ __forceinline__ void exact_fold(const float* __restrict__ acc, int64_
 #pragma unroll
       for (int qq = 0; qq < 4; ++qq) sv[qq] = __shfl_sync(gm, sq[qq], q, kGroup);
       if (!(v > 0.0f)) continue;  // uniform in the group
-      const float* yq = s_Y[gbase + q];
+      const float* yq = s_Y[q];
       const float Yr = row ? yq[r] : 0.0f;
       if (gram) {
         const float vh = v * Yr, vl = fmaf(v, Yr, -vh);
@@ -542,13 +541,17 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
     float* __restrict__ coeffs, uint8_t* __restrict__ status_out, float* __restrict__ chol,
     DevStatus* status, const float* __restrict__ acc, int RS, int n_acc_cams,
     const DevCam* __restrict__ cams, const float* __restrict__ means) {
-  __shared__ float s_Y[MIXED ? kSolveThreads : 1][B + 1];  // per lane: basis of its camera (re-fold)
-  constexpr int NGr = kSolveThreads / kGroup, GF = gram_floats(B), R3 = solve_record_floats(B);
-  __shared__ float s_L[NGr * B * (B + 1)];  // per group: the rows of L
-  // Per group the fold's block of G (its hi, then its lo parts), read as it lies in memory, and the record
-  // before it is written out as it lies; s_pos[r][c] = the place of entry (r, c) in the block.
-  __shared__ __align__(16) float s_G[NGr][MIXED ? 2 : 1][GF];
-  __shared__ __align__(16) float s_rec[NGr][R3];
+  constexpr int NGr = kSolveThreads / kGroup, GF = gram_floats(B), R3 = solve_record_floats(B), P = R3 / 3;
+  // Per group, in turn: the fold's block of G (its hi, then its lo parts), read as it lies in memory; the bases of the
+  // re-fold's cameras, a row a lane; the rows of L; and the record (factor, then A) before it is written out as it
+  // lies. G and the record start at kOff: A's part lies behind the rows of L, the factor's takes their place. (Each on
+  // its own, 40 KB a CTA, left so little L1 that the FP64 solve's spills missed it: 400,000 Gaussians from 10 views
+  // at degree 3, 63,143 of them in FP64, 6.1 ms, and 5.5 so.)
+  constexpr int kL = ((MIXED ? kGroup : B) * (B + 1) + 3) / 4 * 4, kOff = (kL - P + 3) / 4 * 4;
+  constexpr int kG = MIXED ? 2 * GF : GF, kBuf = (kOff + (kG > R3 ? kG : R3) + 3) / 4 * 4;
+  static_assert(kL <= kOff + P && B * (B + 1) <= kL, "A's part behind the bases and the rows of L");
+  __shared__ __align__(16) float s_buf[NGr][kBuf];
+  // s_pos[r][c] = the place of entry (r, c) in the block of G
   __shared__ __align__(16) uint8_t s_pos[B][16];
   for (int e = threadIdx.x; e < B * B; e += kSolveThreads) s_pos[e / B][e % B] = (uint8_t)gram_pos(e / B, e % B, B);
   __syncthreads();
@@ -559,7 +562,6 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
   const bool row = r < B;
   float w = wsum[i];
   const float lam_r = row ? lam[r] : 0.0f;
-  constexpr int P = B * (B + 1) / 2;
   float* rec = chol ? chol + i * solve_record_floats(B) : nullptr;
   if (!(w > 0.0f)) {
     if (row)
@@ -573,8 +575,8 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
 #pragma unroll
   for (int e = 0; e < GF / 4; e += kGroup)
     if (e + r < GF / 4) {
-      reinterpret_cast<float4*>(s_G[grp][0])[e + r] = reinterpret_cast<const float4*>(G + i * GF)[e + r];
-      if (MIXED) reinterpret_cast<float4*>(s_G[grp][MIXED ? 1 : 0])[e + r] = reinterpret_cast<const float4*>(Glo + i * GF)[e + r];
+      reinterpret_cast<float4*>(s_buf[grp] + kOff)[e + r] = reinterpret_cast<const float4*>(G + i * GF)[e + r];
+      if (MIXED) reinterpret_cast<float4*>(s_buf[grp] + kOff + GF)[e + r] = reinterpret_cast<const float4*>(Glo + i * GF)[e + r];
     }
   __syncwarp(group_mask());
   uint32_t pos[4] = {0u, 0u, 0u, 0u};  // the places of this lane's row, a byte each
@@ -585,15 +587,19 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
     pos[2] = u.z;
     pos[3] = u.w;
   }
-  auto gram = [&](int part, int c) -> float { return row ? s_G[grp][part][(pos[c / 4] >> (8 * (c % 4))) & 0xFFu] : 0.0f; };
-  // writes the record out, once it is complete in s_rec
-  float* const rec_s = s_rec[grp];
-  auto write_record = [&]() {
+  float* const rec_s = s_buf[grp] + kOff;
+  float (*const s_Y)[B + 1] = reinterpret_cast<float (*)[B + 1]>(s_buf[grp]);
+  auto gram = [&](int part, int c) -> float {
+    return row ? rec_s[part * GF + ((pos[c / 4] >> (8 * (c % 4))) & 0xFFu)] : 0.0f;
+  };
+  // writes the record out from entry `from` (0 or P) on, once that is complete in rec_s
+  auto write_record = [&](int from) {
     __syncwarp(group_mask());
-    if (R3 % 4 == 0 && (reinterpret_cast<uintptr_t>(chol) & 15u) == 0) {
-      for (int e = r; e < R3 / 4; e += kGroup) reinterpret_cast<float4*>(rec)[e] = reinterpret_cast<const float4*>(rec_s)[e];
+    if (R3 % 4 == 0 && P % 4 == 0 && (reinterpret_cast<uintptr_t>(chol) & 15u) == 0) {
+      for (int e = from / 4 + r; e < R3 / 4; e += kGroup)
+        reinterpret_cast<float4*>(rec)[e] = reinterpret_cast<const float4*>(rec_s)[e];
     } else {
-      for (int e = r; e < R3; e += kGroup) rec[e] = rec_s[e];
+      for (int e = from + r; e < R3; e += kGroup) rec[e] = rec_s[e];
     }
   };
   float a[B];
@@ -602,6 +608,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
     a[c] = gram(0, c);
     if (c == r) a[c] += w * lam_r;
   }
+  if (!MIXED) __syncwarp(group_mask());  // G has been read
   if (!MIXED && rec && row) {  // PLAIN: A in FP32 (no compensation term)
 #pragma unroll
     for (int c = 0; c < B; ++c)
@@ -632,6 +639,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
 #pragma unroll
       for (int c = 0; c < B; ++c) { ghi[c] = 0.0f; glo[c] = 0.0f; }
       w = 0.0f;
+      __syncwarp(group_mask());  // G has been read
       exact_fold<B>(acc, cam_stride, i, RS, n_acc_cams, cams, mu, r, true, 0, K, ghi, glo, w, wl, rb_h, rb_l, s_Y);
 #pragma unroll
       for (int c = 0; c < B; ++c) {
@@ -649,6 +657,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
       }
     }
   }
+  if (MIXED) __syncwarp(group_mask());  // G has been read
   if (MIXED && rec && row) {  // A = (G_hi + G_lo) + (w_hi + w_lo) Lambda in float-float
 #pragma unroll
     for (int c = 0; c < B; ++c)
@@ -668,13 +677,16 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
     const float wl_r = w * lam_r;
     const float wl_lo = MIXED ? wl * lam_r : 0.0f;
     const int steps = refold ? kRefineStepsRefold : kRefineSteps;
-    float* s_Lg = s_L + (threadIdx.x / kGroup) * (B * (B + 1));
-    if (row) {
+    float* s_Lg = s_buf[grp];
+    auto store_L = [&]() {
+      if (row) {
 #pragma unroll
-      for (int c = 0; c < B; ++c)
-        if (c <= r) s_Lg[r * (B + 1) + c] = a[c];
-    }
-    __syncwarp(group_mask());
+        for (int c = 0; c < B; ++c)
+          if (c <= r) s_Lg[r * (B + 1) + c] = a[c];
+      }
+      __syncwarp(group_mask());
+    };
+    store_L();
     for (int k0 = 0; k0 < K; k0 += NR) {
       float bh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, bl[4] = {0.0f, 0.0f, 0.0f, 0.0f};
       if (refold && k0 == 0) {
@@ -682,8 +694,10 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
         for (int q = 0; q < NR; ++q) { bh[q] = rb_h[q]; bl[q] = rb_l[q]; }
       } else if (refold) {
         float gdummy[B], gldummy[B], wdummy = 0.0f, wldummy = 0.0f;
+        __syncwarp(group_mask());  // L has been read
         exact_fold<B>(acc, cam_stride, i, RS, n_acc_cams, cams, mu, r, false, k0, K, gdummy, gldummy, wdummy,
                       wldummy, bh, bl, s_Y);
+        store_L();  // where the bases were
       } else {
 #pragma unroll
         for (int q = 0; q < NR; ++q)
@@ -715,17 +729,19 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
       for (int q = 0; q < NR; ++q)
         if (row && k0 + q < K) coeffs[(i * B + r) * K + k0 + q] = x[q];
     }
+    __syncwarp(group_mask());  // L has been read
     if (rec) {
 #pragma unroll
       for (int c = 0; c < B; ++c)
         if (row && c <= r) rec_s[r * (r + 1) / 2 + c] = a[c];
-      write_record();
+      write_record(0);
     }
     if (r == 0 && status_out) status_out[i] = kGaussOk;
     return;
   }
   // FP64 from (G_hi + G_lo, b_hi + b_lo): the exact re-fold when it ran, else the fold's
   // compensated sums
+  if (rec) write_record(P);  // A; the factor leaves from the registers, so that nothing of the record is held meanwhile
   double ad[B];
   const double wd = (double)w + (double)wl;
 #pragma unroll
@@ -759,11 +775,10 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(
       if (row) coeffs[(i * B + r) * K + k0 + q] = (float)x;
     }
   }
-  if (rec) {
+  if (chol && row) {
 #pragma unroll
     for (int c = 0; c < B; ++c)
-      if (row && c <= r) rec_s[r * (r + 1) / 2 + c] = (float)ad[c];
-    write_record();
+      if (c <= r) chol[i * R3 + r * (r + 1) / 2 + c] = (float)ad[c];
   }
   if (r == 0) {
     if (status_out) status_out[i] = kGaussFp64;
